@@ -154,7 +154,7 @@ int tsd_build_branch_mask(const tsd_layout* layout, const uint64_t* vis, const i
  *              bytes (may be 0, then NULL is accepted).
  *   flags      TSD_ATTN_* bits.
  * The tensor-core kernel (tcgen05 MMAs with TMEM accumulators, TMA-staged
- * tiles) serves bf16 with head_dim 128; other combinations run on CUDA cores.
+ * tiles) serves bf16; fp32 runs on CUDA cores.
  * ------------------------------------------------------------------------- */
 size_t tsd_verify_attention_workspace_bytes(const tsd_layout* layout);
 int tsd_verify_attention(const tsd_layout* layout, const void* mask,

@@ -1,5 +1,5 @@
 // Stage 1b entry point: argument checks and the choice between the tensor-core kernel
-// (bf16, head_dim 128) and the CUDA-core kernel (everything else).
+// (bf16) and the CUDA-core kernel (fp32, and whatever the tensor maps cannot express).
 #include "tsd_common.cuh"
 
 namespace tsd {

@@ -1,5 +1,5 @@
 // Stage 1b on CUDA cores: masked verify attention (paper Section 3.3) for the combinations the
-// tensor-core kernel does not serve (fp32 inputs, head_dim 64) and as a cross-check for it.
+// tensor-core kernel does not serve (fp32 inputs) and as a cross-check for it.
 //
 // One thread block per (sequence, query head, branch).  A warp owns a query row at a time; its
 // lanes stride over the visible keys (the cached tokens, then the rows of every visible draft

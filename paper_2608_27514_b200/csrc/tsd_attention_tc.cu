@@ -1,4 +1,4 @@
-// Stage 1b on tensor cores: masked verify attention (paper Section 3.3) for bf16, head_dim 128.
+// Stage 1b on tensor cores: masked verify attention (paper Section 3.3) for bf16, head_dim 128 or 64.
 //
 // Persistent kernel, one thread block of 20 warps per SM.  A work item is (sequence, query head,
 // tile of 128 draft rows = 128/R branches); a block takes items blockIdx.x, blockIdx.x + gridDim.x,
@@ -63,22 +63,39 @@ constexpr int kNP = 2;                         // P buffers in tensor memory
 constexpr int kKeys = 64;                      // keys per tile
 constexpr int kMaxItems = 512;                 // work items of one block (their tile counts sit in shared memory)
 constexpr uint32_t kSub = 16384;               // bytes of one [128 rows x 64 elements] bf16 sub-tile
-constexpr uint32_t kTileBytes = 2 * kSub;      // a [128 x 128] bf16 tile
 constexpr uint32_t kSubKV = 8192;              // bytes of one [64 keys x 64 elements] bf16 sub-tile
-constexpr uint32_t kKVBytes = 2 * kSubKV;      // a [64 x 128] bf16 K or V tile
-constexpr uint32_t kOffQ = 0;                  // Q staging (TMA destination, copied to tensor memory)
-constexpr uint32_t kOffO = kTileBytes;         // O staging (TMA store source)
-constexpr uint32_t kOffK = 2 * kTileBytes;
-constexpr uint32_t kOffV = kOffK + kNK * kKVBytes;
-constexpr uint32_t kOffBar = kOffV + kNV * kKVBytes;
-constexpr uint32_t kOffMref = kOffBar + 512;   // exponent offset per row (128 floats)
-// partial row sums and the exponent offsets they are on, per softmax warpgroup, for three items in
-// rotation (3 x 3 x 128 floats each): a softmax warpgroup leaves them for the epilogue and moves on
-constexpr uint32_t kOffLpart = kOffMref + 512;
-constexpr uint32_t kOffMpart = kOffLpart + 3 * 3 * 128 * 4;
-constexpr uint32_t kOffItems = kOffMpart + 3 * 3 * 128 * 4;  // key tiles / cache length per item (2 x kMaxItems int32)
-constexpr uint32_t kSmemBytes = kOffItems + 2 * kMaxItems * 4 + 1024;  // + slack to align the base to 1 KB
-constexpr uint32_t kColO = 0, kColQ = 128, kColS = 256, kColP = 448;  // tensor-memory columns
+// Shared-memory layout for a head_dim of D = 64 or 128 (one sub-tile per 64 elements of head_dim).
+template <int D>
+struct TcSmem {
+  static constexpr uint32_t kTileBytes = D / 64 * kSub;   // a [128 x D] bf16 tile
+  static constexpr uint32_t kKVBytes = D / 64 * kSubKV;   // a [64 x D] bf16 K or V tile
+  static constexpr uint32_t kOffQ = 0;                    // Q staging (TMA destination, copied to tensor memory)
+  static constexpr uint32_t kOffO = kTileBytes;           // O staging (TMA store source)
+  static constexpr uint32_t kOffK = 2 * kTileBytes;
+  static constexpr uint32_t kOffV = kOffK + kNK * kKVBytes;
+  static constexpr uint32_t kOffBar = kOffV + kNV * kKVBytes;
+  static constexpr uint32_t kOffMref = kOffBar + 512;     // exponent offset per row (128 floats)
+  // partial row sums and the exponent offsets they are on, per softmax warpgroup, for three items in
+  // rotation (3 x 3 x 128 floats each): a softmax warpgroup leaves them for the epilogue and moves on
+  static constexpr uint32_t kOffLpart = kOffMref + 512;
+  static constexpr uint32_t kOffMpart = kOffLpart + 3 * 3 * 128 * 4;
+  static constexpr uint32_t kOffItems = kOffMpart + 3 * 3 * 128 * 4;  // key tiles / cache length per item (2 x kMaxItems int32)
+  static constexpr uint32_t kBytes = kOffItems + 2 * kMaxItems * 4 + 1024;  // + slack to align the base to 1 KB
+};
+// Tensor-memory columns.  At head_dim 128 everything is in use and P is one bf16 per score.  At head_dim 64
+// the tensor pipe has twice the time it needs (256 of the 512 clocks that a tile's exponentials take) and half
+// of O and Q is free, so P is kept as the sum of two bf16 (high part, residual: 2^-17 relative) and P V issues
+// one MMA more per 16 keys: outputs then carry no rounding but their own, as from fp32 weights.
+// (4 sequences x 16 branches x 32 rows, 32/8 heads, 1472 cached keys: 67.9 us; on CUDA cores, where this head
+// size ran before: 5.96 ms.)
+template <int D>
+struct TcCols {
+  static constexpr bool kSplitP = D == 64;
+  static constexpr uint32_t kPCols = kSplitP ? kKeys : kKeys / 2;   // columns of one P buffer
+  static constexpr uint32_t kO = 0, kQ = D, kQStride = D / 2;       // O, then two Q buffers
+  static constexpr uint32_t kS = 2 * D, kP = kS + kNSb * kKeys;     // three S buffers, two P buffers
+  static_assert(kP + kNP * kPCols <= 512, "tensor memory has 512 columns");
+};
 constexpr uint32_t kSpinLimit = 1u << 21;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -209,13 +226,9 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ float ex2f(float x) {
-#ifdef TSD_EXPERIMENT_NO_EX2  /* timing experiment only: wrong results */
-  return x;
-#else
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-#endif
 }
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   uint32_t r;
@@ -251,34 +264,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-// 2^t for a pair, t in [-126, 16], on the FMA pipe: t = n + f with n = round(t), f in [-0.5, 0.5];
-// 2^f by a degree-3 polynomial (relative error 7.5e-5, well below the bf16 rounding of P), and n
-// added into the exponent field.  Takes load off the 16-per-clock special-function unit.
-__device__ __forceinline__ void exp2_poly2(uint64_t t2, float& p0, float& p1) {
-  float t0, t1;
-  unpack2(t2, t0, t1);
-  t2 = pack2f(fmaxf(t0, -126.f), fmaxf(t1, -126.f));
-  const uint64_t magic = pack2f(12582912.f, 12582912.f);          // 1.5 * 2^23: rounds to an integer
-  const uint64_t y = add2(t2, magic);
-  const uint64_t n = add2(y, pack2f(-12582912.f, -12582912.f));
-  const uint64_t f = fma2(n, pack2f(-1.f, -1.f), t2);
-  uint64_t r = fma2(f, pack2f(0.05517165f, 0.05517165f), pack2f(0.24261113f, 0.24261113f));
-  r = fma2(r, f, pack2f(0.69326097f, 0.69326097f));
-  r = fma2(r, f, pack2f(0.99992806f, 0.99992806f));
-  float y0, y1, r0, r1;
-  unpack2(y, y0, y1);
-  unpack2(r, r0, r1);
-  p0 = __uint_as_float(__float_as_uint(r0) + (__float_as_uint(y0) << 23));
-  p1 = __uint_as_float(__float_as_uint(r1) + (__float_as_uint(y1) << 23));
-}
-#ifndef TSD_SM_SLEEP
-#define TSD_SM_SLEEP 0
-#endif
-#ifndef TSD_POLY_OF8
-#define TSD_POLY_OF8 0
-#endif
-constexpr int kPolyOf8 = TSD_POLY_OF8;  // of every 8 score pairs, this many take the polynomial exp2 (unmasked tiles)
-
 // Shared-memory matrix descriptor, 128-byte swizzle (descriptor version 1 = this architecture).
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
   return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16) |
@@ -331,62 +316,67 @@ struct TcParams {
 // descriptor) is a gap in which the tensor pipe may run dry.  Descriptors are passed as their low
 // words (the address field varies, the high word is the same for all of one operand).
 //
-// One Q K^T: 8 MMAs (K = 16 over head_dim) into the S buffer at tensor-memory address `s_tmem`, Q
+// One Q K^T: D / 16 MMAs (K = 16 over head_dim) into the S buffer at tensor-memory address `s_tmem`, Q
 // from tensor memory at `q_tmem`, K through the descriptors (lo[kk], hi); then the two commits.
+#define TSD_QK_FIRST(lo)                                                            \
+  "mov.b64 dsc, {" lo ", %2};\n"                                                    \
+  "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], dsc, %3, pf;\n"
+#define TSD_QK_NEXT(col, lo)                                                        \
+  "add.u32 a, %1, " col ";\nmov.b64 dsc, {" lo ", %2};\n"                           \
+  "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %3, pt;\n"
+#define TSD_QK_BEGIN "{\n.reg .pred pf, pt;\n.reg .b32 a;\n.reg .b64 dsc;\nsetp.ne.b32 pf, 0, 0;\nsetp.eq.b32 pt, 0, 0;\n"
+#define TSD_QK_END                                                                  \
+  "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%4];\n"   \
+  "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n}"
 __device__ __forceinline__ void issue_qk_mmas(uint32_t s_tmem, uint32_t q_tmem, const uint32_t (&lo)[8], uint32_t hi,
                                               uint32_t s_full, uint32_t k_free) {
   constexpr uint32_t idesc_qk = instr_desc(kKeys, 0);
-  asm volatile(
-      "{\n.reg .pred pf, pt;\n.reg .b32 a;\n.reg .b64 dsc;\n"
-      "setp.ne.b32 pf, 0, 0;\nsetp.eq.b32 pt, 0, 0;\n"
-      "mov.b64 dsc, {%2, %10};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], dsc, %11, pf;\n"
-      "add.u32 a, %1, 8;\nmov.b64 dsc, {%3, %10};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %11, pt;\n"
-      "add.u32 a, %1, 16;\nmov.b64 dsc, {%4, %10};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %11, pt;\n"
-      "add.u32 a, %1, 24;\nmov.b64 dsc, {%5, %10};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %11, pt;\n"
-      "add.u32 a, %1, 32;\nmov.b64 dsc, {%6, %10};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %11, pt;\n"
-      "add.u32 a, %1, 40;\nmov.b64 dsc, {%7, %10};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %11, pt;\n"
-      "add.u32 a, %1, 48;\nmov.b64 dsc, {%8, %10};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %11, pt;\n"
-      "add.u32 a, %1, 56;\nmov.b64 dsc, {%9, %10};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %11, pt;\n"
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%12];\n"
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%13];\n}"
-      ::"r"(s_tmem), "r"(q_tmem), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]), "r"(lo[4]), "r"(lo[5]), "r"(lo[6]),
-        "r"(lo[7]), "r"(hi), "r"(idesc_qk), "r"(s_full), "r"(k_free) : "memory");
+  asm volatile(TSD_QK_BEGIN TSD_QK_FIRST("%6") TSD_QK_NEXT("8", "%7") TSD_QK_NEXT("16", "%8") TSD_QK_NEXT("24", "%9")
+               TSD_QK_NEXT("32", "%10") TSD_QK_NEXT("40", "%11") TSD_QK_NEXT("48", "%12") TSD_QK_NEXT("56", "%13") TSD_QK_END
+      ::"r"(s_tmem), "r"(q_tmem), "r"(hi), "r"(idesc_qk), "r"(s_full), "r"(k_free), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]),
+        "r"(lo[3]), "r"(lo[4]), "r"(lo[5]), "r"(lo[6]), "r"(lo[7]) : "memory");
+}
+__device__ __forceinline__ void issue_qk_mmas(uint32_t s_tmem, uint32_t q_tmem, const uint32_t (&lo)[4], uint32_t hi,
+                                              uint32_t s_full, uint32_t k_free) {
+  constexpr uint32_t idesc_qk = instr_desc(kKeys, 0);
+  asm volatile(TSD_QK_BEGIN TSD_QK_FIRST("%6") TSD_QK_NEXT("8", "%7") TSD_QK_NEXT("16", "%8") TSD_QK_NEXT("24", "%9") TSD_QK_END
+      ::"r"(s_tmem), "r"(q_tmem), "r"(hi), "r"(idesc_qk), "r"(s_full), "r"(k_free), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]),
+        "r"(lo[3]) : "memory");
 }
 // One P V: 4 MMAs (16 keys = 8 packed columns of P each), P from tensor memory at `p_tmem`, V through
 // the descriptors (lo[kk], hi), into O at `o_tmem`; `acc` = 0 starts a new accumulation; then the commit.
+// With P in two parts (head_dim 64) four more MMAs add the residuals, 32 columns further on.
+#define TSD_PV_NEXT(col, lo)                                                        \
+  "add.u32 a, %1, " col ";\nmov.b64 dsc, {" lo ", %2};\n"                           \
+  "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %3, pt;\n"
+#define TSD_PV_BEGIN                                                                \
+  "{\n.reg .pred pa, pt;\n.reg .b32 a;\n.reg .b64 dsc;\n"                           \
+  "setp.ne.b32 pa, %4, 0;\nsetp.eq.b32 pt, 0, 0;\n"                                 \
+  "mov.b64 dsc, {%6, %2};\n"                                                        \
+  "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], dsc, %3, pa;\n"                   \
+  TSD_PV_NEXT("8", "%7") TSD_PV_NEXT("16", "%8") TSD_PV_NEXT("24", "%9")
+#define TSD_PV_END "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n}"
+template <int D>
 __device__ __forceinline__ void issue_pv_mmas(uint32_t o_tmem, uint32_t p_tmem, const uint32_t (&lo)[kKeys / 16], uint32_t hi,
                                               uint32_t acc, uint32_t pv_done) {
-  constexpr uint32_t idesc_pv = instr_desc(128, 1);
-  asm volatile(
-      "{\n.reg .pred pa, pt;\n.reg .b32 a;\n.reg .b64 dsc;\n"
-      "setp.ne.b32 pa, %7, 0;\nsetp.eq.b32 pt, 0, 0;\n"
-      "mov.b64 dsc, {%2, %6};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], dsc, %8, pa;\n"
-      "add.u32 a, %1, 8;\nmov.b64 dsc, {%3, %6};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %8, pt;\n"
-      "add.u32 a, %1, 16;\nmov.b64 dsc, {%4, %6};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %8, pt;\n"
-      "add.u32 a, %1, 24;\nmov.b64 dsc, {%5, %6};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], dsc, %8, pt;\n"
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%9];\n}"
-      ::"r"(o_tmem), "r"(p_tmem), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]), "r"(hi), "r"(acc), "r"(idesc_pv),
-        "r"(pv_done) : "memory");
+  constexpr uint32_t idesc_pv = instr_desc(D, 1);
+  if (TcCols<D>::kSplitP)
+    asm volatile(TSD_PV_BEGIN TSD_PV_NEXT("32", "%6") TSD_PV_NEXT("40", "%7") TSD_PV_NEXT("48", "%8") TSD_PV_NEXT("56", "%9") TSD_PV_END
+        ::"r"(o_tmem), "r"(p_tmem), "r"(hi), "r"(idesc_pv), "r"(acc), "r"(pv_done), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]),
+          "r"(lo[3]) : "memory");
+  else
+    asm volatile(TSD_PV_BEGIN TSD_PV_END
+        ::"r"(o_tmem), "r"(p_tmem), "r"(hi), "r"(idesc_pv), "r"(acc), "r"(pv_done), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]),
+          "r"(lo[3]) : "memory");
 }
 
 // Rarely executed pieces of the softmax warps, kept out of line so that the loop over the key
 // tiles stays small in the instruction cache.
-// One row of O (128 fp32 columns of this thread's tensor-memory lane) times alpha.
+// One row of O (D fp32 columns of this thread's tensor-memory lane) times alpha.
+template <int D>
 __device__ __noinline__ void rescale_o_row(uint32_t t_o, float alpha) {
 #pragma unroll 1
-  for (int q4 = 0; q4 < 4; ++q4) {
+  for (int q4 = 0; q4 < D / 32; ++q4) {
     uint32_t ov[32];
     TSD_TMEM_LD32(ov, 0, t_o + q4 * 32);
     tmem_wait_ld();
@@ -396,11 +386,12 @@ __device__ __noinline__ void rescale_o_row(uint32_t t_o, float alpha) {
   }
 }
 // One row of Q: staging buffer (128-byte swizzle: 16-byte chunk c of row r sits at chunk c ^ (r & 7),
-// one sub-tile per half of head_dim) -> 64 columns of this thread's tensor-memory lane, as the A
+// one sub-tile per 64 elements of head_dim) -> D / 2 columns of this thread's tensor-memory lane, as the A
 // operand of Q K^T (32-bit column i = elements 2i, 2i+1).
+template <int D>
 __device__ __noinline__ void copy_q_row(uint32_t q_smem, int r, uint32_t t_q) {
 #pragma unroll 1
-  for (int sub = 0; sub < 2; ++sub) {
+  for (int sub = 0; sub < D / 64; ++sub) {
     uint32_t w[32];
 #pragma unroll
     for (int ch = 0; ch < 8; ++ch) {
@@ -413,21 +404,26 @@ __device__ __noinline__ void copy_q_row(uint32_t q_smem, int r, uint32_t t_q) {
   tmem_wait_st();
 }
 
+template <int D>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kc,
                     const __grid_constant__ CUtensorMap map_vc, const __grid_constant__ CUtensorMap map_kd,
                     const __grid_constant__ CUtensorMap map_vd, const __grid_constant__ CUtensorMap map_o,
                     const TcParams p) {
+  using L = TcSmem<D>;
+  using C = TcCols<D>;
+  constexpr uint32_t kTileBytes = L::kTileBytes, kKVBytes = L::kKVBytes;
+  constexpr uint32_t kOffQ = L::kOffQ, kOffO = L::kOffO, kOffK = L::kOffK, kOffV = L::kOffV, kOffBar = L::kOffBar;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t bars = base + kOffBar;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + kOffBar + 448);
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(base_ptr + kOffBar + 452);
-  float* mref = reinterpret_cast<float*>(base_ptr + kOffMref);
-  float* lpart = reinterpret_cast<float*>(base_ptr + kOffLpart);
-  float* mpart = reinterpret_cast<float*>(base_ptr + kOffMpart);
-  int32_t* item_T = reinterpret_cast<int32_t*>(base_ptr + kOffItems);
+  float* mref = reinterpret_cast<float*>(base_ptr + L::kOffMref);
+  float* lpart = reinterpret_cast<float*>(base_ptr + L::kOffLpart);
+  float* mpart = reinterpret_cast<float*>(base_ptr + L::kOffMpart);
+  int32_t* item_T = reinterpret_cast<int32_t*>(base_ptr + L::kOffItems);
   int32_t* item_clen = item_T + kMaxItems;
   auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
 
@@ -503,7 +499,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       item_coords(0, s, h, qt);
       mbar_expect_tx(bar(QS_FULL), kTileBytes);
       tma_load_4d(base + kOffQ, &map_q, bar(QS_FULL), 0, h, qt * kTile, s);
-      tma_load_4d(base + kOffQ + kSub, &map_q, bar(QS_FULL), 64, h, qt * kTile, s);
+      if (D == 128) tma_load_4d(base + kOffQ + kSub, &map_q, bar(QS_FULL), 64, h, qt * kTile, s);
     }
   }
   if (warp == kQkWarp) {  // the whole tensor memory of the SM: O, 2 x Q, 3 x S, 2 x P
@@ -547,7 +543,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         item_coords(x, s, h, qt);
         mbar_expect_tx(bar(QS_FULL), kTileBytes);
         tma_load_4d(base + kOffQ, &map_q, bar(QS_FULL), 0, h, qt * kTile, s);
-        tma_load_4d(base + kOffQ + kSub, &map_q, bar(QS_FULL), 64, h, qt * kTile, s);
+        if (D == 128) tma_load_4d(base + kOffQ + kSub, &map_q, bar(QS_FULL), 64, h, qt * kTile, s);
         q_issued = x + 1;
       };
       const CUtensorMap* mc = is_k ? &map_kc : &map_vc;
@@ -567,7 +563,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         mbar_expect_tx(full_bar, kKVBytes);
         if (is_k && t < kNSb) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], 4;" ::"r"(full_bar) : "memory");
         tma_load_4d(dst, mc, full_bar, 0, g_first, t * kKeys, s_first);
-        tma_load_4d(dst + kSubKV, mc, full_bar, 64, g_first, t * kKeys, s_first);
+        if (D == 128) tma_load_4d(dst + kSubKV, mc, full_bar, 64, g_first, t * kKeys, s_first);
       }
       issued = n_pre;
       for (int it = 0; it < n_run && ok; ++it) {
@@ -593,7 +589,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             // no softmax has run before the first three tiles: their S buffers are free from the start
             if (is_k && G < kNSb) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], 4;" ::"r"(full_bar) : "memory");
             tma_load_4d(dst, m, full_bar, 0, g, row, s);
-            tma_load_4d(dst + kSubKV, m, full_bar, 64, g, row, s);
+            if (D == 128) tma_load_4d(dst + kSubKV, m, full_bar, 64, g, row, s);
             issued = G + 1;
           }
           TSD_TR(is_k ? 0 : 1, G);
@@ -628,15 +624,15 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       long long acc_a = 0, acc_c = 0;
       int sb = 0, kb = 0;   // S buffer of tile G = G mod 3, K stage = G mod 5
       uint32_t kph = 0;     // (G / 5) & 1
-      uint32_t kd_lo[8];  // low words of the descriptors of K stage 0; the others differ in the address field only
+      uint32_t kd_lo[D / 16];  // low words of the descriptors of K stage 0; the others differ in the address field only
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk)
+      for (int kk = 0; kk < D / 16; ++kk)
         kd_lo[kk] = (uint32_t)smem_desc(ubase + kOffK + (kk >> 2) * kSubKV + (kk & 3) * 32, 16, 1024);
       const uint32_t kd_hi = (uint32_t)(smem_desc(0, 16, 1024) >> 32);
       bool ready = false;  // the barrier of the tile at hand was seen complete by the early test
       for (int it = 0; it < n_run && ok; ++it) {
         const int T = __shfl_sync(0xffffffffu, item_T[it], 0);
-        const uint32_t q_tmem = utmem + kColQ + (uint32_t)(it & 1) * 64u;
+        const uint32_t q_tmem = utmem + C::kQ + (uint32_t)(it & 1) * C::kQStride;
         ok = mbar_wait(bar(QT_READY + (it & 1)), (it >> 1) & 1, abort_flag);
         for (int j = 0; j < T; ++j, ++G) {
           if (lane == 0) TSD_TR(2, G);
@@ -654,10 +650,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           const bool seen = mbar_test_wait(bar(QK_GO + kb1), kph1);  // used after the MMAs
           if (elect_one()) {
             const uint32_t k_off = (uint32_t)kb * (kKVBytes >> 4);
-            uint32_t lo[8];
+            uint32_t lo[D / 16];
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) lo[kk] = kd_lo[kk] + k_off;
-            issue_qk_mmas(utmem + kColS + (uint32_t)sb * kKeys, q_tmem, lo, kd_hi, bar(S_FULL + sb), bar(K_FREE + kb));
+            for (int kk = 0; kk < D / 16; ++kk) lo[kk] = kd_lo[kk] + k_off;
+            issue_qk_mmas(utmem + C::kS + (uint32_t)sb * kKeys, q_tmem, lo, kd_hi, bar(S_FULL + sb), bar(K_FREE + kb));
           }
           __syncwarp();
           ready = seen;
@@ -718,9 +714,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             if (z0 < z1 || dead) {
               const uint32_t v_stage = base + kOffV + (uint32_t)b * kKVBytes;
               if (dead) { z0 = (dead & 1u) ? 0 : 32; z1 = (dead & 2u) ? kKeys : 32; }
-              // 16 chunks of 16 bytes per row (8 per sub-tile): whole rows, so the swizzle does not matter
-              for (int idx = lane; idx < (z1 - z0) * 16; idx += 32) {
-                const int row = z0 + (idx >> 4), ch = idx & 15;
+              // D / 8 chunks of 16 bytes per row (8 per sub-tile): whole rows, so the swizzle does not matter
+              for (int idx = lane; idx < (z1 - z0) * (D / 8); idx += 32) {
+                const int row = z0 + idx / (D / 8), ch = idx % (D / 8);
                 const uint32_t a = v_stage + (uint32_t)(ch >> 3) * kSubKV + (uint32_t)row * 128u + (uint32_t)(ch & 7) * 16u;
                 asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(a), "r"(0u) : "memory");
               }
@@ -737,7 +733,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             uint32_t lo[kKeys / 16];
 #pragma unroll
             for (int kk = 0; kk < kKeys / 16; ++kk) lo[kk] = vd_lo[kk] + v_off;
-            issue_pv_mmas(utmem + kColO, utmem + kColP + (uint32_t)(b & 1) * 32u, lo, vd_hi, j == 0 ? 0u : 1u, bar(PV_DONE + b));
+            issue_pv_mmas<D>(utmem + C::kO, utmem + C::kP + (uint32_t)(b & 1) * C::kPCols, lo, vd_hi, j == 0 ? 0u : 1u, bar(PV_DONE + b));
           }
           __syncwarp();
           ready = seen;
@@ -766,7 +762,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       ok = ok && mbar_wait(bar(QS_FULL), it & 1, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) return;
-      copy_q_row(base + kOffQ, r, t_lane + kColQ + (uint32_t)(it & 1) * 64u);
+      copy_q_row<D>(base + kOffQ, r, t_lane + C::kQ + (uint32_t)(it & 1) * C::kQStride);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(QT_READY + (it & 1)));
@@ -792,7 +788,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         const int Gj = G + j, pb = Gj & 1;
         const uint32_t ph = (uint32_t)n_done & 1u;
         if (wq == 0 && lane == 0) TSD_TR(9, Gj);
-        ok = ok && mbar_wait(bar(S_FULL + wg), ph, abort_flag, TSD_SM_SLEEP);
+        ok = ok && mbar_wait(bar(S_FULL + wg), ph, abort_flag);
         ok = __all_sync(0xffffffffu, ok);  // leave the loop as a whole warp
         if (!ok) break;
         tc_fence_after();
@@ -800,7 +796,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         // S of a tile of this item is complete, so every Q K^T of the previous item is, and the Q
         // buffer they read can take Q of the next item
         if (j == jc && it + 1 < n_run) { copy_q(it + 1); if (!ok) break; }
-        const uint32_t t_s = t_lane + kColS + wg * kKeys;
+        const uint32_t t_s = t_lane + C::kS + wg * kKeys;
         uint32_t sv[kKeys];
         TSD_TMEM_LD32(sv, 0, t_s);
         TSD_TMEM_LD32(sv, 32, t_s + 32);
@@ -839,11 +835,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 #pragma unroll
         for (int i = 0; i < kKeys / 2; ++i)
           mx4[i & 3] = max3(mx4[i & 3], __uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1]));
-#ifdef TSD_EXPERIMENT_NO_MAX  /* timing experiment only: wrong results */
-        const float mx = __uint_as_float(sv[0]);
-#else
         const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-#endif
 
         // the row's exponent offset: the decision of the previous tile, moved only when this tile's
         // maximum exceeds it by more than 2^8 (always for the first finite maximum)
@@ -872,31 +864,19 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         const float off = (m_use == -CUDART_INF_F) ? 0.f : -m_use;
         const uint64_t c2 = pack2f(c, c), off2 = pack2f(off, off);
         uint64_t rs4[4] = {0ull, 0ull, 0ull, 0ull};
-        uint32_t pk[kKeys / 2];
-        if (masked || kPolyOf8 == 0) {  // every exponential on the special-function unit: 2^(-inf) is exactly 0
+        uint32_t pk[kKeys / 2], pl[kKeys / 2];  // P, and its residuals where it is kept in two parts
 #pragma unroll
-          for (int i = 0; i < kKeys / 2; ++i) {
-            float t0, t1;
-            unpack2(fma2(pack2(sv[2 * i], sv[2 * i + 1]), c2, off2), t0, t1);
-            const float p0 = ex2f(t0), p1 = ex2f(t1);
-            rs4[i & 3] = add2(rs4[i & 3], pack2f(p0, p1));
-            pk[i] = pack_bf16x2(p0, p1);
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < kKeys / 2; ++i) {
-            const uint64_t t2 = fma2(pack2(sv[2 * i], sv[2 * i + 1]), c2, off2);
-            float p0, p1;
-            if ((i & 7) < kPolyOf8) {
-              exp2_poly2(t2, p0, p1);
-            } else {
-              float t0, t1;
-              unpack2(t2, t0, t1);
-              p0 = ex2f(t0);
-              p1 = ex2f(t1);
-            }
-            rs4[i & 3] = add2(rs4[i & 3], pack2f(p0, p1));
-            pk[i] = pack_bf16x2(p0, p1);
+        for (int i = 0; i < kKeys / 2; ++i) {  // 2^(-inf) is exactly 0
+          float t0, t1;
+          unpack2(fma2(pack2(sv[2 * i], sv[2 * i + 1]), c2, off2), t0, t1);
+          const float p0 = ex2f(t0), p1 = ex2f(t1);
+          const uint64_t pp = pack2f(p0, p1);
+          rs4[i & 3] = add2(rs4[i & 3], pp);
+          pk[i] = pack_bf16x2(p0, p1);
+          if (C::kSplitP) {
+            float l0, l1;
+            unpack2(fma2(pack2(pk[i] << 16, pk[i] & 0xffff0000u), pack2f(-1.f, -1.f), pp), l0, l1);
+            pl[i] = pack_bf16x2(l0, l1);
           }
         }
         float r0, r1;
@@ -911,7 +891,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
-          rescale_o_row(t_lane + kColO, alpha);
+          rescale_o_row<D>(t_lane + C::kO, alpha);
         }
         // P (bf16 pairs) into P buffer pb, free once the P V of tile t-2 has completed:
         // column i = keys 2i (low half), 2i+1
@@ -921,7 +901,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           if (!ok) break;
           tc_fence_after();
         }
-        TSD_TMEM_ST32(pk, 0, t_lane + kColP + pb * 32);
+        TSD_TMEM_ST32(pk, 0, t_lane + C::kP + pb * C::kPCols);
+        if (C::kSplitP) TSD_TMEM_ST32(pl, 0, t_lane + C::kP + pb * C::kPCols + kKeys / 2);
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -981,14 +962,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       tc_fence_after();
       if (tid == kFirstEpilogueWarp * 32) TSD_TR(1, 255 - it);
       // staging layout = the output tensor map's: 128-byte swizzle, 16-byte chunk c of row r sits at
-      // chunk c ^ (r & 7); one sub-tile per half of head_dim; rows past the end of the tensor are
+      // chunk c ^ (r & 7); one sub-tile per 64 elements of head_dim; rows past the end of the tensor are
       // clipped by the copy engine
 #pragma unroll
-      for (int q4 = 0; q4 < 4; ++q4) {
+      for (int q4 = 0; q4 < D / 32; ++q4) {
         uint32_t ov[32];
-        TSD_TMEM_LD32(ov, 0, t_lane + kColO + q4 * 32);
+        TSD_TMEM_LD32(ov, 0, t_lane + C::kO + q4 * 32);
         tmem_wait_ld();
-        if (q4 == 3) {
+        if (q4 == D / 32 - 1) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(O_FREE));
@@ -1018,7 +999,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         ok = __all_sync(0xffffffffu, ok);
         if (ok && lane == 0) {
           tma_store_4d(&map_o, base + kOffO, 0, h, qt * kTile, s);
-          tma_store_4d(&map_o, base + kOffO + kSub, 64, h, qt * kTile, s);
+          if (D == 128) tma_store_4d(&map_o, base + kOffO + kSub, 64, h, qt * kTile, s);
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           TSD_TR(4, 255 - it);
         }
@@ -1079,12 +1060,12 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// [S, rows, H, 128] bf16 with element strides (sb, sr, sh): box = box_rows x 64 elements, 128B swizzle.
+// [S, rows, H, D] bf16 with element strides (sb, sr, sh): box = box_rows x 64 elements, 128B swizzle.
 static bool make_map(CUtensorMap* m, const void* ptr, int S, int rows, int H, int64_t sb, int64_t sr, int64_t sh,
-                     int box_rows) {
+                     int box_rows, int D) {
   EncodeTiledFn fn = encode_fn();
   if (!fn || rows < 1) return false;
-  cuuint64_t dims[4] = {128, (cuuint64_t)H, (cuuint64_t)rows, (cuuint64_t)S};
+  cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)rows, (cuuint64_t)S};
   cuuint64_t strides[3] = {(cuuint64_t)sh * 2, (cuuint64_t)sr * 2, (cuuint64_t)sb * 2};
   // a size-1 dimension may carry any stride; give it a harmless valid one
   if (H == 1) strides[0] = 256;
@@ -1125,22 +1106,23 @@ static DeviceFacts device_facts() {
 }
 
 bool attention_tc_supported(const AttnArgs& a) {
-  return a.L.dtype == TSD_BF16 && a.L.head_dim == 128 && a.sm_scale > 0.f && device_facts().state == 1;
+  return a.L.dtype == TSD_BF16 && (a.L.head_dim == 128 || a.L.head_dim == 64) && a.sm_scale > 0.f && device_facts().state == 1;
 }
 
 size_t attention_tc_workspace_bytes(const tsd_layout&) { return 0; }
 
-int launch_attention_tc(const AttnArgs& a) {
+template <int D>
+static int launch_tc(const AttnArgs& a) {
   const tsd_layout& L = a.L;
   const int N = L.n_branches * L.rows_per_branch;
   CUtensorMap mq, mkc, mvc, mkd, mvd, mo;
-  bool ok = make_map(&mq, a.q, L.batch, N, L.n_q_heads, a.qs_b, a.qs_r, a.qs_h, kTile) &&
-            make_map(&mo, a.out, L.batch, N, L.n_q_heads, a.os_b, a.os_r, a.os_h, kTile) &&
-            make_map(&mkd, a.kd, L.batch, N, L.n_kv_heads, a.ds_b, a.ds_r, a.ds_h, kKeys) &&
-            make_map(&mvd, a.vd, L.batch, N, L.n_kv_heads, a.ds_b, a.ds_r, a.ds_h, kKeys);
+  bool ok = make_map(&mq, a.q, L.batch, N, L.n_q_heads, a.qs_b, a.qs_r, a.qs_h, kTile, D) &&
+            make_map(&mo, a.out, L.batch, N, L.n_q_heads, a.os_b, a.os_r, a.os_h, kTile, D) &&
+            make_map(&mkd, a.kd, L.batch, N, L.n_kv_heads, a.ds_b, a.ds_r, a.ds_h, kKeys, D) &&
+            make_map(&mvd, a.vd, L.batch, N, L.n_kv_heads, a.ds_b, a.ds_r, a.ds_h, kKeys, D);
   if (ok && L.n_cache > 0) {
-    ok = make_map(&mkc, a.kc, L.batch, L.n_cache, L.n_kv_heads, a.cs_b, a.cs_r, a.cs_h, kKeys) &&
-         make_map(&mvc, a.vc, L.batch, L.n_cache, L.n_kv_heads, a.cs_b, a.cs_r, a.cs_h, kKeys);
+    ok = make_map(&mkc, a.kc, L.batch, L.n_cache, L.n_kv_heads, a.cs_b, a.cs_r, a.cs_h, kKeys, D) &&
+         make_map(&mvc, a.vc, L.batch, L.n_cache, L.n_kv_heads, a.cs_b, a.cs_r, a.cs_h, kKeys, D);
   } else if (ok) {  // no cache: the cached maps are never dereferenced
     mkc = mkd;
     mvc = mvd;
@@ -1156,7 +1138,7 @@ int launch_attention_tc(const AttnArgs& a) {
     std::lock_guard<std::mutex> lock(mu);
     if (!done[dev]) {
       cudaError_t attr_err =
-          cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+          cudaFuncSetAttribute(attention_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<D>::kBytes);
       if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(attention_tc_kernel)");
       done[dev] = true;
     }
@@ -1175,11 +1157,13 @@ int launch_attention_tc(const AttnArgs& a) {
   const int sms = std::max(device_facts().sms, 1);
   int64_t grid = std::min<int64_t>(n_items, sms);
   grid = std::max<int64_t>(grid, (n_items + kMaxItems - 1) / kMaxItems);
-  attention_tc_kernel<<<(unsigned)grid, kTcThreads, kSmemBytes, a.stream>>>(mq, mkc, mvc, mkd, mvd, mo, p);
+  attention_tc_kernel<D><<<(unsigned)grid, kTcThreads, TcSmem<D>::kBytes, a.stream>>>(mq, mkc, mvc, mkd, mvd, mo, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "attention_tc_kernel");
   return TSD_OK;
 }
+
+int launch_attention_tc(const AttnArgs& a) { return a.L.head_dim == 64 ? launch_tc<64>(a) : launch_tc<128>(a); }
 
 }  // namespace tsd
 

@@ -265,6 +265,25 @@ def test_attention_is_deterministic():
     assert torch.equal(a.out, b.out) and torch.equal(a.attn_lse, b.attn_lse)
 
 
+@pytest.mark.parametrize("R,Bn,Nc,lens", [(32, 1, 1, None), (32, 5, 333, [333, 65]), (64, 3, 64, [64, 0]), (128, 2, 127, [63, 127]),
+                                          (32, 9, 0, None), (64, 4, 1000, None)])
+def test_attention_head_dim_64_tensor_cores(R, Bn, Nc, lens):
+    # 64-wide heads keep P as two bf16 parts: no rounding of the weights shows, so the bound is the bf16 rounding of the output
+    # (half an ulp, 2^-9 relative, taken as 2^-8) plus the weights' 2^-17 and the fp32 sums on values of size up to 6 (6 * 2^-16)
+    cfg = W.small(W.CONFIGS["cfg2"], S=2, B=Bn, R=R, Nc=Nc, Hq=4, Hkv=2, d=64)
+    attn = W.attention_inputs(cfg, DEV, q_gain=2.0)
+    vis = np.zeros((cfg.S, Bn, 1), dtype=np.int64)
+    vis[1, Bn - 1, 0] = 1                     # the last branch of sequence 1 also reads the first
+    vis = torch.from_numpy(vis).to(DEV)
+    lens = None if lens is None else torch.tensor(lens, dtype=torch.int32, device=DEV)
+    _check_attention(cfg, attn, 0, vis=vis, cache_lens=lens)
+    step, _ = _run_attention(cfg, attn, 0, vis, lens)
+    mask = oracle.dense_mask(cfg.S, cfg.B, cfg.R, cfg.Nc, vis.cpu().numpy(), None if lens is None else lens.cpu().numpy())
+    ref, _ = oracle.masked_attention(_np(attn["q"]), _np(attn["k_cache"]), _np(attn["v_cache"]), _np(attn["k_draft"]),
+                                     _np(attn["v_draft"]), mask, attn["sm_scale"])
+    assert (np.abs(_np(step.out) - ref) <= 2.0 ** -8 * np.abs(ref) + 6 * 2.0 ** -16).all()
+
+
 # ----------------------------------------------------------------- confidence / top-k
 def _check_topk(logits, k, rows=None):
     n, V = logits.shape
