@@ -284,6 +284,19 @@ def test_attention_head_dim_64_tensor_cores(R, Bn, Nc, lens):
     assert (np.abs(_np(step.out) - ref) <= 2.0 ** -8 * np.abs(ref) + 6 * 2.0 ** -16).all()
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("S,Bn,R,Nc,Hq,Hkv,lens", [(1, 1, 32, 0, 1, 1, None), (1, 3, 32, 31, 2, 1, None), (2, 2, 64, 97, 2, 2, [97, 1]),
+                                                   (1, 8, 32, 400, 4, 2, None), (2, 3, 128, 64, 3, 1, [33, 64])])
+def test_attention_fp32_rows_per_block_and_key_chunks(d, S, Bn, R, Nc, Hq, Hkv, lens):
+    # both row counts per block (4 up to 592 (head, row) pairs, 8 above), one chunk of keys up to more than the block has warps,
+    # partial chunks, sequences without cached keys, a branch that reads every other one
+    cfg = W.small(W.CONFIGS["cfg1"], S=S, B=Bn, R=R, Nc=Nc, Hq=Hq, Hkv=Hkv, d=d)
+    vis = np.zeros((S, Bn, 1), dtype=np.int64)
+    vis[S - 1, 0, 0] = (1 << Bn) - 1
+    lens = None if lens is None else torch.tensor(lens, dtype=torch.int32, device=DEV)
+    _check_attention(cfg, W.attention_inputs(cfg, DEV), 0, vis=torch.from_numpy(vis).to(DEV), cache_lens=lens)
+
+
 # ----------------------------------------------------------------- confidence / top-k
 def _check_topk(logits, k, rows=None):
     n, V = logits.shape
