@@ -64,6 +64,8 @@ accept_kernel(int B_all, int n_cur, int R, const int32_t* __restrict__ parent, c
   const size_t ts = (size_t)tree * batch + s;  // slot in the tree-major outputs
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   const unsigned full = 0xffffffffu;
+  grid_wait(parent, state, conf, top1);
+  grid_launch_next();
   if (B <= 0) return;
   const int32_t* st = state + ((size_t)s * B_all + lo) * R;
   const float* cf = conf + ((size_t)s * B_all + lo) * R;
@@ -276,11 +278,10 @@ static int accept_launch(int32_t batch, int32_t n_branches, int32_t n_cur, int32
                       : (tree_max * 32 > tsd::kAcceptMaxThreads ? tsd::kAcceptMaxThreads : tree_max * 32);
   auto kernel = rows_per_branch <= 32 ? tsd::accept_kernel<1>
                 : rows_per_branch <= 64 ? tsd::accept_kernel<2> : tsd::accept_kernel<tsd::kRowWords>;
-  kernel<<<grid, threads, 0, stream>>>(
-      n_branches, n_cur, rows_per_branch, parent, state, mask_id, conf, top1_idx, top1_stride, tau, rule,
+  cudaError_t e = tsd::launch(
+      kernel, grid, threads, 0, stream, n_branches, n_cur, rows_per_branch, parent, state, mask_id, conf, top1_idx, top1_stride, tau, rule,
       search, edge_valid, prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag,
       unmask_tok, status, x);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return tsd::cuda_fail(e, "accept_kernel");
   return TSD_OK;
 }

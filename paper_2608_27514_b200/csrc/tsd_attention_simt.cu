@@ -90,6 +90,8 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
   const int b = row0 / R, g = h / (Hq / Hkv), N = B * R;
   const int j = lane % LPK, slots = kTile / R;
   const unsigned full = 0xffffffffu;
+  grid_wait(mask, q, kc, vc, kd, vd);
+  grid_launch_next();
 
   // the block's query rows, 8 dimensions per lane (requested first: nothing else is needed for them)
   float qr[RB][8];
@@ -263,12 +265,11 @@ static cudaError_t launch_rows(const AttnArgs& a, int warps) {
   const tsd_layout& L = a.L;
   const MaskDims md = mask_dims(L);
   const dim3 grid(L.n_branches * L.rows_per_branch / RB, L.n_q_heads, L.batch);
-  attention_rows_kernel<T, D, RB, MAXW><<<grid, std::min(warps, MAXW) * 32, 0, a.stream>>>(
-      L.batch, L.n_branches, L.rows_per_branch, L.n_cache, L.n_q_heads, L.n_kv_heads, md.recs_off, md.n_qt,
+  return launch(
+      attention_rows_kernel<T, D, RB, MAXW>, grid, std::min(warps, MAXW) * 32, 0, a.stream, L.batch, L.n_branches, L.rows_per_branch, L.n_cache, L.n_q_heads, L.n_kv_heads, md.recs_off, md.n_qt,
       md.rec_words, a.mask, static_cast<const T*>(a.q), static_cast<const T*>(a.kc), static_cast<const T*>(a.vc),
       static_cast<const T*>(a.kd), static_cast<const T*>(a.vd), static_cast<T*>(a.out), a.lse, a.qs_b, a.qs_r,
       a.qs_h, a.cs_b, a.cs_r, a.cs_h, a.ds_b, a.ds_r, a.ds_h, a.os_b, a.os_r, a.os_h, a.sm_scale, a.status);
-  return cudaGetLastError();
 }
 
 template <typename T, int D>

@@ -451,27 +451,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     s = item / (p.n_qt * p.Hq);
   };
 
-  const int h_magic = mask[H_MAGIC], h_s = mask[H_S], h_b = mask[H_B], h_r = mask[H_R], h_nc = mask[H_NC];
-  // tile counts of this block's items (the blob's layout follows from the tsd_layout, so no
-  // address depends on a loaded value)
-  for (int it = tid; it < n_my; it += kTcThreads) {
-    int s, h, qt;
-    item_coords(it, s, h, qt);
-    const int clen = min(max(mask[kHdrWords + s], 0), p.Nc);
-    const int n_dt = min(max(mask[p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words], 1), p.n_qt);
-    const int n_ct = (clen + kKeys - 1) / kKeys;
-    item_clen[it] = clen;
-    item_T[it] = n_ct + 2 * n_dt;
-  }
-
-  // Coordinates of the block's first item for the two producer lanes: worked out here, while the
-  // block is still setting up, so that their first requests after the sync are a few instructions.
-  int s_first = 0, g_first = 0;
-  if (lane == 0 && (warp == kKProducerWarp || warp == kVProducerWarp) && n_my > 0) {
-    int h, qt;
-    item_coords(0, s_first, h, qt);
-    g_first = h / p.group;
-  }
   if (warp == kKProducerWarp && lane == 0) {
     abort_flag[0] = 0;
     abort_flag[1] = 0;  // scratch flag for the drain waits
@@ -494,6 +473,33 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     mbar_init(bar(OS_FREE), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
+  }
+  // Everything above runs while the previous kernel of the stream finishes.  Tensor memory is allocated only
+  // after the wait: a block of that kernel may still need it.
+  grid_wait(mask);
+
+  const int h_magic = mask[H_MAGIC], h_s = mask[H_S], h_b = mask[H_B], h_r = mask[H_R], h_nc = mask[H_NC];
+  // tile counts of this block's items (the blob's layout follows from the tsd_layout, so no
+  // address depends on a loaded value)
+  for (int it = tid; it < n_my; it += kTcThreads) {
+    int s, h, qt;
+    item_coords(it, s, h, qt);
+    const int clen = min(max(mask[kHdrWords + s], 0), p.Nc);
+    const int n_dt = min(max(mask[p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words], 1), p.n_qt);
+    const int n_ct = (clen + kKeys - 1) / kKeys;
+    item_clen[it] = clen;
+    item_T[it] = n_ct + 2 * n_dt;
+  }
+
+  // Coordinates of the block's first item for the two producer lanes: worked out here, while the
+  // block is still setting up, so that their first requests after the sync are a few instructions.
+  int s_first = 0, g_first = 0;
+  if (lane == 0 && (warp == kKProducerWarp || warp == kVProducerWarp) && n_my > 0) {
+    int h, qt;
+    item_coords(0, s_first, h, qt);
+    g_first = h / p.group;
+  }
+  if (warp == kKProducerWarp && lane == 0) {
     if (n_my > 0) {  // Q of the first item: its coordinates need nothing from the blob
       int s, h, qt;
       item_coords(0, s, h, qt);
@@ -1157,8 +1163,8 @@ static int launch_tc(const AttnArgs& a) {
   const int sms = std::max(device_facts().sms, 1);
   int64_t grid = std::min<int64_t>(n_items, sms);
   grid = std::max<int64_t>(grid, (n_items + kMaxItems - 1) / kMaxItems);
-  attention_tc_kernel<D><<<(unsigned)grid, kTcThreads, TcSmem<D>::kBytes, a.stream>>>(mq, mkc, mvc, mkd, mvd, mo, p);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch(attention_tc_kernel<D>, (unsigned)grid, kTcThreads, TcSmem<D>::kBytes, a.stream, mq, mkc, mvc, mkd,
+                         mvd, mo, p);
   if (e != cudaSuccess) return cuda_fail(e, "attention_tc_kernel");
   return TSD_OK;
 }

@@ -25,6 +25,8 @@ commit_kernel(int B, int R, int root, const int32_t* __restrict__ parent, const 
               int32_t* __restrict__ n_masked, uint32_t* __restrict__ status) {
   __shared__ int s_path[kCommitMaxBranches];  // accepted node first, root last
   __shared__ int s_depth;
+  grid_wait(parent, state, accepted_node, unmask_flag, unmask_tok, block_start);
+  grid_launch_next();
   const int s = blockIdx.x, lane = threadIdx.x;
   const int32_t* par = parent + (size_t)s * B;
   const int32_t* st = state + (size_t)s * B * R;
@@ -98,6 +100,8 @@ gather_accepted_kv_kernel(int B, int R, int H, int vec_per_head, const int32_t* 
                           int64_t ss_r, int64_t ss_h, uint4* __restrict__ k_dst, uint4* __restrict__ v_dst,
                           int64_t ds_b, int64_t ds_r, int64_t ds_h, const int32_t* __restrict__ dst_row0,
                           int dst_rows, uint32_t* __restrict__ status) {
+  grid_wait(accepted_node, k_src, v_src, dst_row0);
+  grid_launch_next();
   const int s = blockIdx.y;
   const int node = accepted_node ? accepted_node[s] : 0;
   const int64_t row0 = dst_row0 ? dst_row0[s] : 0;
@@ -142,12 +146,11 @@ extern "C" int tsd_gather_accepted_kv(int32_t batch, int32_t n_branches, int32_t
   const int per16 = 16 / esize, vec_per_head = head_dim / per16;
   const int total = rows_per_branch * n_kv_heads * vec_per_head;
   dim3 grid((unsigned)std::min((total + 255) / 256, 64), (unsigned)batch);
-  tsd::gather_accepted_kv_kernel<<<grid, 256, 0, stream>>>(
-      n_branches, rows_per_branch, n_kv_heads, vec_per_head, accepted_node, static_cast<const uint4*>(k_draft),
+  cudaError_t e = tsd::launch(
+      tsd::gather_accepted_kv_kernel, grid, 256, 0, stream, n_branches, rows_per_branch, n_kv_heads, vec_per_head, accepted_node, static_cast<const uint4*>(k_draft),
       static_cast<const uint4*>(v_draft), d_stride_b / per16, d_stride_row / per16, d_stride_head / per16,
       static_cast<uint4*>(k_out), static_cast<uint4*>(v_out), o_stride_b / per16, o_stride_row / per16,
       o_stride_head / per16, out_row0, out_rows, status);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return tsd::cuda_fail(e, "gather_accepted_kv_kernel");
   return TSD_OK;
 }
@@ -166,10 +169,9 @@ extern "C" int tsd_commit_accepted(int32_t batch, int32_t n_branches, int32_t ro
   if (tokens && seq_stride < rows_per_branch) return TSD_ERR_INVALID_ARG;
   if (batch == 0) return TSD_OK;
   if (!parent || !state) return TSD_ERR_INVALID_ARG;
-  tsd::commit_kernel<<<batch, 32, 0, stream>>>(n_branches, rows_per_branch, tree_root, parent, state, accepted_node,
+  cudaError_t e = tsd::launch(tsd::commit_kernel, batch, 32, 0, stream, n_branches, rows_per_branch, tree_root, parent, state, accepted_node,
                                                unmask_flag, unmask_tok, mask_id, tokens, seq_stride, block_start,
                                                root_out, fill_step, step_base, n_masked, status);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return tsd::cuda_fail(e, "commit_kernel");
   return TSD_OK;
 }

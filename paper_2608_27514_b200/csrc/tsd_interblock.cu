@@ -12,6 +12,8 @@
 namespace tsd {
 
 __global__ void interblock_vis_kernel(int B, int n_cur, int words, uint64_t* __restrict__ vis, size_t total) {
+  grid_wait();
+  grid_launch_next();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // one (sequence, branch, word)
   if (i >= total) return;
   const int w = (int)(i % words);
@@ -31,6 +33,8 @@ interblock_trigger_kernel(int B, int R, const int32_t* __restrict__ state, const
                           const int32_t* __restrict__ node_cur, int node_next, int mask_id, float tau,
                           uint8_t* __restrict__ trigger, float* __restrict__ top_conf,
                           uint32_t* __restrict__ status) {
+  grid_wait(state, conf, node_cur);
+  grid_launch_next();
   const int s = blockIdx.x, lane = threadIdx.x;
   int cur = node_cur ? node_cur[s] : 0;
   if (cur < 0 || cur >= B) {
@@ -63,9 +67,8 @@ extern "C" int tsd_build_interblock_vis(int32_t batch, int32_t n_branches, int32
   if (!vis) return TSD_ERR_INVALID_ARG;
   const int words = (n_branches + 63) / 64;
   const size_t total = (size_t)batch * n_branches * words;
-  tsd::interblock_vis_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(n_branches, n_cur, words, vis,
+  cudaError_t e = tsd::launch(tsd::interblock_vis_kernel, (unsigned)((total + 255) / 256), 256, 0, stream, n_branches, n_cur, words, vis,
                                                                                total);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return tsd::cuda_fail(e, "interblock_vis_kernel");
   return TSD_OK;
 }
@@ -79,9 +82,8 @@ extern "C" int tsd_interblock_trigger(int32_t batch, int32_t n_branches, int32_t
     return TSD_ERR_INVALID_ARG;
   if (batch == 0) return TSD_OK;
   if (!state || !conf || !trigger) return TSD_ERR_INVALID_ARG;
-  tsd::interblock_trigger_kernel<<<batch, 32, 0, stream>>>(n_branches, rows_per_branch, state, conf, node_cur,
+  cudaError_t e = tsd::launch(tsd::interblock_trigger_kernel, batch, 32, 0, stream, n_branches, rows_per_branch, state, conf, node_cur,
                                                            node_next, mask_id, tau, trigger, top_conf, status);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return tsd::cuda_fail(e, "interblock_trigger_kernel");
   return TSD_OK;
 }

@@ -16,6 +16,7 @@ dequant_e4m3_kernel(const uint8_t* __restrict__ k_src, const uint8_t* __restrict
                     int64_t ss_h, const float* __restrict__ k_scale, const float* __restrict__ v_scale,
                     const int32_t* __restrict__ mask_blob, __nv_bfloat16* __restrict__ k_dst,
                     __nv_bfloat16* __restrict__ v_dst, int Nc, int H, int d, uint32_t vec_per_seq) {
+  grid_wait(k_src, v_src, k_scale, v_scale, mask_blob);
   const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;  // one vector = 16 consecutive codes of sequence s
   if (v >= vec_per_seq) return;
   const uint32_t vec_per_head = (uint32_t)d / 16u, vec_per_row = vec_per_head * (uint32_t)H;
@@ -97,12 +98,11 @@ extern "C" int tsd_verify_attention_fp8_cache(
     const int64_t vec_per_seq = (int64_t)L->n_cache * L->n_kv_heads * (L->head_dim / 16);
     if (vec_per_seq > 0x7fffff00ll || L->batch > 65535) return TSD_ERR_UNSUPPORTED;  // 32-bit indices, grid y
     const dim3 grid((unsigned)((vec_per_seq + 255) / 256), (unsigned)L->batch, 2);
-    tsd::dequant_e4m3_kernel<<<grid, 256, 0, stream>>>(
-        k_cache_e4m3, v_cache_e4m3, c_stride_b, c_stride_row, c_stride_head, k_scale, v_scale,
+    cudaError_t e = tsd::launch(
+        tsd::dequant_e4m3_kernel, grid, 256, 0, stream, k_cache_e4m3, v_cache_e4m3, c_stride_b, c_stride_row, c_stride_head, k_scale, v_scale,
         static_cast<const int32_t*>(mask), reinterpret_cast<__nv_bfloat16*>(ws + inner),
         reinterpret_cast<__nv_bfloat16*>(ws + inner + half), L->n_cache, L->n_kv_heads, L->head_dim,
         (uint32_t)vec_per_seq);
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return tsd::cuda_fail(e, "dequant_e4m3_kernel");
   }
   return tsd_verify_attention(L, mask, q, q_stride_b, q_stride_row, q_stride_head,

@@ -14,6 +14,8 @@ __device__ __forceinline__ bool branch_sees(const uint64_t* vis, int s, int B, i
 __global__ void build_mask_kernel(int S, int B, int R, int Nc, int n_qt, int rec_words, int lens_off,
                                   int recs_off, const uint64_t* __restrict__ vis,
                                   const int32_t* __restrict__ cache_lens, int32_t* __restrict__ blob) {
+  grid_wait(vis, cache_lens);
+  grid_launch_next();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t == 0) {
     blob[H_MAGIC] = kMaskMagic; blob[H_S] = S; blob[H_B] = B; blob[H_R] = R; blob[H_NC] = Nc;
@@ -47,6 +49,7 @@ __global__ void build_mask_kernel(int S, int B, int R, int Nc, int n_qt, int rec
 
 __global__ void dense_mask_kernel(int S, int B, int R, int Nc, const uint64_t* __restrict__ vis,
                                   const int32_t* __restrict__ cache_lens, uint8_t* __restrict__ dense) {
+  grid_wait(vis, cache_lens);
   const int N = B * R, words = (B + 63) / 64;
   const int64_t L = (int64_t)Nc + N, total = (int64_t)S * N * L;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -84,18 +87,16 @@ int tsd_build_branch_mask(const tsd_layout* L, const uint64_t* vis, const int32_
   if (mask_bytes < m.bytes) return TSD_ERR_WORKSPACE;
   const int threads = 128;
   const int work = max(L->batch * m.n_qt, L->batch);
-  tsd::build_mask_kernel<<<(work + threads - 1) / threads, threads, 0, stream>>>(
-      L->batch, L->n_branches, L->rows_per_branch, L->n_cache, m.n_qt, m.rec_words, m.lens_off,
+  cudaError_t e = tsd::launch(
+      tsd::build_mask_kernel, (work + threads - 1) / threads, threads, 0, stream, L->batch, L->n_branches, L->rows_per_branch, L->n_cache, m.n_qt, m.rec_words, m.lens_off,
       m.recs_off, vis, cache_lens, static_cast<int32_t*>(mask_out));
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return tsd::cuda_fail(e, "build_mask_kernel");
   if (dense_out) {
     const int64_t N = (int64_t)L->n_branches * L->rows_per_branch;
     const int64_t total = (int64_t)L->batch * N * (L->n_cache + N);
     const int blocks = (int)std::min<int64_t>((total + 255) / 256, 148 * 16);
-    tsd::dense_mask_kernel<<<blocks, 256, 0, stream>>>(L->batch, L->n_branches, L->rows_per_branch,
+    e = tsd::launch(tsd::dense_mask_kernel, blocks, 256, 0, stream, L->batch, L->n_branches, L->rows_per_branch,
                                                        L->n_cache, vis, cache_lens, dense_out);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return tsd::cuda_fail(e, "dense_mask_kernel");
   }
   return TSD_OK;

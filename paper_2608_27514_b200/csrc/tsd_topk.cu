@@ -273,6 +273,8 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   const int n_iter = (c1 - c0 + kTopkBatch - 1) / kTopkBatch;  // <= kTopkMaxIter (host-enforced)
   const bool has_tail = seg == n_seg - 1 && tid == 0 && chunks_total * E_ < vocab;
 
+  grid_wait(rowp, rowv);
+
   // ---- phase 1: stream.  Two register buffers: the loads of batch it+1 are in flight while
   // batch it is processed, so a block overlaps memory latency with its own arithmetic.
   float m = -CUDART_INF_F, e = 0.f, s = 0.f;
@@ -541,15 +543,9 @@ static cudaError_t launch_topk(const void* logits, int64_t n_rows, int vocab, in
                                void* ws, cudaStream_t st) {
   Partial<K>* partials = reinterpret_cast<Partial<K>*>(ws);
   unsigned* tickets = reinterpret_cast<unsigned*>(static_cast<char*>(ws) + p.ticket_off);
-  if (p.threads == 512)
-    confidence_topk_kernel<T, K, 512><<<(unsigned)(n_rows * p.n_seg), 512, 0, st>>>(
-        static_cast<const T*>(logits), vocab, row_stride, k, p.n_seg, p.chunks_per_seg, conf, idx, prob,
-        lse, partials, tickets, p.prefetch);
-  else
-    confidence_topk_kernel<T, K, 256><<<(unsigned)(n_rows * p.n_seg), 256, 0, st>>>(
-        static_cast<const T*>(logits), vocab, row_stride, k, p.n_seg, p.chunks_per_seg, conf, idx, prob,
-        lse, partials, tickets, p.prefetch);
-  return cudaGetLastError();
+  auto kernel = p.threads == 512 ? confidence_topk_kernel<T, K, 512> : confidence_topk_kernel<T, K, 256>;
+  return launch(kernel, (unsigned)(n_rows * p.n_seg), p.threads, 0, st, static_cast<const T*>(logits), vocab, row_stride, k,
+                p.n_seg, p.chunks_per_seg, conf, idx, prob, lse, partials, tickets, p.prefetch);
 }
 
 template <typename T>

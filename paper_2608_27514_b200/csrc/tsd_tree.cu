@@ -76,6 +76,8 @@ build_draft_tree_kernel(int prev_branches, int R, int k, const int32_t* __restri
   __shared__ int s_cpar[kTreeMaxWidth], s_crow[kTreeMaxWidth], s_crank[kTreeMaxWidth];
   __shared__ float s_cp[kTreeMaxWidth];
   __shared__ uint32_t s_mask[256][RPL];  // per node: which rows are still masked
+  grid_wait(prev_state, accepted_node, unmask_flag, unmask_tok, topk_idx, topk_prob, enable);
+  grid_launch_next();
   const int s = blockIdx.x, lane = threadIdx.x;
   int acc = accepted_node ? accepted_node[s] : 0;
   if (acc < 0 || acc >= prev_branches) {  // inconsistent device data: report, fall back to node 0
@@ -233,15 +235,15 @@ extern "C" int tsd_build_draft_tree(int32_t batch, int32_t prev_branches, int32_
   if (!prev_state || !topk_idx || !topk_prob || !parent || !state || !node_prob || !n_nodes)
     return TSD_ERR_INVALID_ARG;
   auto launch = [&](auto kernel) {
-    kernel<<<batch, 32, 0, stream>>>(prev_branches, rows_per_branch, k, prev_state, accepted_node, unmask_flag,
+    return tsd::launch(kernel, batch, 32, 0, stream, prev_branches, rows_per_branch, k, prev_state, accepted_node, unmask_flag,
                                      unmask_tok, mask_id, topk_idx, topk_prob, width, depth, max_nodes, out_stride,
                                      node_base, enable, parent, state, node_prob, n_nodes, status);
   };
   const int rpl = (rows_per_branch + 31) / 32;
-  if (rpl == 1 && k <= 4) launch(tsd::build_draft_tree_kernel<1, 4>);
-  else if (rpl <= 2 && k <= 4) launch(tsd::build_draft_tree_kernel<2, 4>);
-  else launch(tsd::build_draft_tree_kernel<tsd::kTreeRowsPerLane, tsd::kTreeMaxK>);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  if (rpl == 1 && k <= 4) e = launch(tsd::build_draft_tree_kernel<1, 4>);
+  else if (rpl <= 2 && k <= 4) e = launch(tsd::build_draft_tree_kernel<2, 4>);
+  else e = launch(tsd::build_draft_tree_kernel<tsd::kTreeRowsPerLane, tsd::kTreeMaxK>);
   if (e != cudaSuccess) return tsd::cuda_fail(e, "build_draft_tree_kernel");
   return TSD_OK;
 }
