@@ -488,6 +488,53 @@ int tsd_accept_joint_trees(int32_t batch, int32_t n_branches, int32_t n_cur, int
                            uint8_t* unmask_flag, int32_t* unmask_tok, uint32_t* status,
                            tsd_stream_t stream);
 
+/* ---------------------------------------------------------------------------
+ * The whole verification step in one call: tsd_verify_attention,
+ * tsd_confidence_topk and tsd_accept_trajectories on one stream, arguments as
+ * for those calls (strides as {batch, row, head}; stage 2's top-1 candidates go
+ * to the acceptance).  Every check of the three runs before the first launch.
+ * The attention and the vocabulary pass may run at the same time on the GPU:
+ * `logits` must not depend on this call's `out` or `attn_lse`, and the outputs
+ * of one must not overlap inputs of the other.  Work enqueued on the stream
+ * before the call is complete when either starts, and work enqueued after it
+ * starts when all three are complete, as with the separate calls.
+ * ------------------------------------------------------------------------- */
+typedef struct {
+  const tsd_layout* layout;
+  const void* mask;
+  const void* q;
+  int64_t q_stride[3];
+  const void *k_cache, *v_cache;
+  int64_t c_stride[3];
+  const void *k_draft, *v_draft;
+  int64_t d_stride[3];
+  void* out;
+  int64_t o_stride[3];
+  float* attn_lse;
+  float sm_scale;
+  uint32_t flags;
+  void* attn_workspace;
+  size_t attn_workspace_bytes;
+  const void* logits;
+  int64_t n_rows, row_stride;
+  int32_t logits_dtype, vocab, k;
+  float* conf;
+  int32_t* topk_idx;
+  float *topk_prob, *lse;
+  void* topk_workspace;
+  size_t topk_workspace_bytes;
+  const int32_t *parent, *state;
+  int32_t mask_id;
+  float tau;
+  int32_t rule, search;
+  uint8_t* edge_valid;
+  int32_t *prefix_len, *accepted_node, *accepted_len, *n_new_tokens;
+  uint8_t* unmask_flag;
+  int32_t* unmask_tok;
+  uint32_t* status;
+} tsd_step_args;
+int tsd_verify_step(const tsd_step_args* args, tsd_stream_t stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -1,4 +1,5 @@
-"""Thin ctypes binding over the libtsd C ABI: same names, argument marshalling only.
+"""Thin binding over the libtsd C ABI: same names, argument marshalling only.  The calls that a decode loop makes
+on every pass go through a small native module, the others through ctypes.
 
 Tensors are torch CUDA tensors used purely as device memory; each call extracts
 raw pointers and strides and enqueues the library's kernels on torch's current
@@ -29,7 +30,7 @@ EXPORTS = (
     "tsd_accept_trajectories", "tsd_build_draft_tree",
     "tsd_build_interblock_vis", "tsd_interblock_trigger", "tsd_accept_joint_trees", "tsd_accept_relaxed",
     "tsd_commit_accepted", "tsd_verify_attention_fp8_cache_workspace_bytes", "tsd_verify_attention_fp8_cache",
-    "tsd_gather_accepted_kv", "tsd_selftest_bounded_wait",
+    "tsd_gather_accepted_kv", "tsd_selftest_bounded_wait", "tsd_verify_step",
 )
 
 
@@ -105,6 +106,23 @@ def lib():
     return _lib
 
 
+_native = None
+
+
+def native():
+    """The module that takes tensors to the library's calls without ctypes; raises like lib() if it is missing."""
+    global _native
+    if _native is None:
+        lib()
+        try:
+            from . import _tsd_native
+        except ImportError as e:
+            raise RuntimeError("_tsd_native.so is missing: build it with `python -m paper_2608_27514_b200.build`") from e
+        _tsd_native.setup(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream, torch.float32, torch.bfloat16, TsdError)
+        _native = _tsd_native
+    return _native
+
+
 def strerror(code):
     return lib().tsd_strerror(int(code)).decode()
 
@@ -125,7 +143,7 @@ def _ptr(t):
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
@@ -152,33 +170,17 @@ def tsd_branch_mask_bytes(layout):
 
 
 def tsd_build_branch_mask(layout, vis, cache_lens, mask_out, dense_out=None, stream=None):
-    rc = lib().tsd_build_branch_mask(ctypes.byref(layout), _ptr(vis), _ptr(cache_lens), _ptr(mask_out),
-                                     mask_out.numel() * mask_out.element_size(), _ptr(dense_out),
-                                     _stream(stream))
-    _check(rc, "tsd_build_branch_mask")
+    native().build_mask(layout, vis, cache_lens, mask_out, dense_out, stream)
 
 
 def tsd_verify_attention_workspace_bytes(layout):
     return int(lib().tsd_verify_attention_workspace_bytes(ctypes.byref(layout)))
 
 
-def _strides3(t):
-    # [batch, rows, heads, dim] -> (batch, row, head) strides in elements
-    assert t.dim() == 4 and t.stride(3) == 1, "head_dim must be contiguous"
-    return t.stride(0), t.stride(1), t.stride(2)
-
-
 def tsd_verify_attention(layout, mask, q, k_cache, v_cache, k_draft, v_draft, out, lse=None,
                          sm_scale=1.0, workspace=None, flags=0, status=None, stream=None):
-    assert v_cache is None or v_cache.stride() == k_cache.stride()
-    assert v_draft.stride() == k_draft.stride()
-    cs = _strides3(k_cache) if k_cache is not None else (0, 0, layout.head_dim)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib().tsd_verify_attention(
-        ctypes.byref(layout), _ptr(mask), _ptr(q), *_strides3(q), _ptr(k_cache), _ptr(v_cache), *cs,
-        _ptr(k_draft), _ptr(v_draft), *_strides3(k_draft), _ptr(out), *_strides3(out), _ptr(lse),
-        float(sm_scale), _ptr(workspace), ws_bytes, int(flags), _ptr(status), _stream(stream))
-    _check(rc, "tsd_verify_attention")
+    native().verify_attention(layout, mask, q, k_cache, v_cache, k_draft, v_draft, out, lse, sm_scale, workspace, flags, status,
+                              stream)
 
 
 def tsd_confidence_topk_workspace_bytes(n_rows, vocab, k):
@@ -187,13 +189,7 @@ def tsd_confidence_topk_workspace_bytes(n_rows, vocab, k):
 
 def tsd_confidence_topk(logits, k, conf, topk_idx, topk_prob, lse=None, workspace=None, status=None,
                         stream=None):
-    assert logits.dim() == 2 and logits.stride(1) == 1
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib().tsd_confidence_topk(
-        _ptr(logits), dtype_code(logits.dtype), logits.shape[0], logits.shape[1], logits.stride(0),
-        int(k), _ptr(conf), _ptr(topk_idx), _ptr(topk_prob), _ptr(lse), _ptr(workspace), ws_bytes,
-        _ptr(status), _stream(stream))
-    _check(rc, "tsd_confidence_topk")
+    native().confidence_topk(logits, k, conf, topk_idx, topk_prob, lse, workspace, status, stream)
 
 
 def tsd_confidence_topk_static_capacity():
@@ -213,18 +209,8 @@ def tsd_confidence_topk_static(logits, k, conf, topk_idx, topk_prob, lse=None, s
 def tsd_accept_trajectories(parent, state, mask_id, conf, top1_idx, top1_stride, tau, rule, search,
                             edge_valid, prefix_len, accepted_node, accepted_len, n_new_tokens,
                             unmask_flag, unmask_tok, status=None, stream=None):
-    S, B, R = state.shape
-    rc = lib().tsd_accept_trajectories(
-        S, B, R, _ptr(parent), _ptr(state), int(mask_id), _ptr(conf), _ptr(top1_idx), int(top1_stride),
-        float(tau), int(rule), int(search), _ptr(edge_valid), _ptr(prefix_len), _ptr(accepted_node),
-        _ptr(accepted_len), _ptr(n_new_tokens), _ptr(unmask_flag), _ptr(unmask_tok), _ptr(status),
-        _stream(stream))
-    _check(rc, "tsd_accept_trajectories")
-
-
-def _slice_ptr(t, first):
-    """Address of branch `first` of sequence 0 in a contiguous [S, B, ...] tensor."""
-    return ctypes.c_void_p(t.data_ptr() + first * t.stride(1) * t.element_size())
+    native().accept(parent, state, None, mask_id, conf, top1_idx, top1_stride, tau, rule, search, edge_valid, prefix_len,
+                    accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, status, stream)
 
 
 def tsd_build_draft_tree(prev_state, accepted_node, unmask_flag, unmask_tok, mask_id, topk_idx, topk_prob,
@@ -234,35 +220,19 @@ def tsd_build_draft_tree(prev_state, accepted_node, unmask_flag, unmask_tok, mas
     outputs parent [S,B], state [S,B,R], node_prob [S,B], n_nodes [S].  With `first`/`max_nodes`
     the tree fills branches [first, first + max_nodes) of the (larger) output arrays and its
     parent indices count from `first`; `enable` uint8 [S] keeps a sequence's tree at its root."""
-    S, Bp, R = prev_state.shape
-    k = topk_idx.shape[-1]
-    B = state.shape[1]
-    max_nodes = B - first if max_nodes is None else int(max_nodes)
     assert state.is_contiguous() and parent.is_contiguous() and node_prob.is_contiguous()
-    assert 0 <= first and first + max_nodes <= B
-    rc = lib().tsd_build_draft_tree(
-        S, Bp, R, k, _ptr(prev_state), _ptr(accepted_node), _ptr(unmask_flag), _ptr(unmask_tok), int(mask_id),
-        _ptr(topk_idx), _ptr(topk_prob), int(width), int(depth), max_nodes, B, int(first), _ptr(enable),
-        _slice_ptr(parent, first), _slice_ptr(state, first), _slice_ptr(node_prob, first), _ptr(n_nodes),
-        _ptr(status), _stream(stream))
-    _check(rc, "tsd_build_draft_tree")
+    native().build_tree(prev_state, accepted_node, unmask_flag, unmask_tok, mask_id, topk_idx, topk_prob, width, depth, parent,
+                        state, node_prob, n_nodes, status, stream, first, max_nodes, enable)
 
 
 def tsd_build_interblock_vis(n_cur, vis, stream=None):
     """vis uint64/int64 [S, B, ceil(B/64)] (written)."""
-    S, B, W = vis.shape
-    assert W == (B + 63) // 64 and vis.is_contiguous() and vis.element_size() == 8
-    _check(lib().tsd_build_interblock_vis(S, B, int(n_cur), _ptr(vis), _stream(stream)),
-           "tsd_build_interblock_vis")
+    native().interblock_vis(n_cur, vis, stream)
 
 
 def tsd_interblock_trigger(state, conf, node_cur, node_next, mask_id, tau, trigger, top_conf=None,
                            status=None, stream=None):
-    S, B, R = state.shape
-    rc = lib().tsd_interblock_trigger(S, B, R, _ptr(state), _ptr(conf), _ptr(node_cur), int(node_next),
-                                      int(mask_id), float(tau), _ptr(trigger), _ptr(top_conf), _ptr(status),
-                                      _stream(stream))
-    _check(rc, "tsd_interblock_trigger")
+    native().interblock_trigger(state, conf, node_cur, node_next, mask_id, tau, trigger, top_conf, status, stream)
 
 
 def tsd_accept_joint_trees(parent, state, n_cur, mask_id, conf, top1_idx, top1_stride, tau, rule, search,
@@ -270,13 +240,8 @@ def tsd_accept_joint_trees(parent, state, n_cur, mask_id, conf, top1_idx, top1_s
                            unmask_flag, unmask_tok, status=None, stream=None):
     """Forest layout: parent/edge_valid/prefix_len [S,B]; accepted_* and n_new_tokens [2,S];
     unmask_* [2,S,R]."""
-    S, B, R = state.shape
-    rc = lib().tsd_accept_joint_trees(
-        S, B, int(n_cur), R, _ptr(parent), _ptr(state), int(mask_id), _ptr(conf), _ptr(top1_idx),
-        int(top1_stride), float(tau), int(rule), int(search), _ptr(edge_valid), _ptr(prefix_len),
-        _ptr(accepted_node), _ptr(accepted_len), _ptr(n_new_tokens), _ptr(unmask_flag), _ptr(unmask_tok),
-        _ptr(status), _stream(stream))
-    _check(rc, "tsd_accept_joint_trees")
+    native().accept(parent, state, n_cur, mask_id, conf, top1_idx, top1_stride, tau, rule, search, edge_valid, prefix_len,
+                    accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, status, stream)
 
 
 def tsd_accept_relaxed(parent, state, n_cur, mask_id, conf, topk_idx, topk_m, logits, lse, tau, rule, search,
@@ -284,17 +249,9 @@ def tsd_accept_relaxed(parent, state, n_cur, mask_id, conf, topk_idx, topk_m, lo
                        unmask_tok, draft_prob=None, status=None, stream=None):
     """Any of the four rules on one tree (n_cur = B) or two; topk_idx [S,B,R,k]; logits
     [S*B*R, V] (or None) with lse [S*B*R]; per-tree outputs [2,S,...] (row 0 only for one tree)."""
-    S, B, R = state.shape
-    if logits is not None:
-        assert logits.dim() == 2 and logits.stride(1) == 1 and logits.shape[0] == S * B * R
-    rc = lib().tsd_accept_relaxed(
-        S, B, int(n_cur), R, _ptr(parent), _ptr(state), int(mask_id), _ptr(conf), _ptr(topk_idx),
-        int(topk_idx.shape[-1]) if topk_idx.dim() == 4 else 1, int(topk_m), _ptr(logits),
-        0 if logits is None else dtype_code(logits.dtype), 0 if logits is None else logits.shape[1],
-        0 if logits is None else logits.stride(0), _ptr(lse), float(tau), int(rule), int(search),
-        _ptr(edge_valid), _ptr(prefix_len), _ptr(accepted_node), _ptr(accepted_len), _ptr(n_new_tokens),
-        _ptr(unmask_flag), _ptr(unmask_tok), _ptr(draft_prob), _ptr(status), _stream(stream))
-    _check(rc, "tsd_accept_relaxed")
+    native().accept_relaxed(parent, state, n_cur, mask_id, conf, topk_idx, topk_m, logits, lse, tau, rule, search, edge_valid,
+                            prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, draft_prob, status,
+                            stream)
 
 
 def tsd_commit_accepted(parent, state, accepted_node, unmask_flag, unmask_tok, mask_id, tokens=None,
@@ -302,14 +259,8 @@ def tsd_commit_accepted(parent, state, accepted_node, unmask_flag, unmask_tok, m
                         status=None, stream=None, tree_root=0):
     """parent [S,B], state [S,B,R]; tokens [S,L] (row stride = tokens.stride(0)); the rest [S] / [S,R];
     tree_root = forest index of the tree's root (the next block's tree of a joint pass)."""
-    S, B, R = state.shape
-    if tokens is not None:
-        assert tokens.dim() == 2 and tokens.stride(1) == 1
-    rc = lib().tsd_commit_accepted(
-        S, B, R, int(tree_root), _ptr(parent), _ptr(state), _ptr(accepted_node), _ptr(unmask_flag), _ptr(unmask_tok),
-        int(mask_id), _ptr(tokens), 0 if tokens is None else tokens.stride(0), _ptr(block_start), _ptr(root_out),
-        _ptr(fill_step), _ptr(step_base), _ptr(n_masked), _ptr(status), _stream(stream))
-    _check(rc, "tsd_commit_accepted")
+    native().commit(parent, state, accepted_node, unmask_flag, unmask_tok, mask_id, tokens, block_start, root_out, fill_step,
+                    step_base, n_masked, status, stream, tree_root)
 
 
 def tsd_gather_accepted_kv(accepted_node, rows_per_branch, k_draft, v_draft, k_out, v_out, out_row0=None,
@@ -341,12 +292,14 @@ def tsd_verify_attention_fp8_cache_workspace_bytes(layout):
 def tsd_verify_attention_fp8_cache(layout, mask, q, k_cache_e4m3, v_cache_e4m3, k_scale, v_scale, k_draft, v_draft,
                                    out, workspace, lse=None, sm_scale=1.0, flags=0, status=None, stream=None):
     """k/v_cache_e4m3: uint8 (or float8_e4m3fn) tensors [S, Nc, Hkv, d]; k/v_scale fp32 [S, Hkv] or None."""
-    assert v_cache_e4m3 is None or v_cache_e4m3.stride() == k_cache_e4m3.stride()
-    assert v_draft.stride() == k_draft.stride()
-    cs = _strides3(k_cache_e4m3) if k_cache_e4m3 is not None else (0, 0, layout.head_dim)
-    rc = lib().tsd_verify_attention_fp8_cache(
-        ctypes.byref(layout), _ptr(mask), _ptr(q), *_strides3(q), _ptr(k_cache_e4m3), _ptr(v_cache_e4m3), *cs,
-        _ptr(k_scale), _ptr(v_scale), _ptr(k_draft), _ptr(v_draft), *_strides3(k_draft), _ptr(out), *_strides3(out),
-        _ptr(lse), float(sm_scale), _ptr(workspace), workspace.numel() * workspace.element_size(), int(flags),
-        _ptr(status), _stream(stream))
-    _check(rc, "tsd_verify_attention_fp8_cache")
+    native().verify_attention_fp8(layout, mask, q, k_cache_e4m3, v_cache_e4m3, k_scale, v_scale, k_draft, v_draft, out, workspace,
+                                  lse, sm_scale, flags, status, stream)
+
+
+def tsd_verify_step(layout, mask, q, k_cache, v_cache, k_draft, v_draft, out, attn_lse, sm_scale, attn_workspace, flags, logits, k,
+                    conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search, edge_valid,
+                    prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, status=None, stream=None):
+    """Attention, vocabulary pass and acceptance in one call (arguments as for the three calls)."""
+    native().verify_step(layout, mask, q, k_cache, v_cache, k_draft, v_draft, out, attn_lse, sm_scale, attn_workspace, flags, logits,
+                         k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search, edge_valid,
+                         prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, status, stream)

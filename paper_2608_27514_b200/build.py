@@ -1,12 +1,15 @@
-"""Builds libtsd.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libtsd.so (the C-ABI CUDA library) with nvcc for sm_100a, and _tsd_native.so (its Python side), in-tree."""
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libtsd.so")
+NATIVE_SRC = os.path.join(CSRC, "tsd_python.cpp")
+NATIVE = os.path.join(HERE, "_tsd_native.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "--use_fast_math=false"]
@@ -17,10 +20,10 @@ def sources():
 
 
 def stale():
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
+    deps = sources() + [NATIVE_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         [os.path.join(os.path.dirname(HERE), "include", "tsd.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -51,6 +54,10 @@ def build(force=False, verbose=False):
     tmp = LIB + ".%d.tmp" % os.getpid()
     subprocess.check_call([NVCC, "-shared", "-o", tmp] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"])
     os.replace(tmp, LIB)
+    tmp = NATIVE + ".%d.tmp" % os.getpid()
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"], NATIVE_SRC,
+                           "-o", tmp, "-L" + HERE, "-l:libtsd.so", "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, NATIVE)
     return LIB
 
 

@@ -17,6 +17,7 @@
 // keep their position in the forest, per-tree outputs are tree-major ([2, batch, ...]).
 #include <limits.h>
 #include <math_constants.h>
+#include <algorithm>
 #include "tsd_common.cuh"
 
 namespace tsd {
@@ -249,42 +250,48 @@ accept_kernel(int B_all, int n_cur, int R, const int32_t* __restrict__ parent, c
 
 }  // namespace tsd
 
-static int accept_launch(int32_t batch, int32_t n_branches, int32_t n_cur, int32_t rows_per_branch,
-                         const int32_t* parent, const int32_t* state, int32_t mask_id, const float* conf,
-                         const int32_t* top1_idx, int32_t top1_stride, float tau, int32_t rule,
-                         int32_t search, uint8_t* edge_valid, int32_t* prefix_len, int32_t* accepted_node,
-                         int32_t* accepted_len, int32_t* n_new_tokens, uint8_t* unmask_flag,
-                         int32_t* unmask_tok, uint32_t* status, tsd_stream_t stream,
-                         const tsd::RelaxedArgs& x) {
-  if (batch < 0 || n_cur < 1 || n_cur > n_branches || n_branches < 1 || n_branches > tsd::kMaxBranches || rows_per_branch < 1 ||
-      rows_per_branch > tsd::kMaxRows || top1_stride < 1)
+namespace tsd {
+
+static int check_accept(const AcceptArgs& a, const RelaxedArgs& x) {
+  if (a.batch < 0 || a.n_cur < 1 || a.n_cur > a.n_branches || a.n_branches < 1 || a.n_branches > kMaxBranches ||
+      a.rows_per_branch < 1 || a.rows_per_branch > kMaxRows || a.top1_stride < 1)
     return TSD_ERR_INVALID_ARG;
-  if (rule < TSD_ACCEPT_EXACT || rule > TSD_ACCEPT_PROB) return TSD_ERR_INVALID_ARG;
-  if (rule == TSD_ACCEPT_TOPK && (x.topk_m < 1 || x.topk_m > top1_stride)) return TSD_ERR_INVALID_ARG;
-  if (rule == TSD_ACCEPT_PROB && !x.logits) return TSD_ERR_INVALID_ARG;
+  if (a.rule < TSD_ACCEPT_EXACT || a.rule > TSD_ACCEPT_PROB) return TSD_ERR_INVALID_ARG;
+  if (a.rule == TSD_ACCEPT_TOPK && (x.topk_m < 1 || x.topk_m > a.top1_stride)) return TSD_ERR_INVALID_ARG;
+  if (a.rule == TSD_ACCEPT_PROB && !x.logits) return TSD_ERR_INVALID_ARG;
   if (x.logits) {
     if (x.dtype != TSD_F32 && x.dtype != TSD_BF16) return TSD_ERR_UNSUPPORTED;
     if (!x.lse || x.vocab < 1 || x.ld < x.vocab) return TSD_ERR_INVALID_ARG;
   }
-  if (search != TSD_SEARCH_GREEDY && search != TSD_SEARCH_LONGEST) return TSD_ERR_INVALID_ARG;
-  if (!(tau == tau)) return TSD_ERR_INVALID_ARG;  // NaN threshold
-  if (batch == 0) return TSD_OK;
-  if (!parent || !state || !conf || !top1_idx || !edge_valid || !prefix_len || !accepted_node ||
-      !accepted_len || !n_new_tokens || !unmask_flag || !unmask_tok)
+  if (a.search != TSD_SEARCH_GREEDY && a.search != TSD_SEARCH_LONGEST) return TSD_ERR_INVALID_ARG;
+  if (!(a.tau == a.tau)) return TSD_ERR_INVALID_ARG;  // NaN threshold
+  if (a.batch == 0) return TSD_OK;
+  if (!a.parent || !a.state || !a.conf || !a.top1_idx || !a.edge_valid || !a.prefix_len || !a.accepted_node ||
+      !a.accepted_len || !a.n_new_tokens || !a.unmask_flag || !a.unmask_tok)
     return TSD_ERR_INVALID_ARG;
-  const dim3 grid(batch, n_cur < n_branches ? 2 : 1);
-  const int tree_max = n_cur > n_branches - n_cur ? n_cur : n_branches - n_cur;
-  const int threads = tree_max * 32 < tsd::kAcceptThreads ? tsd::kAcceptThreads
-                      : (tree_max * 32 > tsd::kAcceptMaxThreads ? tsd::kAcceptMaxThreads : tree_max * 32);
-  auto kernel = rows_per_branch <= 32 ? tsd::accept_kernel<1>
-                : rows_per_branch <= 64 ? tsd::accept_kernel<2> : tsd::accept_kernel<tsd::kRowWords>;
-  cudaError_t e = tsd::launch(
-      kernel, grid, threads, 0, stream, n_branches, n_cur, rows_per_branch, parent, state, mask_id, conf, top1_idx, top1_stride, tau, rule,
-      search, edge_valid, prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag,
-      unmask_tok, status, x);
-  if (e != cudaSuccess) return tsd::cuda_fail(e, "accept_kernel");
   return TSD_OK;
 }
+
+static int launch_accept(const AcceptArgs& a, const RelaxedArgs& x) {
+  if (a.batch == 0) return TSD_OK;
+  const dim3 grid(a.batch, a.n_cur < a.n_branches ? 2 : 1);
+  const int tree_max = std::max(a.n_cur, a.n_branches - a.n_cur);
+  const int threads = std::min(std::max(tree_max * 32, kAcceptThreads), kAcceptMaxThreads);
+  auto kernel = a.rows_per_branch <= 32 ? accept_kernel<1> : a.rows_per_branch <= 64 ? accept_kernel<2> : accept_kernel<kRowWords>;
+  cudaError_t e = launch(kernel, grid, threads, 0, a.stream, a.n_branches, a.n_cur, a.rows_per_branch, a.parent, a.state,
+                         a.mask_id, a.conf, a.top1_idx, a.top1_stride, a.tau, a.rule, a.search, a.edge_valid,
+                         a.prefix_len, a.accepted_node, a.accepted_len, a.n_new_tokens, a.unmask_flag, a.unmask_tok,
+                         a.status, x);
+  return e != cudaSuccess ? cuda_fail(e, "accept_kernel") : TSD_OK;
+}
+
+int check_accept_exact(const AcceptArgs& a) {
+  if (a.rule != TSD_ACCEPT_EXACT && a.rule != TSD_ACCEPT_TOP1) return TSD_ERR_INVALID_ARG;
+  return check_accept(a, RelaxedArgs{});
+}
+int launch_accept_exact(const AcceptArgs& a) { return launch_accept(a, RelaxedArgs{}); }
+
+}  // namespace tsd
 
 extern "C" int tsd_accept_trajectories(int32_t batch, int32_t n_branches, int32_t rows_per_branch,
                                        const int32_t* parent, const int32_t* state, int32_t mask_id,
@@ -294,10 +301,9 @@ extern "C" int tsd_accept_trajectories(int32_t batch, int32_t n_branches, int32_
                                        int32_t* accepted_len, int32_t* n_new_tokens,
                                        uint8_t* unmask_flag, int32_t* unmask_tok, uint32_t* status,
                                        tsd_stream_t stream) {
-  if (rule != TSD_ACCEPT_EXACT && rule != TSD_ACCEPT_TOP1) return TSD_ERR_INVALID_ARG;
-  return accept_launch(batch, n_branches, n_branches, rows_per_branch, parent, state, mask_id, conf, top1_idx,
-                       top1_stride, tau, rule, search, edge_valid, prefix_len, accepted_node, accepted_len,
-                       n_new_tokens, unmask_flag, unmask_tok, status, stream, tsd::RelaxedArgs{});
+  return tsd_accept_joint_trees(batch, n_branches, n_branches, rows_per_branch, parent, state, mask_id, conf, top1_idx,
+                                top1_stride, tau, rule, search, edge_valid, prefix_len, accepted_node, accepted_len,
+                                n_new_tokens, unmask_flag, unmask_tok, status, stream);
 }
 
 extern "C" int tsd_accept_joint_trees(int32_t batch, int32_t n_branches, int32_t n_cur,
@@ -307,10 +313,11 @@ extern "C" int tsd_accept_joint_trees(int32_t batch, int32_t n_branches, int32_t
                                       uint8_t* edge_valid, int32_t* prefix_len, int32_t* accepted_node,
                                       int32_t* accepted_len, int32_t* n_new_tokens, uint8_t* unmask_flag,
                                       int32_t* unmask_tok, uint32_t* status, tsd_stream_t stream) {
-  if (rule != TSD_ACCEPT_EXACT && rule != TSD_ACCEPT_TOP1) return TSD_ERR_INVALID_ARG;
-  return accept_launch(batch, n_branches, n_cur, rows_per_branch, parent, state, mask_id, conf, top1_idx,
-                       top1_stride, tau, rule, search, edge_valid, prefix_len, accepted_node, accepted_len,
-                       n_new_tokens, unmask_flag, unmask_tok, status, stream, tsd::RelaxedArgs{});
+  const tsd::AcceptArgs a = {batch, n_branches, n_cur, rows_per_branch, parent, state, mask_id, conf, top1_idx, top1_stride,
+                             tau, rule, search, edge_valid, prefix_len, accepted_node, accepted_len, n_new_tokens,
+                             unmask_flag, unmask_tok, status, stream};
+  const int rc = tsd::check_accept_exact(a);
+  return rc != TSD_OK ? rc : tsd::launch_accept_exact(a);
 }
 
 extern "C" int tsd_accept_relaxed(int32_t batch, int32_t n_branches, int32_t n_cur, int32_t rows_per_branch,
@@ -330,7 +337,9 @@ extern "C" int tsd_accept_relaxed(int32_t batch, int32_t n_branches, int32_t n_c
   x.ld = row_stride;
   x.lse = lse;
   x.draft_prob = logits ? draft_prob : nullptr;
-  return accept_launch(batch, n_branches, n_cur, rows_per_branch, parent, state, mask_id, conf, topk_idx,
-                       topk_stride, tau, rule, search, edge_valid, prefix_len, accepted_node, accepted_len,
-                       n_new_tokens, unmask_flag, unmask_tok, status, stream, x);
+  const tsd::AcceptArgs a = {batch, n_branches, n_cur, rows_per_branch, parent, state, mask_id, conf, topk_idx, topk_stride,
+                             tau, rule, search, edge_valid, prefix_len, accepted_node, accepted_len, n_new_tokens,
+                             unmask_flag, unmask_tok, status, stream};
+  const int rc = tsd::check_accept(a, x);
+  return rc != TSD_OK ? rc : tsd::launch_accept(a, x);
 }

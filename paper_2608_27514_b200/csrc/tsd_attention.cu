@@ -32,6 +32,10 @@ int check_attention_args(const tsd_layout* L, const void* mask, const void* q, i
   return TSD_OK;
 }
 
+int launch_attention(const AttnArgs& a, uint32_t flags) {
+  return !(flags & TSD_ATTN_FORCE_SIMT) && attention_tc_supported(a) ? launch_attention_tc(a) : launch_attention_simt(a);
+}
+
 }  // namespace tsd
 
 extern "C" {
@@ -68,11 +72,8 @@ int tsd_verify_attention(const tsd_layout* L, const void* mask, const void* q, i
   a.workspace_bytes = workspace_bytes;
   a.status = status;
   a.stream = stream;
-  if (!(flags & TSD_ATTN_FORCE_SIMT) && tsd::attention_tc_supported(a)) {
-    if (workspace_bytes < tsd::attention_tc_workspace_bytes(*L)) return TSD_ERR_WORKSPACE;
-    return tsd::launch_attention_tc(a);
-  }
-  return tsd::launch_attention_simt(a);
+  a.launch_next = false;
+  return tsd::launch_attention(a, flags);
 }
 
 }  // extern "C"

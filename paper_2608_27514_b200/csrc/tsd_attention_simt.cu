@@ -71,7 +71,8 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
                       const T* __restrict__ vc, const T* __restrict__ kd, const T* __restrict__ vd,
                       T* __restrict__ out, float* __restrict__ lse, int64_t qs_b, int64_t qs_r, int64_t qs_h,
                       int64_t cs_b, int64_t cs_r, int64_t cs_h, int64_t ds_b, int64_t ds_r, int64_t ds_h,
-                      int64_t os_b, int64_t os_r, int64_t os_h, float sm_scale, uint32_t* __restrict__ status) {
+                      int64_t os_b, int64_t os_r, int64_t os_h, float sm_scale, uint32_t* __restrict__ status,
+                      int launch_next) {
   constexpr int LPK = D / 8;            // lanes per key
   constexpr int KPI = 32 / LPK;         // keys read at once
   constexpr int SUB = LPK / RB;         // reads per group: SUB * RB scores per key lane, one per lane after the scatter
@@ -91,7 +92,7 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
   const int j = lane % LPK, slots = kTile / R;
   const unsigned full = 0xffffffffu;
   grid_wait(mask, q, kc, vc, kd, vd);
-  grid_launch_next();
+  if (launch_next) grid_launch_next();
 
   // the block's query rows, 8 dimensions per lane (requested first: nothing else is needed for them)
   float qr[RB][8];
@@ -269,7 +270,8 @@ static cudaError_t launch_rows(const AttnArgs& a, int warps) {
       attention_rows_kernel<T, D, RB, MAXW>, grid, std::min(warps, MAXW) * 32, 0, a.stream, L.batch, L.n_branches, L.rows_per_branch, L.n_cache, L.n_q_heads, L.n_kv_heads, md.recs_off, md.n_qt,
       md.rec_words, a.mask, static_cast<const T*>(a.q), static_cast<const T*>(a.kc), static_cast<const T*>(a.vc),
       static_cast<const T*>(a.kd), static_cast<const T*>(a.vd), static_cast<T*>(a.out), a.lse, a.qs_b, a.qs_r,
-      a.qs_h, a.cs_b, a.cs_r, a.cs_h, a.ds_b, a.ds_r, a.ds_h, a.os_b, a.os_r, a.os_h, a.sm_scale, a.status);
+      a.qs_h, a.cs_b, a.cs_r, a.cs_h, a.ds_b, a.ds_r, a.ds_h, a.os_b, a.os_r, a.os_h, a.sm_scale, a.status,
+      (int)a.launch_next);
 }
 
 template <typename T, int D>

@@ -63,11 +63,51 @@ struct AttnArgs {
   size_t workspace_bytes;
   uint32_t* status;
   cudaStream_t stream;
+  bool launch_next;  // let the next kernel of the stream start as soon as every block of this one runs
 };
 int launch_attention_simt(const AttnArgs& a);
 bool attention_tc_supported(const AttnArgs& a);
 size_t attention_tc_workspace_bytes(const tsd_layout& L);
 int launch_attention_tc(const AttnArgs& a);
+int launch_attention(const AttnArgs& a, uint32_t flags);
+
+// The vocabulary pass and the acceptance behind their entry points.  `concurrent`: the pass reads nothing
+// that the kernel before it in the stream writes, and may run beside it.
+struct TopkArgs {
+  const void* logits;
+  int32_t dtype;
+  int64_t n_rows;
+  int32_t vocab;
+  int64_t row_stride;
+  int32_t k;
+  float* conf;
+  int32_t* topk_idx;
+  float *topk_prob, *lse;
+  void* workspace;
+  size_t workspace_bytes;
+  cudaStream_t stream;
+  bool concurrent;
+};
+int check_topk(const TopkArgs& a);
+int launch_topk(const TopkArgs& a);
+struct AcceptArgs {
+  int32_t batch, n_branches, n_cur, rows_per_branch;
+  const int32_t *parent, *state;
+  int32_t mask_id;
+  const float* conf;
+  const int32_t* top1_idx;
+  int32_t top1_stride;
+  float tau;
+  int32_t rule, search;
+  uint8_t* edge_valid;
+  int32_t *prefix_len, *accepted_node, *accepted_len, *n_new_tokens;
+  uint8_t* unmask_flag;
+  int32_t* unmask_tok;
+  uint32_t* status;
+  cudaStream_t stream;
+};
+int check_accept_exact(const AcceptArgs& a);  // rules EXACT and TOP1
+int launch_accept_exact(const AcceptArgs& a);
 
 // ---- programmatic dependent launch ----
 // Every kernel is launched so that it may be set up while its predecessor in the stream still runs, and

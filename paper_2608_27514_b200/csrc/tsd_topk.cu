@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(THREADS)
 confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, int k, int n_seg,
                        int chunks_per_seg, float* __restrict__ conf, int32_t* __restrict__ topk_idx,
                        float* __restrict__ topk_prob, float* __restrict__ lse,
-                       Partial<K>* __restrict__ partials, unsigned* __restrict__ tickets, int prefetch) {
+                       Partial<K>* __restrict__ partials, unsigned* __restrict__ tickets, int prefetch, int concurrent) {
   constexpr int E_ = Unpack<T>::kElems;
   constexpr int kTopkThreads = THREADS, kTopkWarps = THREADS / 32;
   constexpr int kTopkBatch = THREADS * kTopkUnroll;        // chunks per block per batch
@@ -273,7 +273,17 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   const int n_iter = (c1 - c0 + kTopkBatch - 1) / kTopkBatch;  // <= kTopkMaxIter (host-enforced)
   const bool has_tail = seg == n_seg - 1 && tid == 0 && chunks_total * E_ < vocab;
 
-  grid_wait(rowp, rowv);
+  // Normally the kernel before this one may have written the logits.  A concurrent pass reads only what was
+  // there before that kernel started; it takes an acquire fence in place of the wait, so that no line the SM
+  // still holds from earlier kernels is used, and its last block stays until that kernel has completed, so that
+  // a kernel which waits for this one has waited for both.
+  if (concurrent) {
+    __threadfence();
+    settle(rowp, rowv);
+  } else {
+    grid_wait(rowp, rowv);
+  }
+  const bool stay = concurrent && warp == 1 && blockIdx.x == gridDim.x - 1;
 
   // ---- phase 1: stream.  Two register buffers: the loads of batch it+1 are in flight while
   // batch it is processed, so a block overlaps memory latency with its own arithmetic.
@@ -435,6 +445,7 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
       for (int j = 0; j < K; ++j) { s_part[warp].v[j] = a.v[j]; s_part[warp].i[j] = a.i[j]; }
     }
     __syncthreads();
+    if (stay) grid_wait();
     if (warp != 0) return;
     a.init();
     if (lane < kTopkWarps) {
@@ -446,6 +457,7 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
     }
     warp_merge(a);
   } else {
+    if (stay) grid_wait();
     if (warp != 0) return;
     // sum of the warps' sums (fixed tree), and the pool's best K by rank: every lane counts the
     // entries that come before its own (keys are unique), so rank r goes to slot r without a sort
@@ -538,45 +550,71 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
 }
 
 template <typename T, int K>
-static cudaError_t launch_topk(const void* logits, int64_t n_rows, int vocab, int64_t row_stride, int k,
-                               const TopkPlan& p, float* conf, int32_t* idx, float* prob, float* lse,
-                               void* ws, cudaStream_t st) {
+static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   Partial<K>* partials = reinterpret_cast<Partial<K>*>(ws);
   unsigned* tickets = reinterpret_cast<unsigned*>(static_cast<char*>(ws) + p.ticket_off);
   auto kernel = p.threads == 512 ? confidence_topk_kernel<T, K, 512> : confidence_topk_kernel<T, K, 256>;
-  return launch(kernel, (unsigned)(n_rows * p.n_seg), p.threads, 0, st, static_cast<const T*>(logits), vocab, row_stride, k,
-                p.n_seg, p.chunks_per_seg, conf, idx, prob, lse, partials, tickets, p.prefetch);
+  return launch(kernel, (unsigned)(a.n_rows * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
+                a.row_stride, a.k, p.n_seg, p.chunks_per_seg, a.conf, a.topk_idx, a.topk_prob, a.lse, partials, tickets,
+                p.prefetch, (int)a.concurrent);
 }
 
 template <typename T>
-static cudaError_t dispatch_k(int K, const void* logits, int64_t n_rows, int vocab, int64_t row_stride,
-                              int k, const TopkPlan& p, float* conf, int32_t* idx, float* prob,
-                              float* lse, void* ws, cudaStream_t st) {
-  switch (K) {
-    case 1: return launch_topk<T, 1>(logits, n_rows, vocab, row_stride, k, p, conf, idx, prob, lse, ws, st);
-    case 2: return launch_topk<T, 2>(logits, n_rows, vocab, row_stride, k, p, conf, idx, prob, lse, ws, st);
-    case 3: return launch_topk<T, 3>(logits, n_rows, vocab, row_stride, k, p, conf, idx, prob, lse, ws, st);
-    case 4: return launch_topk<T, 4>(logits, n_rows, vocab, row_stride, k, p, conf, idx, prob, lse, ws, st);
-    case 6: return launch_topk<T, 6>(logits, n_rows, vocab, row_stride, k, p, conf, idx, prob, lse, ws, st);
-    default: return launch_topk<T, 8>(logits, n_rows, vocab, row_stride, k, p, conf, idx, prob, lse, ws, st);
+static cudaError_t dispatch_k(const TopkArgs& a, const TopkPlan& p, void* ws) {
+  switch (p.K) {
+    case 1: return run_plan<T, 1>(a, p, ws);
+    case 2: return run_plan<T, 2>(a, p, ws);
+    case 3: return run_plan<T, 3>(a, p, ws);
+    case 4: return run_plan<T, 4>(a, p, ws);
+    case 6: return run_plan<T, 6>(a, p, ws);
+    default: return run_plan<T, 8>(a, p, ws);
   }
+}
+
+static int check_shape(int64_t n_rows, int32_t vocab, int32_t k) {
+  if (n_rows < 0 || vocab < 1 || k < 1 || k > 8 || k > vocab) return TSD_ERR_INVALID_ARG;
+  if (n_rows * (int64_t)kMaxSegments > 0x7fffffffLL) return TSD_ERR_INVALID_ARG;
+  // rows longer than kMaxSegments segments of kTopkMaxIter batches (4 Mi fp32 / 8 Mi bf16 logits)
+  if ((int64_t)vocab / 4 > (int64_t)kTopkSegChunks * kMaxSegments) return TSD_ERR_INVALID_ARG;
+  return TSD_OK;
+}
+
+// Everything but the workspace.
+static int check_pointers(const TopkArgs& a) {
+  int rc = check_shape(a.n_rows, a.vocab, a.k);
+  if (rc != TSD_OK) return rc;
+  if (a.dtype != TSD_F32 && a.dtype != TSD_BF16) return TSD_ERR_UNSUPPORTED;
+  if (a.n_rows == 0) return TSD_OK;
+  const int esize = a.dtype == TSD_F32 ? 4 : 2;
+  if (!a.logits || !a.conf || !a.topk_idx || !a.topk_prob) return TSD_ERR_INVALID_ARG;
+  if (a.row_stride < a.vocab || !aligned16(a.logits) || (a.row_stride * esize) % 16 != 0) return TSD_ERR_INVALID_ARG;
+  return TSD_OK;
+}
+
+int check_topk(const TopkArgs& a) {
+  int rc = check_pointers(a);
+  if (rc != TSD_OK || a.n_rows == 0) return rc;
+  const size_t need = tsd_confidence_topk_workspace_bytes(a.n_rows, a.vocab, a.k);
+  if (need > 0) {  // the documented size is required whichever dtype is passed
+    if (!a.workspace || !aligned16(a.workspace)) return TSD_ERR_INVALID_ARG;
+    if (a.workspace_bytes < need) return TSD_ERR_WORKSPACE;
+  }
+  return TSD_OK;
+}
+
+int launch_topk(const TopkArgs& a) {
+  if (a.n_rows == 0) return TSD_OK;
+  const TopkPlan p = topk_plan(a.n_rows, a.vocab, a.k, a.dtype == TSD_F32 ? 4 : 8);
+  cudaError_t e = a.dtype == TSD_F32 ? dispatch_k<float>(a, p, a.workspace) : dispatch_k<__nv_bfloat16>(a, p, a.workspace);
+  return e != cudaSuccess ? cuda_fail(e, "confidence_topk_kernel") : TSD_OK;
 }
 
 }  // namespace tsd
 
 extern "C" {
 
-static int topk_check(int64_t n_rows, int32_t vocab, int32_t k) {
-  if (n_rows < 0 || vocab < 1 || k < 1 || k > 8 || k > vocab) return TSD_ERR_INVALID_ARG;
-  if (n_rows * (int64_t)tsd::kMaxSegments > 0x7fffffffLL) return TSD_ERR_INVALID_ARG;
-  // rows longer than kMaxSegments segments of kTopkMaxIter batches (4 Mi fp32 / 8 Mi bf16 logits)
-  if ((int64_t)vocab / 4 > (int64_t)tsd::kTopkSegChunks * tsd::kMaxSegments)
-    return TSD_ERR_INVALID_ARG;
-  return TSD_OK;
-}
-
 size_t tsd_confidence_topk_workspace_bytes(int64_t n_rows, int32_t vocab, int32_t k) {
-  if (topk_check(n_rows, vocab, k) != TSD_OK || n_rows == 0) return 0;
+  if (tsd::check_shape(n_rows, vocab, k) != TSD_OK || n_rows == 0) return 0;
   // sized for the narrower element type (more chunks per row can only mean more segments)
   const size_t a = tsd::topk_plan(n_rows, vocab, k, 8).total_bytes;
   const size_t b = tsd::topk_plan(n_rows, vocab, k, 4).total_bytes;
@@ -588,27 +626,10 @@ int tsd_confidence_topk(const void* logits, int32_t dtype, int64_t n_rows, int32
                         float* topk_prob, float* lse, void* workspace, size_t workspace_bytes,
                         uint32_t* status, tsd_stream_t stream) {
   (void)status;
-  int rc = topk_check(n_rows, vocab, k);
-  if (rc != TSD_OK) return rc;
-  if (dtype != TSD_F32 && dtype != TSD_BF16) return TSD_ERR_UNSUPPORTED;
-  if (n_rows == 0) return TSD_OK;
-  const int esize = dtype == TSD_F32 ? 4 : 2;
-  if (!logits || !conf || !topk_idx || !topk_prob) return TSD_ERR_INVALID_ARG;
-  if (row_stride < vocab || !tsd::aligned16(logits) || (row_stride * esize) % 16 != 0)
-    return TSD_ERR_INVALID_ARG;
-  const tsd::TopkPlan p = tsd::topk_plan(n_rows, vocab, k, 16 / esize);
-  const size_t need = tsd_confidence_topk_workspace_bytes(n_rows, vocab, k);
-  if (need > 0) {  // the documented size is required whichever dtype is passed
-    if (!workspace || !tsd::aligned16(workspace)) return TSD_ERR_INVALID_ARG;
-    if (workspace_bytes < need) return TSD_ERR_WORKSPACE;
-  }
-  cudaError_t e = dtype == TSD_F32
-      ? tsd::dispatch_k<float>(p.K, logits, n_rows, vocab, row_stride, k, p, conf, topk_idx, topk_prob,
-                               lse, workspace, stream)
-      : tsd::dispatch_k<__nv_bfloat16>(p.K, logits, n_rows, vocab, row_stride, k, p, conf, topk_idx,
-                                       topk_prob, lse, workspace, stream);
-  if (e != cudaSuccess) return tsd::cuda_fail(e, "confidence_topk_kernel");
-  return TSD_OK;
+  const tsd::TopkArgs a = {logits, dtype, n_rows, vocab, row_stride, k, conf, topk_idx, topk_prob, lse, workspace,
+                           workspace_bytes, stream, false};
+  int rc = tsd::check_topk(a);
+  return rc != TSD_OK ? rc : tsd::launch_topk(a);
 }
 
 }  // extern "C"
@@ -647,33 +668,20 @@ extern "C" int tsd_confidence_topk_static(const void* logits, int32_t dtype, int
                                           float* topk_prob, float* lse, uint32_t* status,
                                           tsd_stream_t stream) {
   (void)status;
-  int rc = topk_check(n_rows, vocab, k);
-  if (rc != TSD_OK) return rc;
-  if (dtype != TSD_F32 && dtype != TSD_BF16) return TSD_ERR_UNSUPPORTED;
-  if (n_rows == 0) return TSD_OK;
-  const int esize = dtype == TSD_F32 ? 4 : 2;
-  if (!logits || !conf || !topk_idx || !topk_prob) return TSD_ERR_INVALID_ARG;
-  if (row_stride < vocab || !tsd::aligned16(logits) || (row_stride * esize) % 16 != 0)
-    return TSD_ERR_INVALID_ARG;
-  const tsd::TopkPlan p = tsd::topk_plan(n_rows, vocab, k, 16 / esize);
+  tsd::TopkArgs a = {logits, dtype, n_rows, vocab, row_stride, k, conf, topk_idx, topk_prob, lse, nullptr, 0, stream, false};
+  int rc = tsd::check_pointers(a);
+  if (rc != TSD_OK || n_rows == 0) return rc;
   // this shape would need more scratch than the library carries: the caller has to use
   // tsd_confidence_topk with a workspace of its own.  The test is on the documented size
   // (tsd_confidence_topk_workspace_bytes, the larger of the two dtypes' needs), so that the check a
   // caller makes beforehand and this one agree.
   if (tsd_confidence_topk_workspace_bytes(n_rows, vocab, k) > tsd::kStaticScratchBytes) return TSD_ERR_WORKSPACE;
-  void* scratch = nullptr;
-  if (p.total_bytes > 0) {
-    cudaError_t e = tsd::static_scratch_address(&scratch);
+  if (tsd::topk_plan(n_rows, vocab, k, dtype == TSD_F32 ? 4 : 8).total_bytes > 0) {
+    cudaError_t e = tsd::static_scratch_address(&a.workspace);
     if (e != cudaSuccess) return tsd::cuda_fail(e, "cudaGetSymbolAddress(g_topk_scratch)");
   }
   // ticket words need no clearing (a word that does not carry the in-use tag counts as idle, and
   // the last arrival of a row returns it to idle); the partial-result slots are fully rewritten by
   // every call that reads them
-  cudaError_t e = dtype == TSD_F32
-      ? tsd::dispatch_k<float>(p.K, logits, n_rows, vocab, row_stride, k, p, conf, topk_idx, topk_prob,
-                               lse, scratch, stream)
-      : tsd::dispatch_k<__nv_bfloat16>(p.K, logits, n_rows, vocab, row_stride, k, p, conf, topk_idx,
-                                       topk_prob, lse, scratch, stream);
-  if (e != cudaSuccess) return tsd::cuda_fail(e, "confidence_topk_kernel (static scratch)");
-  return TSD_OK;
+  return tsd::launch_topk(a);
 }

@@ -96,10 +96,14 @@ class VerifyStep:
     def run(self, attn, logits, parent, state, mask_id, tau, rule=B.TSD_ACCEPT_EXACT,
             search=B.TSD_SEARCH_GREEDY, flags=0):
         """The whole hot path: attention -> confidence/top-k -> acceptance."""
-        self.attention(attn["q"], attn["k_cache"], attn["v_cache"], attn["k_draft"], attn["v_draft"],
-                       attn["sm_scale"], flags)
-        self.confidence_topk(logits)
-        return self.accept(parent, state, mask_id, tau, rule, search)
+        if not self.mask_built:
+            self.build_mask()
+        B.tsd_verify_step(self.layout, self.mask, attn["q"], attn["k_cache"], attn["v_cache"], attn["k_draft"], attn["v_draft"],
+                          self.out, self.attn_lse, attn["sm_scale"], self.attn_ws, flags, logits, self.k, self.conf,
+                          self.topk_idx, self.topk_prob, self.lse, self.topk_ws, parent, state, mask_id, tau, rule, search,
+                          self.edge_valid, self.prefix_len, self.accepted_node, self.accepted_len, self.n_new_tokens,
+                          self.unmask_flag, self.unmask_tok, self.status)
+        return self.accept_outputs()
 
     def check_status(self):
         rc = B.tsd_check_status(self.status)

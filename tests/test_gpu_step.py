@@ -1,0 +1,35 @@
+"""The step in one call (attention beside the vocabulary pass) against the three calls it stands for."""
+import pytest
+import torch
+
+from paper_2608_27514_b200 import workloads as W
+from paper_2608_27514_b200.step import VerifyStep
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("kw", [dict(Hq=2, Hkv=2, V=4096), dict(Hq=32, Hkv=8, B=1, Nc=64, V=152064), dict(S=3, B=9, Hq=8, Hkv=4, Nc=1000, V=32000),
+                                dict(B=64, V=126464), dict(d=64, Hq=4, Hkv=4, V=126464), dict(dtype="f32", d=64, Hq=4, Hkv=4, Nc=100, V=4096)])
+def test_step_in_one_call_equals_the_three_calls(kw):
+    # few and many rows against few and many attention items; the logits are rewritten in place before every pass, so that a
+    # pass that ran ahead of its inputs, or read what an SM had kept of the old ones, would show; every result bit for bit
+    cfg = W.small(W.CONFIGS["cfg2"], name="case", **kw)
+    attn, vi = W.attention_inputs(cfg, DEV), W.verify_inputs(cfg, DEV)
+    one, three = VerifyStep.for_config(cfg, DEV), VerifyStep.for_config(cfg, DEV)
+    logits = vi["logits"]
+    for i in range(8):
+        logits = torch.roll(logits, 1 + 37 * i, 1)
+        vi["logits"].copy_(logits)
+        attn["q"].mul_(-1.0)
+        a = one.run(attn, vi["logits"], vi["parent"], vi["state"], vi["mask_id"], cfg.tau)
+        after = one.out.clone(), one.attn_lse.clone(), one.conf.clone()
+        three.attention(attn["q"], attn["k_cache"], attn["v_cache"], attn["k_draft"], attn["v_draft"], attn["sm_scale"])
+        three.confidence_topk(vi["logits"])
+        b = three.accept(vi["parent"], vi["state"], vi["mask_id"], cfg.tau)
+        assert torch.equal(after[0], three.out) and torch.equal(after[1], three.attn_lse) and torch.equal(after[2], three.conf)
+        for x, y in ((one.topk_idx, three.topk_idx), (one.topk_prob, three.topk_prob), (one.lse, three.lse)):
+            assert torch.equal(x, y)
+        for key in a:
+            assert torch.equal(a[key], b[key]), key
+    one.check_status()
