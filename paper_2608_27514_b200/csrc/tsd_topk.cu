@@ -241,8 +241,8 @@ struct Unpack<__nv_bfloat16> {
   }
 };
 
-// grid.x = n_rows * n_seg; block = THREADS (256 when many blocks share an SM; 512 when there are so
-// few rows that a block has to keep the SM busy on its own: twice the warps per row).
+// grid.x = n_rows * n_seg; block = THREADS (256 when many blocks share an SM; 384 or 512 when there are so
+// few rows that two or three blocks have to keep the SM busy: more warps per row).
 template <typename T, int K, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, int k, int n_seg,
@@ -252,7 +252,7 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   constexpr int E_ = Unpack<T>::kElems;
   constexpr int kTopkThreads = THREADS, kTopkWarps = THREADS / 32;
   constexpr int kTopkBatch = THREADS * kTopkUnroll;        // chunks per block per batch
-  constexpr int kTopkMaxIter = kTopkSegChunks / kTopkBatch;  // batches per segment
+  constexpr int kTopkMaxIter = (kTopkSegChunks + kTopkBatch - 1) / kTopkBatch;  // batches per segment
   __shared__ float s_bmax[kTopkMaxIter][kTopkThreads];  // per-thread batch maxima
   __shared__ __align__(16) float s_wmax[kTopkWarps];  // per-warp maxima
   __shared__ float s_wsum[kTopkWarps];                // per-warp sums on the block's exponent base
@@ -522,30 +522,49 @@ struct TopkPlan {
 
 static int round_k(int k) { return k <= 4 ? k : (k <= 6 ? 6 : 8); }
 
+static void scratch_layout(int64_t n_rows, TopkPlan& p) {
+  const size_t rec = 8 + 8 * (size_t)p.K;
+  p.partial_bytes = p.n_seg > 1 ? (size_t)n_rows * p.n_seg * rec : 0;
+  p.ticket_off = (p.partial_bytes + 15) / 16 * 16;
+  p.total_bytes = p.n_seg > 1 ? p.ticket_off + ((size_t)n_rows * 4 + 15) / 16 * 16 : 0;
+}
+
+// The workspace query's answer: room for as many segments as give every SM at least one block, whether or not a
+// plan uses as many, so that the size a caller has to provide does not follow the tuning of the plans.
+static size_t workspace_bytes(int64_t n_rows, int vocab, int k, int elems_per_chunk) {
+  const int chunks = vocab / elems_per_chunk;
+  TopkPlan p;
+  p.K = round_k(k);
+  const int64_t n_seg = std::min<int64_t>(std::min<int64_t>((148 + n_rows - 1) / n_rows, kMaxSegments), std::max(1, chunks / 2048));
+  p.n_seg = (int)std::max<int64_t>(n_seg, (chunks + kTopkSegChunks - 1) / kTopkSegChunks);
+  scratch_layout(n_rows, p);
+  return p.total_bytes;
+}
+
 static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk) {
   TopkPlan p;
   p.K = round_k(k);
   const int chunks = vocab / elems_per_chunk;
-  // Few rows: split rows only until every SM has a block (more segments add per-block latency
-  // and merge work faster than they add parallelism; measured on cfg2- and cfg3-sized inputs).
-  const int64_t target_units = 148;
-  int64_t n_seg = n_rows >= target_units ? 1 : (target_units + n_rows - 1) / n_rows;
+  // Few rows: split rows as long as every segment has an SM of its own.  (One more segment per row, so that every
+  // SM has one and some have two, costs more than the idle SMs: 32 rows x 152064 bf16 in 5 segments 10.2 us, in
+  // 4 segments 9.4; 100 x 126464 in 2 segments 13.4, whole 11.8.)
+  int64_t n_seg = n_rows > 0 ? 148 / n_rows : 1;
   n_seg = std::min<int64_t>(n_seg, kMaxSegments);
   n_seg = std::min<int64_t>(n_seg, std::max(1, chunks / 2048));
   // a segment may span at most kTopkSegChunks chunks (its batch maxima live in shared memory)
   n_seg = std::max<int64_t>(n_seg, (chunks + kTopkSegChunks - 1) / kTopkSegChunks);
   p.n_seg = (int)std::max<int64_t>(n_seg, 1);
-  // up to two 512-thread blocks fit an SM: use them while that still gives every block a slot at once
-  p.threads = (n_rows * p.n_seg <= 2 * 148) ? 512 : 256;
-  // L2 prefetch distance in batches (measured): with several waves of blocks, requesting lines
-  // three batches ahead adds 3 % of bandwidth; with few blocks it only delays the demand loads
-  p.prefetch = (n_rows * p.n_seg >= 2048) ? 3 : 0;
+  // As many warps per row as still give every block a slot at once: 256 x 126464 bf16 with 512 threads 17.0 us, with
+  // 384 17.9, with 256 18.8; 444 x 126464 25.0 / 23.5 / 24.4; 960 x 126464 50.2 / 48.2 / 46.0.
+  const int64_t units = n_rows * p.n_seg;
+  p.threads = units <= 2 * 148 ? 512 : (units <= 3 * 148 ? 384 : 256);
+  // L2 prefetch distance in batches (measured): with very many waves of blocks, requesting lines three batches ahead
+  // adds 2 % of bandwidth (16384 x 126464: 687 us, without 700); with fewer it delays the demand loads (4096 x 32000:
+  // 57.0 us, without 53.6; 4096 x 126464: 171 and 167; 4096 x 152064: 189.7 and 190.8)
+  p.prefetch = units >= 8192 ? 3 : 0;
   p.chunks_per_seg = (chunks + p.n_seg - 1) / p.n_seg;
   if (p.chunks_per_seg == 0) p.chunks_per_seg = 1;
-  const size_t rec = 8 + 8 * (size_t)p.K;
-  p.partial_bytes = p.n_seg > 1 ? (size_t)n_rows * p.n_seg * rec : 0;
-  p.ticket_off = (p.partial_bytes + 15) / 16 * 16;
-  p.total_bytes = p.n_seg > 1 ? p.ticket_off + ((size_t)n_rows * 4 + 15) / 16 * 16 : 0;
+  scratch_layout(n_rows, p);
   return p;
 }
 
@@ -553,7 +572,8 @@ template <typename T, int K>
 static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   Partial<K>* partials = reinterpret_cast<Partial<K>*>(ws);
   unsigned* tickets = reinterpret_cast<unsigned*>(static_cast<char*>(ws) + p.ticket_off);
-  auto kernel = p.threads == 512 ? confidence_topk_kernel<T, K, 512> : confidence_topk_kernel<T, K, 256>;
+  auto kernel = p.threads == 512 ? confidence_topk_kernel<T, K, 512>
+              : p.threads == 384 ? confidence_topk_kernel<T, K, 384> : confidence_topk_kernel<T, K, 256>;
   return launch(kernel, (unsigned)(a.n_rows * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
                 a.row_stride, a.k, p.n_seg, p.chunks_per_seg, a.conf, a.topk_idx, a.topk_prob, a.lse, partials, tickets,
                 p.prefetch, (int)a.concurrent);
@@ -616,9 +636,7 @@ extern "C" {
 size_t tsd_confidence_topk_workspace_bytes(int64_t n_rows, int32_t vocab, int32_t k) {
   if (tsd::check_shape(n_rows, vocab, k) != TSD_OK || n_rows == 0) return 0;
   // sized for the narrower element type (more chunks per row can only mean more segments)
-  const size_t a = tsd::topk_plan(n_rows, vocab, k, 8).total_bytes;
-  const size_t b = tsd::topk_plan(n_rows, vocab, k, 4).total_bytes;
-  return a > b ? a : b;
+  return std::max(tsd::workspace_bytes(n_rows, vocab, k, 8), tsd::workspace_bytes(n_rows, vocab, k, 4));
 }
 
 int tsd_confidence_topk(const void* logits, int32_t dtype, int64_t n_rows, int32_t vocab,

@@ -345,6 +345,16 @@ def test_topk_ragged_vocab_and_heavy_ties(dtype, k):
         _check_topk(buf[:, :V], min(k, V))
 
 
+@pytest.mark.parametrize("n,V", [(73, 40000), (75, 40000), (148, 5000), (149, 5000), (296, 3000), (297, 3000), (444, 3000), (445, 3000),
+                                 (8191, 300), (8192, 300), (320, 262136)])
+def test_topk_at_the_borders_of_its_plans(n, V):
+    # either side of every row count at which segments, threads per block or prefetch change, and the longest row of one segment
+    # under 384 threads, whose last batch is a partial one
+    g = torch.Generator(device=DEV).manual_seed(n)
+    x = (torch.randn((n, (V + 7) // 8 * 8), generator=g, device=DEV) * 3).bfloat16()[:, :V]
+    _check_topk(x, 3, rows=sorted({0, 1, n // 2, n - 2, n - 1}))
+
+
 @pytest.mark.parametrize("seed", range(10))
 def test_topk_random_rows_vocab_k_and_dtype(seed):
     # sizes drawn at random: one value per row up to a wide vocabulary, one row up to several waves of
