@@ -535,6 +535,71 @@ typedef struct {
 } tsd_step_args;
 int tsd_verify_step(const tsd_step_args* args, tsd_stream_t stream);
 
+/* ---------------------------------------------------------------------------
+ * The decode loop of one block (Alg. 1) in two calls.
+ *
+ * tsd_begin_block starts a block from root_state [batch, R]: parent [batch, B],
+ * state [batch, B, R] and n_nodes [batch] become the tree that is its root alone
+ * (copies in the unused slots), root_out = root_state, fill_step [batch, R] = -1,
+ * step_base [batch] = 0, n_masked [batch] = rows still masked.
+ *
+ * tsd_advance_block is one pass after the model's forward: tsd_confidence_topk on
+ * the logits of every node (batch * B * R rows), the acceptance under `rule`
+ * (TSD_ACCEPT_TOPK with topk_m = k; draft_prob, nullable, is written under
+ * TSD_ACCEPT_PROB only), tsd_commit_accepted and tsd_build_draft_tree into next_*,
+ * arguments as for those calls (max_nodes = B, a tree of its own).  next_* must not
+ * overlap the tree that is verified.
+ *
+ * report, ticket: how the host learns the number of masked rows without a copy or a
+ * synchronisation.  report is memory that host and device both address (pinned host
+ * memory), one 64-bit word per sequence, 8-byte aligned, nullable in tsd_advance_block:
+ * ticket << 32 | status bits << 16 | rows still masked.  tsd_wait_block waits until
+ * every word carries `ticket`, then gives the largest count and the OR of the status
+ * bits (as the words of the device status array stood when they were reported); it
+ * fails instead of waiting for good when the stream has failed or has run dry.
+ * tsd_report_block writes the words from n_masked as it stands.
+ * ------------------------------------------------------------------------- */
+int tsd_begin_block(int32_t batch, int32_t n_branches, int32_t rows_per_branch, int32_t mask_id,
+                    const int32_t* root_state, int32_t* parent, int32_t* state, int32_t* n_nodes,
+                    int32_t* root_out, int32_t* fill_step, int32_t* step_base, int32_t* n_masked,
+                    tsd_stream_t stream);
+typedef struct {
+  int32_t batch, n_branches, rows_per_branch;
+  const void* logits;
+  int64_t row_stride;
+  int32_t logits_dtype, vocab, k;
+  float* conf;
+  int32_t* topk_idx;
+  float *topk_prob, *lse;
+  void* topk_workspace;
+  size_t topk_workspace_bytes;
+  const int32_t *parent, *state;
+  int32_t mask_id;
+  float tau;
+  int32_t rule, search;
+  uint8_t* edge_valid;
+  int32_t *prefix_len, *accepted_node, *accepted_len, *n_new_tokens;
+  uint8_t* unmask_flag;
+  int32_t* unmask_tok;
+  float* draft_prob;
+  int32_t* tokens;
+  int64_t seq_stride;
+  const int32_t* block_start;
+  int32_t *root_out, *fill_step, *step_base, *n_masked;
+  int32_t width, depth;
+  int32_t *next_parent, *next_state;
+  float* next_prob;
+  int32_t* next_n;
+  uint64_t* report;
+  uint32_t ticket;
+  uint32_t* status;
+} tsd_advance_args;
+int tsd_advance_block(const tsd_advance_args* args, tsd_stream_t stream);
+int tsd_report_block(int32_t batch, const int32_t* n_masked, const uint32_t* status, uint64_t* report,
+                     uint32_t ticket, tsd_stream_t stream);
+int tsd_wait_block(int32_t batch, const uint64_t* report, uint32_t ticket, int32_t* max_masked,
+                   uint32_t* status_bits, tsd_stream_t stream);
+
 #ifdef __cplusplus
 }
 #endif

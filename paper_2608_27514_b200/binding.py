@@ -31,6 +31,7 @@ EXPORTS = (
     "tsd_build_interblock_vis", "tsd_interblock_trigger", "tsd_accept_joint_trees", "tsd_accept_relaxed",
     "tsd_commit_accepted", "tsd_verify_attention_fp8_cache_workspace_bytes", "tsd_verify_attention_fp8_cache",
     "tsd_gather_accepted_kv", "tsd_selftest_bounded_wait", "tsd_verify_step",
+    "tsd_begin_block", "tsd_advance_block", "tsd_report_block", "tsd_wait_block",
 )
 
 
@@ -303,3 +304,28 @@ def tsd_verify_step(layout, mask, q, k_cache, v_cache, k_draft, v_draft, out, at
     native().verify_step(layout, mask, q, k_cache, v_cache, k_draft, v_draft, out, attn_lse, sm_scale, attn_workspace, flags, logits,
                          k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search, edge_valid,
                          prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, status, stream)
+
+
+def tsd_begin_block(root_state, mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, stream=None):
+    """root_state int32 [S,R]; everything else is written."""
+    native().begin_block(root_state, mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, stream)
+
+
+def tsd_advance_block(logits, k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search, edge_valid,
+                      prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, draft_prob, tokens, block_start,
+                      root_out, fill_step, step_base, n_masked, width, depth, next_parent, next_state, next_prob, next_n, report=None,
+                      ticket=0, status=None, stream=None):
+    """Vocabulary pass, acceptance, commit and next tree of one pass; report: pinned int64 [S] or None."""
+    native().advance_block(logits, k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search,
+                           edge_valid, prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, draft_prob,
+                           tokens, block_start, root_out, fill_step, step_base, n_masked, width, depth, next_parent, next_state,
+                           next_prob, next_n, report, ticket, status, stream)
+
+
+def tsd_report_block(n_masked, status, report, ticket, stream=None):
+    native().report_block(n_masked, status, report, ticket, stream)
+
+
+def tsd_wait_block(report, ticket, stream=None):
+    """(largest number of masked rows, status bits) of the pass that reported `ticket`."""
+    return native().wait_block(report, ticket, stream)

@@ -8,87 +8,14 @@
 // next root is written into the sequence's token buffer at the block's position, and the block's
 // step counter moves on by depth + 1 (depth, if the accepted node had nothing left to unmask).
 #include <algorithm>
-#include "tsd_common.cuh"
+#include "tsd_commit.cuh"
 
 namespace tsd {
 
-constexpr int kCommitMaxRows = 128;
-constexpr int kCommitRowsPerLane = kCommitMaxRows / 32;
-constexpr int kCommitMaxBranches = 256;
-
-__global__ void __launch_bounds__(32)
-commit_kernel(int B, int R, int root, const int32_t* __restrict__ parent, const int32_t* __restrict__ state,
-              const int32_t* __restrict__ accepted_node, const uint8_t* __restrict__ unmask_flag,
-              const int32_t* __restrict__ unmask_tok, int mask_id, int32_t* __restrict__ tokens,
-              int64_t seq_stride, const int32_t* __restrict__ block_start, int32_t* __restrict__ root_out,
-              int32_t* __restrict__ fill_step, int32_t* __restrict__ step_base,
-              int32_t* __restrict__ n_masked, uint32_t* __restrict__ status) {
-  __shared__ int s_path[kCommitMaxBranches];  // accepted node first, root last
-  __shared__ int s_depth;
-  grid_wait(parent, state, accepted_node, unmask_flag, unmask_tok, block_start);
+__global__ void __launch_bounds__(32) commit_kernel(const CommitArgs a) {
+  grid_wait();
   grid_launch_next();
-  const int s = blockIdx.x, lane = threadIdx.x;
-  const int32_t* par = parent + (size_t)s * B;
-  const int32_t* st = state + (size_t)s * B * R;
-  if (lane == 0) {
-    // `root` is the forest index of this tree's root (0 for a tree of its own); node and parent
-    // indices are forest indices, and a tree's nodes follow its root
-    int b = accepted_node ? accepted_node[s] : root, n = 0;
-    bool bad = b < root || b >= B;
-    if (bad) b = root;
-    s_path[0] = b;
-    while (b > root && n < B) {  // parents precede their children, so this ends within B steps
-      const int p = par[b];
-      if (p < root || p >= b) { bad = true; break; }
-      b = p;
-      s_path[++n] = b;
-    }
-    if (bad) {  // inconsistent tree: commit nothing but U(root)
-      if (status) atomicOr(status, TSD_STATUS_BAD_PARENT);
-      s_path[0] = root;
-      n = 0;
-    }
-    s_depth = n;
-  }
-  __syncwarp();
-  const int depth = s_depth, acc = s_path[0];
-  const int base = step_base ? step_base[s] : 0;
-  const int64_t start = block_start ? block_start[s] : 0;
-  const bool in_range = start >= 0 && start + R <= seq_stride;
-  if (tokens && !in_range && lane == 0 && status) atomicOr(status, TSD_STATUS_BAD_INDEX);
-  int still = 0, open_rows = 0;
-#pragma unroll
-  for (int i = 0; i < kCommitRowsPerLane; ++i) {
-    const int r = lane + 32 * i;
-    if (r >= R) continue;
-    int v = st[(size_t)acc * R + r];
-    int step = -1;
-    if (v == mask_id) {
-      ++open_rows;
-      if (unmask_flag && unmask_flag[(size_t)s * R + r]) {
-        v = unmask_tok[(size_t)s * R + r];
-        step = base + depth;
-      }
-    } else if (st[(size_t)root * R + r] == mask_id) {
-      // filled somewhere on the path: by the shallowest node that holds it
-      int j = depth;  // s_path[depth - j] is the path node at depth j
-      while (j > 1 && st[(size_t)s_path[depth - j + 1] * R + r] != mask_id) --j;
-      step = base + j - 1;
-    }
-    if (v == mask_id) ++still;
-    if (root_out) root_out[(size_t)s * R + r] = v;
-    if (tokens && in_range) tokens[(size_t)s * seq_stride + start + r] = v;
-    if (fill_step && step >= 0) fill_step[(size_t)s * R + r] = step;
-  }
-#pragma unroll
-  for (int off = 16; off; off >>= 1) {
-    still += __shfl_xor_sync(0xffffffffu, still, off);
-    open_rows += __shfl_xor_sync(0xffffffffu, open_rows, off);
-  }
-  if (lane == 0) {
-    if (n_masked) n_masked[s] = still;
-    if (step_base) step_base[s] = base + depth + (open_rows > 0 ? 1 : 0);
-  }
+  commit_sequence(a, blockIdx.x, threadIdx.x);
 }
 
 // The accepted node's draft K/V rows -> a destination of the caller's (one layer per call): 16-byte
@@ -169,9 +96,9 @@ extern "C" int tsd_commit_accepted(int32_t batch, int32_t n_branches, int32_t ro
   if (tokens && seq_stride < rows_per_branch) return TSD_ERR_INVALID_ARG;
   if (batch == 0) return TSD_OK;
   if (!parent || !state) return TSD_ERR_INVALID_ARG;
-  cudaError_t e = tsd::launch(tsd::commit_kernel, batch, 32, 0, stream, n_branches, rows_per_branch, tree_root, parent, state, accepted_node,
-                                               unmask_flag, unmask_tok, mask_id, tokens, seq_stride, block_start,
-                                               root_out, fill_step, step_base, n_masked, status);
+  const tsd::CommitArgs a = {n_branches, rows_per_branch, tree_root, parent, state, accepted_node, unmask_flag, unmask_tok,
+                             mask_id, tokens, seq_stride, block_start, root_out, fill_step, step_base, n_masked, status};
+  cudaError_t e = tsd::launch(tsd::commit_kernel, batch, 32, 0, stream, a);
   if (e != cudaSuccess) return tsd::cuda_fail(e, "commit_kernel");
   return TSD_OK;
 }

@@ -336,6 +336,73 @@ PyObject* verify_step(Args a) {
   return done(call(tsd_verify_step, &t, stream_of(a[33])), "tsd_verify_step");
 }
 
+// root_state [S, R], mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, stream
+PyObject* begin_block(Args a) {
+  int64_t s[4];
+  shape3(a[3], s);
+  return done(call(tsd_begin_block, (int32_t)s[0], (int32_t)s[1], (int32_t)s[2], to_i32(a[1]), ptr<int32_t>(a[0]), ptr<int32_t>(a[2]),
+                   ptr<int32_t>(a[3]), ptr<int32_t>(a[4]), ptr<int32_t>(a[5]), ptr<int32_t>(a[6]), ptr<int32_t>(a[7]),
+                   ptr<int32_t>(a[8]), stream_of(a[9])),
+              "tsd_begin_block");
+}
+
+// logits, k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search, edge_valid, prefix_len,
+// accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, draft_prob, tokens, block_start, root_out, fill_step,
+// step_base, n_masked, width, depth, next_parent, next_state, next_prob, next_n, report, ticket, status, stream
+PyObject* advance_block(Args a) {
+  int64_t s[4], st[4] = {0, 0, 0, 0};
+  shape3(a[8], s);
+  const Logits x(a[0]);
+  want(x.n == s[0] * s[1] * s[2], "logits have a row for every (sequence, branch, row)");
+  if (a[21] != Py_None) want(strides(a[21], st) == 2 && st[1] == 1, "tokens are [sequences, length], contiguous");
+  tsd_advance_args t = {};
+  t.batch = (int32_t)s[0]; t.n_branches = (int32_t)s[1]; t.rows_per_branch = (int32_t)s[2];
+  t.logits = ptr(a[0]);
+  t.row_stride = x.pitch; t.logits_dtype = x.dtype; t.vocab = x.vocab;
+  t.k = to_i32(a[1]);
+  t.conf = ptr<float>(a[2]); t.topk_idx = ptr<int32_t>(a[3]); t.topk_prob = ptr<float>(a[4]); t.lse = ptr<float>(a[5]);
+  t.topk_workspace = ptr(a[6]);
+  t.topk_workspace_bytes = nbytes(a[6]);
+  t.parent = ptr<int32_t>(a[7]); t.state = ptr<int32_t>(a[8]);
+  t.mask_id = to_i32(a[9]);
+  t.tau = to_float(a[10]);
+  t.rule = to_i32(a[11]);
+  t.search = to_i32(a[12]);
+  t.edge_valid = ptr<uint8_t>(a[13]); t.prefix_len = ptr<int32_t>(a[14]); t.accepted_node = ptr<int32_t>(a[15]);
+  t.accepted_len = ptr<int32_t>(a[16]); t.n_new_tokens = ptr<int32_t>(a[17]); t.unmask_flag = ptr<uint8_t>(a[18]);
+  t.unmask_tok = ptr<int32_t>(a[19]); t.draft_prob = ptr<float>(a[20]);
+  t.tokens = ptr<int32_t>(a[21]);
+  t.seq_stride = st[0];
+  t.block_start = ptr<int32_t>(a[22]);
+  t.root_out = ptr<int32_t>(a[23]); t.fill_step = ptr<int32_t>(a[24]); t.step_base = ptr<int32_t>(a[25]); t.n_masked = ptr<int32_t>(a[26]);
+  t.width = to_i32(a[27]); t.depth = to_i32(a[28]);
+  t.next_parent = ptr<int32_t>(a[29]); t.next_state = ptr<int32_t>(a[30]); t.next_prob = ptr<float>(a[31]); t.next_n = ptr<int32_t>(a[32]);
+  t.report = ptr<uint64_t>(a[33]);
+  t.ticket = (uint32_t)to_int(a[34]);
+  t.status = ptr<uint32_t>(a[35]);
+  return done(call(tsd_advance_block, &t, stream_of(a[36])), "tsd_advance_block");
+}
+
+// n_masked [S], status, report, ticket, stream
+PyObject* report_block(Args a) {
+  int64_t s[4];
+  want(shape(a[0], s) == 1, "n_masked is [sequences]");
+  return done(call(tsd_report_block, (int32_t)s[0], ptr<int32_t>(a[0]), ptr<uint32_t>(a[1]), ptr<uint64_t>(a[2]), (uint32_t)to_int(a[3]),
+                   stream_of(a[4])),
+              "tsd_report_block");
+}
+
+// report [S], ticket, stream -> (largest count of masked rows, status bits)
+PyObject* wait_block(Args a) {
+  int64_t s[4];
+  want(shape(a[0], s) == 1, "report is [sequences]");
+  int32_t masked = 0;
+  uint32_t bits = 0;
+  const int rc = call(tsd_wait_block, (int32_t)s[0], ptr<uint64_t>(a[0]), (uint32_t)to_int(a[1]), &masked, &bits, stream_of(a[2]));
+  if (rc != TSD_OK) raise_error(rc, "tsd_wait_block");
+  return Py_BuildValue("iI", masked, bits);
+}
+
 // METH_FASTCALL entry: argument count, then C++ to Python errors
 template <PyObject* (*F)(Args), int N>
 PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
@@ -355,6 +422,8 @@ PyMethodDef methods[] = {TSD_METHOD(setup, 5),           TSD_METHOD(verify_atten
                          TSD_METHOD(confidence_topk, 9), TSD_METHOD(accept, 19),           TSD_METHOD(accept_relaxed, 22),
                          TSD_METHOD(commit, 15),         TSD_METHOD(build_tree, 18),       TSD_METHOD(build_mask, 6),
                          TSD_METHOD(verify_step, 34),    TSD_METHOD(interblock_vis, 3),    TSD_METHOD(interblock_trigger, 10),
+                         TSD_METHOD(begin_block, 10),    TSD_METHOD(advance_block, 37),    TSD_METHOD(report_block, 5),
+                         TSD_METHOD(wait_block, 3),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_tsd_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

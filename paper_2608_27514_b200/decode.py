@@ -4,13 +4,13 @@
 
     caller's model forward over every node of the tree   (its attention layers call
                                                           ``VerifyStep.attention``)
-    -> tsd_confidence_topk      scores of this pass = candidate pool of the next (Section 3.1)
-    -> tsd_accept_trajectories  longest verified trajectory (Section 3.3)
-    -> tsd_commit_accepted      next root into the token buffer, sequential step indices
-    -> tsd_build_draft_tree     tree of the next pass (Alg. 1 Phase 2)
+    -> tsd_advance_block        scores of this pass = candidate pool of the next (Section 3.1), longest
+                                verified trajectory (Section 3.3), next root into the token buffer with
+                                its sequential step indices, tree of the next pass (Alg. 1 Phase 2)
 
-All of it is enqueued on the current stream; the only thing read back per pass is the count of
-rows still masked (4 bytes per sequence), which ends the loop.  The class allocates and marshals;
+All of it is enqueued on the current stream; the only thing that comes back per pass is the count of
+rows still masked, which ends the loop: the pass writes it to pinned host memory (8 bytes per sequence)
+and the loop watches that.  The class allocates and marshals;
 every step of the arithmetic runs in the library's kernels.
 """
 import torch
@@ -34,6 +34,8 @@ class BlockDecoder:
         self.fill_step = i32(S, R)
         self.step_base = i32(S)
         self.n_masked = i32(S)
+        self.report = torch.zeros(S, dtype=torch.int64, pin_memory=True)
+        self.ticket = 0
         self.n_forward = 0
 
     @property
@@ -43,42 +45,44 @@ class BlockDecoder:
     def start(self, root_state):
         """Begin a block from root_state int32 [S, R]; the first pass has no candidate pool yet, so
         its tree is the root alone (copies in the unused slots)."""
-        t = self.tree
-        t["state"].copy_(root_state.to(torch.int32)[:, None, :].expand_as(t["state"]))
-        t["parent"].zero_()
-        t["parent"][:, 0] = -1
-        t["n"].fill_(1)
-        self.fill_step.fill_(-1)
-        self.step_base.zero_()
-        # the root alone, nothing accepted, nothing to unmask: the commit kernel copies it to
-        # self.root and counts its masked rows
-        B.tsd_commit_accepted(t["parent"], t["state"], None, None, None, self.mask_id, root_out=self.root,
-                              n_masked=self.n_masked, status=self.step.status)
+        st, t = self.step, self.tree
+        root = root_state.to(device=st.device, dtype=torch.int32).expand(st.S, st.R).contiguous()
+        B.tsd_begin_block(root, self.mask_id, t["parent"], t["state"], t["n"], self.root, self.fill_step, self.step_base, self.n_masked)
         self.n_forward = 0
 
     def advance(self, logits, tokens=None, block_start=None):
         """One pass after the caller's forward: logits [S*B*R, V] of the current tree's nodes."""
+        self._advance(logits, tokens, block_start, None)
+
+    def _advance(self, logits, tokens, block_start, report):
         st, t, nxt = self.step, self.tree, self.trees[1 - self.cur]
-        st.confidence_topk(logits)
-        if self.rule in (B.TSD_ACCEPT_EXACT, B.TSD_ACCEPT_TOP1):
-            st.accept(t["parent"], t["state"], self.mask_id, self.tau, self.rule, self.search)
-        else:
-            st.accept_relaxed(t["parent"], t["state"], self.mask_id, self.tau, self.rule, self.search,
-                              logits if self.rule == B.TSD_ACCEPT_PROB else None)
-        B.tsd_commit_accepted(t["parent"], t["state"], st.accepted_node, st.unmask_flag, st.unmask_tok,
-                              self.mask_id, tokens, block_start, self.root, self.fill_step, self.step_base,
-                              self.n_masked, st.status)
-        B.tsd_build_draft_tree(t["state"], st.accepted_node, st.unmask_flag, st.unmask_tok, self.mask_id,
-                               st.topk_idx, st.topk_prob, self.width, self.depth, nxt["parent"], nxt["state"],
-                               nxt["prob"], nxt["n"], st.status)
+        if self.rule == B.TSD_ACCEPT_PROB and not hasattr(st, "draft_prob"):
+            st.draft_prob = torch.empty((st.S, st.B, st.R), dtype=torch.float32, device=st.device)
+        B.tsd_advance_block(logits, st.k, st.conf, st.topk_idx, st.topk_prob, st.lse, st.topk_ws, t["parent"], t["state"], self.mask_id,
+                            self.tau, self.rule, self.search, st.edge_valid, st.prefix_len, st.accepted_node, st.accepted_len,
+                            st.n_new_tokens, st.unmask_flag, st.unmask_tok, getattr(st, "draft_prob", None), tokens, block_start,
+                            self.root, self.fill_step, self.step_base, self.n_masked, self.width, self.depth, nxt["parent"],
+                            nxt["state"], nxt["prob"], nxt["n"], report, self.ticket, st.status)
         self.cur = 1 - self.cur
         self.n_forward += 1
+
+    def _next_ticket(self):
+        self.ticket = self.ticket % 0x7fffffff + 1
 
     def decode(self, forward, tokens=None, block_start=None, max_passes=None):
         """Run passes until no sequence has a masked row left.  forward(state int32 [S,B,R]) must
         return the logits [S*B*R, V] of every node (a device tensor the vocabulary pass accepts)."""
         limit = self.step.R + 1 if max_passes is None else max_passes
-        while self.n_forward < limit and int(self.n_masked.max().item()) > 0:
-            self.advance(forward(self.tree["state"]), tokens, block_start)
-        self.step.check_status()
+        status = 1  # not known from a report
+        if self.n_forward < limit:
+            self._next_ticket()
+            B.tsd_report_block(self.n_masked, self.step.status, self.report, self.ticket)
+            masked, status = B.tsd_wait_block(self.report, self.ticket)
+            while self.n_forward < limit and masked > 0:
+                logits = forward(self.tree["state"])
+                self._next_ticket()
+                self._advance(logits, tokens, block_start, self.report)
+                masked, status = B.tsd_wait_block(self.report, self.ticket)
+        if status:
+            self.step.check_status()
         return self.root

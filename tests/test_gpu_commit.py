@@ -254,3 +254,59 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable()
     step.attention(attn["q"], attn["k_cache"], attn["v_cache"], attn["k_draft"], attn["v_draft"], attn["sm_scale"])
     torch.cuda.synchronize()
     assert B.tsd_check_status(step.status) == B.TSD_OK
+
+
+@pytest.mark.parametrize("S,Bn,R,k,width,depth,rule", [(1, 1, 32, 1, 1, 1, B.TSD_ACCEPT_EXACT), (3, 10, 32, 4, 3, 3, B.TSD_ACCEPT_TOP1),
+                                                       (2, 7, 64, 3, 2, 3, B.TSD_ACCEPT_TOPK), (2, 9, 32, 5, 3, 2, B.TSD_ACCEPT_PROB),
+                                                       (5, 4, 128, 8, 32, 4, B.TSD_ACCEPT_EXACT), (2, 256, 32, 3, 8, 40, B.TSD_ACCEPT_PROB)])
+def test_advance_in_one_launch_equals_the_single_calls(S, Bn, R, k, width, depth, rule):
+    # every (rows, candidates) variant of the kernel and all four rules; three passes, everything bit for bit, and the report
+    V, M = 600, 599
+    mk = lambda: VerifyStep(S, Bn, R, 0, 1, 1, 64, V, k, torch.bfloat16, DEV)
+    dec = BlockDecoder(mk(), width, depth, 0.3, M, rule, B.TSD_SEARCH_LONGEST)
+    g = torch.Generator(device=DEV).manual_seed(S * 100 + Bn)
+    root = torch.randint(0, M, (S, R), generator=g, device=DEV, dtype=torch.int32)
+    root[:, ::2] = M
+    tokens, tokens2 = (torch.full((S, 2 * R), -5, dtype=torch.int32, device=DEV) for _ in range(2))
+    start = torch.arange(S, dtype=torch.int32, device=DEV)
+    st, i32 = mk(), lambda *shape: torch.zeros(shape, dtype=torch.int32, device=DEV)
+    parent, state, fill, base, masked, out = i32(S, Bn), root[:, None].repeat(1, Bn, 1), i32(S, R) - 1, i32(S), i32(S), i32(S, R)
+    parent[:, 0] = -1
+    dec.start(root)
+    assert torch.equal(dec.tree["state"], state) and torch.equal(dec.tree["parent"], parent) and (dec.tree["n"] == 1).all()
+    assert torch.equal(dec.root, root) and torch.equal(dec.fill_step, fill) and (dec.n_masked == R // 2).all()
+    rows = torch.randn((1, 1, R, V), generator=g, device=DEV) * 2  # a row's scores hardly move from pass to pass
+    for i in range(3):
+        x = (rows + 0.1 * torch.randn((S, Bn, R, V), generator=g, device=DEV)).bfloat16().reshape(-1, V)
+        dec._next_ticket()
+        dec._advance(x, tokens, start, dec.report)
+        most, status = B.tsd_wait_block(dec.report, dec.ticket)
+        st.confidence_topk(x)
+        if rule in (B.TSD_ACCEPT_EXACT, B.TSD_ACCEPT_TOP1):
+            st.accept(parent, state, M, 0.3, rule, B.TSD_SEARCH_LONGEST)
+        else:
+            st.accept_relaxed(parent, state, M, 0.3, rule, B.TSD_SEARCH_LONGEST, x if rule == B.TSD_ACCEPT_PROB else None)
+        B.tsd_commit_accepted(parent, state, st.accepted_node, st.unmask_flag, st.unmask_tok, M, tokens2, start, out, fill, base, masked,
+                              st.status)
+        parent2, state2, prob, n = i32(S, Bn), i32(S, Bn, R), torch.zeros((S, Bn), device=DEV), i32(S)
+        B.tsd_build_draft_tree(state, st.accepted_node, st.unmask_flag, st.unmask_tok, M, st.topk_idx, st.topk_prob, width, depth,
+                               parent2, state2, prob, n, st.status)
+        parent, state = parent2, state2
+        t = dec.tree
+        for a, b in ((t["parent"], parent), (t["state"], state), (t["prob"], prob), (t["n"], n), (dec.root, out), (tokens, tokens2),
+                     (dec.fill_step, fill), (dec.step_base, base), (dec.n_masked, masked), (dec.step.conf, st.conf),
+                     *((v, st.accept_outputs()[key]) for key, v in dec.step.accept_outputs().items())):
+            assert torch.equal(a, b)
+        if rule == B.TSD_ACCEPT_PROB:
+            assert torch.equal(dec.step.draft_prob, st.draft_prob)
+        assert status == 0 and most == int(masked.max())
+
+
+def test_wait_for_a_report_that_never_comes_fails():
+    report = torch.zeros(2, dtype=torch.int64).pin_memory()
+    with pytest.raises(B.TsdError):
+        B.tsd_wait_block(report, 7)
+    n = torch.tensor([3, 5], dtype=torch.int32, device=DEV)
+    status = torch.tensor([2], dtype=torch.int32, device=DEV)
+    B.tsd_report_block(n, status, report, 7)
+    assert B.tsd_wait_block(report, 7) == (5, 2)
