@@ -22,6 +22,7 @@ namespace tsd {
 
 template <int WORDS>
 __global__ void __launch_bounds__(kAcceptMaxThreads, 1) accept_kernel(const AcceptArgs a, const RelaxedArgs x) {
+  accept_prefetch(a, blockIdx.x);
   grid_wait();
   grid_launch_next();
   const int tree = blockIdx.y;

@@ -29,6 +29,18 @@ struct RelaxedArgs {
 
 int check_accept(const AcceptArgs& a, const RelaxedArgs& x);
 
+// Asks for the sequence's tree (parents and states), which usually comes from DRAM, to be brought to L2 while the
+// vocabulary pass still runs: a hint only, nothing is read before grid_wait().
+__device__ __forceinline__ void accept_prefetch(const AcceptArgs& a, int s) {
+  const size_t cells = (size_t)a.n_branches * a.rows_per_branch;
+  const char* st = reinterpret_cast<const char*>(a.state + s * cells);
+  for (size_t i = threadIdx.x * 128; i < cells * 4; i += blockDim.x * 128)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(st + i));
+  const char* par = reinterpret_cast<const char*>(a.parent + (size_t)s * a.n_branches);
+  for (size_t i = threadIdx.x * 128; i < (size_t)a.n_branches * 4; i += blockDim.x * 128)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(par + i));
+}
+
 // WORDS = 32-row words per node that the unrolled loops cover (R <= 32 * WORDS).  Called by a whole block of at least
 // a warp; returns the accepted node (an index in the tree) to every thread.
 template <int WORDS>

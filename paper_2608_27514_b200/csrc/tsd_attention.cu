@@ -72,7 +72,7 @@ int tsd_verify_attention(const tsd_layout* L, const void* mask, const void* q, i
   a.workspace_bytes = workspace_bytes;
   a.status = status;
   a.stream = stream;
-  a.launch_next = false;
+  a.concurrent = false;
   return tsd::launch_attention(a, flags);
 }
 

@@ -72,7 +72,7 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
                       T* __restrict__ out, float* __restrict__ lse, int64_t qs_b, int64_t qs_r, int64_t qs_h,
                       int64_t cs_b, int64_t cs_r, int64_t cs_h, int64_t ds_b, int64_t ds_r, int64_t ds_h,
                       int64_t os_b, int64_t os_r, int64_t os_h, float sm_scale, uint32_t* __restrict__ status,
-                      int launch_next) {
+                      int concurrent) {
   constexpr int LPK = D / 8;            // lanes per key
   constexpr int KPI = 32 / LPK;         // keys read at once
   constexpr int SUB = LPK / RB;         // reads per group: SUB * RB scores per key lane, one per lane after the scatter
@@ -91,8 +91,12 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
   const int b = row0 / R, g = h / (Hq / Hkv), N = B * R;
   const int j = lane % LPK, slots = kTile / R;
   const unsigned full = 0xffffffffu;
-  grid_wait(mask, q, kc, vc, kd, vd);
-  if (launch_next) grid_launch_next();
+  if (concurrent) {  // beside the kernel before it, see tsd_attention_tc.cu
+    __threadfence();
+    settle(mask, q, kc, vc, kd, vd);
+  } else {
+    grid_wait(mask, q, kc, vc, kd, vd);
+  }
 
   // the block's query rows, 8 dimensions per lane (requested first: nothing else is needed for them)
   float qr[RB][8];
@@ -108,6 +112,7 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
   const int clen = min(max(mask[kHdrWords + s], 0), Nc);
   if (!hdr_ok) {  // a blob built for another layout: report, write nothing
     if (threadIdx.x == 0 && status) atomicOr(status, TSD_STATUS_BAD_MASK);
+    if (concurrent) grid_wait();
     return;
   }
   if (warp == 0) {
@@ -259,6 +264,7 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
     from_float(out[s * os_b + (int64_t)(row0 + r) * os_r + h * os_h + c], o / lt);
     if (lse && c == 0) lse[((size_t)s * Hq + h) * N + row0 + r] = M + logf(lt);
   }
+  if (concurrent) grid_wait();
 }
 
 template <typename T, int D, int RB, int MAXW>
@@ -271,7 +277,7 @@ static cudaError_t launch_rows(const AttnArgs& a, int warps) {
       md.rec_words, a.mask, static_cast<const T*>(a.q), static_cast<const T*>(a.kc), static_cast<const T*>(a.vc),
       static_cast<const T*>(a.kd), static_cast<const T*>(a.vd), static_cast<T*>(a.out), a.lse, a.qs_b, a.qs_r,
       a.qs_h, a.cs_b, a.cs_r, a.cs_h, a.ds_b, a.ds_r, a.ds_h, a.os_b, a.os_r, a.os_h, a.sm_scale, a.status,
-      (int)a.launch_next);
+      (int)a.concurrent);
 }
 
 template <typename T, int D>

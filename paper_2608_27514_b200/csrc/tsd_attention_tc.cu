@@ -309,7 +309,7 @@ struct TcParams {
   int recs_off, n_qt, rec_words;  // layout of the mask blob, computed on the host from the same tsd_layout
   int n_items;                    // S * Hq * n_qt
   float scale_log2e;              // sm_scale * log2(e), > 0
-  int launch_next;
+  int concurrent;
 };
 
 // The MMAs of a tile go out as ONE block of instructions: the issuing lane shares its scheduler with
@@ -477,8 +477,15 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   }
   // Everything above runs while the previous kernel of the stream finishes.  Tensor memory is allocated only
   // after the wait: a block of that kernel may still need it.
-  grid_wait(mask);
-  if (p.launch_next) grid_launch_next();
+  // Beside the kernel before it nothing is waited for but an acquire fence, so that no line the SM still holds from
+  // earlier kernels is used; the block then leaves only after that kernel has completed, so that a kernel which waits
+  // for this one has waited for both.
+  if (p.concurrent) {
+    __threadfence();
+    settle(mask);
+  } else {
+    grid_wait(mask);
+  }
 
   const int h_magic = mask[H_MAGIC], h_s = mask[H_S], h_b = mask[H_B], h_r = mask[H_R], h_nc = mask[H_NC];
   // tile counts of this block's items (the blob's layout follows from the tsd_layout, so no
@@ -1030,6 +1037,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
   if (tid == 0 && *abort_flag && p.status) atomicOr(p.status, TSD_STATUS_TIMEOUT);
+  if (p.concurrent) grid_wait();
 }
 
 // The bounded wait of this file on a barrier that nothing ever completes: it gives up after
@@ -1160,7 +1168,7 @@ static int launch_tc(const AttnArgs& a) {
   p.recs_off = md.recs_off; p.n_qt = md.n_qt; p.rec_words = md.rec_words;
   p.n_items = (int)n_items;
   p.scale_log2e = a.sm_scale * kLog2e;
-  p.launch_next = a.launch_next;
+  p.concurrent = a.concurrent;
   // one block per SM, each walking its share of the items; more blocks only when a block's share
   // would not fit the per-block item table
   const int sms = std::max(device_facts().sms, 1);

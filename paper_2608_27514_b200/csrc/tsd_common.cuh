@@ -63,7 +63,7 @@ struct AttnArgs {
   size_t workspace_bytes;
   uint32_t* status;
   cudaStream_t stream;
-  bool launch_next;  // let the next kernel of the stream start as soon as every block of this one runs
+  bool concurrent;  // reads nothing that the kernel before it in the stream writes: may run beside it
 };
 int launch_attention_simt(const AttnArgs& a);
 bool attention_tc_supported(const AttnArgs& a);
@@ -72,7 +72,9 @@ int launch_attention_tc(const AttnArgs& a);
 int launch_attention(const AttnArgs& a, uint32_t flags);
 
 // The vocabulary pass and the acceptance behind their entry points.  `concurrent`: the pass reads nothing
-// that the kernel before it in the stream writes, and may run beside it.
+// that the kernel before it in the stream writes, and may run beside it.  `launch_next`: when the next kernel may be
+// brought up.
+enum { kNextAfter = 0, kNextAtTail = 1, kNextAtOnce = 2 };  // when this one is done; at the end of its rows; with its last blocks
 struct TopkArgs {
   const void* logits;
   int32_t dtype;
@@ -86,7 +88,7 @@ struct TopkArgs {
   void* workspace;
   size_t workspace_bytes;
   cudaStream_t stream;
-  bool concurrent;
+  int launch_next;
 };
 int check_topk(const TopkArgs& a);
 int launch_topk(const TopkArgs& a);

@@ -1,12 +1,14 @@
 // The whole verification step in one call (Section 3.3): verify attention, vocabulary pass, acceptance.
 //
-// The vocabulary pass reads none of what the attention call writes, so the two may run side by side: the
-// attention kernel lets its successor start once all its blocks run, and the vocabulary pass starts right
-// away on the SMs that attention leaves idle instead of waiting for its last block; the acceptance waits for
-// both.  Done where attention has fewer work items than the GPU has SMs (256 draft rows, 32 heads, 768 cached
-// keys: 64 items; the step 41.5 -> 34.2 us).  With more items than SMs only the last round leaves SMs free,
-// and rows that start early there upset the balance of the vocabulary pass: 1024 rows, 256 items, 95.2 us
-// side by side and 89.8 us one after the other.
+// The attention reads none of what the vocabulary pass writes, so the two may run side by side: the vocabulary
+// pass lets its successor start once all its blocks run, and the attention takes the SMs as the first rows are finished
+// instead of waiting for the last one; the acceptance waits for both.  Done where attention has fewer work items
+// than the GPU has SMs (256 draft rows, 32 heads, 768 cached keys, 64 items: the step takes 32.9 us; attention first and the
+// vocabulary pass beside it 33.5; one after the other 40.8).  With more items than SMs neither leaves SMs
+// free before its end, and what starts early there upsets the balance: 1024 rows, 256 items, 95.2 us side by side
+// and 89.8 us one after the other.
+//
+// The acceptance is brought up while the last rows are finished and asks for the trees ahead of time.
 #include "tsd_common.cuh"
 
 extern "C" int tsd_verify_step(const tsd_step_args* x, tsd_stream_t stream) {
@@ -25,13 +27,19 @@ extern "C" int tsd_verify_step(const tsd_step_args* x, tsd_stream_t stream) {
                            x->o_stride[1], x->o_stride[2], x->sm_scale, x->attn_workspace, x->attn_workspace_bytes,
                            x->status, stream, beside};
   const tsd::TopkArgs t = {x->logits, x->logits_dtype, x->n_rows, x->vocab, x->row_stride, x->k, x->conf, x->topk_idx,
-                           x->topk_prob, x->lse, x->topk_workspace, x->topk_workspace_bytes, stream, beside};
+                           x->topk_prob, x->lse, x->topk_workspace, x->topk_workspace_bytes, stream,
+                           beside ? tsd::kNextAtOnce : tsd::kNextAtTail};
   const tsd::AcceptArgs c = {L->batch, L->n_branches, L->n_branches, L->rows_per_branch, x->parent, x->state, x->mask_id,
                              x->conf, x->topk_idx, x->k, x->tau, x->rule, x->search, x->edge_valid, x->prefix_len,
                              x->accepted_node, x->accepted_len, x->n_new_tokens, x->unmask_flag, x->unmask_tok, x->status,
                              stream};
   if ((rc = tsd::check_topk(t)) != TSD_OK || (rc = tsd::check_accept_exact(c)) != TSD_OK) return rc;
-  if ((rc = tsd::launch_attention(a, x->flags)) != TSD_OK) return rc;
-  if ((rc = tsd::launch_topk(t)) != TSD_OK) return rc;
+  if (beside) {
+    if ((rc = tsd::launch_topk(t)) != TSD_OK) return rc;
+    if ((rc = tsd::launch_attention(a, x->flags)) != TSD_OK) return rc;
+  } else {
+    if ((rc = tsd::launch_attention(a, x->flags)) != TSD_OK) return rc;
+    if ((rc = tsd::launch_topk(t)) != TSD_OK) return rc;
+  }
   return tsd::launch_accept_exact(c);
 }

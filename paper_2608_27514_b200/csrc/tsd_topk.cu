@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(THREADS)
 confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, int k, int n_seg,
                        int chunks_per_seg, float* __restrict__ conf, int32_t* __restrict__ topk_idx,
                        float* __restrict__ topk_prob, float* __restrict__ lse,
-                       Partial<K>* __restrict__ partials, unsigned* __restrict__ tickets, int prefetch, int concurrent) {
+                       Partial<K>* __restrict__ partials, unsigned* __restrict__ tickets, int prefetch, int launch_next) {
   constexpr int E_ = Unpack<T>::kElems;
   constexpr int kTopkThreads = THREADS, kTopkWarps = THREADS / 32;
   constexpr int kTopkBatch = THREADS * kTopkUnroll;        // chunks per block per batch
@@ -273,17 +273,8 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   const int n_iter = (c1 - c0 + kTopkBatch - 1) / kTopkBatch;  // <= kTopkMaxIter (host-enforced)
   const bool has_tail = seg == n_seg - 1 && tid == 0 && chunks_total * E_ < vocab;
 
-  // Normally the kernel before this one may have written the logits.  A concurrent pass reads only what was
-  // there before that kernel started; it takes an acquire fence in place of the wait, so that no line the SM
-  // still holds from earlier kernels is used, and its last block stays until that kernel has completed, so that
-  // a kernel which waits for this one has waited for both.
-  if (concurrent) {
-    __threadfence();
-    settle(rowp, rowv);
-  } else {
-    grid_wait(rowp, rowv);
-  }
-  const bool stay = concurrent && warp == 1 && blockIdx.x == gridDim.x - 1;
+  grid_wait(rowp, rowv);
+  if (launch_next == kNextAtOnce) grid_launch_next();
 
   // ---- phase 1: stream.  Two register buffers: the loads of batch it+1 are in flight while
   // batch it is processed, so a block overlaps memory latency with its own arithmetic.
@@ -350,6 +341,8 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
     e = e_new;
     for (int x = chunks_total * E_; x < vocab; ++x) s += ex2_approx(fmaf(to_float(rowp[x]), kLog2e, -e));
   }
+
+  if (launch_next == kNextAtTail) grid_launch_next();
 
   // ---- phase 2: bound = k-th largest of the warps' maxima.  Each of the k best warps holds a
   // value equal to its maximum, so at least k values of the segment reach the bound.  One shuffle
@@ -445,7 +438,6 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
       for (int j = 0; j < K; ++j) { s_part[warp].v[j] = a.v[j]; s_part[warp].i[j] = a.i[j]; }
     }
     __syncthreads();
-    if (stay) grid_wait();
     if (warp != 0) return;
     a.init();
     if (lane < kTopkWarps) {
@@ -457,7 +449,6 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
     }
     warp_merge(a);
   } else {
-    if (stay) grid_wait();
     if (warp != 0) return;
     // sum of the warps' sums (fixed tree), and the pool's best K by rank: every lane counts the
     // entries that come before its own (keys are unique), so rank r goes to slot r without a sort
@@ -576,7 +567,7 @@ static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
               : p.threads == 384 ? confidence_topk_kernel<T, K, 384> : confidence_topk_kernel<T, K, 256>;
   return launch(kernel, (unsigned)(a.n_rows * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
                 a.row_stride, a.k, p.n_seg, p.chunks_per_seg, a.conf, a.topk_idx, a.topk_prob, a.lse, partials, tickets,
-                p.prefetch, (int)a.concurrent);
+                p.prefetch, a.launch_next);
 }
 
 template <typename T>
@@ -645,7 +636,7 @@ int tsd_confidence_topk(const void* logits, int32_t dtype, int64_t n_rows, int32
                         uint32_t* status, tsd_stream_t stream) {
   (void)status;
   const tsd::TopkArgs a = {logits, dtype, n_rows, vocab, row_stride, k, conf, topk_idx, topk_prob, lse, workspace,
-                           workspace_bytes, stream, false};
+                           workspace_bytes, stream, tsd::kNextAfter};
   int rc = tsd::check_topk(a);
   return rc != TSD_OK ? rc : tsd::launch_topk(a);
 }
@@ -686,7 +677,7 @@ extern "C" int tsd_confidence_topk_static(const void* logits, int32_t dtype, int
                                           float* topk_prob, float* lse, uint32_t* status,
                                           tsd_stream_t stream) {
   (void)status;
-  tsd::TopkArgs a = {logits, dtype, n_rows, vocab, row_stride, k, conf, topk_idx, topk_prob, lse, nullptr, 0, stream, false};
+  tsd::TopkArgs a = {logits, dtype, n_rows, vocab, row_stride, k, conf, topk_idx, topk_prob, lse, nullptr, 0, stream, tsd::kNextAfter};
   int rc = tsd::check_pointers(a);
   if (rc != TSD_OK || n_rows == 0) return rc;
   // this shape would need more scratch than the library carries: the caller has to use
