@@ -25,7 +25,7 @@
 namespace tsd {
 
 constexpr int kRowsChunk = 32;      // keys per chunk
-constexpr int kRowsMaxBranches = 256;
+constexpr int kRowsMaxGroups = 1024;  // 32-row groups of a sequence's draft rows at most (256 branches x 128 rows)
 
 // 8 dimensions of a row for lane j of LPK: two 16-byte reads LPK * 16 bytes apart (fp32), or one (bf16).
 template <int LPK>
@@ -80,7 +80,7 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
   constexpr int NG = kRowsChunk / KG;
   constexpr int VC = D / 32;            // value dimensions per lane
   static_assert(LPK % RB == 0, "RB divides D / 8");
-  __shared__ int s_vis[kRowsMaxBranches];                              // visible draft branches of this branch
+  __shared__ int s_vis[kRowsMaxGroups];                                // visible groups of 32 draft rows of this branch
   __shared__ int s_nvis;
   __shared__ __align__(16) float s_p[MAXW][kRowsChunk][RB];            // weights of a warp's chunk
   __shared__ __align__(16) float s_alpha[MAXW][RB];
@@ -117,16 +117,15 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
   }
   if (warp == 0) {
     const int32_t* rec = mask + recs_off + (size_t)(s * n_qt + b / slots) * rec_words;
-    const int qs = b % slots, n_entries = min(rec[0], n_qt);
+    const int qs = b % slots, n_list = rec_words / 2 - 1, n_entries = min(rec[0], n_list);
     int n = 0;
-    for (int e0 = 0; e0 < n_qt; e0 += 32) {
+    for (int e0 = 0; e0 < n_list; e0 += 32) {
       const int e = e0 + lane;
       int kt = 0, nib = 0;
-      if (e < n_qt) {
+      if (e < n_entries) {
         kt = rec[2 + 2 * e];
-        nib = (rec[3 + 2 * e] >> (qs * 4)) & ((1 << slots) - 1);
+        nib = (rec[3 + 2 * e] >> (qs * 2)) & 3;
       }
-      if (e >= n_entries) nib = 0;
       int at = __popc(nib);  // inclusive prefix sum of the lanes' counts
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
@@ -135,15 +134,14 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
       }
       const int total = __shfl_sync(full, at, 31);
       at += n - __popc(nib);
-      for (int ks = 0; ks < slots; ++ks)
-        if ((nib >> ks) & 1) { if (at < kRowsMaxBranches) s_vis[at] = min(kt * slots + ks, B - 1); ++at; }
+      for (int w = 0; w < 2; ++w)
+        if ((nib >> w) & 1) { if (at < kRowsMaxGroups) s_vis[at] = min(kt * 2 + w, N / kRowsChunk - 1); ++at; }
       n += total;
     }
-    if (lane == 0) s_nvis = min(n, kRowsMaxBranches);
+    if (lane == 0) s_nvis = min(n, kRowsMaxGroups);
   }
   __syncthreads();
-  const int n_cc = (clen + kRowsChunk - 1) / kRowsChunk, per_branch = R / kRowsChunk;
-  const int n_chunks = n_cc + s_nvis * per_branch;
+  const int n_cc = (clen + kRowsChunk - 1) / kRowsChunk, n_chunks = n_cc + s_nvis;
 
   float m = -CUDART_INF_F, l = 0.f;  // of row lane % RB
   float acc[RB][VC];
@@ -162,8 +160,7 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
       stride = cs_r;
       valid = min(kRowsChunk, clen - ch * kRowsChunk);
     } else {
-      const int e = ch - n_cc;
-      const int64_t row = (int64_t)s_vis[e / per_branch] * R + (e % per_branch) * kRowsChunk;
+      const int64_t row = (int64_t)s_vis[ch - n_cc] * kRowsChunk;
       kp = kd + s * ds_b + row * ds_r + g * ds_h;
       vp = vd + s * ds_b + row * ds_r + g * ds_h;
       stride = ds_r;

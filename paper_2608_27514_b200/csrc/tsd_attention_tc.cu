@@ -82,6 +82,7 @@ struct TcSmem {
   static constexpr uint32_t kOffItems = kOffMpart + 3 * 3 * 128 * 4;  // key tiles / cache length per item (2 x kMaxItems int32)
   static constexpr uint32_t kBytes = kOffItems + 2 * kMaxItems * 4 + 1024;  // + slack to align the base to 1 KB
 };
+static_assert(kKeys == kKeyTile, "the mask blob lists tiles of this many keys");
 // Tensor-memory columns.  At head_dim 128 everything is in use and P is one bf16 per score.  At head_dim 64
 // the tensor pipe has twice the time it needs (256 of the 512 clocks that a tile's exponentials take) and half
 // of O and Q is free, so P is kept as the sum of two bf16 (high part, residual: 2^-17 relative) and P V issues
@@ -494,10 +495,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     int s, h, qt;
     item_coords(it, s, h, qt);
     const int clen = min(max(mask[kHdrWords + s], 0), p.Nc);
-    const int n_dt = min(max(mask[p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words], 1), p.n_qt);
+    const int n_dt = min(max(mask[p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words], 1), p.rec_words / 2 - 1);
     const int n_ct = (clen + kKeys - 1) / kKeys;
     item_clen[it] = clen;
-    item_T[it] = n_ct + 2 * n_dt;
+    item_T[it] = n_ct + n_dt;
   }
 
   // Coordinates of the block's first item for the two producer lanes: worked out here, while the
@@ -596,8 +597,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           if (!ok) break;
           if (G >= n_pre) {
             const bool cached = j < n_ct;
-            const int e = j - n_ct;  // draft key tile e = half (e & 1) of the listed 128-row tile e >> 1
-            const int row = cached ? j * kKeys : rec[2 + 2 * (e >> 1)] * kTile + (e & 1) * kKeys;
+            const int row = (cached ? j : rec[2 + 2 * (j - n_ct)]) * kKeys;
             const CUtensorMap* m = cached ? mc : md;
             const uint32_t dst = stage0 + b * kKVBytes, full_bar = bar(full0 + b);
             mbar_expect_tx(full_bar, kKVBytes);
@@ -718,13 +718,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
               if (j == n_ct - 1) z0 = clen - j * kKeys;  // 1..64 valid rows
             } else {
               const int e = j - n_ct;
-              const unsigned bits = e < 2 ? bits0 : (unsigned)__ldg(rec + 3 + 2 * (e >> 1));  // bit qs*4+ks
-              unsigned seen_slots = 0;
-#pragma unroll
-              for (int qs = 0; qs < 4; ++qs) seen_slots |= (bits >> (4 * qs)) & 15u;
-#pragma unroll
-              for (int w = 0; w < 2; ++w)
-                if (!((seen_slots >> (((e & 1) * kKeys + w * 32) / p.R)) & 1u)) dead |= 1u << w;
+              const unsigned bits = e == 0 ? bits0 : (unsigned)__ldg(rec + 3 + 2 * e);  // bit qs * 2 + w
+              dead = ~(bits | bits >> 2 | bits >> 4 | bits >> 6) & 3u;
             }
             if (z0 < z1 || dead) {
               const uint32_t v_stage = base + kOffV + (uint32_t)b * kKVBytes;
@@ -836,10 +831,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           }
         } else {
           const int e = j - n_ct;
-          const uint32_t nib = ((uint32_t)rec[3 + 2 * (e >> 1)] >> (qs * 4)) & 15u;  // visible key slots
+          const uint32_t see = (uint32_t)rec[3 + 2 * e] >> (qs * 2);  // bit w: this row may read the tile's 32 keys from 32 w on
           masked = true;
 #pragma unroll
-          for (int w = 0; w < 2; ++w) cm[w] = ((nib >> (((e & 1) * kKeys + w * 32) / p.R)) & 1u) ? 0xffffffffu : 0u;
+          for (int w = 0; w < 2; ++w) cm[w] = ((see >> w) & 1u) ? 0xffffffffu : 0u;
         }
         if (masked) {
 #pragma unroll

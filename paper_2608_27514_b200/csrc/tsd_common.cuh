@@ -14,11 +14,12 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 // ---- branch-mask blob (written by tsd_build_branch_mask, read by the attention kernels) ----
 // int32 words: header[8] | cache_len[round4(S)] | records[S * n_qt], each record =
-// { count, 0, (draft_tile, bits) * n_qt }.  A query tile is 128 consecutive draft rows of one
-// sequence = 128/R branch slots; bit (qs*4 + ks) of `bits` = slot qs of the query tile may read
-// slot ks of draft tile `draft_tile`.
-constexpr int kMaskMagic = 0x54534431;
+// { count, 0, (key_tile, bits) * n_kt }.  A query tile is 128 consecutive draft rows of one
+// sequence = 128/R branch slots, a key tile 64 consecutive draft rows; bit (qs * 2 + w) of `bits` = slot qs of
+// the query tile may read rows [32 w, 32 w + 32) of key tile `key_tile`.
+constexpr int kMaskMagic = 0x54534432;
 constexpr int kTile = 128;
+constexpr int kKeyTile = 64;
 constexpr int kHdrWords = 8;
 enum { H_MAGIC = 0, H_S, H_B, H_R, H_NC, H_NQT, H_REC_WORDS, H_RECS_OFF };
 
@@ -34,7 +35,7 @@ inline MaskDims mask_dims(const tsd_layout& L) {
   MaskDims m;
   const int N = L.n_branches * L.rows_per_branch;
   m.n_qt = (N + kTile - 1) / kTile;
-  m.rec_words = 2 + 2 * m.n_qt;
+  m.rec_words = 2 + 2 * ((N + kKeyTile - 1) / kKeyTile);
   m.lens_off = kHdrWords;
   m.recs_off = kHdrWords + ((L.batch + 3) / 4) * 4;
   m.bytes = (size_t)(m.recs_off + (size_t)L.batch * m.n_qt * m.rec_words) * 4;

@@ -11,9 +11,9 @@ __device__ __forceinline__ bool branch_sees(const uint64_t* vis, int s, int B, i
   return (vis[((size_t)s * B + bq) * words + (bk >> 6)] >> (bk & 63)) & 1ull;
 }
 
-// A warp per (sequence, query tile), a lane per draft tile: the slots of a draft tile are 1, 2 or 4 neighbouring bits of
-// one visibility word, so a lane reads one word per query slot.  (A thread per query tile that tested every pair
-// of branches with a load of its own took 9.3 us for 2 sequences x 20 branches of 32 rows; this takes 2.6.)
+// A warp per (sequence, query tile), a lane per key tile, which holds one or two branches (or half a one).
+// (A thread per query tile that tested every pair of branches with a load of its own took 9.3 us for 2 sequences x 20
+// branches of 32 rows; this takes 2.6.)
 __global__ void __launch_bounds__(128)
 build_mask_kernel(int S, int B, int R, int Nc, int n_qt, int rec_words, int lens_off, int recs_off,
                   const uint64_t* __restrict__ vis, const int32_t* __restrict__ cache_lens, int32_t* __restrict__ blob) {
@@ -30,21 +30,21 @@ build_mask_kernel(int S, int B, int R, int Nc, int n_qt, int rec_words, int lens
   }
   if (t >= S * n_qt) return;
   const int s = t / n_qt, qt = t % n_qt;
-  const int slots = kTile / R, words = (B + 63) / 64;
+  const int slots = kTile / R, words = (B + 63) / 64, n_kt = (B * R + kKeyTile - 1) / kKeyTile;
   int32_t* rec = blob + recs_off + (size_t)t * rec_words;
   int count = 0;
-  for (int kt0 = 0; kt0 < n_qt; kt0 += 32) {
-    const int kt = kt0 + lane, b0 = kt * slots;  // first branch of the draft tile
+  for (int kt0 = 0; kt0 < n_kt; kt0 += 32) {
+    const int kt = kt0 + lane;
+    const int bk[2] = {kt * kKeyTile / R, (kt * kKeyTile + 32) / R};  // branches of the tile's two groups of 32 rows
     unsigned bits = 0;
-    if (kt < n_qt) {
-      const unsigned exist = (1u << min(slots, B - b0)) - 1u;  // slots that hold a branch
+    if (kt < n_kt) {
 #pragma unroll
       for (int qs = 0; qs < 4; ++qs) {
         const int bq = qt * slots + qs;
         if (qs >= slots || bq >= B) continue;
-        unsigned seen = vis ? (unsigned)(vis[((size_t)s * B + bq) * words + (b0 >> 6)] >> (b0 & 63)) & exist : 0u;
-        if (kt == qt) seen |= 1u << qs;  // bidirectional inside the own block
-        bits |= seen << (qs * 4);
+#pragma unroll
+        for (int w = 0; w < 2; ++w)
+          if (bk[w] < B && branch_sees(vis, s, B, words, bq, bk[w])) bits |= 1u << (qs * 2 + w);
       }
     }
     const unsigned listed = __ballot_sync(0xffffffffu, bits != 0);

@@ -105,7 +105,7 @@ def test_mask_dense_matches_oracle_with_vis_and_ragged_cache():
 @pytest.mark.parametrize("R,Bn", [(32, 1), (32, 63), (32, 130), (32, 256), (64, 2), (64, 65), (128, 40), (128, 256)])
 @pytest.mark.parametrize("isolated", [True, False])
 def test_mask_lists_of_many_and_odd_branches(R, Bn, isolated):
-    # the compact lists themselves (one warp per query tile, 32 draft tiles at a time, up to 4 visibility words per branch)
+    # the compact lists themselves (one warp per query tile, 32 key tiles at a time, up to 4 visibility words per branch)
     S, Nc, slots = 2, 70, 128 // R
     layout = B.make_layout(S, Bn, R, Nc, 1, 1, 64, B.TSD_BF16)
     rng = np.random.default_rng(Bn)
@@ -119,17 +119,18 @@ def test_mask_lists_of_many_and_odd_branches(R, Bn, isolated):
     blob = torch.full((B.tsd_branch_mask_bytes(layout) // 4,), -7, dtype=torch.int32, device=DEV)
     B.tsd_build_branch_mask(layout, vis, lens, blob)
     got = blob.cpu().numpy()
-    n_qt = (Bn + slots - 1) // slots
+    n_qt, n_kt = (Bn + slots - 1) // slots, (Bn * R + 63) // 64
     assert got[1:6].tolist() == [S, Bn, R, Nc, n_qt] and got[8:10].tolist() == [70, 0]
     sees |= np.eye(Bn, dtype=bool)
     for s_ in range(S):
         for qt in range(n_qt):
             want = []
-            for kt in range(n_qt):
-                part = sees[s_, qt * slots:(qt + 1) * slots, kt * slots:(kt + 1) * slots]
-                bits = sum(1 << (q * 4 + k) for q, k in zip(*np.nonzero(part)))
+            for kt in range(n_kt):
+                part = sees[s_, qt * slots:(qt + 1) * slots]
+                bits = sum(1 << (q * 2 + w) for q in range(len(part)) for w in range(2)
+                           if (kt * 64 + w * 32) // R < Bn and part[q, (kt * 64 + w * 32) // R])
                 want += [kt, bits] if bits else []
-            rec = got[12 + (s_ * n_qt + qt) * (2 + 2 * n_qt):]
+            rec = got[12 + (s_ * n_qt + qt) * (2 + 2 * n_kt):]
             assert rec[0] == len(want) // 2 and rec[2:2 + len(want)].tolist() == want
 
 
