@@ -14,9 +14,11 @@
 //      (a handful per row, served by L2); the values >= bound go into a small pool in shared
 //      memory, from which one warp picks the k best by counting ranks (no sort, no shuffles).
 //      A pool that would overflow (heavy ties) falls back to merging per-lane lists by shuffles.
-// With few rows a row is split into segments handled by different blocks; the last block to finish
-// a row (a ticket word in the workspace, no spinning, no clearing between calls) merges the
-// segment partials in segment order, so the result does not depend on arrival order.
+// With few rows a row is split into segments handled by different blocks.  Up to eight of them form a thread-block
+// cluster and leave their partials in the shared memory of its first block; with more, the last block to finish a row
+// (a ticket word in the workspace, no spinning, no clearing between calls) merges the partials.  Either way in
+// segment order, so the result does not depend on arrival order.  (32 rows x 152064 in 4 segments: 9.2 us with
+// tickets, 6.8 with clusters: publish, fence, ticket and re-read are a chain of global round trips.)
 //
 // Ordering is (logit descending, index ascending) on the raw input values (bf16 and fp32 both
 // widen to fp32 exactly), so indices are uniquely defined.
@@ -30,6 +32,7 @@ namespace tsd {
 constexpr int kTopkUnroll = 4;            // chunks per thread per batch
 constexpr int kTopkSegChunks = 32768;     // chunks per segment at most (batch maxima: 32 KB of smem)
 constexpr int kMaxSegments = 32;
+constexpr int kMaxCluster = 8;            // blocks of a cluster at most (the portable size)
 constexpr int kPoolCap = 64;              // candidate pool of a block (entries)
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -76,6 +79,19 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+
+// Thread-block clusters: shared memory of another block, and the barrier over all threads that have not left.
+__device__ __forceinline__ uint32_t cluster_address(const void* p, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t bmax2(uint32_t a, uint32_t b) {
   uint32_t r;
@@ -262,6 +278,7 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   __shared__ float s_res_v[K];
   __shared__ int s_res_i[K];
   __shared__ Partial<K> s_part[kTopkWarps];           // shuffle-merge path only
+  __shared__ Partial<K> s_seg[kMaxCluster];           // the segments of a row (first block of a cluster)
   const int64_t row = blockIdx.x / n_seg;
   const int seg = blockIdx.x % n_seg;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -272,6 +289,8 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   const int c1 = min(c0 + chunks_per_seg, chunks_total);
   const int n_iter = (c1 - c0 + kTopkBatch - 1) / kTopkBatch;  // <= kTopkMaxIter (host-enforced)
   const bool has_tail = seg == n_seg - 1 && tid == 0 && chunks_total * E_ < vocab;
+  const bool clustered = n_seg > 1 && n_seg <= kMaxCluster;
+  if (clustered) cluster_arrive_relaxed();  // "has started": waited for before anything is written to another block
 
   grid_wait(rowp, rowv);
   if (launch_next == kNextAtOnce) grid_launch_next();
@@ -479,7 +498,36 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
     finalize(a, k, row, lane, conf, topk_idx, topk_prob, lse);
     return;
   }
-  // several segments per row: publish this one, the last to arrive merges all of them
+  if (clustered) {
+    cluster_wait();
+    const uint32_t to = cluster_address(&s_seg[seg], 0);
+    if (lane == 0) {
+      st_cluster(to, a.seen ? a.e : -CUDART_INF_F);
+      st_cluster(to + 4, a.s);
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+      if (lane == j) {
+        st_cluster(to + 8 + 4 * j, a.v[j]);
+        st_cluster(to + 8 + 4 * K + 4 * j, __int_as_float(a.i[j]));
+      }
+    cluster_arrive();
+    if (seg != 0) return;
+    cluster_wait();
+    a.init();
+    if (lane < n_seg) {
+      const float pe = s_seg[lane].e;
+      a.seen = pe != -CUDART_INF_F;
+      a.e = a.seen ? pe : 0.f;
+      a.s = s_seg[lane].s;
+#pragma unroll
+      for (int j = 0; j < K; ++j) { a.v[j] = s_seg[lane].v[j]; a.i[j] = s_seg[lane].i[j]; }
+    }
+    warp_merge(a);
+    finalize(a, k, row, lane, conf, topk_idx, topk_prob, lse);
+    return;
+  }
+  // many segments per row: publish this one, the last to arrive merges all of them
   bool last = false;
   if (lane == 0) {
     Partial<K>* p = partials + row * n_seg + seg;
@@ -515,7 +563,7 @@ static int round_k(int k) { return k <= 4 ? k : (k <= 6 ? 6 : 8); }
 
 static void scratch_layout(int64_t n_rows, TopkPlan& p) {
   const size_t rec = 8 + 8 * (size_t)p.K;
-  p.partial_bytes = p.n_seg > 1 ? (size_t)n_rows * p.n_seg * rec : 0;
+  p.partial_bytes = (size_t)n_rows * p.n_seg * rec;
   p.ticket_off = (p.partial_bytes + 15) / 16 * 16;
   p.total_bytes = p.n_seg > 1 ? p.ticket_off + ((size_t)n_rows * 4 + 15) / 16 * 16 : 0;
 }
@@ -536,12 +584,19 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
   TopkPlan p;
   p.K = round_k(k);
   const int chunks = vocab / elems_per_chunk;
-  // Few rows: split rows as long as every segment has an SM of its own.  (One more segment per row, so that every
-  // SM has one and some have two, costs more than the idle SMs: 32 rows x 152064 bf16 in 5 segments 10.2 us, in
-  // 4 segments 9.4; 100 x 126464 in 2 segments 13.4, whole 11.8.)
-  int64_t n_seg = n_rows > 0 ? 148 / n_rows : 1;
-  n_seg = std::min<int64_t>(n_seg, kMaxSegments);
-  n_seg = std::min<int64_t>(n_seg, std::max(1, chunks / 2048));
+  // Few rows are split into 2, 4 or 8 segments where that shortens what the busiest SM streams, in rows of 126464 bf16
+  // (7.3 us each), by more than a split costs (1.2 us and a little per segment).  Measured, 126464 bf16: 8 rows whole
+  // 9.1 us, in 8 segments 5.7; 50 rows 11.0, in 2 9.1, in 8 8.6; 74 rows 11.2, in 2 9.8, in 4 10.4; 100 rows 11.6, in 4
+  // 11.2; 148 rows 12.3, in 2 12.7; 200 rows 16.7, in 2 15.8; 256 rows 17.1, in 2 18.1; of 32000: 32 rows 5.0, in 4 5.5.
+  int64_t n_seg = 1;
+  if (n_rows > 0 && n_rows <= 222) {
+    double best = 1e30;
+    for (int n = 1; n <= (n_rows <= 148 ? kMaxCluster : 2); n *= 2) {
+      const double rounds = (double)((n_rows * n + 147) / 148) / n;
+      const double cost = rounds * chunks / 15808 + (n > 1 ? 0.17 + 0.005 * n : 0.0);
+      if (cost < best) { best = cost; n_seg = n; }
+    }
+  }
   // a segment may span at most kTopkSegChunks chunks (its batch maxima live in shared memory)
   n_seg = std::max<int64_t>(n_seg, (chunks + kTopkSegChunks - 1) / kTopkSegChunks);
   p.n_seg = (int)std::max<int64_t>(n_seg, 1);
@@ -549,6 +604,8 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
   // 384 17.9, with 256 18.8; 444 x 126464 25.0 / 23.5 / 24.4; 960 x 126464 50.2 / 48.2 / 46.0.
   const int64_t units = n_rows * p.n_seg;
   p.threads = units <= 2 * 148 ? 512 : (units <= 3 * 148 ? 384 : 256);
+  // clusters of large blocks are hard to place: 74 x 126464 in 4 segments 12.8 us with 512 threads, 10.4 with 256
+  if (p.n_seg > 1 && units > 148) p.threads = 256;
   // L2 prefetch distance in batches (measured): with very many waves of blocks, requesting lines three batches ahead
   // adds 2 % of bandwidth (16384 x 126464: 687 us, without 700); with fewer it delays the demand loads (4096 x 32000:
   // 57.0 us, without 53.6; 4096 x 126464: 171 and 167; 4096 x 152064: 189.7 and 190.8)
@@ -556,6 +613,7 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
   p.chunks_per_seg = (chunks + p.n_seg - 1) / p.n_seg;
   if (p.chunks_per_seg == 0) p.chunks_per_seg = 1;
   scratch_layout(n_rows, p);
+  if (p.n_seg <= kMaxCluster) p.total_bytes = 0;  // the segments meet in shared memory
   return p;
 }
 
@@ -565,7 +623,7 @@ static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   unsigned* tickets = reinterpret_cast<unsigned*>(static_cast<char*>(ws) + p.ticket_off);
   auto kernel = p.threads == 512 ? confidence_topk_kernel<T, K, 512>
               : p.threads == 384 ? confidence_topk_kernel<T, K, 384> : confidence_topk_kernel<T, K, 256>;
-  return launch(kernel, (unsigned)(a.n_rows * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
+  return launch_clusters(p.n_seg <= kMaxCluster ? p.n_seg : 1, kernel, (unsigned)(a.n_rows * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
                 a.row_stride, a.k, p.n_seg, p.chunks_per_seg, a.conf, a.topk_idx, a.topk_prob, a.lse, partials, tickets,
                 p.prefetch, a.launch_next);
 }

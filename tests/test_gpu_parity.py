@@ -377,14 +377,14 @@ def test_topk_ragged_vocab_and_heavy_ties(dtype, k):
         _check_topk(buf[:, :V], min(k, V))
 
 
-@pytest.mark.parametrize("n,V", [(73, 40000), (75, 40000), (148, 5000), (149, 5000), (296, 3000), (297, 3000), (444, 3000), (445, 3000),
+@pytest.mark.parametrize("n,V", [(1, 126464), (18, 70001), (19, 126464), (37, 126464), (73, 80000), (75, 126464), (148, 5000), (149, 126464), (222, 126464), (223, 80000), (296, 3000), (297, 3000), (444, 3000), (445, 3000),
                                  (8191, 300), (8192, 300), (320, 262136)])
 def test_topk_at_the_borders_of_its_plans(n, V):
-    # either side of every row count at which segments, threads per block or prefetch change, and the longest row of one segment
-    # under 384 threads, whose last batch is a partial one
+    # either side of every row count at which segments, threads per block or prefetch change (1, 2, 4 and 8 segments per row), and
+    # the longest row of one segment under 384 threads, whose last batch is a partial one
     g = torch.Generator(device=DEV).manual_seed(n)
     x = (torch.randn((n, (V + 7) // 8 * 8), generator=g, device=DEV) * 3).bfloat16()[:, :V]
-    _check_topk(x, 3, rows=sorted({0, 1, n // 2, n - 2, n - 1}))
+    _check_topk(x, 3, rows=sorted({0, min(1, n - 1), n // 2, max(n - 2, 0), n - 1}))
 
 
 @pytest.mark.parametrize("seed", range(10))
