@@ -28,13 +28,10 @@ dequant_e4m3_kernel(const uint8_t* __restrict__ k_src, const uint8_t* __restrict
   const float* scale = is_v ? v_scale : k_scale;
   __nv_bfloat16* dst = is_v ? v_dst : k_dst;
   uint4* o = reinterpret_cast<uint4*>(dst + (((s * Nc + row) * H + h) * (int64_t)d + c * 16));
-  // rows at or past the sequence's cache length (from the mask blob) hold whatever the caller left
-  // there, the NaN codes 0x7f / 0xff included: they are written as zeros and never decoded
-  if ((int)row >= min(max(mask_blob[kHdrWords + s], 0), Nc)) {
-    o[0] = make_uint4(0u, 0u, 0u, 0u);
-    o[1] = make_uint4(0u, 0u, 0u, 0u);
-    return;
-  }
+  // Rows at or past the sequence's cache length (from the mask blob) hold whatever the caller left there, the NaN codes
+  // 0x7f / 0xff included: they are not decoded, and what their places in the copy hold does not matter (keys past
+  // the length are masked, their V rows zeroed on chip).
+  if ((int)row >= min(max(mask_blob[kHdrWords + s], 0), Nc)) return;
   const uint4 w = *reinterpret_cast<const uint4*>(src + s * ss_b + row * ss_r + h * ss_h + c * 16);
   const float sc = scale ? scale[s * H + h] : 1.f;
   const uint32_t words[4] = {w.x, w.y, w.z, w.w};
