@@ -122,10 +122,11 @@ enum Bar {
                   //     is why this is a ring of four although there are only two P buffers.
   DEC = 24,       // [4][4] exponent offsets of a tile decided, per tile mod 4 and warp quarter
   O_FREE = 40,    // the epilogue has read O into registers
-  LPART = 41,     // every softmax warp has published its partial row sums of an item
-  STAGED = 42,    // the output tile is complete in the staging buffer
-  OS_FREE = 43,   // the previous item's store has read the staging buffer
-  N_BARS = 44
+  LPART = 41,     // [3] every softmax warp has published its partial row sums of an item, per item mod 3: a warpgroup
+                  //     without a tile in an item arrives for it while others are still at the item before
+  STAGED = 44,    // the output tile is complete in the staging buffer
+  OS_FREE = 45,   // the previous item's store has read the staging buffer
+  N_BARS = 46
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -470,7 +471,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     }
     for (int i = 0; i < 16; ++i) mbar_init(bar(DEC + i), 1);
     mbar_init(bar(O_FREE), 4);
-    mbar_init(bar(LPART), kSoftmaxWarps);
+    for (int i = 0; i < 3; ++i) mbar_init(bar(LPART + i), kSoftmaxWarps);
     mbar_init(bar(STAGED), 4);
     mbar_init(bar(OS_FREE), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -927,7 +928,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       lpart[(it % 3) * 384 + wg * kTile + r] = l;
       mpart[(it % 3) * 384 + wg * kTile + r] = m_mine;
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(LPART));
+      if (lane == 0) mbar_arrive(bar(LPART + it % 3));
       G += T;
     }
   } else {
@@ -946,7 +947,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       item_coords(it, s, h, qt);
       const int T = item_T[it], Gl = G + T - 1;
       if (tid == kFirstEpilogueWarp * 32) TSD_TR(5, 255 - it);
-      ok = mbar_wait(bar(LPART), it & 1, abort_flag, 200);
+      ok = mbar_wait(bar(LPART + it % 3), (it / 3) & 1, abort_flag, 200);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       if (tid == kFirstEpilogueWarp * 32) TSD_TR(0, 255 - it);

@@ -316,6 +316,15 @@ def test_attention_head_dim_64_tensor_cores(R, Bn, Nc, lens):
     assert (np.abs(_np(step.out) - ref) <= 2.0 ** -8 * np.abs(ref) + 6 * 2.0 ** -16).all()
 
 
+@pytest.mark.parametrize("S,Bn,Nc,d", [(300, 2, 0, 128), (300, 2, 0, 64), (160, 2, 64, 128), (200, 4, 30, 64)])
+def test_attention_many_items_of_few_key_tiles(S, Bn, Nc, d):
+    """Blocks that walk several work items of one or two key tiles: fewer than there are softmax warpgroups, so that
+    some warpgroups pass an item without a tile of it while others are still at the one before."""
+    cfg = W.small(W.CONFIGS["cfg2"], S=S, B=Bn, R=32, Nc=Nc, Hq=2, Hkv=2, d=d)
+    lens = torch.tensor([(7 * s) % (Nc + 1) for s in range(S)], dtype=torch.int32, device=DEV)
+    _check_attention(cfg, W.attention_inputs(cfg, DEV), 0, cache_lens=lens, seqs=[0, 1, S // 2, S - 2, S - 1])
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("S,Bn,R,Nc,Hq,Hkv,lens", [(1, 1, 32, 0, 1, 1, None), (1, 3, 32, 31, 2, 1, None), (2, 2, 64, 97, 2, 2, [97, 1]),
                                                    (1, 8, 32, 400, 4, 2, None), (2, 3, 128, 64, 3, 1, [33, 64])])
