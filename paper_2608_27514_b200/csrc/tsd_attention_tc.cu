@@ -37,6 +37,11 @@
 // buffer during the current item, its first Q K^T are issued while the last softmax tiles of the
 // current item run, the softmax warpgroups go on to it without waiting for the epilogue, and its
 // first P V waits only until the epilogue has read O into registers.
+// Few items (kCut): an item is shared by the blocks of a cluster, each with a stretch of its key tiles; at the end every block hands
+// every other one a share of the columns of its O through distributed shared memory and finishes the share that is
+// its own.  Bound by the serial chain of one item otherwise: 28 items of 81 key tiles took 40.6 us on 28 SMs and take 18.7 on 112,
+// 56 items 41.6 -> 27.6, 16 items of 81 tiles 40.8 -> 18.2 (64-wide heads: 4 items of 34 tiles 24.3 -> 11.7).  A
+// kernel of its own, so that the loops of whole items keep their registers (in one kernel: 256 items 31.7 -> 36.4 us).
 // Every mbarrier wait is bounded: on expiry the block raises TSD_STATUS_TIMEOUT, stops issuing
 // work, waits (bounded) for its copies in flight, frees its tensor memory and returns.
 #include <cuda.h>
@@ -50,7 +55,7 @@ constexpr int kTcThreads = 640;
 constexpr int kSoftmaxWarps = 12;              // three warpgroups: warps 4-15
 // The issuing roles take the lowest warp indices: the schedulers favour them over the softmax
 // warps they share a sub-partition with, and a late MMA or copy stalls the whole pipeline.
-constexpr int kQkWarp = 0, kKProducerWarp = 1, kPvWarp = 2, kVProducerWarp = 3, kFirstSoftmaxWarp = 4;
+constexpr int kQkWarp = 0, kKProducerWarp = 1, kVProducerWarp = 3, kFirstSoftmaxWarp = 4;  // P V: warp 2
 constexpr int kFirstEpilogueWarp = kFirstSoftmaxWarp + kSoftmaxWarps;  // warps 16-19
 // Registers per thread after the warpgroups have traded them (the block starts with 96 each):
 // what the softmax threads gain (384 x 24) is exactly what the others release (128 x 40 + 128 x 32):
@@ -97,6 +102,10 @@ struct TcCols {
   static constexpr uint32_t kS = 2 * D, kP = kS + kNSb * kKeys;     // three S buffers, two P buffers
   static_assert(kP + kNP * kPCols <= 512, "tensor memory has 512 columns");
 };
+// What putting two parts of an item together takes, in key tiles of 0.43 us; 2 more with each doubling.  (56 items of 81
+// tiles in halves: 27.6 us, 40 tiles less than 41.6; 28 in quarters: 18.7, 60 tiles less than 40.6.  Two thirds of it is the way of the
+// columns between the SMs, ~20 bytes per clock and SM.  64 items of 14 tiles would gain nothing: 12.7 whole, 13.0 in halves.)
+constexpr int kMeetTiles = 7;
 constexpr uint32_t kSpinLimit = 1u << 21;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -126,7 +135,9 @@ enum Bar {
                   //     without a tile in an item arrives for it while others are still at the item before
   STAGED = 44,    // the output tile is complete in the staging buffer
   OS_FREE = 45,   // the previous item's store has read the staging buffer
-  N_BARS = 46
+  ROOM = 46,      // cut items: every other block of the cluster has room for this one's part
+  PARTS = 47,     // [4] cut items: the other blocks' parts are here, per epilogue warp
+  N_BARS = 51     // (the words behind them start at 56)
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -175,6 +186,39 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
       ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+}
+
+// Blocks of a cluster.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_address(uint32_t addr, int rank) {  // the same address in another block's shared memory
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void cluster_arrive_at(uint32_t remote_bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote_bar) : "memory");
+}
+// Stores to another block that count their bytes on a barrier there.
+__device__ __forceinline__ void cluster_store4(uint32_t addr, const uint32_t* v, uint32_t remote_bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(remote_bar) : "memory");
+}
+__device__ __forceinline__ void cluster_store2(uint32_t addr, float x, float y, uint32_t remote_bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+               ::"r"(addr), "r"(__float_as_uint(x)), "r"(__float_as_uint(y)), "r"(remote_bar) : "memory");
+}
+// mbar_wait on what other blocks of the cluster did.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
+  for (uint32_t it = 0; it < kSpinLimit; ++it) {
+    uint32_t ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return true;
+    if ((it & 255u) == 255u && *abort_flag) return false;
+  }
+  *abort_flag = 1u;
+  return false;
 }
 
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
@@ -312,6 +356,9 @@ struct TcParams {
   int n_items;                    // S * Hq * n_qt
   float scale_log2e;              // sm_scale * log2(e), > 0
   int concurrent;
+  int cut;                        // blocks per item (a cluster), each with a stretch of its key tiles; 1: whole items
+  __nv_bfloat16* out;             // where cut items are written without a tensor map
+  int64_t os_b, os_r, os_h;
 };
 
 // The MMAs of a tile go out as ONE block of instructions: the issuing lane shares its scheduler with
@@ -407,7 +454,7 @@ __device__ __noinline__ void copy_q_row(uint32_t q_smem, int r, uint32_t t_q) {
   tmem_wait_st();
 }
 
-template <int D>
+template <int D, bool kCut>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kc,
                     const __grid_constant__ CUtensorMap map_vc, const __grid_constant__ CUtensorMap map_kd,
@@ -423,6 +470,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   const uint32_t bars = base + kOffBar;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + kOffBar + 448);
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(base_ptr + kOffBar + 452);
+  volatile int32_t* parts = reinterpret_cast<volatile int32_t*>(base_ptr + kOffBar + 464);  // of a cut item
+  volatile int32_t* tile_first = reinterpret_cast<volatile int32_t*>(base_ptr + kOffBar + 460);  // of the block's first item
   float* mref = reinterpret_cast<float*>(base_ptr + L::kOffMref);
   float* lpart = reinterpret_cast<float*>(base_ptr + L::kOffLpart);
   float* mpart = reinterpret_cast<float*>(base_ptr + L::kOffMpart);
@@ -444,11 +493,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     prefetch_tensormap(&map_o);
   }
   const int32_t* mask = p.mask;
-  const int n_my = (int)blockIdx.x < p.n_items ? (p.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+  const int n_my = kCut ? 1 : (int)blockIdx.x < p.n_items ? (p.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+  const int rank = kCut ? (int)blockIdx.x % p.cut : 0;
   // item -> (sequence, query head, query tile); query tiles of a head, then heads, then sequences
   // are neighbours, so that blocks running at the same time share K/V in L2
   auto item_coords = [&](int it, int& s, int& h, int& qt) {
-    const int item = (int)blockIdx.x + it * (int)gridDim.x;
+    const int item = kCut ? (int)blockIdx.x / p.cut : (int)blockIdx.x + it * (int)gridDim.x;
     qt = item % p.n_qt;
     h = (item / p.n_qt) % p.Hq;
     s = item / (p.n_qt * p.Hq);
@@ -474,9 +524,17 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     for (int i = 0; i < 3; ++i) mbar_init(bar(LPART + i), kSoftmaxWarps);
     mbar_init(bar(STAGED), 4);
     mbar_init(bar(OS_FREE), 1);
+    if (kCut) {
+      mbar_init(bar(ROOM), p.cut - 1);
+      for (int i = 0; i < 4; ++i) {  // a part comes as bytes: D / cut columns and (m, l) of 32 rows from each other block
+        mbar_init(bar(PARTS + i), 1);
+        mbar_expect_tx(bar(PARTS + i), (uint32_t)(p.cut - 1) * 32u * (uint32_t)(D / p.cut * 4 + 8));
+      }
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
+  if (kCut) cluster_arrive();  // "barriers set up"; waited for before another block's are touched
   // Everything above runs while the previous kernel of the stream finishes.  Tensor memory is allocated only
   // after the wait: a block of that kernel may still need it.
   // Beside the kernel before it nothing is waited for but an acquire fence, so that no line the SM still holds from
@@ -499,7 +557,15 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     const int n_dt = min(max(mask[p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words], 1), p.rec_words / 2 - 1);
     const int n_ct = (clen + kKeys - 1) / kKeys;
     item_clen[it] = clen;
-    item_T[it] = n_ct + n_dt;
+    int T = n_ct + n_dt, first = 0;
+    if (kCut) {  // this block's stretch; the first block alone takes an item of few tiles
+      const bool whole = T < 2 * p.cut;
+      first = whole ? 0 : rank * T / p.cut;
+      T = whole ? (rank == 0 ? T : 0) : (rank + 1) * T / p.cut - first;
+      *parts = whole ? 1 : p.cut;
+    }
+    if (kCut) *tile_first = first;
+    item_T[it] = T;
   }
 
   // Coordinates of the block's first item for the two producer lanes: worked out here, while the
@@ -527,11 +593,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   // still waited for before the block leaves).
   const bool hdr_ok = h_magic == kMaskMagic && h_s == p.S && h_b == p.B && h_r == p.R && h_nc == p.Nc;
   if (!hdr_ok && tid == 0 && blockIdx.x == 0 && p.status) atomicOr(p.status, TSD_STATUS_BAD_MASK);
-  const int n_run = hdr_ok ? n_my : 0;
 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  const int n_run = hdr_ok && (!kCut || item_T[0] > 0) ? n_my : 0;
   const uint32_t tmem = *tmem_slot;
   if (tid == 0) TSD_TR_ALWAYS(1, 200);
 
@@ -574,13 +640,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       // below is entered: on its first pass that loop costs ~1.5 k clocks of instruction fetches and
       // single-lane index arithmetic before its first request (measured), and the whole block
       // waits for these tiles.
-      const int n_pre = n_run > 0 ? min(n_stage, (item_clen[0] + kKeys - 1) / kKeys) : 0;
+      const int t_first = kCut ? *tile_first : 0;
+      const int n_pre = n_run > 0 ? max(0, min(kCut ? min(n_stage, item_T[0]) : n_stage, (item_clen[0] + kKeys - 1) / kKeys - t_first)) : 0;
       for (int t = 0; t < n_pre; ++t) {
         const uint32_t dst = stage0 + t * kKVBytes, full_bar = bar(full0 + t);
         mbar_expect_tx(full_bar, kKVBytes);
         if (is_k && t < kNSb) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], 4;" ::"r"(full_bar) : "memory");
-        tma_load_4d(dst, mc, full_bar, 0, g_first, t * kKeys, s_first);
-        if (D == 128) tma_load_4d(dst + kSubKV, mc, full_bar, 64, g_first, t * kKeys, s_first);
+        tma_load_4d(dst, mc, full_bar, 0, g_first, (t_first + t) * kKeys, s_first);
+        if (D == 128) tma_load_4d(dst + kSubKV, mc, full_bar, 64, g_first, (t_first + t) * kKeys, s_first);
       }
       issued = n_pre;
       for (int it = 0; it < n_run && ok; ++it) {
@@ -590,7 +657,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         item_coords(it, s, h, qt);
         const int g = h / p.group, n_ct = (item_clen[it] + kKeys - 1) / kKeys, T = item_T[it];
         const int32_t* rec = mask + p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words;
-        for (int j = 0; j < T && ok; ++j, ++G) {
+        const int j0 = kCut ? *tile_first : 0;
+        for (int j = j0; j < j0 + T && ok; ++j, ++G) {
           if (is_k) issue_q(false);
           if (!ok) break;
           // the stage is free once the MMAs that read its previous tile have completed
@@ -612,7 +680,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           if (++b == n_stage) { b = 0; ph ^= 1u; }
         }
       }
-      if (*abort_flag || !hdr_ok) {
+      if (*abort_flag || n_run == 0) {
         // leaving early: give the copies already issued a bounded time to land before the block exits
         volatile uint32_t* scratch = abort_flag + 1;
         if (q_issued > 0) mbar_wait(bar(QS_FULL), (q_issued - 1) & 1, scratch);
@@ -699,7 +767,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         const unsigned bits0 = (unsigned)__ldg(rec + 3);  // visibility of the first listed draft tile, asked for early
         // the first P V of an item overwrites O: the epilogue of the previous item must have read it
         if (it > 0) ok = mbar_wait(bar(O_FREE), (it - 1) & 1, abort_flag);
-        for (int j = 0; j < T; ++j, ++G) {
+        const int j0 = kCut ? __shfl_sync(0xffffffffu, *tile_first, 0) : 0;
+        for (int j = j0; j < j0 + T; ++j, ++G) {
           const int b = G & 3;  // V stage; P buffer = G & 1
           if (lane == 0) TSD_TR(5, G);
           const long long c0 = TSD_CLK();
@@ -744,7 +813,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             uint32_t lo[kKeys / 16];
 #pragma unroll
             for (int kk = 0; kk < kKeys / 16; ++kk) lo[kk] = vd_lo[kk] + v_off;
-            issue_pv_mmas<D>(utmem + C::kO, utmem + C::kP + (uint32_t)(b & 1) * C::kPCols, lo, vd_hi, j == 0 ? 0u : 1u, bar(PV_DONE + b));
+            issue_pv_mmas<D>(utmem + C::kO, utmem + C::kP + (uint32_t)(b & 1) * C::kPCols, lo, vd_hi, j == j0 ? 0u : 1u, bar(PV_DONE + b));
           }
           __syncwarp();
           ready = seen;
@@ -790,7 +859,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       item_coords(it, s, h, qt);
       const int32_t* rec = mask + p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words;
       const int clen = item_clen[it];
-      const int n_ct = (clen + kKeys - 1) / kKeys, T = item_T[it];
+      const int T = item_T[it], j0 = kCut ? *tile_first : 0;  // tiles of the item from j0 on
+      const int n_ct = (clen + kKeys - 1) / kKeys - j0;  // the cached ones among them (negative: behind the first draft tiles)
       const int jc = min(4, T - 1);  // the tile at which Q of the next item is copied
       float m_mine = -CUDART_INF_F, l = 0.f;  // the exponent offset this thread used last, its partial row sum
       // tile t goes to warpgroup t mod 3, which is also its S buffer; n_done counts this
@@ -821,7 +891,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         uint32_t cm[2] = {0xffffffffu, 0xffffffffu};
         bool masked = false;
         if (j < n_ct) {
-          const int valid = clen - j * kKeys;  // keys past the sequence's cache length are invisible
+          const int valid = clen - (j0 + j) * kKeys;  // keys past the sequence's cache length are invisible
           if (valid < kKeys) {
             masked = true;
 #pragma unroll
@@ -942,7 +1012,100 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     const uint32_t t_lane = tmem + ((uint32_t)(wq * 32) << 16);
     bool ok = true;
     int G = 0;
-    for (int it = 0; it < n_run && ok; ++it) {
+    if (kCut) cluster_wait();
+    const bool shared = kCut && n_run > 0 && *parts > 1;
+    if (shared) {
+      // A part of an item, the block's only work: each block of the cluster hands every other one D / cut columns of O and
+      // (m, l) of all rows and finishes the columns that are its own.  Warps of the same rows do this among themselves.
+      int s, h, qt;
+      item_coords(0, s, h, qt);
+      const int n = p.cut, cols = D / n, row = qt * kTile + r, last = item_T[0] - 1;
+      constexpr uint32_t kOffMl = D == 128 ? 57344 : 24576;  // in the staging buffers of Q and O, behind the parts
+      static_assert(kOffMl + (D == 128 ? 8 : 4) * 1024 <= 2 * kTileBytes, "room for parts");
+      // once Q is in tensor memory, the staging buffers take what the other blocks send
+      if (warp == kFirstEpilogueWarp) {
+        ok = mbar_wait(bar(QT_READY), 0, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok && lane < n && lane != rank) cluster_arrive_at(cluster_address(bar(ROOM), lane));
+      }
+      // [source block without this one][cols / 4][128 rows] of 4 columns
+      auto at = [&](int of, int to, int col) { return (uint32_t)((((of < to ? of : of - 1) * cols + col) >> 2) * 128 + r) * 16u; };
+      ok = ok && mbar_wait(bar(LPART), 0, abort_flag, 100);
+      ok = __all_sync(0xffffffffu, ok);
+      const float m0 = mpart[r], m1 = mpart[kTile + r], m2 = mpart[2 * kTile + r];
+      const float m = fmaxf(m0, fmaxf(m1, m2));  // the offsets only grow along the tiles
+      auto weight = [&](float of, float to) { return of == -CUDART_INF_F ? 0.f : ex2f(of - to); };
+      const float l = (lpart[r] * weight(m0, m) + lpart[kTile + r] * weight(m1, m)) + lpart[2 * kTile + r] * weight(m2, m);
+      ok = ok && mbar_wait_cluster(bar(ROOM), 0, abort_flag) && mbar_wait(bar(PV_DONE + (last & 3)), (last >> 2) & 1, abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+        tc_fence_after();
+#pragma unroll 1
+        for (int col = 0; col < D; col += 16) {
+          const int to = col / cols, c = col - to * cols;
+          if (to == rank) continue;
+          const uint32_t there = cluster_address(base, to), there_bar = cluster_address(bar(PARTS + wq), to);
+          uint32_t ov[16];
+          TSD_TMEM_LD16(ov, 0, t_lane + C::kO + col);
+          if (c == 0) cluster_store2(there + kOffMl + (uint32_t)(rank * kTile + r) * 8u, m, l, there_bar);
+          tmem_wait_ld();
+#pragma unroll
+          for (int x = 0; x < 4; ++x) cluster_store4(there + at(rank, to, c + 4 * x), ov + 4 * x, there_bar);
+        }
+        ok = mbar_wait_cluster(bar(PARTS + wq), 0, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+      }
+      if (ok) {
+        auto ml_of = [&](int i) {
+          float2 v = make_float2(m, l);
+          if (i != rank)
+            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(base + kOffMl + (uint32_t)(i * kTile + r) * 8u) : "memory");
+          return v;
+        };
+        float m_all = -CUDART_INF_F, l_all = 0.f;  // over the parts in their order, so that every block has the same
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) m_all = fmaxf(m_all, ml_of(i).x);
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) {
+          const float2 v = ml_of(i);
+          l_all = fmaf(v.y, weight(v.x, m_all), l_all);
+        }
+        const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+        __nv_bfloat16* o_row = p.out + s * p.os_b + row * p.os_r + h * p.os_h + rank * cols;
+#pragma unroll 1
+        for (int col = 0; col < cols; col += 16) {
+          uint32_t ov[16];
+          float acc[16];
+          TSD_TMEM_LD16(ov, 0, t_lane + C::kO + rank * cols + col);
+          tmem_wait_ld();
+          const float f_own = weight(m, m_all) * inv;
+#pragma unroll
+          for (int c = 0; c < 16; ++c) acc[c] = __uint_as_float(ov[c]) * f_own;
+#pragma unroll 1
+          for (int i = 0; i < n; ++i) {
+            if (i == rank) continue;
+            const uint32_t from = base + at(i, rank, col);
+            const float f = weight(ml_of(i).x, m_all) * inv;
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+              float4 v;
+              asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(from + x * 2048) : "memory");
+              acc[4 * x] = fmaf(v.x, f, acc[4 * x]);
+              acc[4 * x + 1] = fmaf(v.y, f, acc[4 * x + 1]);
+              acc[4 * x + 2] = fmaf(v.z, f, acc[4 * x + 2]);
+              acc[4 * x + 3] = fmaf(v.w, f, acc[4 * x + 3]);
+            }
+          }
+          if (row < p.N) {
+            uint4* dst = reinterpret_cast<uint4*>(o_row + col);
+            dst[0] = make_uint4(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]), pack_bf16x2(acc[4], acc[5]), pack_bf16x2(acc[6], acc[7]));
+            dst[1] = make_uint4(pack_bf16x2(acc[8], acc[9]), pack_bf16x2(acc[10], acc[11]), pack_bf16x2(acc[12], acc[13]), pack_bf16x2(acc[14], acc[15]));
+          }
+        }
+        if (rank == 0 && p.lse && row < p.N) p.lse[((size_t)s * p.Hq + h) * p.N + row] = (m_all + log2f(l_all)) * kLn2;
+      }
+    }
+    for (int it = 0; it < (shared ? 0 : n_run) && ok; ++it) {
       int s, h, qt;
       item_coords(it, s, h, qt);
       const int T = item_T[it], Gl = G + T - 1;
@@ -1025,6 +1188,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
   // ---------------------------------------------------------------- teardown (all threads)
   if (tid == 0) TSD_TR_ALWAYS(2, 200);
+  if (kCut) {
+    if (warp < kFirstEpilogueWarp) cluster_wait();  // the first phase, which the epilogue has waited for
+    cluster_arrive();
+  }
   tc_fence_before();
   __syncthreads();
   if (tid == 0) TSD_TR_ALWAYS(3, 200);
@@ -1033,6 +1200,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
   if (tid == 0 && *abort_flag && p.status) atomicOr(p.status, TSD_STATUS_TIMEOUT);
+  if (kCut) cluster_wait();  // no block leaves while another may write to its shared memory
   if (p.concurrent) grid_wait();
 }
 
@@ -1123,6 +1291,42 @@ bool attention_tc_supported(const AttnArgs& a) {
 
 size_t attention_tc_workspace_bytes(const tsd_layout&) { return 0; }
 
+// Blocks per item: a launch with fewer items than SMs leaves SMs idle, so an item's key tiles (T of them, over a full cache) are
+// cut over the 2, 4 or 8 blocks of a cluster, as far as the GPU holds all clusters at one time.
+template <int D>
+static int cut_items(int64_t n_items, int T) {
+  static std::mutex mu;
+  static int clusters[kMaxDevices][9];  // clusters of that many blocks that run at one time, + 1
+  const int dev = current_device();
+  if (dev < 0) return 1;
+  std::lock_guard<std::mutex> lock(mu);
+  int best = 1, best_time = T;  // in key tiles
+  for (int n = 2, meet = kMeetTiles; n <= (D == 128 ? 8 : 4); n *= 2, meet += 2) {
+    const int time = (T + n - 1) / n + meet;
+    if (time >= best_time) continue;
+    int& c = clusters[dev][n];
+    if (c == 0) {
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = (unsigned)n;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)n * 64);
+      cfg.blockDim = dim3(kTcThreads);
+      cfg.dynamicSmemBytes = TcSmem<D>::kBytes;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      int found = 0;
+      c = cudaOccupancyMaxActiveClusters(&found, attention_tc_kernel<D, true>, &cfg) == cudaSuccess ? found + 1 : 1;
+      if (c == 1) cudaGetLastError();
+    }
+    if (n_items > c - 1) break;
+    best = n;
+    best_time = time;
+  }
+  return best;
+}
+
 template <int D>
 static int launch_tc(const AttnArgs& a) {
   const tsd_layout& L = a.L;
@@ -1150,7 +1354,9 @@ static int launch_tc(const AttnArgs& a) {
     std::lock_guard<std::mutex> lock(mu);
     if (!done[dev]) {
       cudaError_t attr_err =
-          cudaFuncSetAttribute(attention_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<D>::kBytes);
+          cudaFuncSetAttribute(attention_tc_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<D>::kBytes);
+      if (attr_err == cudaSuccess)
+        attr_err = cudaFuncSetAttribute(attention_tc_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<D>::kBytes);
       if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(attention_tc_kernel)");
       done[dev] = true;
     }
@@ -1169,8 +1375,16 @@ static int launch_tc(const AttnArgs& a) {
   // would not fit the per-block item table
   const int sms = std::max(device_facts().sms, 1);
   int64_t grid = std::min<int64_t>(n_items, sms);
+  p.cut = n_items < sms ? cut_items<D>(n_items, (L.n_cache + kKeys - 1) / kKeys + std::min(2, md.rec_words / 2 - 1)) : 1;
+  p.out = static_cast<__nv_bfloat16*>(a.out);
+  p.os_b = a.os_b; p.os_r = a.os_r; p.os_h = a.os_h;
+  if (p.cut > 1) {
+    cudaError_t e = launch_clusters(p.cut, attention_tc_kernel<D, true>, (unsigned)(n_items * p.cut), kTcThreads, TcSmem<D>::kBytes, a.stream,
+                                    mq, mkc, mvc, mkd, mvd, mo, p);
+    return e != cudaSuccess ? cuda_fail(e, "attention_tc_kernel") : TSD_OK;
+  }
   grid = std::max<int64_t>(grid, (n_items + kMaxItems - 1) / kMaxItems);
-  cudaError_t e = launch(attention_tc_kernel<D>, (unsigned)grid, kTcThreads, TcSmem<D>::kBytes, a.stream, mq, mkc, mvc, mkd,
+  cudaError_t e = launch(attention_tc_kernel<D, false>, (unsigned)grid, kTcThreads, TcSmem<D>::kBytes, a.stream, mq, mkc, mvc, mkd,
                          mvd, mo, p);
   if (e != cudaSuccess) return cuda_fail(e, "attention_tc_kernel");
   return TSD_OK;

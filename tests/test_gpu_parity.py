@@ -325,6 +325,23 @@ def test_attention_many_items_of_few_key_tiles(S, Bn, Nc, d):
     _check_attention(cfg, W.attention_inputs(cfg, DEV), 0, cache_lens=lens, seqs=[0, 1, S // 2, S - 2, S - 1])
 
 
+@pytest.mark.parametrize("S,Bn,R,Nc,Hq,Hkv,d,lens", [
+    (1, 3, 32, 1500, 8, 4, 128, None),                  # 8 items in 8 parts, rows past the last branch
+    (1, 6, 64, 1500, 4, 2, 128, [1499]),                # 12 items in 8 parts of 3 or 4 tiles
+    (2, 5, 32, 1300, 4, 2, 128, [1300, 0]),             # 16 items in 4 parts, the second sequence's too short to be cut
+    (3, 4, 32, 1700, 16, 16, 128, [1700, 65, 1111]),    # 48 items in halves; 4 tiles: as short as a cut item gets
+    (2, 3, 32, 1600, 4, 1, 64, [1600, 1027]),           # 64-wide heads, 4 parts
+    (2, 4, 32, 1400, 24, 8, 64, None),                  # 64-wide heads, halves
+])
+def test_attention_items_shared_by_the_blocks_of_a_cluster(S, Bn, R, Nc, Hq, Hkv, d, lens):
+    cfg = W.small(W.CONFIGS["cfg2"], S=S, B=Bn, R=R, Nc=Nc, Hq=Hq, Hkv=Hkv, d=d)
+    attn = W.attention_inputs(cfg, DEV)
+    lens = None if lens is None else torch.tensor(lens, dtype=torch.int32, device=DEV)
+    _check_attention(cfg, attn, 0, cache_lens=lens)
+    a, b = (_run_attention(cfg, attn, 0, cache_lens=lens)[0] for _ in range(2))
+    assert torch.equal(a.out, b.out) and torch.equal(a.attn_lse, b.attn_lse)
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("S,Bn,R,Nc,Hq,Hkv,lens", [(1, 1, 32, 0, 1, 1, None), (1, 3, 32, 31, 2, 1, None), (2, 2, 64, 97, 2, 2, [97, 1]),
                                                    (1, 8, 32, 400, 4, 2, None), (2, 3, 128, 64, 3, 1, [33, 64])])
