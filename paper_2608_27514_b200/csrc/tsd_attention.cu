@@ -72,7 +72,7 @@ int tsd_verify_attention(const tsd_layout* L, const void* mask, const void* q, i
   a.workspace_bytes = workspace_bytes;
   a.status = status;
   a.stream = stream;
-  a.concurrent = false;
+  a.concurrent = a.next_at_once = false;
   return tsd::launch_attention(a, flags);
 }
 

@@ -72,7 +72,7 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
                       T* __restrict__ out, float* __restrict__ lse, int64_t qs_b, int64_t qs_r, int64_t qs_h,
                       int64_t cs_b, int64_t cs_r, int64_t cs_h, int64_t ds_b, int64_t ds_r, int64_t ds_h,
                       int64_t os_b, int64_t os_r, int64_t os_h, float sm_scale, uint32_t* __restrict__ status,
-                      int concurrent) {
+                      int concurrent, int next_at_once) {
   constexpr int LPK = D / 8;            // lanes per key
   constexpr int KPI = 32 / LPK;         // keys read at once
   constexpr int SUB = LPK / RB;         // reads per group: SUB * RB scores per key lane, one per lane after the scatter
@@ -97,6 +97,7 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
   } else {
     grid_wait(mask, q, kc, vc, kd, vd);
   }
+  if (next_at_once) grid_launch_next();
 
   // the block's query rows, 8 dimensions per lane (requested first: nothing else is needed for them)
   float qr[RB][8];
@@ -274,7 +275,7 @@ static cudaError_t launch_rows(const AttnArgs& a, int warps) {
       md.rec_words, a.mask, static_cast<const T*>(a.q), static_cast<const T*>(a.kc), static_cast<const T*>(a.vc),
       static_cast<const T*>(a.kd), static_cast<const T*>(a.vd), static_cast<T*>(a.out), a.lse, a.qs_b, a.qs_r,
       a.qs_h, a.cs_b, a.cs_r, a.cs_h, a.ds_b, a.ds_r, a.ds_h, a.os_b, a.os_r, a.os_h, a.sm_scale, a.status,
-      (int)a.concurrent);
+      (int)a.concurrent, (int)a.next_at_once);
 }
 
 template <typename T, int D>

@@ -355,7 +355,7 @@ struct TcParams {
   int recs_off, n_qt, rec_words;  // layout of the mask blob, computed on the host from the same tsd_layout
   int n_items;                    // S * Hq * n_qt
   float scale_log2e;              // sm_scale * log2(e), > 0
-  int concurrent;
+  int concurrent, next_at_once;
   int cut;                        // blocks per item (a cluster), each with a stretch of its key tiles; 1: whole items
   __nv_bfloat16* out;             // where cut items are written without a tensor map
   int64_t os_b, os_r, os_h;
@@ -540,12 +540,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   // Beside the kernel before it nothing is waited for but an acquire fence, so that no line the SM still holds from
   // earlier kernels is used; the block then leaves only after that kernel has completed, so that a kernel which waits
   // for this one has waited for both.
-  if (p.concurrent) {
-    __threadfence();
-    settle(mask);
-  } else {
-    grid_wait(mask);
-  }
+  asm volatile("{\n.reg .pred c, n;\nsetp.ne.b32 c, %0, 0;\nsetp.ne.b32 n, %1, 0;\n@c fence.acq_rel.gpu;\n@!c griddepcontrol.wait;\n"
+               "@n griddepcontrol.launch_dependents;\n}" ::"r"(p.concurrent), "r"(p.next_at_once) : "memory");
+  settle(mask);
 
   const int h_magic = mask[H_MAGIC], h_s = mask[H_S], h_b = mask[H_B], h_r = mask[H_R], h_nc = mask[H_NC];
   // tile counts of this block's items (the blob's layout follows from the tsd_layout, so no
@@ -1328,6 +1325,21 @@ static int cut_items(int64_t n_items, int T) {
 }
 
 template <int D>
+static int blocks_per_item(const tsd_layout& L) {
+  const MaskDims md = mask_dims(L);
+  const int64_t n_items = (int64_t)L.batch * L.n_q_heads * md.n_qt;
+  if (n_items >= device_facts().sms) return 1;
+  return cut_items<D>(n_items, (L.n_cache + kKeys - 1) / kKeys + std::min(2, md.rec_words / 2 - 1));
+}
+
+int attention_tc_blocks(const tsd_layout& L) {
+  const int64_t n_items = (int64_t)L.batch * L.n_q_heads * mask_dims(L).n_qt;
+  const int sms = device_facts().sms;
+  if (n_items >= sms) return sms;
+  return (int)n_items * (L.head_dim == 64 ? blocks_per_item<64>(L) : blocks_per_item<128>(L));
+}
+
+template <int D>
 static int launch_tc(const AttnArgs& a) {
   const tsd_layout& L = a.L;
   const int N = L.n_branches * L.rows_per_branch;
@@ -1371,11 +1383,12 @@ static int launch_tc(const AttnArgs& a) {
   p.n_items = (int)n_items;
   p.scale_log2e = a.sm_scale * kLog2e;
   p.concurrent = a.concurrent;
+  p.next_at_once = a.next_at_once;
   // one block per SM, each walking its share of the items; more blocks only when a block's share
   // would not fit the per-block item table
   const int sms = std::max(device_facts().sms, 1);
   int64_t grid = std::min<int64_t>(n_items, sms);
-  p.cut = n_items < sms ? cut_items<D>(n_items, (L.n_cache + kKeys - 1) / kKeys + std::min(2, md.rec_words / 2 - 1)) : 1;
+  p.cut = blocks_per_item<D>(L);
   p.out = static_cast<__nv_bfloat16*>(a.out);
   p.os_b = a.os_b; p.os_r = a.os_r; p.os_h = a.os_h;
   if (p.cut > 1) {

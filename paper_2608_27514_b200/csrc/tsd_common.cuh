@@ -64,17 +64,18 @@ struct AttnArgs {
   size_t workspace_bytes;
   uint32_t* status;
   cudaStream_t stream;
-  bool concurrent;  // reads nothing that the kernel before it in the stream writes: may run beside it
+  bool concurrent;    // reads nothing that the kernel before it in the stream writes: may run beside it
+  bool next_at_once;  // the next kernel may be brought up once all blocks of this one run
 };
 int launch_attention_simt(const AttnArgs& a);
 bool attention_tc_supported(const AttnArgs& a);
 size_t attention_tc_workspace_bytes(const tsd_layout& L);
 int launch_attention_tc(const AttnArgs& a);
+int attention_tc_blocks(const tsd_layout& L);  // that it takes, one per SM
 int launch_attention(const AttnArgs& a, uint32_t flags);
 
-// The vocabulary pass and the acceptance behind their entry points.  `concurrent`: the pass reads nothing
-// that the kernel before it in the stream writes, and may run beside it.  `launch_next`: when the next kernel may be
-// brought up.
+// The vocabulary pass and the acceptance behind their entry points.  `launch_next`: when the next kernel may be
+// brought up.  `concurrent`: the pass reads nothing that the kernel before it in the stream writes, and may run beside it.
 enum { kNextAfter = 0, kNextAtTail = 1, kNextAtOnce = 2 };  // when this one is done; at the end of its rows; with its last blocks
 struct TopkArgs {
   const void* logits;
@@ -90,9 +91,11 @@ struct TopkArgs {
   size_t workspace_bytes;
   cudaStream_t stream;
   int launch_next;
+  bool concurrent;
 };
 int check_topk(const TopkArgs& a);
 int launch_topk(const TopkArgs& a);
+int64_t topk_threads(const TopkArgs& a);  // of all blocks of the pass
 struct AcceptArgs {
   int32_t batch, n_branches, n_cur, rows_per_branch;
   const int32_t *parent, *state;

@@ -94,7 +94,7 @@ extern "C" int tsd_advance_block(const tsd_advance_args* x, tsd_stream_t stream)
   const int32_t S = x->batch, B = x->n_branches, R = x->rows_per_branch;
   const bool relaxed = x->rule != TSD_ACCEPT_EXACT && x->rule != TSD_ACCEPT_TOP1;
   const tsd::TopkArgs t = {x->logits, x->logits_dtype, (int64_t)S * B * R, x->vocab, x->row_stride, x->k, x->conf, x->topk_idx,
-                           x->topk_prob, x->lse, x->topk_workspace, x->topk_workspace_bytes, stream, tsd::kNextAfter};
+                           x->topk_prob, x->lse, x->topk_workspace, x->topk_workspace_bytes, stream, tsd::kNextAfter, false};
   tsd::AdvanceArgs a = {};
   a.accept = {S, B, B, R, x->parent, x->state, x->mask_id, x->conf, x->topk_idx, x->k, x->tau, x->rule, x->search, x->edge_valid,
               x->prefix_len, x->accepted_node, x->accepted_len, x->n_new_tokens, x->unmask_flag, x->unmask_tok, x->status, stream};

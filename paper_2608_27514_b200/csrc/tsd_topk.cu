@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(THREADS)
 confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, int k, int n_seg,
                        int chunks_per_seg, float* __restrict__ conf, int32_t* __restrict__ topk_idx,
                        float* __restrict__ topk_prob, float* __restrict__ lse,
-                       Partial<K>* __restrict__ partials, unsigned* __restrict__ tickets, int prefetch, int launch_next) {
+                       Partial<K>* __restrict__ partials, unsigned* __restrict__ tickets, int prefetch, int launch_next, int rows_beside) {
   constexpr int E_ = Unpack<T>::kElems;
   constexpr int kTopkThreads = THREADS, kTopkWarps = THREADS / 32;
   constexpr int kTopkBatch = THREADS * kTopkUnroll;        // chunks per block per batch
@@ -290,9 +290,17 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   const int n_iter = (c1 - c0 + kTopkBatch - 1) / kTopkBatch;  // <= kTopkMaxIter (host-enforced)
   const bool has_tail = seg == n_seg - 1 && tid == 0 && chunks_total * E_ < vocab;
   const bool clustered = n_seg > 1 && n_seg <= kMaxCluster;
+  if (rows_beside && row >= rows_beside) {
+    grid_wait();
+    return;
+  }
   if (clustered) cluster_arrive_relaxed();  // "has started": waited for before anything is written to another block
 
-  grid_wait(rowp, rowv);
+  // Beside the kernel before it (rows_beside = rows, else 0) nothing is waited for but an acquire fence, so that no line
+  // the SM still holds from earlier kernels is used.  The blocks of one row more wait for that kernel, so that a
+  // kernel which waits for this one has waited for both.  (A wait by a block of the last row, at its end, cost every pass 0.1 us.)
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %0, 0;\n@p fence.acq_rel.gpu;\n@!p griddepcontrol.wait;\n}" ::"r"(rows_beside) : "memory");
+  settle(rowp, rowv);
   if (launch_next == kNextAtOnce) grid_launch_next();
 
   // ---- phase 1: stream.  Two register buffers: the loads of batch it+1 are in flight while
@@ -604,6 +612,9 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
   // 384 17.9, with 256 18.8; 444 x 126464 25.0 / 23.5 / 24.4; 960 x 126464 50.2 / 48.2 / 46.0.
   const int64_t units = n_rows * p.n_seg;
   p.threads = units <= 2 * 148 ? 512 : (units <= 3 * 148 ? 384 : 256);
+  // Rows that even 256 threads walk in one batch or two: 256 x 4096 fp32 with 512 threads 4.75 us, with 256 4.42 (bf16 4.79
+  // and 4.41); 128 x 8000 4.30 and 4.5, 128 x 16000 5.0 and 5.8.
+  if (chunks <= 1024) p.threads = 256;
   // clusters of large blocks are hard to place: 74 x 126464 in 4 segments 12.8 us with 512 threads, 10.4 with 256
   if (p.n_seg > 1 && units > 148) p.threads = 256;
   // L2 prefetch distance in batches (measured): with very many waves of blocks, requesting lines three batches ahead
@@ -623,9 +634,9 @@ static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   unsigned* tickets = reinterpret_cast<unsigned*>(static_cast<char*>(ws) + p.ticket_off);
   auto kernel = p.threads == 512 ? confidence_topk_kernel<T, K, 512>
               : p.threads == 384 ? confidence_topk_kernel<T, K, 384> : confidence_topk_kernel<T, K, 256>;
-  return launch_clusters(p.n_seg <= kMaxCluster ? p.n_seg : 1, kernel, (unsigned)(a.n_rows * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
+  return launch_clusters(p.n_seg <= kMaxCluster ? p.n_seg : 1, kernel, (unsigned)((a.n_rows + a.concurrent) * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
                 a.row_stride, a.k, p.n_seg, p.chunks_per_seg, a.conf, a.topk_idx, a.topk_prob, a.lse, partials, tickets,
-                p.prefetch, a.launch_next);
+                p.prefetch, a.launch_next, a.concurrent ? (int)a.n_rows : 0);
 }
 
 template <typename T>
@@ -671,6 +682,11 @@ int check_topk(const TopkArgs& a) {
   return TSD_OK;
 }
 
+int64_t topk_threads(const TopkArgs& a) {
+  const TopkPlan p = topk_plan(a.n_rows, a.vocab, a.k, a.dtype == TSD_F32 ? 4 : 8);
+  return a.n_rows * p.n_seg * p.threads;
+}
+
 int launch_topk(const TopkArgs& a) {
   if (a.n_rows == 0) return TSD_OK;
   const TopkPlan p = topk_plan(a.n_rows, a.vocab, a.k, a.dtype == TSD_F32 ? 4 : 8);
@@ -694,7 +710,7 @@ int tsd_confidence_topk(const void* logits, int32_t dtype, int64_t n_rows, int32
                         uint32_t* status, tsd_stream_t stream) {
   (void)status;
   const tsd::TopkArgs a = {logits, dtype, n_rows, vocab, row_stride, k, conf, topk_idx, topk_prob, lse, workspace,
-                           workspace_bytes, stream, tsd::kNextAfter};
+                           workspace_bytes, stream, tsd::kNextAfter, false};
   int rc = tsd::check_topk(a);
   return rc != TSD_OK ? rc : tsd::launch_topk(a);
 }
@@ -735,7 +751,7 @@ extern "C" int tsd_confidence_topk_static(const void* logits, int32_t dtype, int
                                           float* topk_prob, float* lse, uint32_t* status,
                                           tsd_stream_t stream) {
   (void)status;
-  tsd::TopkArgs a = {logits, dtype, n_rows, vocab, row_stride, k, conf, topk_idx, topk_prob, lse, nullptr, 0, stream, tsd::kNextAfter};
+  tsd::TopkArgs a = {logits, dtype, n_rows, vocab, row_stride, k, conf, topk_idx, topk_prob, lse, nullptr, 0, stream, tsd::kNextAfter, false};
   int rc = tsd::check_pointers(a);
   if (rc != TSD_OK || n_rows == 0) return rc;
   // this shape would need more scratch than the library carries: the caller has to use

@@ -33,3 +33,24 @@ def test_step_in_one_call_equals_the_three_calls(kw):
         for key in a:
             assert torch.equal(a[key], b[key]), key
     one.check_status()
+
+
+@pytest.mark.parametrize("kw", [dict(B=2, Nc=300, Hq=32, Hkv=8, V=32000), dict(B=2, Nc=5056, Hq=4, Hkv=2, V=126464),
+                                dict(B=1, Nc=1500, Hq=28, Hkv=4, V=152064), dict(B=2, Nc=700, Hq=28, Hkv=4, V=50008, d=64),
+                                dict(dtype="f32", B=3, d=128, Hq=4, Hkv=2, Nc=100, V=5004), dict(dtype="f32", B=4, d=64, Hq=4, Hkv=4, Nc=100, V=32768)])
+def test_step_with_the_vocabulary_pass_beside_the_attention(kw):
+    # both orders of the two kernels, whole items and items shared by a cluster; a kernel of the caller's right behind the step
+    # sees both results, and the next step may follow at once on the same buffers
+    test_step_in_one_call_equals_the_three_calls(kw)
+    cfg = W.small(W.CONFIGS["cfg2"], name="case", **kw)
+    attn, vi = W.attention_inputs(cfg, DEV), W.verify_inputs(cfg, DEV)
+    step = VerifyStep.for_config(cfg, DEV)
+    seen = []
+    for _ in range(6):
+        step.out.zero_()
+        step.conf.zero_()
+        step.run(attn, vi["logits"], vi["parent"], vi["state"], vi["mask_id"], cfg.tau)
+        seen.append((step.out.clone(), step.conf.clone()))
+    for out, conf in seen:
+        assert torch.equal(out, seen[0][0]) and torch.equal(conf, seen[0][1]) and bool((conf > 0).all())
+        assert bool((out.float().abs().amax(-1) > 0).all())
