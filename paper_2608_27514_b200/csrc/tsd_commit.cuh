@@ -21,8 +21,9 @@ struct CommitArgs {
   uint32_t* status;
 };
 
-// Returns the number of rows still masked, to every lane.
-__device__ __forceinline__ int commit_sequence(const CommitArgs& a, int s, int lane) {
+// Returns the number of rows still masked, to every lane.  `accepted`: the accepted node where the caller has it at hand
+// (else -1 and it is loaded).
+__device__ __forceinline__ int commit_sequence(const CommitArgs& a, int s, int lane, int accepted = -1) {
   __shared__ int s_path[kCommitMaxBranches];  // accepted node first, root last
   __shared__ int s_depth;
   const int B = a.B, R = a.R, root = a.root;
@@ -32,7 +33,7 @@ __device__ __forceinline__ int commit_sequence(const CommitArgs& a, int s, int l
   if (lane == 0) {
     // `root` is the forest index of this tree's root (0 for a tree of its own); node and parent
     // indices are forest indices, and a tree's nodes follow its root
-    int b = a.accepted_node ? a.accepted_node[s] : root, n = 0;
+    int b = accepted >= 0 ? accepted : a.accepted_node ? a.accepted_node[s] : root, n = 0;
     bool bad = b < root || b >= B;
     if (bad) b = root;
     s_path[0] = b;

@@ -33,13 +33,13 @@ __global__ void __launch_bounds__(kAcceptMaxThreads, 1) advance_kernel(const __g
   grid_wait();
   grid_launch_next();
   const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  accept_tree<WORDS>(a.accept, a.relaxed, s, 0);
-  __syncthreads();  // the accepted node and its unmask set are read below
+  const int accepted = accept_tree<WORDS>(a.accept, a.relaxed, s, 0);
+  __syncthreads();  // the unmask set is read below
   if (warp == 0) {
-    const int masked = commit_sequence(a.commit, s, lane);
+    const int masked = commit_sequence(a.commit, s, lane, accepted);
     if (a.report && lane == 0) report_sequence(a.report, a.ticket, s, masked, a.commit.status);
   } else if (warp == 1) {
-    build_tree<WORDS, KK>(a.tree, s, lane);
+    build_tree<WORDS, KK>(a.tree, s, lane, accepted);
   }
 }
 

@@ -60,17 +60,19 @@ struct TreeArgs {
 // RPL = rows per lane (R <= 32 * RPL), KK = candidates per row held in registers (k <= KK): the
 // selection loops are unrolled over RPL x KK, so the common block of 32 rows with k <= 4 runs a
 // tenth of the instructions of the largest case (a single warp is bound by instruction latency).
-// The selection touches registers and shared memory only: a node is its parent and the (row, rank) it adds, and the
-// tokens are looked up once, at the end, when every node's path is written over its slot's copy of the root.
+// The selection touches registers and shared memory only: a node is its parent and the (row, rank) it adds; at the end
+// every node's path is written over its slot's copy of the root.  The candidates' tokens are asked for together with
+// everything else, in one round trip.  `accepted`: the accepted node where the caller has it at hand (else -1 and it is loaded).
 template <int RPL, int KK>
-__device__ __forceinline__ void build_tree(const TreeArgs& a, int s, int lane) {
+__device__ __forceinline__ void build_tree(const TreeArgs& a, int s, int lane, int accepted = -1) {
   __shared__ int s_front[kTreeMaxWidth];
   __shared__ int s_cpar[kTreeMaxWidth], s_crow[kTreeMaxWidth], s_crank[kTreeMaxWidth];
   __shared__ float s_cp[kTreeMaxWidth];
   __shared__ uint32_t s_mask[kTreeMaxNodes][RPL];  // per node: which rows are still masked
   __shared__ int s_link[kTreeMaxNodes];            // per node: parent | row << 8 | rank << 16
+  __shared__ int32_t s_tok[RPL * 32][KK];          // the candidates' tokens
   const int R = a.R, k = a.k, max_nodes = a.max_nodes;
-  int acc = a.accepted_node ? a.accepted_node[s] : 0;
+  int acc = accepted >= 0 ? accepted : a.accepted_node ? a.accepted_node[s] : 0;
   if (acc < 0 || acc >= a.prev_branches) {  // inconsistent device data: report, fall back to node 0
     if (lane == 0 && a.status) atomicOr(a.status, TSD_STATUS_BAD_PARENT);
     acc = 0;
@@ -98,6 +100,9 @@ __device__ __forceinline__ void build_tree(const TreeArgs& a, int s, int lane) {
     }
 #pragma unroll
     for (int j = 0; j < KK; ++j) pool[i][j] = (r < R && j < k) ? prb[(size_t)r * k + j] : -1.f;
+#pragma unroll
+    for (int j = 0; j < KK; ++j)
+      if (r < R && j < k) s_tok[r][j] = idx[(size_t)r * k + j];
   }
   bool root_masked[RPL];
 #pragma unroll
@@ -193,7 +198,7 @@ __device__ __forceinline__ void build_tree(const TreeArgs& a, int s, int lane) {
   for (int node = 1 + lane; node < n; node += 32) {
     for (int q = node; q > 0;) {
       const int link = s_link[q], row = (link >> 8) & 0xff, rank = link >> 16;
-      st[(size_t)node * R + row] = idx[(size_t)row * k + rank];
+      st[(size_t)node * R + row] = s_tok[row][rank];
       q = link & 0xff;
     }
   }
