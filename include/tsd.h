@@ -541,7 +541,8 @@ int tsd_verify_step(const tsd_step_args* args, tsd_stream_t stream);
  * tsd_begin_block starts a block from root_state [batch, R]: parent [batch, B],
  * state [batch, B, R] and n_nodes [batch] become the tree that is its root alone
  * (copies in the unused slots), root_out = root_state, fill_step [batch, R] = -1,
- * step_base [batch] = 0, n_masked [batch] = rows still masked.
+ * step_base [batch] = 0, n_masked [batch] = rows still masked, and report (nullable,
+ * see below) gets them with `ticket`.
  *
  * tsd_advance_block is one pass after the model's forward: tsd_confidence_topk on
  * the logits of every node (batch * B * R rows), the acceptance under `rule`
@@ -552,7 +553,7 @@ int tsd_verify_step(const tsd_step_args* args, tsd_stream_t stream);
  *
  * report, ticket: how the host learns the number of masked rows without a copy or a
  * synchronisation.  report is memory that host and device both address (pinned host
- * memory), one 64-bit word per sequence, 8-byte aligned, nullable in tsd_advance_block:
+ * memory), one 64-bit word per sequence, 8-byte aligned, nullable in the two calls above:
  * ticket << 32 | status bits << 16 | rows still masked.  tsd_wait_block waits until
  * every word carries `ticket`, then gives the largest count and the OR of the status
  * bits (as the words of the device status array stood when they were reported); it
@@ -562,7 +563,7 @@ int tsd_verify_step(const tsd_step_args* args, tsd_stream_t stream);
 int tsd_begin_block(int32_t batch, int32_t n_branches, int32_t rows_per_branch, int32_t mask_id,
                     const int32_t* root_state, int32_t* parent, int32_t* state, int32_t* n_nodes,
                     int32_t* root_out, int32_t* fill_step, int32_t* step_base, int32_t* n_masked,
-                    tsd_stream_t stream);
+                    uint64_t* report, uint32_t ticket, const uint32_t* status, tsd_stream_t stream);
 typedef struct {
   int32_t batch, n_branches, rows_per_branch;
   const void* logits;

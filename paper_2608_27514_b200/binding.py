@@ -306,9 +306,11 @@ def tsd_verify_step(layout, mask, q, k_cache, v_cache, k_draft, v_draft, out, at
                          prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, status, stream)
 
 
-def tsd_begin_block(root_state, mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, stream=None):
-    """root_state int32 [S,R]; everything else is written."""
-    native().begin_block(root_state, mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, stream)
+def tsd_begin_block(root_state, mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, report=None, ticket=0,
+                    status=None, stream=None):
+    """root_state int32 [S,R]; everything else is written; report: pinned int64 [S] or None."""
+    native().begin_block(root_state, mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, report, ticket, status,
+                         stream)
 
 
 def tsd_advance_block(logits, k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search, edge_valid,

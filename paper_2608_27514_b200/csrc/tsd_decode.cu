@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kAcceptMaxThreads, 1) advance_kernel(const __g
 // Start of a block: the tree is the root alone (copies in the unused slots).
 __global__ void __launch_bounds__(256) begin_kernel(int B, int R, int mask_id, const int32_t* root, int32_t* parent, int32_t* state,
                                                     int32_t* n_nodes, int32_t* root_out, int32_t* fill_step, int32_t* step_base,
-                                                    int32_t* n_masked) {
+                                                    int32_t* n_masked, uint64_t* report, uint32_t ticket, const uint32_t* status) {
   grid_wait();
   grid_launch_next();
   const int s = blockIdx.x, t = threadIdx.x;
@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(256) begin_kernel(int B, int R, int mask_id, c
     n_nodes[s] = 1;
     step_base[s] = 0;
     n_masked[s] = count;
+    if (report) report_sequence(report, ticket, s, count, status);
   }
 }
 
@@ -79,13 +80,14 @@ __global__ void __launch_bounds__(256) report_kernel(int batch, const int32_t* n
 
 extern "C" int tsd_begin_block(int32_t batch, int32_t n_branches, int32_t rows_per_branch, int32_t mask_id, const int32_t* root_state,
                                int32_t* parent, int32_t* state, int32_t* n_nodes, int32_t* root_out, int32_t* fill_step,
-                               int32_t* step_base, int32_t* n_masked, tsd_stream_t stream) {
+                               int32_t* step_base, int32_t* n_masked, uint64_t* report, uint32_t ticket, const uint32_t* status,
+                               tsd_stream_t stream) {
   if (batch < 0 || n_branches < 1 || n_branches > tsd::kMaxBranches || rows_per_branch < 1 || rows_per_branch > tsd::kMaxRows)
     return TSD_ERR_INVALID_ARG;
   if (batch == 0) return TSD_OK;
   if (!root_state || !parent || !state || !n_nodes || !root_out || !fill_step || !step_base || !n_masked) return TSD_ERR_INVALID_ARG;
   cudaError_t e = tsd::launch(tsd::begin_kernel, batch, 256, 0, stream, n_branches, rows_per_branch, mask_id, root_state, parent, state,
-                              n_nodes, root_out, fill_step, step_base, n_masked);
+                              n_nodes, root_out, fill_step, step_base, n_masked, report, ticket, status);
   return e != cudaSuccess ? tsd::cuda_fail(e, "begin_kernel") : TSD_OK;
 }
 

@@ -336,13 +336,13 @@ PyObject* verify_step(Args a) {
   return done(call(tsd_verify_step, &t, stream_of(a[33])), "tsd_verify_step");
 }
 
-// root_state [S, R], mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, stream
+// root_state [S, R], mask_id, parent, state, n_nodes, root_out, fill_step, step_base, n_masked, report, ticket, status, stream
 PyObject* begin_block(Args a) {
   int64_t s[4];
   shape3(a[3], s);
   return done(call(tsd_begin_block, (int32_t)s[0], (int32_t)s[1], (int32_t)s[2], to_i32(a[1]), ptr<int32_t>(a[0]), ptr<int32_t>(a[2]),
                    ptr<int32_t>(a[3]), ptr<int32_t>(a[4]), ptr<int32_t>(a[5]), ptr<int32_t>(a[6]), ptr<int32_t>(a[7]),
-                   ptr<int32_t>(a[8]), stream_of(a[9])),
+                   ptr<int32_t>(a[8]), ptr<uint64_t>(a[9]), (uint32_t)to_int(a[10]), ptr<uint32_t>(a[11]), stream_of(a[12])),
               "tsd_begin_block");
 }
 
@@ -422,7 +422,7 @@ PyMethodDef methods[] = {TSD_METHOD(setup, 5),           TSD_METHOD(verify_atten
                          TSD_METHOD(confidence_topk, 9), TSD_METHOD(accept, 19),           TSD_METHOD(accept_relaxed, 22),
                          TSD_METHOD(commit, 15),         TSD_METHOD(build_tree, 18),       TSD_METHOD(build_mask, 6),
                          TSD_METHOD(verify_step, 34),    TSD_METHOD(interblock_vis, 3),    TSD_METHOD(interblock_trigger, 10),
-                         TSD_METHOD(begin_block, 10),    TSD_METHOD(advance_block, 37),    TSD_METHOD(report_block, 5),
+                         TSD_METHOD(begin_block, 13),    TSD_METHOD(advance_block, 37),    TSD_METHOD(report_block, 5),
                          TSD_METHOD(wait_block, 3),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_tsd_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -36,6 +36,7 @@ class BlockDecoder:
         self.n_masked = i32(S)
         self.report = torch.zeros(S, dtype=torch.int64, pin_memory=True)
         self.ticket = 0
+        self.begun = False  # the block has just begun, and that call has reported its masked rows
         self.n_forward = 0
 
     @property
@@ -47,8 +48,11 @@ class BlockDecoder:
         its tree is the root alone (copies in the unused slots)."""
         st, t = self.step, self.tree
         root = root_state.to(device=st.device, dtype=torch.int32).expand(st.S, st.R).contiguous()
-        B.tsd_begin_block(root, self.mask_id, t["parent"], t["state"], t["n"], self.root, self.fill_step, self.step_base, self.n_masked)
+        self._next_ticket()
+        B.tsd_begin_block(root, self.mask_id, t["parent"], t["state"], t["n"], self.root, self.fill_step, self.step_base, self.n_masked,
+                          self.report, self.ticket, st.status)
         self.n_forward = 0
+        self.begun = True
 
     def advance(self, logits, tokens=None, block_start=None):
         """One pass after the caller's forward: logits [S*B*R, V] of the current tree's nodes."""
@@ -65,6 +69,7 @@ class BlockDecoder:
                             nxt["state"], nxt["prob"], nxt["n"], report, self.ticket, st.status)
         self.cur = 1 - self.cur
         self.n_forward += 1
+        self.begun = False
 
     def _next_ticket(self):
         self.ticket = self.ticket % 0x7fffffff + 1
@@ -75,9 +80,12 @@ class BlockDecoder:
         limit = self.step.R + 1 if max_passes is None else max_passes
         status = 1  # not known from a report
         if self.n_forward < limit:
-            self._next_ticket()
-            B.tsd_report_block(self.n_masked, self.step.status, self.report, self.ticket)
+            if not self.begun:
+                self._next_ticket()
+                B.tsd_report_block(self.n_masked, self.step.status, self.report, self.ticket)
             masked, status = B.tsd_wait_block(self.report, self.ticket)
+            if masked == 0:
+                status = 1
             while self.n_forward < limit and masked > 0:
                 logits = forward(self.tree["state"])
                 self._next_ticket()
