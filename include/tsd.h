@@ -225,9 +225,10 @@ int tsd_verify_attention_fp8_cache(const tsd_layout* layout, const void* mask, c
  *   conf       device fp32 [n_rows];  topk_idx device int32 [n_rows, k];
  *   topk_prob  device fp32 [n_rows, k];  lse device fp32 [n_rows], nullable.
  *   workspace  device, 16-byte aligned, tsd_confidence_topk_workspace_bytes()
- *              bytes: per-segment partial results and per-row ticket words when
- *              a row is split across thread blocks (few rows); 0 bytes when it
- *              is not.  Zero it once before its first use (cudaMemsetAsync);
+ *              bytes: per-segment partial results and per-row ticket words for
+ *              rows split across more thread blocks than a cluster holds (the
+ *              blocks of a cluster meet in shared memory); 0 bytes where no row
+ *              can be split.  Zero it once before its first use (cudaMemsetAsync);
  *              after that it can be reused by later calls of any shape without
  *              clearing: a completed call leaves every ticket word it used at 0
  *              and the next call rewrites the partial slots it reads.  (A word
