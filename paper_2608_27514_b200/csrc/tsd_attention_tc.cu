@@ -91,8 +91,9 @@ static_assert(kKeys == kKeyTile, "the mask blob lists tiles of this many keys");
 // Tensor-memory columns.  At head_dim 128 everything is in use and P is one bf16 per score.  At head_dim 64
 // the tensor pipe has twice the time it needs (256 of the 512 clocks that a tile's exponentials take) and half
 // of O and Q is free, so P is kept as the sum of two bf16 (high part, residual: 2^-17 relative) and P V issues
-// one MMA more per 16 keys: outputs then carry no rounding but their own, as from fp32 weights.
-// (4 sequences x 16 branches x 32 rows, 32/8 heads, 1472 cached keys: 67.9 us; on CUDA cores, where this head
+// one MMA more per 16 keys: the outputs' error against fp64 is then that of fp32 weights up to bf16 roundings that fall the other
+// way (relative, 2-norm: 1.6594e-3 for either; over drawn sizes the two are apart by 2e-5 of the error at most).
+// (4 sequences x 16 branches x 32 rows, 32/8 heads, 1472 cached keys: 65.6 us; on CUDA cores, where this head
 // size ran before: 5.96 ms.)
 template <int D>
 struct TcCols {
@@ -109,6 +110,8 @@ constexpr int kMeetTiles = 7;
 constexpr uint32_t kSpinLimit = 1u << 21;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
+constexpr double kLog2eExact = 1.4426950408889634;
+constexpr double kSumsShrink = 1.0 + 1.0 / (1 << 24);  // see row_lse()
 
 // Barriers.  Tile t (counted over all items of the block) uses S buffer t mod 3, K stage t mod 5,
 // V stage t mod 4 and P buffer t mod 2.  A test of a barrier costs the issuing warps a
@@ -355,6 +358,7 @@ struct TcParams {
   int recs_off, n_qt, rec_words;  // layout of the mask blob, computed on the host from the same tsd_layout
   int n_items;                    // S * Hq * n_qt
   float scale_log2e;              // sm_scale * log2(e), > 0
+  float unscale_hi, unscale_lo;   // natural units of an exponent offset, to twice the precision of a float
   int concurrent, next_at_once;
   int cut;                        // blocks per item (a cluster), each with a stretch of its key tiles; 1: whole items
   __nv_bfloat16* out;             // where cut items are written without a tensor map
@@ -418,6 +422,18 @@ __device__ __forceinline__ void issue_pv_mmas(uint32_t o_tmem, uint32_t p_tmem, 
     asm volatile(TSD_PV_BEGIN TSD_PV_END
         ::"r"(o_tmem), "r"(p_tmem), "r"(hi), "r"(idesc_pv), "r"(acc), "r"(pv_done), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]),
           "r"(lo[3]) : "memory");
+}
+
+// Log-sum-exp of a row from its exponent offset `m` (in units of scale_log2e) and the sum `l` on that offset.
+// 64-wide heads ran on CUDA cores before, and their log-sum-exp keeps that accuracy: the offset goes back to natural units with a
+// factor that undoes the rounding of scale_log2e, the result is rounded once, and kSumsShrink makes up for the tensor pipe's
+// fp32 sums, which are rounded towards zero (scores come out 2^-24 of themselves too small on average).  Relative error against fp64
+// (2-norm), 4 x 16 branches x 32 rows, 32 heads, 1472 keys: 2.60e-8; on CUDA cores 2.73e-8; in the form that 128-wide heads
+// have 3.95e-8.
+template <int D>
+__device__ __forceinline__ float row_lse(const TcParams& p, float m, float l) {
+  if (D == 64) return fmaf(m, p.unscale_hi, fmaf(m, p.unscale_lo, logf(l)));
+  return (m + log2f(l)) * kLn2;
 }
 
 // Rarely executed pieces of the softmax warps, kept out of line so that the loop over the key
@@ -1099,7 +1115,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             dst[1] = make_uint4(pack_bf16x2(acc[8], acc[9]), pack_bf16x2(acc[10], acc[11]), pack_bf16x2(acc[12], acc[13]), pack_bf16x2(acc[14], acc[15]));
           }
         }
-        if (rank == 0 && p.lse && row < p.N) p.lse[((size_t)s * p.Hq + h) * p.N + row] = (m_all + log2f(l_all)) * kLn2;
+        if (rank == 0 && p.lse && row < p.N) p.lse[((size_t)s * p.Hq + h) * p.N + row] = row_lse<D>(p, m_all, l_all);
       }
     }
     for (int it = 0; it < (shared ? 0 : n_run) && ok; ++it) {
@@ -1160,7 +1176,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         }
       }
       const int i_row = qt * kTile + r;
-      if (p.lse && i_row < p.N) p.lse[((size_t)s * p.Hq + h) * p.N + i_row] = (m_fin + log2f(lt)) * kLn2;
+      if (p.lse && i_row < p.N) p.lse[((size_t)s * p.Hq + h) * p.N + i_row] = row_lse<D>(p, m_fin, lt);
       fence_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(STAGED));
@@ -1381,7 +1397,10 @@ static int launch_tc(const AttnArgs& a) {
   p.Hq = L.n_q_heads; p.group = L.n_q_heads / L.n_kv_heads;
   p.recs_off = md.recs_off; p.n_qt = md.n_qt; p.rec_words = md.rec_words;
   p.n_items = (int)n_items;
-  p.scale_log2e = a.sm_scale * kLog2e;
+  p.scale_log2e = D == 64 ? (float)(a.sm_scale * kLog2eExact * kSumsShrink) : a.sm_scale * kLog2e;
+  const double unscale = a.sm_scale * kSumsShrink / p.scale_log2e;
+  p.unscale_hi = (float)unscale;
+  p.unscale_lo = (float)(unscale - (double)p.unscale_hi);
   p.concurrent = a.concurrent;
   p.next_at_once = a.next_at_once;
   // one block per SM, each walking its share of the items; more blocks only when a block's share

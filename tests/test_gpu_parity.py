@@ -300,7 +300,7 @@ def test_attention_is_deterministic():
 @pytest.mark.parametrize("R,Bn,Nc,lens", [(32, 1, 1, None), (32, 5, 333, [333, 65]), (64, 3, 64, [64, 0]), (128, 2, 127, [63, 127]),
                                           (32, 9, 0, None), (64, 4, 1000, None)])
 def test_attention_head_dim_64_tensor_cores(R, Bn, Nc, lens):
-    # 64-wide heads keep P as two bf16 parts: no rounding of the weights shows, so the bound is the bf16 rounding of the output
+    # 64-wide heads keep P as two bf16 parts (2^-17 of a weight is lost), so the bound is the bf16 rounding of the output
     # (half an ulp, 2^-9 relative, taken as 2^-8) plus the weights' 2^-17 and the fp32 sums on values of size up to 6 (6 * 2^-16)
     cfg = W.small(W.CONFIGS["cfg2"], S=2, B=Bn, R=R, Nc=Nc, Hq=4, Hkv=2, d=64)
     attn = W.attention_inputs(cfg, DEV, q_gain=2.0)
@@ -314,6 +314,23 @@ def test_attention_head_dim_64_tensor_cores(R, Bn, Nc, lens):
     ref, _ = oracle.masked_attention(_np(attn["q"]), _np(attn["k_cache"]), _np(attn["v_cache"]), _np(attn["k_draft"]),
                                      _np(attn["v_draft"]), mask, attn["sm_scale"])
     assert (np.abs(_np(step.out) - ref) <= 2.0 ** -8 * np.abs(ref) + 6 * 2.0 ** -16).all()
+
+
+@pytest.mark.parametrize("S,Bn,R,Nc,scale", [(2, 5, 32, 333, 0.125), (4, 4, 64, 1472, 0.125), (1, 2, 32, 3000, 0.1), (3, 1, 32, 90, 0.37)])
+def test_attention_head_dim_64_is_as_accurate_as_on_cuda_cores(S, Bn, R, Nc, scale):
+    # the tensor-core kernel against the fp32 arithmetic of the CUDA-core one, both measured against fp64: the root mean square
+    # error of the log-sum-exp may be no larger (10 % for the sample: thousands of rows), that of the bf16 outputs the same to 0.1 %
+    cfg = W.small(W.CONFIGS["cfg2"], S=S, B=Bn, R=R, Nc=Nc, Hq=8, Hkv=4, d=64)
+    attn = dict(W.attention_inputs(cfg, DEV, q_gain=2.0), sm_scale=float(np.float32(scale)))
+    mask = oracle.dense_mask(cfg.S, cfg.B, cfg.R, cfg.Nc, None, None)
+    ref, ref_lse = oracle.masked_attention(_np(attn["q"]), _np(attn["k_cache"]), _np(attn["v_cache"]), _np(attn["k_draft"]),
+                                           _np(attn["v_draft"]), mask, attn["sm_scale"])
+    err = {}
+    for flags in (0, B.TSD_ATTN_FORCE_SIMT):
+        step, _ = _run_attention(cfg, attn, flags)
+        err[flags] = [np.sqrt(np.mean((_np(x).astype(np.float64) - y) ** 2)) for x, y in ((step.out, ref), (step.attn_lse, ref_lse))]
+    tensor, cuda = err[0], err[B.TSD_ATTN_FORCE_SIMT]
+    assert tensor[0] <= 1.001 * cuda[0] and tensor[1] <= 1.1 * cuda[1], (tensor, cuda)
 
 
 @pytest.mark.parametrize("S,Bn,Nc,d", [(300, 2, 0, 128), (300, 2, 0, 64), (160, 2, 64, 128), (200, 4, 30, 64)])
