@@ -1304,14 +1304,28 @@ bool attention_tc_supported(const AttnArgs& a) {
 
 size_t attention_tc_workspace_bytes(const tsd_layout&) { return 0; }
 
+// The kernels' dynamic shared memory limit, an attribute per device; needed by launches and by questions about them.
+template <int D>
+static cudaError_t allow_smem(int dev) {
+  static std::mutex mu;
+  static bool done[kMaxDevices];
+  std::lock_guard<std::mutex> lock(mu);
+  if (done[dev]) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(attention_tc_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<D>::kBytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(attention_tc_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<D>::kBytes);
+  done[dev] = e == cudaSuccess;
+  return e;
+}
+
 // Blocks per item: a launch with fewer items than SMs leaves SMs idle, so an item's key tiles (T of them, over a full cache) are
 // cut over the 2, 4 or 8 blocks of a cluster, as far as the GPU holds all clusters at one time.
 template <int D>
 static int cut_items(int64_t n_items, int T) {
   static std::mutex mu;
-  static int clusters[kMaxDevices][9];  // clusters of that many blocks that run at one time, + 1
+  static int clusters[kMaxDevices][9];  // clusters of that many blocks that run at one time, + 1; 0: not asked yet
   const int dev = current_device();
-  if (dev < 0) return 1;
+  if (dev < 0 || allow_smem<D>(dev) != cudaSuccess) return 1;
   std::lock_guard<std::mutex> lock(mu);
   int best = 1, best_time = T;  // in key tiles
   for (int n = 2, meet = kMeetTiles; n <= (D == 128 ? 8 : 4); n *= 2, meet += 2) {
@@ -1330,8 +1344,8 @@ static int cut_items(int64_t n_items, int T) {
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
       int found = 0;
-      c = cudaOccupancyMaxActiveClusters(&found, attention_tc_kernel<D, true>, &cfg) == cudaSuccess ? found + 1 : 1;
-      if (c == 1) cudaGetLastError();
+      if (cudaOccupancyMaxActiveClusters(&found, attention_tc_kernel<D, true>, &cfg) != cudaSuccess) return best;  // asked again next time
+      c = found + 1;
     }
     if (n_items > c - 1) break;
     best = n;
@@ -1374,21 +1388,10 @@ static int launch_tc(const AttnArgs& a) {
   const MaskDims md = mask_dims(L);
   const int64_t n_items = (int64_t)L.batch * L.n_q_heads * md.n_qt;
   if (!ok || n_items > 0x7fffffffLL / 4) return launch_attention_simt(a);  // strides the tensor maps cannot express
-  {  // the dynamic shared memory limit is an attribute of the kernel on each device
-    static std::mutex mu;
-    static bool done[kMaxDevices];
-    const int dev = current_device();
-    if (dev < 0) return cuda_fail(cudaErrorInvalidDevice, "cudaGetDevice");
-    std::lock_guard<std::mutex> lock(mu);
-    if (!done[dev]) {
-      cudaError_t attr_err =
-          cudaFuncSetAttribute(attention_tc_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<D>::kBytes);
-      if (attr_err == cudaSuccess)
-        attr_err = cudaFuncSetAttribute(attention_tc_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<D>::kBytes);
-      if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(attention_tc_kernel)");
-      done[dev] = true;
-    }
-  }
+  const int dev = current_device();
+  if (dev < 0) return cuda_fail(cudaErrorInvalidDevice, "cudaGetDevice");
+  const cudaError_t attr_err = allow_smem<D>(dev);
+  if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(attention_tc_kernel)");
   TcParams p;
   p.mask = a.mask;
   p.lse = a.lse;

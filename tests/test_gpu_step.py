@@ -1,4 +1,7 @@
 """The step in one call (attention beside the vocabulary pass) against the three calls it stands for."""
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -54,3 +57,30 @@ def test_step_with_the_vocabulary_pass_beside_the_attention(kw):
     for out, conf in seen:
         assert torch.equal(out, seen[0][0]) and torch.equal(conf, seen[0][1]) and bool((conf > 0).all())
         assert bool((out.float().abs().amax(-1) > 0).all())
+
+
+FIRST_CALL = """
+import hashlib, sys
+import torch
+from paper_2608_27514_b200 import workloads as W
+from paper_2608_27514_b200.step import VerifyStep
+first, d = sys.argv[1], int(sys.argv[2])
+cfg = W.small(W.CONFIGS["cfg2"], name="case", B=4, Nc=5056, Hq=28, Hkv=4, V=4096, d=d)
+attn, vi = W.attention_inputs(cfg, "cuda:0"), W.verify_inputs(cfg, "cuda:0")
+step = VerifyStep.for_config(cfg, "cuda:0")
+if first == "step":
+    step.run(attn, vi["logits"], vi["parent"], vi["state"], vi["mask_id"], cfg.tau)
+    torch.cuda.synchronize()
+    step.out.zero_()
+step.attention(*(attn[k] for k in ("q", "k_cache", "v_cache", "k_draft", "v_draft", "sm_scale")))
+print(hashlib.sha1(step.out.view(torch.int16).cpu().numpy().tobytes()).hexdigest())
+"""
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_results_do_not_depend_on_the_entry_point_that_ran_first(d):
+    # whether items are cut over clusters is asked of the runtime once per process: the answer, and with it the order of the sums,
+    # has to be the same whichever call asks first (a fresh process each)
+    seen = {subprocess.run([sys.executable, "-c", FIRST_CALL, first, str(d)], check=True, capture_output=True, text=True, timeout=300).stdout
+            for first in ("step", "attention")}
+    assert len(seen) == 1
