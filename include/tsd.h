@@ -494,6 +494,9 @@ int tsd_accept_joint_trees(int32_t batch, int32_t n_branches, int32_t n_cur, int
  * tsd_confidence_topk and tsd_accept_trajectories on one stream, arguments as
  * for those calls (strides as {batch, row, head}; stage 2's top-1 candidates go
  * to the acceptance).  Every check of the three runs before the first launch.
+ * conf, topk_idx, topk_prob and lse hold batch * n_branches * rows_per_branch
+ * rows, which the acceptance reads; logits for more rows are rejected, with fewer
+ * (unused nodes of a padded tree) the rows past n_rows are what they were.
  * The attention and the vocabulary pass may run at the same time on the GPU:
  * `logits` must not depend on this call's `out` or `attn_lse`, and the outputs
  * of one must not overlap inputs of the other.  Work enqueued on the stream

@@ -34,7 +34,6 @@ extern "C" int tsd_verify_step(const tsd_step_args* x, tsd_stream_t stream) {
                                      x->d_stride[0], x->d_stride[1], x->d_stride[2], x->out, x->o_stride[0],
                                      x->o_stride[1], x->o_stride[2], x->sm_scale, x->attn_workspace);
   if (rc != TSD_OK) return rc;
-  const bool beside = (int64_t)L->batch * L->n_q_heads * tsd::mask_dims(*L).n_qt < 148;
   tsd::AttnArgs a = {*L, static_cast<const int32_t*>(x->mask), x->q, x->k_cache, x->v_cache, x->k_draft, x->v_draft,
                            x->out, x->attn_lse, x->q_stride[0], x->q_stride[1], x->q_stride[2], x->c_stride[0],
                            x->c_stride[1], x->c_stride[2], x->d_stride[0], x->d_stride[1], x->d_stride[2], x->o_stride[0],
@@ -48,6 +47,9 @@ extern "C" int tsd_verify_step(const tsd_step_args* x, tsd_stream_t stream) {
                              x->accepted_node, x->accepted_len, x->n_new_tokens, x->unmask_flag, x->unmask_tok, x->status,
                              stream};
   if ((rc = tsd::check_topk(t)) != TSD_OK || (rc = tsd::check_accept_exact(c)) != TSD_OK) return rc;
+  if (x->n_rows > (int64_t)L->batch * L->n_branches * L->rows_per_branch) return TSD_ERR_INVALID_ARG;  // conf, topk_* hold one row each
+  // without a vocabulary pass in between there is nothing that the attention might run beside but what came before the step
+  const bool beside = x->n_rows > 0 && (int64_t)L->batch * L->n_q_heads * tsd::mask_dims(*L).n_qt < 148;
   if (beside && attention_first(*x, a, t)) {
     a.next_at_once = t.concurrent = true;
   } else if (beside) {

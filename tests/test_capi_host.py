@@ -110,6 +110,32 @@ def test_attention_validation(lib):
     assert call(scale=float("nan")) == B.TSD_ERR_INVALID_ARG
 
 
+def test_step_rejects_logits_for_more_rows_than_the_tree_has(lib):
+    # the outputs of the vocabulary pass hold a row per (sequence, branch, row); nothing may be launched for more
+    class Args(ctypes.Structure):
+        _fields_ = [("layout", ctypes.c_void_p), ("mask", ctypes.c_void_p), ("q", ctypes.c_void_p), ("q_stride", ctypes.c_int64 * 3),
+                    ("k_cache", ctypes.c_void_p), ("v_cache", ctypes.c_void_p), ("c_stride", ctypes.c_int64 * 3),
+                    ("k_draft", ctypes.c_void_p), ("v_draft", ctypes.c_void_p), ("d_stride", ctypes.c_int64 * 3),
+                    ("out", ctypes.c_void_p), ("o_stride", ctypes.c_int64 * 3), ("attn_lse", ctypes.c_void_p),
+                    ("sm_scale", ctypes.c_float), ("flags", ctypes.c_uint32), ("attn_workspace", ctypes.c_void_p),
+                    ("attn_workspace_bytes", ctypes.c_size_t), ("logits", ctypes.c_void_p), ("n_rows", ctypes.c_int64),
+                    ("row_stride", ctypes.c_int64), ("logits_dtype", ctypes.c_int32), ("vocab", ctypes.c_int32), ("k", ctypes.c_int32)] + [
+            (name, ctypes.c_void_p) for name in ("conf", "topk_idx", "topk_prob", "lse", "topk_workspace")] + [
+            ("topk_workspace_bytes", ctypes.c_size_t), ("parent", ctypes.c_void_p), ("state", ctypes.c_void_p), ("mask_id", ctypes.c_int32),
+            ("tau", ctypes.c_float), ("rule", ctypes.c_int32), ("search", ctypes.c_int32)] + [
+            (name, ctypes.c_void_p) for name in ("edge_valid", "prefix_len", "accepted_node", "accepted_len", "n_new_tokens", "unmask_flag",
+                                                 "unmask_tok", "status")]
+    layout = B.make_layout(2, 4, 32, 64, 2, 2, 64, B.TSD_F32)
+    a = Args(**{name: 4096 for name, kind in Args._fields_ if kind is ctypes.c_void_p})
+    a.layout, a.status = ctypes.addressof(layout), None
+    a.q_stride = a.c_stride = a.d_stride = a.o_stride = (1 << 20, 128, 64)
+    a.sm_scale, a.tau, a.k, a.vocab, a.row_stride, a.logits_dtype, a.topk_workspace_bytes = 0.1, 0.9, 3, 1024, 1024, B.TSD_F32, 1 << 30
+    lib.tsd_verify_step.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    for rows in (257, 1 << 20):
+        a.n_rows = rows
+        assert lib.tsd_verify_step(ctypes.byref(a), None) == B.TSD_ERR_INVALID_ARG
+
+
 def test_missing_library_is_loud(monkeypatch):
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "LIB_PATH", "/nonexistent/libtsd.so")

@@ -59,6 +59,30 @@ def test_step_with_the_vocabulary_pass_beside_the_attention(kw):
         assert bool((out.float().abs().amax(-1) > 0).all())
 
 
+@pytest.mark.parametrize("kw,rows", [(dict(B=8, Nc=300, Hq=4, Hkv=2, V=32000), 160), (dict(B=8, Nc=300, Hq=4, Hkv=2, V=32000), 0),
+                                     (dict(dtype="f32", d=64, B=16, Hq=4, Hkv=4, Nc=100, V=4096), 0)])
+def test_step_with_logits_for_fewer_rows_than_the_tree_has(kw, rows):
+    # a padded tree's unused nodes need no logits: their rows of the outputs stay; without any logits there is no vocabulary pass
+    # and the attention must not start before what the caller enqueued in front of the step (here: its queries)
+    cfg = W.small(W.CONFIGS["cfg2"], name="case", **kw)
+    attn, vi = W.attention_inputs(cfg, DEV), W.verify_inputs(cfg, DEV)
+    one, three = VerifyStep.for_config(cfg, DEV), VerifyStep.for_config(cfg, DEV)
+    q = attn["q"].clone()
+    for st in (one, three):
+        st.conf.fill_(0.25)
+        st.topk_idx.fill_(3)
+    for i in range(4):
+        torch.cuda._sleep(200000)
+        attn["q"].copy_(q if i % 2 else -q)
+        a = one.run(attn, vi["logits"][:rows], vi["parent"], vi["state"], vi["mask_id"], cfg.tau)
+        out = one.out.clone()
+        three.attention(attn["q"], attn["k_cache"], attn["v_cache"], attn["k_draft"], attn["v_draft"], attn["sm_scale"])
+        three.confidence_topk(vi["logits"][:rows])
+        b = three.accept(vi["parent"], vi["state"], vi["mask_id"], cfg.tau)
+        assert torch.equal(out, three.out) and torch.equal(one.conf, three.conf) and torch.equal(one.topk_idx, three.topk_idx)
+        assert bool((one.conf[rows:] == 0.25).all()) and all(torch.equal(a[key], b[key]) for key in a)
+
+
 FIRST_CALL = """
 import hashlib, sys
 import torch
