@@ -18,6 +18,21 @@ import torch
 from . import binding as B
 
 
+# Report words of decoders that are gone while a kernel may still have to write to them: the allocator of pinned memory knows
+# nothing of that kernel and would give them to the next one who asks.  Given back once the words have arrived.
+_unreported = {}
+
+
+def _arrived(report, ticket):
+    return bool((report >> 32 == ticket).all())
+
+
+def _give_back():
+    for key, words in list(_unreported.items()):
+        if _arrived(*words):
+            _unreported.pop(key, None)
+
+
 class BlockDecoder:
     def __init__(self, step, width, depth, tau, mask_id, rule=B.TSD_ACCEPT_EXACT, search=B.TSD_SEARCH_GREEDY):
         """step: a VerifyStep whose layout (batch, branches, rows) fixes the tree size: every pass
@@ -34,10 +49,16 @@ class BlockDecoder:
         self.fill_step = i32(S, R)
         self.step_base = i32(S)
         self.n_masked = i32(S)
+        _give_back()
         self.report = torch.zeros(S, dtype=torch.int64, pin_memory=True)
         self.ticket = 0
+        self.in_flight = None  # the ticket of a report that has been enqueued and not seen yet
         self.begun = False  # the block has just begun, and that call has reported its masked rows
         self.n_forward = 0
+
+    def __del__(self):
+        if getattr(self, "in_flight", None) and not _arrived(self.report, self.in_flight):
+            _unreported[id(self.report)] = (self.report, self.in_flight)
 
     @property
     def tree(self):
@@ -48,11 +69,12 @@ class BlockDecoder:
         its tree is the root alone (copies in the unused slots)."""
         st, t = self.step, self.tree
         root = root_state.to(device=st.device, dtype=torch.int32).expand(st.S, st.R).contiguous()
-        self._next_ticket()
-        B.tsd_begin_block(root, self.mask_id, t["parent"], t["state"], t["n"], self.root, self.fill_step, self.step_base, self.n_masked,
-                          self.report, self.ticket, st.status)
+        # a captured call is replayed for as long as its graph lives, which this object knows nothing of: it reports nothing
+        begin = lambda report: B.tsd_begin_block(root, self.mask_id, t["parent"], t["state"], t["n"], self.root, self.fill_step,
+                                                 self.step_base, self.n_masked, report, self.ticket, st.status)
+        self.begun = not torch.cuda.is_current_stream_capturing()
+        self._reported(begin) if self.begun else begin(None)
         self.n_forward = 0
-        self.begun = True
 
     def advance(self, logits, tokens=None, block_start=None):
         """One pass after the caller's forward: logits [S*B*R, V] of the current tree's nodes."""
@@ -74,6 +96,21 @@ class BlockDecoder:
     def _next_ticket(self):
         self.ticket = self.ticket % 0x7fffffff + 1
 
+    def _reported(self, enqueue):
+        """enqueue(report words) with a new ticket; a call that is rejected reports nothing."""
+        self._next_ticket()
+        before, self.in_flight = self.in_flight, self.ticket
+        try:
+            enqueue(self.report)
+        except Exception:
+            self.in_flight = before
+            raise
+
+    def _wait(self):
+        found = B.tsd_wait_block(self.report, self.ticket)
+        self.in_flight = None
+        return found
+
     def decode(self, forward, tokens=None, block_start=None, max_passes=None):
         """Run passes until no sequence has a masked row left.  forward(state int32 [S,B,R]) must
         return the logits [S*B*R, V] of every node (a device tensor the vocabulary pass accepts)."""
@@ -81,16 +118,14 @@ class BlockDecoder:
         status = 1  # not known from a report
         if self.n_forward < limit:
             if not self.begun:
-                self._next_ticket()
-                B.tsd_report_block(self.n_masked, self.step.status, self.report, self.ticket)
-            masked, status = B.tsd_wait_block(self.report, self.ticket)
+                self._reported(lambda report: B.tsd_report_block(self.n_masked, self.step.status, report, self.ticket))
+            masked, status = self._wait()
             if masked == 0:
                 status = 1
             while self.n_forward < limit and masked > 0:
                 logits = forward(self.tree["state"])
-                self._next_ticket()
-                self._advance(logits, tokens, block_start, self.report)
-                masked, status = B.tsd_wait_block(self.report, self.ticket)
+                self._reported(lambda report: self._advance(logits, tokens, block_start, report))
+                masked, status = self._wait()
         if status:
             self.step.check_status()
         return self.root
