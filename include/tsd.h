@@ -562,6 +562,10 @@ int tsd_verify_step(const tsd_step_args* args, tsd_stream_t stream);
  * every word carries `ticket`, then gives the largest count and the OR of the status
  * bits (as the words of the device status array stood when they were reported); it
  * fails instead of waiting for good when the stream has failed or has run dry.
+ * The words come as early as they can, while the call may still be building the next tree:
+ * a ticket that has arrived there says nothing of its other outputs.  `done` (nullable, like
+ * report) gets the ticket last: once every word of it carries the ticket, all outputs of the
+ * call are complete, for the host and for any stream; tsd_wait_block waits for it as well.
  * tsd_report_block writes the words from n_masked as it stands.
  * ------------------------------------------------------------------------- */
 int tsd_begin_block(int32_t batch, int32_t n_branches, int32_t rows_per_branch, int32_t mask_id,
@@ -595,7 +599,7 @@ typedef struct {
   int32_t *next_parent, *next_state;
   float* next_prob;
   int32_t* next_n;
-  uint64_t* report;
+  uint64_t *report, *done;
   uint32_t ticket;
   uint32_t* status;
 } tsd_advance_args;

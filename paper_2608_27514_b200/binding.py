@@ -316,12 +316,12 @@ def tsd_begin_block(root_state, mask_id, parent, state, n_nodes, root_out, fill_
 def tsd_advance_block(logits, k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search, edge_valid,
                       prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, draft_prob, tokens, block_start,
                       root_out, fill_step, step_base, n_masked, width, depth, next_parent, next_state, next_prob, next_n, report=None,
-                      ticket=0, status=None, stream=None):
-    """Vocabulary pass, acceptance, commit and next tree of one pass; report: pinned int64 [S] or None."""
+                      ticket=0, status=None, stream=None, done=None):
+    """Vocabulary pass, acceptance, commit and next tree of one pass; report, done: pinned int64 [S] or None."""
     native().advance_block(logits, k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search,
                            edge_valid, prefix_len, accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, draft_prob,
                            tokens, block_start, root_out, fill_step, step_base, n_masked, width, depth, next_parent, next_state,
-                           next_prob, next_n, report, ticket, status, stream)
+                           next_prob, next_n, report, ticket, status, stream, done)
 
 
 def tsd_report_block(n_masked, status, report, ticket, stream=None):

@@ -18,7 +18,7 @@ struct AdvanceArgs {
   RelaxedArgs relaxed;
   CommitArgs commit;
   TreeArgs tree;
-  uint64_t* report;
+  uint64_t *report, *done;
   uint32_t ticket;
 };
 
@@ -40,6 +40,13 @@ __global__ void __launch_bounds__(kAcceptMaxThreads, 1) advance_kernel(const __g
     if (a.report && lane == 0) report_sequence(a.report, a.ticket, s, masked, a.commit.status);
   } else if (warp == 1) {
     build_tree<WORDS, KK>(a.tree, s, lane, accepted);
+  }
+  if (a.done) {  // behind everything the block has written, for whoever sees the word: host, other streams
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence_system();
+      report_sequence(a.done, a.ticket, s, 0, nullptr);
+    }
   }
 }
 
@@ -114,6 +121,7 @@ extern "C" int tsd_advance_block(const tsd_advance_args* x, tsd_stream_t stream)
   a.tree = {B, R, x->k, x->state, x->accepted_node, x->unmask_flag, x->unmask_tok, x->mask_id, x->topk_idx, x->topk_prob, x->width,
             x->depth, B, B, 0, nullptr, x->next_parent, x->next_state, x->next_prob, x->next_n, x->status};
   a.report = x->report;
+  a.done = x->done;
   a.ticket = x->ticket;
   int rc = tsd::check_topk(t);
   if (rc == TSD_OK) rc = tsd::check_accept(a.accept, a.relaxed);

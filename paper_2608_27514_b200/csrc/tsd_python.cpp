@@ -348,7 +348,7 @@ PyObject* begin_block(Args a) {
 
 // logits, k, conf, topk_idx, topk_prob, lse, topk_workspace, parent, state, mask_id, tau, rule, search, edge_valid, prefix_len,
 // accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, draft_prob, tokens, block_start, root_out, fill_step,
-// step_base, n_masked, width, depth, next_parent, next_state, next_prob, next_n, report, ticket, status, stream
+// step_base, n_masked, width, depth, next_parent, next_state, next_prob, next_n, report, ticket, status, stream, done
 PyObject* advance_block(Args a) {
   int64_t s[4], st[4] = {0, 0, 0, 0};
   shape3(a[8], s);
@@ -378,6 +378,7 @@ PyObject* advance_block(Args a) {
   t.width = to_i32(a[27]); t.depth = to_i32(a[28]);
   t.next_parent = ptr<int32_t>(a[29]); t.next_state = ptr<int32_t>(a[30]); t.next_prob = ptr<float>(a[31]); t.next_n = ptr<int32_t>(a[32]);
   t.report = ptr<uint64_t>(a[33]);
+  t.done = ptr<uint64_t>(a[37]);
   t.ticket = (uint32_t)to_int(a[34]);
   t.status = ptr<uint32_t>(a[35]);
   return done(call(tsd_advance_block, &t, stream_of(a[36])), "tsd_advance_block");
@@ -422,7 +423,7 @@ PyMethodDef methods[] = {TSD_METHOD(setup, 5),           TSD_METHOD(verify_atten
                          TSD_METHOD(confidence_topk, 9), TSD_METHOD(accept, 19),           TSD_METHOD(accept_relaxed, 22),
                          TSD_METHOD(commit, 15),         TSD_METHOD(build_tree, 18),       TSD_METHOD(build_mask, 6),
                          TSD_METHOD(verify_step, 34),    TSD_METHOD(interblock_vis, 3),    TSD_METHOD(interblock_trigger, 10),
-                         TSD_METHOD(begin_block, 13),    TSD_METHOD(advance_block, 37),    TSD_METHOD(report_block, 5),
+                         TSD_METHOD(begin_block, 13),    TSD_METHOD(advance_block, 38),    TSD_METHOD(report_block, 5),
                          TSD_METHOD(wait_block, 3),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_tsd_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -50,15 +50,17 @@ class BlockDecoder:
         self.step_base = i32(S)
         self.n_masked = i32(S)
         _give_back()
-        self.report = torch.zeros(S, dtype=torch.int64, pin_memory=True)
+        # words that the calls write a ticket to: the count of masked rows as soon as it is known, and behind all outputs
+        self.report, self.done = torch.zeros((2, S), dtype=torch.int64, pin_memory=True)
         self.ticket = 0
-        self.in_flight = None  # the ticket of a report that has been enqueued and not seen yet
+        self.in_flight = None  # (words, ticket) that the last such call enqueued has yet to write, or None once seen
         self.begun = False  # the block has just begun, and that call has reported its masked rows
         self.n_forward = 0
 
     def __del__(self):
-        if getattr(self, "in_flight", None) and not _arrived(self.report, self.in_flight):
-            _unreported[id(self.report)] = (self.report, self.in_flight)
+        words = getattr(self, "in_flight", None)
+        if words and not _arrived(*words):
+            _unreported[id(words)] = words
 
     @property
     def tree(self):
@@ -70,17 +72,24 @@ class BlockDecoder:
         st, t = self.step, self.tree
         root = root_state.to(device=st.device, dtype=torch.int32).expand(st.S, st.R).contiguous()
         # a captured call is replayed for as long as its graph lives, which this object knows nothing of: it reports nothing
-        begin = lambda report: B.tsd_begin_block(root, self.mask_id, t["parent"], t["state"], t["n"], self.root, self.fill_step,
-                                                 self.step_base, self.n_masked, report, self.ticket, st.status)
-        self.begun = not torch.cuda.is_current_stream_capturing()
-        self._reported(begin) if self.begun else begin(None)
+        report = None if torch.cuda.is_current_stream_capturing() else self.report
+        before = self.in_flight
+        if report is not None:
+            self._next_ticket(report)
+        try:
+            B.tsd_begin_block(root, self.mask_id, t["parent"], t["state"], t["n"], self.root, self.fill_step, self.step_base,
+                              self.n_masked, report, self.ticket, st.status)
+        except Exception:
+            self.in_flight = before  # a call that is rejected writes nothing
+            raise
         self.n_forward = 0
+        self.begun = report is not None
 
     def advance(self, logits, tokens=None, block_start=None):
         """One pass after the caller's forward: logits [S*B*R, V] of the current tree's nodes."""
         self._advance(logits, tokens, block_start, None)
 
-    def _advance(self, logits, tokens, block_start, report):
+    def _advance(self, logits, tokens, block_start, report, done=None):
         st, t, nxt = self.step, self.tree, self.trees[1 - self.cur]
         if self.rule == B.TSD_ACCEPT_PROB and not hasattr(st, "draft_prob"):
             st.draft_prob = torch.empty((st.S, st.B, st.R), dtype=torch.float32, device=st.device)
@@ -88,44 +97,43 @@ class BlockDecoder:
                             self.tau, self.rule, self.search, st.edge_valid, st.prefix_len, st.accepted_node, st.accepted_len,
                             st.n_new_tokens, st.unmask_flag, st.unmask_tok, getattr(st, "draft_prob", None), tokens, block_start,
                             self.root, self.fill_step, self.step_base, self.n_masked, self.width, self.depth, nxt["parent"],
-                            nxt["state"], nxt["prob"], nxt["n"], report, self.ticket, st.status)
+                            nxt["state"], nxt["prob"], nxt["n"], report, self.ticket, st.status, None, done)
         self.cur = 1 - self.cur
         self.n_forward += 1
         self.begun = False
 
-    def _next_ticket(self):
+    def _next_ticket(self, words=None):
         self.ticket = self.ticket % 0x7fffffff + 1
-
-    def _reported(self, enqueue):
-        """enqueue(report words) with a new ticket; a call that is rejected reports nothing."""
-        self._next_ticket()
-        before, self.in_flight = self.in_flight, self.ticket
-        try:
-            enqueue(self.report)
-        except Exception:
-            self.in_flight = before
-            raise
-
-    def _wait(self):
-        found = B.tsd_wait_block(self.report, self.ticket)
-        self.in_flight = None
-        return found
+        if words is not None:
+            self.in_flight = (words, self.ticket)
 
     def decode(self, forward, tokens=None, block_start=None, max_passes=None):
         """Run passes until no sequence has a masked row left.  forward(state int32 [S,B,R]) must
-        return the logits [S*B*R, V] of every node (a device tensor the vocabulary pass accepts)."""
+        return the logits [S*B*R, V] of every node (a device tensor the vocabulary pass accepts).  When it
+        returns, all its outputs are complete, for the host and for any stream."""
         limit = self.step.R + 1 if max_passes is None else max_passes
         status = 1  # not known from a report
         if self.n_forward < limit:
             if not self.begun:
-                self._reported(lambda report: B.tsd_report_block(self.n_masked, self.step.status, report, self.ticket))
-            masked, status = self._wait()
+                self._next_ticket(self.report)
+                B.tsd_report_block(self.n_masked, self.step.status, self.report, self.ticket)
+            masked, status = B.tsd_wait_block(self.report, self.ticket)
+            self.in_flight = None
             if masked == 0:
                 status = 1
             while self.n_forward < limit and masked > 0:
                 logits = forward(self.tree["state"])
-                self._reported(lambda report: self._advance(logits, tokens, block_start, report))
-                masked, status = self._wait()
+                before = self.in_flight
+                self._next_ticket(self.done)
+                try:
+                    self._advance(logits, tokens, block_start, self.report, self.done)
+                except Exception:
+                    self.in_flight = before
+                    raise
+                masked, status = B.tsd_wait_block(self.report, self.ticket)
+            if self.in_flight is not None:
+                B.tsd_wait_block(self.done, self.ticket)
+                self.in_flight = None
         if status:
             self.step.check_status()
         return self.root

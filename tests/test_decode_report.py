@@ -26,7 +26,7 @@ def calls(monkeypatch):
     monkeypatch.setattr(torch, "zeros", lambda *a, pin_memory=False, **kw: zeros(*a, **kw))
     monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: False)
     monkeypatch.setattr(decode.B, "tsd_begin_block", lambda *a: seen.append((weakref.ref(a[9]) if a[9] is not None else None, a[10])))
-    monkeypatch.setattr(decode.B, "tsd_advance_block", lambda *a: seen.append((weakref.ref(a[33]) if a[33] is not None else None, a[34])))
+    monkeypatch.setattr(decode.B, "tsd_advance_block", lambda *a: seen.append((weakref.ref(a[37]) if a[37] is not None else None, a[34])))
     return seen
 
 
@@ -77,3 +77,20 @@ def test_a_captured_start_reports_nothing(calls, monkeypatch):
     d = decode.BlockDecoder(_Step(), 2, 2, 0.9, 99)
     d.start(torch.zeros(2, 32, dtype=torch.int32))
     assert calls[0][0] is None and not d.begun
+
+
+def test_words_outlive_a_decoder_dropped_between_two_passes(calls, monkeypatch):
+    # the second forward fails while the first pass is still writing its tree: its last word has not arrived
+    monkeypatch.setattr(decode.B, "tsd_wait_block", lambda report, ticket, stream=None: (5, 0))
+    d = decode.BlockDecoder(_Step(), 2, 2, 0.9, 99)
+    d.start(torch.zeros(2, 32, dtype=torch.int32))
+    passes = iter([torch.zeros(1)])
+    with pytest.raises(StopIteration):
+        d.decode(lambda state: next(passes))
+    del d
+    gc.collect()
+    assert calls[1][0]() is not None
+    _write(calls[1])
+    decode.BlockDecoder(_Step(), 2, 2, 0.9, 99)
+    gc.collect()
+    assert calls[1][0]() is None

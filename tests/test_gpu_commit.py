@@ -310,3 +310,23 @@ def test_wait_for_a_report_that_never_comes_fails():
     status = torch.tensor([2], dtype=torch.int32, device=DEV)
     B.tsd_report_block(n, status, report, 7)
     assert B.tsd_wait_block(report, 7) == (5, 2)
+
+
+def test_everything_is_complete_when_decode_returns():
+    # the report arrives before the next tree is built (here a large one, one that differs from block to block): a caller may all
+    # the same read the decoder's buffers on another stream, as after a read-back
+    S, Bn, R, V, k = 1, 256, 128, 600, 8
+    dec = BlockDecoder(VerifyStep(S, Bn, R, 0, 1, 1, 64, V, k, torch.bfloat16, DEV), 32, 64, 0.9, V - 1)
+    g = torch.Generator(device=DEV).manual_seed(5)
+    logits = [torch.randn((S * Bn * R, V), generator=g, device=DEV).bfloat16() for _ in range(6)]
+    root = torch.full((S, R), V - 1, dtype=torch.int32, device=DEV)
+    other = torch.cuda.Stream()
+    for i in range(10):
+        dec.start(root)
+        torch.cuda.synchronize()
+        passes = iter(logits[i % 5:])
+        dec.decode(lambda state: next(passes), max_passes=1 + i % 2)
+        with torch.cuda.stream(other):
+            seen = [dec.tree[key].clone() for key in ("state", "parent", "n")]
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, dec.tree[key]) for a, key in zip(seen, ("state", "parent", "n")))
