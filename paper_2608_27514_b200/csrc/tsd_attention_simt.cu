@@ -91,13 +91,13 @@ attention_rows_kernel(int S, int B, int R, int Nc, int Hq, int Hkv, int recs_off
   const int b = row0 / R, g = h / (Hq / Hkv), N = B * R;
   const int j = lane % LPK, slots = kTile / R;
   const unsigned full = 0xffffffffu;
-  if (concurrent) {  // beside the kernel before it, see tsd_attention_tc.cu
-    __threadfence();
+  if (concurrent) {  // beside the kernel before it
+    beside_fence();
     settle(mask, q, kc, vc, kd, vd);
   } else {
     grid_wait(mask, q, kc, vc, kd, vd);
   }
-  if (next_at_once) grid_launch_next();
+  if (next_at_once) grid_launch_beside();
 
   // the block's query rows, 8 dimensions per lane (requested first: nothing else is needed for them)
   float qr[RB][8];

@@ -553,11 +553,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   if (kCut) cluster_arrive();  // "barriers set up"; waited for before another block's are touched
   // Everything above runs while the previous kernel of the stream finishes.  Tensor memory is allocated only
   // after the wait: a block of that kernel may still need it.
-  // Beside the kernel before it nothing is waited for but an acquire fence, so that no line the SM still holds from
-  // earlier kernels is used; the block then leaves only after that kernel has completed, so that a kernel which waits
-  // for this one has waited for both.
-  asm volatile("{\n.reg .pred c, n;\nsetp.ne.b32 c, %0, 0;\nsetp.ne.b32 n, %1, 0;\n@c fence.acq_rel.gpu;\n@!c griddepcontrol.wait;\n"
-               "@n griddepcontrol.launch_dependents;\n}" ::"r"(p.concurrent), "r"(p.next_at_once) : "memory");
+  // Beside the kernel before it nothing is waited for but beside_fence(); the block then leaves only after that kernel has
+  // completed, so that a kernel which waits for this one has waited for both.
+  asm volatile("{\n.reg .pred c, n;\nsetp.ne.b32 c, %0, 0;\nsetp.ne.b32 n, %1, 0;\n"
+               "@c fence.acq_rel.gpu;\n@c fence.proxy.async.global;\n@!c griddepcontrol.wait;\n"
+               "@n fence.acq_rel.gpu;\n@n griddepcontrol.launch_dependents;\n}" ::"r"(p.concurrent), "r"(p.next_at_once) : "memory");
   settle(mask);
 
   const int h_magic = mask[H_MAGIC], h_s = mask[H_S], h_b = mask[H_B], h_r = mask[H_R], h_nc = mask[H_NC];

@@ -141,6 +141,18 @@ __device__ __forceinline__ void grid_wait(P&... inputs) {
   settle(inputs...);
 }
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A kernel that may run BESIDE its predecessor A in the stream does not call grid_wait() before it reads.  What it reads was
+// written before A, and A's blocks have waited for that.  Handing it on rests on
+//   A: grid_wait(), grid_launch_beside() in every block   ->   this kernel's blocks start   ->   this kernel: beside_fence()
+// that is, a release by all blocks of A in front of the signal that lets this kernel start, and an acquire behind the start.
+// The manuals define the fences, but they name only grid_wait() as what makes memory visible across that signal:
+// that a start which the signal has caused comes after it for the fences as well is an assumption of this library, and
+// test_step_with_the_vocabulary_pass_beside_the_attention is what watches it (inputs rewritten in place before every step).
+// The copy engine (TMA) reads through the async proxy, hence the second fence.
+__device__ __forceinline__ void grid_launch_beside() {
+  asm volatile("fence.acq_rel.gpu;\ngriddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void beside_fence() { asm volatile("fence.acq_rel.gpu;\nfence.proxy.async.global;" ::: "memory"); }
 
 // `cluster`: blocks per thread-block cluster (along x).
 template <typename... P, typename... A>

@@ -296,12 +296,12 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   }
   if (clustered) cluster_arrive_relaxed();  // "has started": waited for before anything is written to another block
 
-  // Beside the kernel before it (rows_beside = rows, else 0) nothing is waited for but an acquire fence, so that no line
-  // the SM still holds from earlier kernels is used.  The blocks of one row more wait for that kernel, so that a
-  // kernel which waits for this one has waited for both.  (A wait by a block of the last row, at its end, cost every pass 0.1 us.)
+  // Beside the kernel before it (rows_beside = rows, else 0) nothing is waited for but beside_fence() (no copy engine here).  The
+  // blocks of one row more wait for that kernel, so that a kernel which waits for this one has waited for both.  (A wait by a
+  // block of the last row, at its end, cost every pass 0.1 us.)
   asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %0, 0;\n@p fence.acq_rel.gpu;\n@!p griddepcontrol.wait;\n}" ::"r"(rows_beside) : "memory");
   settle(rowp, rowv);
-  if (launch_next == kNextAtOnce) grid_launch_next();
+  if (launch_next == kNextAtOnce) grid_launch_beside();
 
   // ---- phase 1: stream.  Two register buffers: the loads of batch it+1 are in flight while
   // batch it is processed, so a block overlaps memory latency with its own arithmetic.
