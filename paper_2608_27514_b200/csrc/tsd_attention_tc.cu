@@ -140,7 +140,8 @@ enum Bar {
   OS_FREE = 45,   // the previous item's store has read the staging buffer
   ROOM = 46,      // cut items: every other block of the cluster has room for this one's part
   PARTS = 47,     // [4] cut items: the other blocks' parts are here, per epilogue warp
-  N_BARS = 51     // (the words behind them start at 56)
+  LPART_FREE = 51,  // [3] the epilogue has read the partial row sums of an item, per item mod 3
+  N_BARS = 54     // (the words behind them start at 56)
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -537,7 +538,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     }
     for (int i = 0; i < 16; ++i) mbar_init(bar(DEC + i), 1);
     mbar_init(bar(O_FREE), 4);
-    for (int i = 0; i < 3; ++i) mbar_init(bar(LPART + i), kSoftmaxWarps);
+    for (int i = 0; i < 3; ++i) {
+      mbar_init(bar(LPART + i), kSoftmaxWarps);
+      mbar_init(bar(LPART_FREE + i), 4);
+    }
     mbar_init(bar(STAGED), 4);
     mbar_init(bar(OS_FREE), 1);
     if (kCut) {
@@ -875,6 +879,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       const int T = item_T[it], j0 = kCut ? *tile_first : 0;  // tiles of the item from j0 on
       const int n_ct = (clen + kKeys - 1) / kKeys - j0;  // the cached ones among them (negative: behind the first draft tiles)
       const int jc = min(4, T - 1);  // the tile at which Q of the next item is copied
+      // A warpgroup's sums of this item go where those of item it-3 were, and its arrival must not count for that item.  With a tile in
+      // this item it has waited for the P V of a tile of item it-2 or later (for its P buffer) before it publishes them, and the
+      // first P V of item it-2 comes after the epilogue's reading of item it-3.  Without one it has waited for nothing of the
+      // kind (with items of one tile it is up to two items ahead), so it waits here.  (Here, and not where the sums are
+      // written: there it changes the registers of the loop below, 5 ragged sequences of 28 heads 46.3 -> 50.7 us.)
+      if (it >= 3 && T < 3 && ((wg - G) % 3 + 3) % 3 >= T)
+        ok = __all_sync(0xffffffffu, mbar_wait(bar(LPART_FREE + it % 3), (it / 3 - 1) & 1, abort_flag));
       float m_mine = -CUDART_INF_F, l = 0.f;  // the exponent offset this thread used last, its partial row sum
       // tile t goes to warpgroup t mod 3, which is also its S buffer; n_done counts this
       // warpgroup's tiles, so the buffer's barriers are in phase n_done & 1
@@ -1005,9 +1016,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       }
       if (!ok) break;
 
-      // ---- the item's partial row sum of this thread, and the offset it is on, go to the epilogue
-      // warpgroup (three sets in rotation: a warpgroup that runs ahead writes the set of item it+3
-      // only after a P of item it+1 or later, whose buffer needs a P V that follows the epilogue's read of O)
+      // ---- the item's partial row sum of this thread, and the offset it is on, go to the epilogue warpgroup (three sets in rotation)
       lpart[(it % 3) * 384 + wg * kTile + r] = l;
       mpart[(it % 3) * 384 + wg * kTile + r] = m_mine;
       __syncwarp();
@@ -1134,6 +1143,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       const float m_fin = fmaxf(m0, fmaxf(m1, m2));
       auto on_final = [&](float lg, float mg) { return mg == -CUDART_INF_F ? 0.f : lg * ex2f(mg - m_fin); };
       const float lt = (on_final(lp[0], m0) + on_final(lp[kTile], m1)) + on_final(lp[2 * kTile], m2);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(LPART_FREE + it % 3));
       const float inv = lt > 0.f ? 1.f / lt : 0.f;
       // the previous item's store must have read the staging buffer before it is written again
       if (warp == kFirstEpilogueWarp && lane == 0) {
