@@ -1355,7 +1355,10 @@ static int cut_items(int64_t n_items, int T) {
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
       int found = 0;
-      if (cudaOccupancyMaxActiveClusters(&found, attention_tc_kernel<D, true>, &cfg) != cudaSuccess) return best;  // asked again next time
+      if (cudaOccupancyMaxActiveClusters(&found, attention_tc_kernel<D, true>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return best;  // asked again next time
+      }
       c = found + 1;
     }
     if (n_items > c - 1) break;

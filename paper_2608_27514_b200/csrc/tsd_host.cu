@@ -10,6 +10,7 @@ static thread_local char g_last_cuda_error[256] = "";
 int cuda_fail(cudaError_t e, const char* where) {
   snprintf(g_last_cuda_error, sizeof(g_last_cuda_error), "%s: %s (%s)", where,
            cudaGetErrorName(e), cudaGetErrorString(e));
+  cudaGetLastError();  // reported here: a later call must not find it again
   return TSD_ERR_CUDA;
 }
 

@@ -330,3 +330,13 @@ def test_everything_is_complete_when_decode_returns():
             seen = [dec.tree[key].clone() for key in ("state", "parent", "n")]
         torch.cuda.synchronize()
         assert all(torch.equal(a, dec.tree[key]) for a, key in zip(seen, ("state", "parent", "n")))
+
+
+def test_a_refused_launch_is_not_reported_again_by_a_later_call():
+    # the runtime keeps a launch that it refused as its last error until somebody asks
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    many = torch.zeros((70000, 1, 1, 8), dtype=torch.bfloat16, device=DEV)
+    with pytest.raises(B.TsdError):                 # more sequences than a grid has rows
+        B.tsd_gather_accepted_kv(None, 1, many, None, torch.zeros_like(many), None)
+    B.tsd_selftest_bounded_wait(status)
+    assert B.tsd_check_status(status) == B.TSD_ERR_TIMEOUT
