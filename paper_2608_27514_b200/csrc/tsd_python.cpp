@@ -9,7 +9,7 @@
 
 namespace {
 
-PyObject *n_data_ptr, *n_stride, *n_shape, *n_nbytes, *n_dtype, *n_cuda_stream;
+PyObject *n_data_ptr, *n_stride, *n_shape, *n_nbytes, *n_dtype, *n_cuda_stream, *n_is_contiguous;
 PyObject *get_device, *get_raw_stream, *dtype_f32, *dtype_bf16, *error_type;  // set by setup()
 
 struct Failed {};  // a Python exception is set
@@ -56,8 +56,17 @@ int read_tuple(const Ref& t, int64_t* v, int most) {
   for (int i = 0; i < n && i < most; ++i) v[i] = to_int(PyTuple_GET_ITEM(t.p, i));
   return n;
 }
+int64_t last_size(PyObject* t) {
+  Ref s(PyObject_GetAttr(t, n_shape));
+  Ref last(PySequence_GetItem(s.p, -1));
+  return to_int(last.p);
+}
 int shape(PyObject* t, int64_t (&v)[4]) { return read_tuple(Ref(PyObject_GetAttr(t, n_shape)), v, 4); }
 int strides(PyObject* t, int64_t (&v)[4]) { return read_tuple(Ref(PyObject_CallMethodNoArgs(t, n_stride)), v, 4); }
+bool contiguous(PyObject* t) {  // as torch has it: the stride of a dimension of size 1 does not matter
+  Ref c(PyObject_CallMethodNoArgs(t, n_is_contiguous));
+  return c.p == Py_True;
+}
 void want(bool ok, const char* what) {
   if (ok) return;
   PyErr_SetString(PyExc_AssertionError, what);
@@ -259,14 +268,13 @@ PyObject* commit(Args a) {
 // prev_state, accepted_node, unmask_flag, unmask_tok, mask_id, topk_idx, topk_prob, width, depth, parent, state, node_prob,
 // n_nodes, status, stream, first, max_nodes (None = the rest), enable
 PyObject* build_tree(Args a) {
-  int64_t s[4], k[4], o[4];
+  int64_t s[4], o[4];
   shape3(a[0], s);
-  const int nk = shape(a[5], k);
+  const int64_t k = last_size(a[5]);
   shape3(a[10], o);
   const int64_t first = to_int(a[15]), B = o[1], max_nodes = a[16] == Py_None ? B - first : to_int(a[16]);
-  want(nk >= 1 && nk <= 4, "topk_idx has 1 to 4 dimensions");
   want(0 <= first && first + max_nodes <= B, "the tree fits the output arrays");
-  return done(call(tsd_build_draft_tree, (int32_t)s[0], (int32_t)s[1], (int32_t)s[2], (int32_t)k[nk - 1], ptr<int32_t>(a[0]),
+  return done(call(tsd_build_draft_tree, (int32_t)s[0], (int32_t)s[1], (int32_t)s[2], (int32_t)k, ptr<int32_t>(a[0]),
                                    ptr<int32_t>(a[1]), ptr<uint8_t>(a[2]), ptr<int32_t>(a[3]), to_i32(a[4]), ptr<int32_t>(a[5]),
                                    ptr<float>(a[6]), to_i32(a[7]), to_i32(a[8]), (int32_t)max_nodes, (int32_t)B, (int32_t)first,
                                    ptr<uint8_t>(a[17]), ptr<int32_t>(a[9], first * 4), ptr<int32_t>(a[10], first * o[2] * 4),
@@ -284,9 +292,8 @@ PyObject* build_mask(Args a) {
 
 // n_cur, vis, stream
 PyObject* interblock_vis(Args a) {
-  int64_t s[4], st[4];
-  want(shape(a[1], s) == 3 && strides(a[1], st) == 3 && s[2] == (s[1] + 63) / 64 && st[2] == 1 && st[1] == s[2] &&
-           (s[0] == 1 || st[0] == s[1] * s[2]) && (int64_t)nbytes(a[1]) == 8 * s[0] * s[1] * s[2],
+  int64_t s[4];
+  want(shape(a[1], s) == 3 && s[2] == (s[1] + 63) / 64 && contiguous(a[1]) && (int64_t)nbytes(a[1]) == 8 * s[0] * s[1] * s[2],
        "vis is a contiguous 64-bit [sequences, branches, words]");
   return done(call(tsd_build_interblock_vis, (int32_t)s[0], (int32_t)s[1], to_i32(a[0]), ptr<uint64_t>(a[1]), stream_of(a[2])),
               "tsd_build_interblock_vis");
@@ -437,5 +444,6 @@ PyMODINIT_FUNC PyInit__tsd_native(void) {
   n_nbytes = PyUnicode_InternFromString("nbytes");
   n_dtype = PyUnicode_InternFromString("dtype");
   n_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+  n_is_contiguous = PyUnicode_InternFromString("is_contiguous");
   return PyModule_Create(&module);
 }

@@ -35,6 +35,14 @@ def test_vis_matches_oracle(Bn, n_cur):
         assert np.array_equal(got[s], ref)
 
 
+def test_vis_in_memory_whose_last_dimension_has_an_odd_stride():
+    # one word per branch: contiguous in torch's terms whatever the stride of that dimension is
+    vis = torch.full((3 * 7,), -1, dtype=torch.int64, device=DEV).as_strided((3, 7, 1), (7, 1, 5))
+    assert vis.is_contiguous()
+    B.tsd_build_interblock_vis(4, vis)
+    assert torch.equal(vis, _gpu_vis(3, 7, 4))
+
+
 def test_trigger_matches_oracle():
     rng = np.random.default_rng(11)
     S, Bn, R, M, tau = 64, 6, 32, 1000, 0.75

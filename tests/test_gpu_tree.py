@@ -64,6 +64,16 @@ def test_tree_matches_oracle_random_pools(R, k, Wd, D, Bn, lowest):
         assert np.array_equal(got[3][s], nprob)
 
 
+def test_candidates_with_a_dimension_more():
+    # only the last dimension of topk_idx is looked at
+    rng = np.random.default_rng(3)
+    prev = np.full((2, 1, 32), 99, dtype=np.int32)
+    idx, prob = rng.integers(0, 99, (2, 1, 32, 3)).astype(np.int32), -np.sort(-rng.random((2, 1, 32, 3)).astype(np.float32), axis=-1)
+    a = _gpu_tree(prev, None, None, None, 99, idx, prob, 3, 3, 7)
+    b = _gpu_tree(prev, None, None, None, 99, idx[None], prob[None], 3, 3, 7)
+    assert all(np.array_equal(x, y) for x, y in zip(a, b)) and a[0].tolist() == [7, 7]
+
+
 def test_tree_without_acceptance_inputs_and_bad_node():
     rng = np.random.default_rng(1)
     S, R, k, M = 3, 32, 3, 500
