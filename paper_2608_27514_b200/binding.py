@@ -241,7 +241,7 @@ def tsd_accept_joint_trees(parent, state, n_cur, mask_id, conf, top1_idx, top1_s
                            unmask_flag, unmask_tok, status=None, stream=None):
     """Forest layout: parent/edge_valid/prefix_len [S,B]; accepted_* and n_new_tokens [2,S];
     unmask_* [2,S,R]."""
-    native().accept(parent, state, n_cur, mask_id, conf, top1_idx, top1_stride, tau, rule, search, edge_valid, prefix_len,
+    native().accept(parent, state, int(n_cur), mask_id, conf, top1_idx, top1_stride, tau, rule, search, edge_valid, prefix_len,
                     accepted_node, accepted_len, n_new_tokens, unmask_flag, unmask_tok, status, stream)
 
 

@@ -155,6 +155,7 @@ struct AttnViews {
       strides3(kc, c);
       if (vc != Py_None) same_strides(c, vc);
     } else {
+      want(vc == Py_None, "V rows of the cache without K rows");
       c[2] = L->head_dim;
     }
     strides3(kd, d);
@@ -179,6 +180,7 @@ PyObject* verify_attention(Args a) {
 PyObject* verify_attention_fp8(Args a) {
   Layout L(a[0]);
   const AttnViews v(L.get(), a[2], a[3], a[4], a[7], a[8], a[9]);
+  want(a[10] != Py_None, "a workspace is wanted");
   return done(call(tsd_verify_attention_fp8_cache, L.get(), ptr(a[1]), ptr(a[2]), v.q[0], v.q[1], v.q[2], ptr<uint8_t>(a[3]), ptr<uint8_t>(a[4]), v.c[0], v.c[1],
                   v.c[2], ptr<float>(a[5]), ptr<float>(a[6]), ptr(a[7]), ptr(a[8]), v.d[0], v.d[1], v.d[2], ptr(a[9]), v.o[0],
                   v.o[1], v.o[2], ptr<float>(a[11]), to_float(a[12]), ptr(a[10]), nbytes(a[10]), (uint32_t)to_int(a[13]),

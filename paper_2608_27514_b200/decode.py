@@ -70,6 +70,8 @@ class BlockDecoder:
         """Begin a block from root_state int32 [S, R]; the first pass has no candidate pool yet, so
         its tree is the root alone (copies in the unused slots)."""
         st, t = self.step, self.tree
+        if root_state.dim() != 2:
+            raise IndexError("root_state is [sequences, rows]")
         root = root_state.to(device=st.device, dtype=torch.int32).expand(st.S, st.R).contiguous()
         # a captured call is replayed for as long as its graph lives, which this object knows nothing of: it reports nothing
         report = None if torch.cuda.is_current_stream_capturing() else self.report

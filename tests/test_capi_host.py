@@ -3,11 +3,14 @@ header declares, and rejects bad arguments before launching anything."""
 import ctypes
 import os
 import re
+from types import SimpleNamespace
 
 import pytest
+import torch
 
 import __graft_entry__  # noqa: F401  (builds the library on first use)
 from paper_2608_27514_b200 import binding as B
+from paper_2608_27514_b200.decode import BlockDecoder
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -134,6 +137,28 @@ def test_step_rejects_logits_for_more_rows_than_the_tree_has(lib):
     for rows in (257, 1 << 20):
         a.n_rows = rows
         assert lib.tsd_verify_step(ctypes.byref(a), None) == B.TSD_ERR_INVALID_ARG
+
+
+def test_arguments_that_the_ctypes_calls_refused_are_refused(lib):
+    # nothing may be launched: the tensors are host memory (and there need be no device)
+    layout = B.make_layout(1, 1, 32, 0, 1, 1, 64, B.TSD_BF16)      # no cached tokens: the library itself asks for no cache
+    x = torch.zeros((1, 32, 1, 64), dtype=torch.bfloat16)
+    mask = torch.zeros(B.tsd_branch_mask_bytes(layout), dtype=torch.uint8)
+    with pytest.raises((AssertionError, AttributeError)):
+        B.tsd_verify_attention(layout, mask, x, None, x, x, x, x, stream=0)
+    with pytest.raises((AssertionError, AttributeError)):
+        B.tsd_verify_attention_fp8_cache(layout, mask, x, None, None, None, None, x, x, x, None, stream=0)
+    i32 = lambda *shape: torch.zeros(shape, dtype=torch.int32)
+    with pytest.raises(TypeError):
+        B.tsd_accept_joint_trees(i32(1, 2), i32(1, 2, 32), None, 99, torch.zeros(64), i32(64, 1), 1, 0.9, 0, 0, *[i32(64)] * 7, stream=0)
+
+
+@pytest.mark.parametrize("shape", [(), (32,), (2, 32, 1)])
+def test_a_block_starts_from_rows_per_sequence(shape):
+    decoder = BlockDecoder.__new__(BlockDecoder)
+    decoder.step, decoder.trees, decoder.cur = SimpleNamespace(S=2, R=32, device=torch.device("cpu")), [dict(state=None)], 0
+    with pytest.raises(IndexError):
+        decoder.start(torch.zeros(shape, dtype=torch.int32))
 
 
 def test_missing_library_is_loud(monkeypatch):
