@@ -549,7 +549,8 @@ int tsd_verify_step(const tsd_step_args* args, tsd_stream_t stream);
  * see below) gets them with `ticket`.
  *
  * tsd_advance_block is one pass after the model's forward: tsd_confidence_topk on
- * the logits of every node (batch * B * R rows), the acceptance under `rule`
+ * the logits of every node (n_rows = batch * B * R; fewer, as for tsd_verify_step, unless
+ * the rule is TSD_ACCEPT_PROB), the acceptance under `rule`
  * (TSD_ACCEPT_TOPK with topk_m = k; draft_prob, nullable, is written under
  * TSD_ACCEPT_PROB only), tsd_commit_accepted and tsd_build_draft_tree into next_*,
  * arguments as for those calls (max_nodes = B, a tree of its own).  next_* must not
@@ -575,7 +576,7 @@ int tsd_begin_block(int32_t batch, int32_t n_branches, int32_t rows_per_branch, 
 typedef struct {
   int32_t batch, n_branches, rows_per_branch;
   const void* logits;
-  int64_t row_stride;
+  int64_t n_rows, row_stride;
   int32_t logits_dtype, vocab, k;
   float* conf;
   int32_t* topk_idx;

@@ -102,7 +102,7 @@ extern "C" int tsd_advance_block(const tsd_advance_args* x, tsd_stream_t stream)
   if (!x) return TSD_ERR_INVALID_ARG;
   const int32_t S = x->batch, B = x->n_branches, R = x->rows_per_branch;
   const bool relaxed = x->rule != TSD_ACCEPT_EXACT && x->rule != TSD_ACCEPT_TOP1;
-  const tsd::TopkArgs t = {x->logits, x->logits_dtype, (int64_t)S * B * R, x->vocab, x->row_stride, x->k, x->conf, x->topk_idx,
+  const tsd::TopkArgs t = {x->logits, x->logits_dtype, x->n_rows, x->vocab, x->row_stride, x->k, x->conf, x->topk_idx,
                            x->topk_prob, x->lse, x->topk_workspace, x->topk_workspace_bytes, stream, tsd::kNextAfter, false};
   tsd::AdvanceArgs a = {};
   a.accept = {S, B, B, R, x->parent, x->state, x->mask_id, x->conf, x->topk_idx, x->k, x->tau, x->rule, x->search, x->edge_valid,
@@ -127,6 +127,8 @@ extern "C" int tsd_advance_block(const tsd_advance_args* x, tsd_stream_t stream)
   if (rc == TSD_OK) rc = tsd::check_accept(a.accept, a.relaxed);
   if (rc != TSD_OK) return rc;
   if (x->width < 1 || x->width > tsd::kTreeMaxWidth || x->depth < 0 || x->k > tsd::kTreeMaxK) return TSD_ERR_INVALID_ARG;
+  const int64_t rows = (int64_t)S * B * R;  // conf, topk_* hold one each; the probability rule reads the logits of any of them
+  if (x->n_rows > rows || (x->rule == TSD_ACCEPT_PROB && x->n_rows != rows)) return TSD_ERR_INVALID_ARG;
   if (x->tokens && x->seq_stride < R) return TSD_ERR_INVALID_ARG;
   if (S == 0) return TSD_OK;
   if (!x->next_parent || !x->next_state || !x->next_prob || !x->next_n || x->next_state == x->state) return TSD_ERR_INVALID_ARG;

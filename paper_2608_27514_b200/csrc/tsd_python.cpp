@@ -362,12 +362,13 @@ PyObject* advance_block(Args a) {
   int64_t s[4], st[4] = {0, 0, 0, 0};
   shape3(a[8], s);
   const Logits x(a[0]);
-  want(x.n == s[0] * s[1] * s[2], "logits have a row for every (sequence, branch, row)");
+  want(to_i32(a[11]) == TSD_ACCEPT_PROB ? x.n == s[0] * s[1] * s[2] : x.n <= s[0] * s[1] * s[2],
+       "logits have a row for every (sequence, branch, row)");
   if (a[21] != Py_None) want(strides(a[21], st) == 2 && st[1] == 1, "tokens are [sequences, length], contiguous");
   tsd_advance_args t = {};
   t.batch = (int32_t)s[0]; t.n_branches = (int32_t)s[1]; t.rows_per_branch = (int32_t)s[2];
   t.logits = ptr(a[0]);
-  t.row_stride = x.pitch; t.logits_dtype = x.dtype; t.vocab = x.vocab;
+  t.n_rows = x.n; t.row_stride = x.pitch; t.logits_dtype = x.dtype; t.vocab = x.vocab;
   t.k = to_i32(a[1]);
   t.conf = ptr<float>(a[2]); t.topk_idx = ptr<int32_t>(a[3]); t.topk_prob = ptr<float>(a[4]); t.lse = ptr<float>(a[5]);
   t.topk_workspace = ptr(a[6]);

@@ -340,3 +340,28 @@ def test_a_refused_launch_is_not_reported_again_by_a_later_call():
         B.tsd_gather_accepted_kv(None, 1, many, None, torch.zeros_like(many), None)
     B.tsd_selftest_bounded_wait(status)
     assert B.tsd_check_status(status) == B.TSD_ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("rule", [B.TSD_ACCEPT_EXACT, B.TSD_ACCEPT_TOPK])
+def test_a_pass_with_logits_for_the_used_nodes_only(rule):
+    # one sequence, a tree of 4 nodes in 9 slots: the padding needs no logits
+    S, Bn, R, V, M = 1, 9, 32, 600, 599
+    g = torch.Generator(device=DEV).manual_seed(2)
+    root = torch.full((S, R), M, dtype=torch.int32, device=DEV)
+    rows = torch.randn((1, R, V), generator=g, device=DEV) * 2
+    logits = [(rows + 0.1 * torch.randn((Bn, R, V), generator=g, device=DEV)).bfloat16().reshape(-1, V) for _ in range(2)]
+    seen = []
+    for used in (Bn, 4):
+        dec = BlockDecoder(VerifyStep(S, Bn, R, 0, 1, 1, 64, V, 3, torch.bfloat16, DEV), 3, 1, 0.2, M, rule)
+        dec.step.conf.fill_(0.5)
+        dec.step.topk_idx.zero_()
+        dec.start(root)
+        for x in logits:
+            dec.advance(x[:used * R])
+        assert int(dec.tree["n"]) == 4
+        seen.append([dec.root, dec.fill_step, dec.n_masked, dec.tree["parent"], dec.tree["state"], dec.step.accepted_node])
+    assert all(torch.equal(a, b) for a, b in zip(*seen)) and int(seen[0][2]) < R
+    dec = BlockDecoder(VerifyStep(S, Bn, R, 0, 1, 1, 64, V, 3, torch.bfloat16, DEV), 3, 1, 0.2, M, rule)
+    dec.start(root)
+    with pytest.raises(AssertionError):
+        dec.advance(torch.cat(logits))
