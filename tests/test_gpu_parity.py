@@ -467,9 +467,8 @@ def test_topk_minus_inf_and_split_rows():
 
 @pytest.mark.parametrize("fill", ["ones", "random", "last_call"])
 def test_topk_workspace_needs_no_clearing(fill):
-    # few rows: each row is split over several blocks that meet through ticket words in the
-    # workspace; whatever the workspace held before (all bits set, noise, the previous call's
-    # leftovers), the results are the oracle's
+    # few rows of an ordinary vocabulary: the blocks of a row meet in a cluster, but a workspace is asked for all the same; whatever
+    # it held before (all bits set, noise, the previous call's leftovers), the results are the oracle's
     V, k = 50000, 3
     g = torch.Generator(device=DEV).manual_seed(11)
     x = (torch.randn((5, V), generator=g, device=DEV) * 3).bfloat16()
@@ -489,6 +488,48 @@ def test_topk_workspace_needs_no_clearing(fill):
         assert np.array_equal(idx.cpu().numpy(), r_idx)
         assert np.abs(conf.cpu().numpy() - r_conf).max() <= 1e-5
         assert np.abs(prob.cpu().numpy() - r_prob).max() <= 1e-5
+
+
+@pytest.mark.parametrize("dtype,n,V", [("bf16", 3, 2200000), ("f32", 2, 1200000), ("f32", 1, 4194304), ("bf16", 160, 2100003)])
+def test_topk_rows_of_more_segments_than_a_cluster_holds(dtype, n, V):
+    # more than 8 segments per row: these meet through partial results and ticket words in the workspace, which needs clearing
+    # neither before a call nor between calls (all bits set, noise, what the call before it left), of this shape or another
+    k = 3
+    g = torch.Generator(device=DEV).manual_seed(V % 1000 + n)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    x = torch.empty((n, (V + 7) // 8 * 8), dtype=dt, device=DEV)
+    for r in range(n):
+        x[r] = torch.randn(x.shape[1], generator=g, device=DEV) * 3
+    x = x[:, :V]
+    x[0, V // 3:V // 3 + 50] = 40.0                     # the best of row 0 tie, across a pool
+    nbytes = B.tsd_confidence_topk_workspace_bytes(n, V, k)
+    rows = [0, n // 2, n - 1]
+    want = oracle.confidence_topk(_np(x[torch.as_tensor(rows, device=DEV)]), k)
+    ws = torch.full((nbytes,), 0xFF, dtype=torch.uint8, device=DEV)
+    other = torch.randn((5, 50000), generator=g, device=DEV).bfloat16()
+    for fill in ("ones", "last call", "noise", "last call", "another shape"):
+        if fill == "noise":
+            ws.copy_(torch.randint(0, 256, (nbytes,), generator=g, device=DEV, dtype=torch.uint8))
+        out = [torch.full(shape, -1, dtype=t, device=DEV) for shape, t in (((n,), torch.float32), ((n, k), torch.int32), ((n, k), torch.float32),
+                                                                           ((n,), torch.float32))]
+        if fill == "another shape" and nbytes >= B.tsd_confidence_topk_workspace_bytes(5, 50000, k):
+            small = [torch.empty(shape, dtype=t, device=DEV) for shape, t in (((5,), torch.float32), ((5, k), torch.int32), ((5, k), torch.float32))]
+            B.tsd_confidence_topk(other, k, *small, None, ws)
+        B.tsd_confidence_topk(x, k, *out, ws)
+        conf, idx, prob, lse = (_np(t)[rows] for t in out)
+        assert np.array_equal(idx, want[1])
+        assert np.abs(conf - want[0]).max() <= 1e-5 and np.abs(prob - want[2]).max() <= 1e-5 and np.abs(lse - want[3]).max() <= 1e-4
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 600001), ("f32", 300000), ("bf16", 1200000), ("bf16", 1500004), ("bf16", 1800000), ("f32", 1000000)])
+def test_topk_rows_in_clusters_of_any_size(dtype, V):
+    # long rows need 3, 5, 6, 7 or 8 segments (32768 vectors each at most) where the number of rows alone would ask for one or two
+    n = 150
+    g = torch.Generator(device=DEV).manual_seed(V % 1000)
+    x = torch.empty((n, (V + 7) // 8 * 8), dtype=torch.bfloat16 if dtype == "bf16" else torch.float32, device=DEV)
+    for r in range(n):
+        x[r] = torch.randn(x.shape[1], generator=g, device=DEV) * 3
+    _check_topk(x[:, :V], 5, rows=[0, 1, n - 1])
 
 
 def test_topk_all_equal_rows_whole_and_split():
@@ -748,7 +789,7 @@ def test_topk_k_equals_vocab_and_single_row():
     x = torch.randn((5, 8), generator=g, device=DEV).bfloat16()
     _check_topk(x, 8)                                  # every entry is a candidate
     y = torch.randn((1, 300000), generator=g, device=DEV)
-    _check_topk(y, 8)                                  # one long fp32 row: segments + ticket merge
+    _check_topk(y, 8)                                  # one long fp32 row: 8 segments, which meet in a cluster
     z = torch.randn((3, 16), generator=g, device=DEV)
     _check_topk(z[:, :1], 1)                           # vocabulary of one
 

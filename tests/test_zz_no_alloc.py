@@ -4,8 +4,8 @@ that stops at the first failure has already run everything else.
 
 Who needs it: a caller that receives only input and output buffers and cannot get more device
 memory when the call is made (a plug-in with a frozen memory pool, a decode step that must not
-call cudaMalloc).  The test uses few rows so that rows are split into segments, which is the case
-that needs scratch at all."""
+call cudaMalloc).  Scratch is used by rows of more segments than a cluster of blocks holds: more than
+2 Mi bf16 or 1 Mi fp32 logits."""
 import ctypes
 
 import numpy as np
@@ -54,10 +54,8 @@ def _check_against_oracle(x, k, got):
 def test_static_scratch_matches_workspace_entry_point_twice_in_a_row():
     g = torch.Generator(device=DEV).manual_seed(77)
     k = 3
-    # different inputs back to back: each call finds the previous call's leftovers in the shared
-    # array and must not be affected by them.  The shapes differ in segments per row and in k, so
-    # that the partial-result slots of one call overlap the ticket words of another, and both
-    # element types take part.
+    # different inputs back to back, split rows of ordinary vocabularies: the size asked for is that of a split into
+    # segments, and the two entry points give the same
     xa = (torch.randn((100, 126464), generator=g, device=DEV) * 3).bfloat16()
     xb = (torch.randn((40, 50000), generator=g, device=DEV) * 3).bfloat16()
     xc = torch.randn((7, 90000), generator=g, device=DEV) * 3                  # fp32
@@ -71,6 +69,21 @@ def test_static_scratch_matches_workspace_entry_point_twice_in_a_row():
             assert (a - b).abs().max().item() <= 1e-5
         assert (got[3] - ref[3]).abs().max().item() <= 1e-4
         _check_against_oracle(x, kk, got)                          # and the definition itself
+
+
+def test_static_scratch_is_shared_by_calls_of_different_shapes():
+    # rows long enough to use the array: each call finds the previous call's leftovers there and must not be affected by
+    # them.  The shapes differ in segments per row, rows and k, so that the partial-result slots of one call overlap the
+    # ticket words of another, and both element types take part.
+    g = torch.Generator(device=DEV).manual_seed(78)
+    xa = (torch.randn((3, 2200000), generator=g, device=DEV) * 3).bfloat16()
+    xb = torch.randn((2, 1200000), generator=g, device=DEV) * 3
+    xc = (torch.randn((9, 2400000), generator=g, device=DEV) * 3).bfloat16()
+    for x, k in ((xa, 3), (xb, 8), (xc, 1), (xa, 3), (xc, 5), (xb, 2)):
+        assert 0 < B.tsd_confidence_topk_workspace_bytes(*x.shape, k) <= B.tsd_confidence_topk_static_capacity()
+        got = _static(x, k)
+        assert all(torch.equal(a, b) for a, b in zip(got, _regular(x, k)))
+        _check_against_oracle(x[:2], k, [t[:2] for t in got])
 
 
 def test_static_scratch_rejects_what_does_not_fit():
