@@ -16,7 +16,9 @@
 // rows, 800 keys, D = 128, which take 7.4 and 95 us here.
 // What bounds it: on the sizes fp32 is used for (checking; a few heads, hundreds of keys) the chain of
 // dependent loads and the number of blocks, at larger ones the fp32 pipe (3 of 4 instructions are
-// multiply-adds) and the L2 reads of K and V, once per RB rows.
+// multiply-adds) and the L2 reads of K and V, once per RB rows.  Eight rows of 128 dimensions do not fit the 128 registers that two
+// blocks per SM leave a thread: that form spills (fp32 332 bytes of stores and 476 of loads, bf16 368 and 480; the others
+// 0 to 28).
 #include <limits.h>
 #include <math_constants.h>
 #include <algorithm>

@@ -10,6 +10,10 @@ namespace tsd {
 // Records a failed CUDA runtime call for tsd_last_cuda_error(); returns TSD_ERR_CUDA.
 int cuda_fail(cudaError_t e, const char* where);
 
+// SMs of the GPU that the plans of the vocabulary pass and of the step were measured for.  A constant, because the workspace
+// queries answer without a device; the attention, which asks for none, counts the SMs of the device it runs on.
+constexpr int kPlanSms = 148;
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // ---- branch-mask blob (written by tsd_build_branch_mask, read by the attention kernels) ----
@@ -197,11 +201,6 @@ __device__ __forceinline__ bool ticket_arrive(unsigned* t, int n) {
     old = atomicCAS(t, assumed, next);
   } while (old != assumed);
   return cnt + 1 == (unsigned)n;
-}
-// Arrivals so far (a snapshot: more may follow at any time).
-__device__ __forceinline__ unsigned ticket_count(const unsigned* t) {
-  const unsigned v = *reinterpret_cast<const volatile unsigned*>(t);
-  return (v >> 8) == kTicketTag ? (v & 0xffu) : 0u;
 }
 #endif
 

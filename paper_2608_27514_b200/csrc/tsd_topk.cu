@@ -582,7 +582,7 @@ static size_t workspace_bytes(int64_t n_rows, int vocab, int k, int elems_per_ch
   const int chunks = vocab / elems_per_chunk;
   TopkPlan p;
   p.K = round_k(k);
-  const int64_t n_seg = std::min<int64_t>(std::min<int64_t>((148 + n_rows - 1) / n_rows, kMaxSegments), std::max(1, chunks / 2048));
+  const int64_t n_seg = std::min<int64_t>(std::min<int64_t>((kPlanSms + n_rows - 1) / n_rows, kMaxSegments), std::max(1, chunks / 2048));
   p.n_seg = (int)std::max<int64_t>(n_seg, (chunks + kTopkSegChunks - 1) / kTopkSegChunks);
   scratch_layout(n_rows, p);
   return p.total_bytes;
@@ -599,8 +599,8 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
   int64_t n_seg = 1;
   if (n_rows > 0 && n_rows <= 222) {
     double best = 1e30;
-    for (int n = 1; n <= (n_rows <= 148 ? kMaxCluster : 2); n *= 2) {
-      const double rounds = (double)((n_rows * n + 147) / 148) / n;
+    for (int n = 1; n <= (n_rows <= kPlanSms ? kMaxCluster : 2); n *= 2) {
+      const double rounds = (double)((n_rows * n + kPlanSms - 1) / kPlanSms) / n;
       const double cost = rounds * chunks / 15808 + (n > 1 ? 0.17 + 0.005 * n : 0.0);
       if (cost < best) { best = cost; n_seg = n; }
     }
@@ -611,12 +611,12 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
   // As many warps per row as still give every block a slot at once: 256 x 126464 bf16 with 512 threads 17.0 us, with
   // 384 17.9, with 256 18.8; 444 x 126464 25.0 / 23.5 / 24.4; 960 x 126464 50.2 / 48.2 / 46.0.
   const int64_t units = n_rows * p.n_seg;
-  p.threads = units <= 2 * 148 ? 512 : (units <= 3 * 148 ? 384 : 256);
-  // Rows that even 256 threads walk in one batch or two: 256 x 4096 fp32 with 512 threads 4.75 us, with 256 4.42 (bf16 4.79
-  // and 4.41); 128 x 8000 4.30 and 4.5, 128 x 16000 5.0 and 5.8.
+  p.threads = units <= 2 * kPlanSms ? 512 : (units <= 3 * kPlanSms ? 384 : 256);
+  // Rows that even 256 threads walk in one batch: with 512 threads 256 x 4096 fp32 takes 4.6 us and with 256 4.3, bf16 4.7 and 4.4,
+  // 256 x 8192 bf16 4.8 and 4.6, 296 x 8000 bf16 5.2 and 4.9; 128 x 8000 and fewer rows the same (4.3).  128 x 16000: 5.0 and 5.8.
   if (chunks <= 1024) p.threads = 256;
   // clusters of large blocks are hard to place: 74 x 126464 in 4 segments 12.8 us with 512 threads, 10.4 with 256
-  if (p.n_seg > 1 && units > 148) p.threads = 256;
+  if (p.n_seg > 1 && units > kPlanSms) p.threads = 256;
   // L2 prefetch distance in batches (measured): with very many waves of blocks, requesting lines three batches ahead
   // adds 2 % of bandwidth (16384 x 126464: 687 us, without 700); with fewer it delays the demand loads (4096 x 32000:
   // 57.0 us, without 53.6; 4096 x 126464: 171 and 167; 4096 x 152064: 189.7 and 190.8)

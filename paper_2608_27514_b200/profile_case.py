@@ -2,7 +2,8 @@
 ncu captures summarised under profiles/ (small enough for a full-set capture, larger than L2).
 
   python -m paper_2608_27514_b200.profile_case topk [--rows 2048] [--vocab 126464] [--k 3]
-  python -m paper_2608_27514_b200.profile_case attention [--workload cfg4] [--batch 4]
+  python -m paper_2608_27514_b200.profile_case attention [--workload cfg4] [--batch 4] [--set d=64 Hkv=8 ...]
+  python -m paper_2608_27514_b200.profile_case decode [--workload cfg2] [--batch 3] [--set B=10 ...]
 
 Prints the CUDA-event time of the last call.  Nothing here is timed for the benchmark.
 """
@@ -12,17 +13,19 @@ import torch
 
 from . import binding as B
 from . import workloads as W
+from .decode import BlockDecoder
 from .step import VerifyStep
 
 
 def main():
     ap = argparse.ArgumentParser()
-    ap.add_argument("stage", choices=["topk", "attention"])
+    ap.add_argument("stage", choices=["topk", "attention", "decode"])
     ap.add_argument("--rows", type=int, default=2048)
     ap.add_argument("--vocab", type=int, default=126464)
     ap.add_argument("--k", type=int, default=3)
     ap.add_argument("--workload", default="cfg4")
     ap.add_argument("--batch", type=int, default=4)
+    ap.add_argument("--set", nargs="*", default=[], help="other sizes than the workload's: name=value")
     ap.add_argument("--calls", type=int, default=4)
     args = ap.parse_args()
     dev = "cuda:0"
@@ -39,7 +42,19 @@ def main():
         call = lambda: B.tsd_confidence_topk(x, args.k, conf, idx, prob, lse, ws)
         work, unit = args.rows * args.vocab * 2 / 1e9, "GB"
     else:
-        cfg = W.small(W.CONFIGS[args.workload], S=args.batch)
+        sizes = dict(item.split("=") for item in args.set)
+        cfg = W.small(W.CONFIGS[args.workload], name="case", S=args.batch, **{n: v if n == "dtype" else int(v) for n, v in sizes.items()})
+    if args.stage == "decode":
+        st = VerifyStep.for_config(cfg, dev)
+        logits = W.verify_inputs(cfg, dev)["logits"]
+        dec = BlockDecoder(st, 3, 3, cfg.tau, cfg.V - 1, B.TSD_ACCEPT_PROB, B.TSD_SEARCH_LONGEST)
+        root = torch.full((cfg.S, cfg.R), cfg.V - 1, dtype=torch.int32, device=dev)
+
+        def call():
+            dec.start(root)
+            dec.decode(lambda state: logits, max_passes=2)
+        work, unit = 2 * cfg.rows * cfg.V * 2 / 1e9, "GB"
+    if args.stage == "attention":
         attn = W.attention_inputs(cfg, dev)
         st = VerifyStep.for_config(cfg, dev)
         st.build_mask()
