@@ -22,7 +22,7 @@
 //               memory, fp32 accumulation in tensor memory.
 // All rows share one O accumulator, so the warpgroups agree on the exponent offset of a row
 // through a chain of decisions in tile order: the thread that owns row r in tile t waits for the
-// decision of tile t-1 (a per-warp mbarrier and one float per row in shared memory), keeps that
+// decision of tile t-1 (a word of shared memory per row that holds the offset and the tile), keeps that
 // offset unless the tile's maximum exceeds it by more than 2^8, publishes its decision and only
 // then starts on the exponentials.  The chain is short; the expensive part of the tiles overlaps.
 // A thread that moves the offset rescales the row of O before it publishes P (the P V of its tile
@@ -36,7 +36,7 @@
 // Items overlap: Q of the next item is loaded into shared memory and copied into the other Q
 // buffer during the current item, its first Q K^T are issued while the last softmax tiles of the
 // current item run, the softmax warpgroups go on to it without waiting for the epilogue, and its
-// first P V waits only until the epilogue has read O into registers.
+// first P V waits only until the epilogue has read O into registers (at head_dim 64 not even that: tensor memory has room for two O).
 // Few items (kCut): an item is shared by the blocks of a cluster, each with a stretch of its key tiles; at the end every block hands
 // every other one a share of the columns of its O through distributed shared memory and finishes the share that is
 // its own.  Bound by the serial chain of one item otherwise: 28 items of 81 key tiles took 40.6 us on 28 SMs and take 18.7 on 112,
@@ -66,7 +66,7 @@ constexpr int kNK = 5;                         // K stages: a K tile is needed w
 constexpr int kNV = 4;                         // V stages
 constexpr int kNP = 2;                         // P buffers in tensor memory
 constexpr int kKeys = 64;                      // keys per tile
-constexpr int kMaxItems = 512;                 // work items of one block (their tile counts sit in shared memory)
+constexpr int kMaxItems = 256;                 // work items of one block (what the warps need to know of them sits in shared memory)
 constexpr uint32_t kSub = 16384;               // bytes of one [128 rows x 64 elements] bf16 sub-tile
 constexpr uint32_t kSubKV = 8192;              // bytes of one [64 keys x 64 elements] bf16 sub-tile
 // Shared-memory layout for a head_dim of D = 64 or 128 (one sub-tile per 64 elements of head_dim).
@@ -79,13 +79,13 @@ struct TcSmem {
   static constexpr uint32_t kOffK = 2 * kTileBytes;
   static constexpr uint32_t kOffV = kOffK + kNK * kKVBytes;
   static constexpr uint32_t kOffBar = kOffV + kNV * kKVBytes;
-  static constexpr uint32_t kOffMref = kOffBar + 512;     // exponent offset per row (128 floats)
+  static constexpr uint32_t kOffMref = kOffBar + 512;     // per row: exponent offset and the tile after the one that decided it (128 x 8 bytes)
   // partial row sums and the exponent offsets they are on, per softmax warpgroup, for three items in
   // rotation (3 x 3 x 128 floats each): a softmax warpgroup leaves them for the epilogue and moves on
-  static constexpr uint32_t kOffLpart = kOffMref + 512;
+  static constexpr uint32_t kOffLpart = kOffMref + 1024;
   static constexpr uint32_t kOffMpart = kOffLpart + 3 * 3 * 128 * 4;
-  static constexpr uint32_t kOffItems = kOffMpart + 3 * 3 * 128 * 4;  // key tiles / cache length per item (2 x kMaxItems int32)
-  static constexpr uint32_t kBytes = kOffItems + 2 * kMaxItems * 4 + 1024;  // + slack to align the base to 1 KB
+  static constexpr uint32_t kOffItems = kOffMpart + 3 * 3 * 128 * 4;  // key tiles / cache length / mask record / sequence and kv head per item
+  static constexpr uint32_t kBytes = kOffItems + 4 * kMaxItems * 4 + 1024;  // + slack to align the base to 1 KB
 };
 static_assert(kKeys == kKeyTile, "the mask blob lists tiles of this many keys");
 // Tensor-memory columns.  At head_dim 128 everything is in use and P is one bf16 per score.  At head_dim 64
@@ -99,8 +99,10 @@ template <int D>
 struct TcCols {
   static constexpr bool kSplitP = D == 64;
   static constexpr uint32_t kPCols = kSplitP ? kKeys : kKeys / 2;   // columns of one P buffer
-  static constexpr uint32_t kO = 0, kQ = D, kQStride = D / 2;       // O, then two Q buffers
-  static constexpr uint32_t kS = 2 * D, kP = kS + kNSb * kKeys;     // three S buffers, two P buffers
+  // O, in two buffers at head_dim 64: the P V of an item then do not wait until the epilogue has read O of the item before
+  static constexpr int kNO = D == 64 ? 2 : 1;
+  static constexpr uint32_t kO = 0, kQ = kNO * D, kQStride = D / 2;  // then two Q buffers
+  static constexpr uint32_t kS = kQ + D, kP = kS + kNSb * kKeys;     // three S buffers, two P buffers
   static_assert(kP + kNP * kPCols <= 512, "tensor memory has 512 columns");
 };
 // What putting two parts of an item together takes, in key tiles of 0.43 us; 2 more with each doubling.  (56 items of 81
@@ -132,8 +134,8 @@ enum Bar {
                   //     its P buffer are free, O is up to date.  Waiters look at most one phase ahead of
                   //     what they know to be complete (a parity wait cannot tell two phases apart), which
                   //     is why this is a ring of four although there are only two P buffers.
-  DEC = 24,       // [4][4] exponent offsets of a tile decided, per tile mod 4 and warp quarter
-  O_FREE = 40,    // the epilogue has read O into registers
+  O_FULL = 24,    // [2] every P V of an item is complete, per O buffer
+  O_FREE = 26,    // [2] the epilogue has read O into registers, per O buffer
   LPART = 41,     // [3] every softmax warp has published its partial row sums of an item, per item mod 3: a warpgroup
                   //     without a tile in an item arrives for it while others are still at the item before
   STAGED = 44,    // the output tile is complete in the staging buffer
@@ -355,7 +357,7 @@ struct TcParams {
   const int32_t* mask;
   float* lse;
   uint32_t* status;
-  int S, B, R, Nc, N, Hq, group;
+  int S, B, R, Nc, N, Hq, Hkv, group;
   int recs_off, n_qt, rec_words;  // layout of the mask blob, computed on the host from the same tsd_layout
   int n_items;                    // S * Hq * n_qt
   float scale_log2e;              // sm_scale * log2(e), > 0
@@ -437,6 +439,19 @@ __device__ __forceinline__ float row_lse(const TcParams& p, float m, float l) {
   return (m + log2f(l)) * kLn2;
 }
 
+// A row's exponent offset and the count of tiles that have decided on it, in one word of shared memory: written by the thread that owns
+// the row in one tile, read by the one that owns it in the next.  (A barrier per warp with the offset beside it cost a test
+// of the barrier, a vote, the load and an arrival per tile, one behind the other: 512 items of 64-wide heads 65.3 us, with
+// the word 62.4, and with O in two buffers 59.5.)
+__device__ __forceinline__ void st_decision(uint32_t addr, float m, int count) {
+  asm volatile("st.volatile.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(__float_as_uint(m)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void ld_decision(uint32_t addr, float& m, int& count) {
+  uint32_t bits;
+  asm volatile("ld.volatile.shared.v2.b32 {%0, %1}, [%2];" : "=r"(bits), "=r"(count) : "r"(addr));
+  m = __uint_as_float(bits);
+}
+
 // Rarely executed pieces of the softmax warps, kept out of line so that the loop over the key
 // tiles stays small in the instruction cache.
 // One row of O (D fp32 columns of this thread's tensor-memory lane) times alpha.
@@ -489,11 +504,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(base_ptr + kOffBar + 452);
   volatile int32_t* parts = reinterpret_cast<volatile int32_t*>(base_ptr + kOffBar + 464);  // of a cut item
   volatile int32_t* tile_first = reinterpret_cast<volatile int32_t*>(base_ptr + kOffBar + 460);  // of the block's first item
-  float* mref = reinterpret_cast<float*>(base_ptr + L::kOffMref);
+  const uint32_t decisions = base + L::kOffMref;
   float* lpart = reinterpret_cast<float*>(base_ptr + L::kOffLpart);
   float* mpart = reinterpret_cast<float*>(base_ptr + L::kOffMpart);
   int32_t* item_T = reinterpret_cast<int32_t*>(base_ptr + L::kOffItems);
   int32_t* item_clen = item_T + kMaxItems;
+  uint32_t* item_rec = reinterpret_cast<uint32_t*>(item_clen + kMaxItems);  // word of the mask blob at which the lists of its query tile begin
+  int32_t* item_sg = item_clen + 2 * kMaxItems;  // sequence * kv heads + kv head
   auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -536,8 +553,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       mbar_init(bar(PV_GO + i), 5);
       mbar_init(bar(PV_DONE + i), 1);
     }
-    for (int i = 0; i < 16; ++i) mbar_init(bar(DEC + i), 1);
-    mbar_init(bar(O_FREE), 4);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(O_FULL + i), 1);
+      mbar_init(bar(O_FREE + i), 4);
+    }
     for (int i = 0; i < 3; ++i) {
       mbar_init(bar(LPART + i), kSoftmaxWarps);
       mbar_init(bar(LPART_FREE + i), 4);
@@ -567,13 +586,17 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   const int h_magic = mask[H_MAGIC], h_s = mask[H_S], h_b = mask[H_B], h_r = mask[H_R], h_nc = mask[H_NC];
   // tile counts of this block's items (the blob's layout follows from the tsd_layout, so no
   // address depends on a loaded value)
+  if (tid < kTile) st_decision(decisions + 8u * (uint32_t)tid, 0.f, 0);
   for (int it = tid; it < n_my; it += kTcThreads) {
     int s, h, qt;
     item_coords(it, s, h, qt);
     const int clen = min(max(mask[kHdrWords + s], 0), p.Nc);
-    const int n_dt = min(max(mask[p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words], 1), p.rec_words / 2 - 1);
+    const uint32_t rec = (uint32_t)p.recs_off + (uint32_t)(s * p.n_qt + qt) * (uint32_t)p.rec_words;
+    const int n_dt = min(max(mask[rec], 1), p.rec_words / 2 - 1);
     const int n_ct = (clen + kKeys - 1) / kKeys;
     item_clen[it] = clen;
+    item_rec[it] = rec;
+    item_sg[it] = s * p.Hkv + h / p.group;
     int T = n_ct + n_dt, first = 0;
     if (kCut) {  // this block's stretch; the first block alone takes an item of few tiles
       const bool whole = T < 2 * p.cut;
@@ -670,10 +693,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       for (int it = 0; it < n_run && ok; ++it) {
         // Q of this item must be on its way before its K tiles queue behind it
         while (is_k && ok && q_issued <= it) issue_q(true);
-        int s, h, qt;
-        item_coords(it, s, h, qt);
-        const int g = h / p.group, n_ct = (item_clen[it] + kKeys - 1) / kKeys, T = item_T[it];
-        const int32_t* rec = mask + p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words;
+        const int s = item_sg[it] / p.Hkv, g = item_sg[it] - s * p.Hkv, n_ct = (item_clen[it] + kKeys - 1) / kKeys, T = item_T[it];
+        const int32_t* rec = mask + item_rec[it];
         const int j0 = kCut ? *tile_first : 0;
         for (int j = j0; j < j0 + T && ok; ++j, ++G) {
           if (is_k) issue_q(false);
@@ -778,12 +799,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         const int T = __shfl_sync(0xffffffffu, item_T[it], 0);
         const int clen = __shfl_sync(0xffffffffu, item_clen[it], 0);
         const int n_ct = (clen + kKeys - 1) / kKeys;
-        int s, h, qt;
-        item_coords(it, s, h, qt);
-        const int32_t* rec = mask + p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words;
+        const int32_t* rec = mask + item_rec[it];
         const unsigned bits0 = (unsigned)__ldg(rec + 3);  // visibility of the first listed draft tile, asked for early
-        // the first P V of an item overwrites O: the epilogue of the previous item must have read it
-        if (it > 0) ok = mbar_wait(bar(O_FREE), (it - 1) & 1, abort_flag);
+        // the first P V of an item overwrites O: the epilogue must have read what was there before
+        const int ob = it % C::kNO;
+        if (it >= C::kNO) ok = mbar_wait(bar(O_FREE + ob), (it / C::kNO - 1) & 1, abort_flag);
         const int j0 = kCut ? __shfl_sync(0xffffffffu, *tile_first, 0) : 0;
         for (int j = j0; j < j0 + T; ++j, ++G) {
           const int b = G & 3;  // V stage; P buffer = G & 1
@@ -830,7 +850,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             uint32_t lo[kKeys / 16];
 #pragma unroll
             for (int kk = 0; kk < kKeys / 16; ++kk) lo[kk] = vd_lo[kk] + v_off;
-            issue_pv_mmas<D>(utmem + C::kO, utmem + C::kP + (uint32_t)(b & 1) * C::kPCols, lo, vd_hi, j == j0 ? 0u : 1u, bar(PV_DONE + b));
+            issue_pv_mmas<D>(utmem + C::kO + (uint32_t)(D * ob), utmem + C::kP + (uint32_t)(b & 1) * C::kPCols, lo, vd_hi, j == j0 ? 0u : 1u, bar(PV_DONE + b));
+            if (C::kNO == 2 && j == j0 + T - 1)
+              asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar(O_FULL + ob)) : "memory");
           }
           __syncwarp();
           ready = seen;
@@ -872,19 +894,17 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
     int G = 0, n_done = 0;
     for (int it = 0; it < n_run && ok; ++it) {
-      int s, h, qt;
-      item_coords(it, s, h, qt);
-      const int32_t* rec = mask + p.recs_off + (size_t)(s * p.n_qt + qt) * p.rec_words;
+      const int32_t* rec = mask + item_rec[it];
       const int clen = item_clen[it];
       const int T = item_T[it], j0 = kCut ? *tile_first : 0;  // tiles of the item from j0 on
       const int n_ct = (clen + kKeys - 1) / kKeys - j0;  // the cached ones among them (negative: behind the first draft tiles)
       const int jc = min(4, T - 1);  // the tile at which Q of the next item is copied
       // A warpgroup's sums of this item go where those of item it-3 were, and its arrival must not count for that item.  With a tile in
       // this item it has waited for the P V of a tile of item it-2 or later (for its P buffer) before it publishes them, and the
-      // first P V of item it-2 comes after the epilogue's reading of item it-3.  Without one it has waited for nothing of the
+      // first P V of item it-2 comes after the epilogue's reading of item it-3 (not with two O buffers).  Without one it has waited for nothing of the
       // kind (with items of one tile it is up to two items ahead), so it waits here.  (Here, and not where the sums are
       // written: there it changes the registers of the loop below, 5 ragged sequences of 28 heads 46.3 -> 50.7 us.)
-      if (it >= 3 && T < 3 && ((wg - G) % 3 + 3) % 3 >= T)
+      if (it >= 3 && (C::kNO == 2 || (T < 3 && ((wg - G) % 3 + 3) % 3 >= T)))
         ok = __all_sync(0xffffffffu, mbar_wait(bar(LPART_FREE + it % 3), (it / 3 - 1) & 1, abort_flag));
       float m_mine = -CUDART_INF_F, l = 0.f;  // the exponent offset this thread used last, its partial row sum
       // tile t goes to warpgroup t mod 3, which is also its S buffer; n_done counts this
@@ -936,30 +956,33 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           for (int i = 0; i < kKeys; ++i)
             if (!((cm[i >> 5] >> (i & 31)) & 1u)) sv[i] = 0xff800000u;  // -inf: weight exactly 0
         }
+        // The row's exponent offset: the decision of the previous tile, moved only when this tile's maximum exceeds it by more
+        // than 2^8 (always for the first finite maximum).  It is asked for here and looked at behind the maximum.
+        const uint32_t decision = decisions + 8u * (uint32_t)r;
+        float m_prev;
+        int decided;
+        ld_decision(decision, m_prev, decided);
         float mx4[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};  // independent chains
 #pragma unroll
         for (int i = 0; i < kKeys / 2; ++i)
           mx4[i & 3] = max3(mx4[i & 3], __uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1]));
         const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-
-        // the row's exponent offset: the decision of the previous tile, moved only when this tile's
-        // maximum exceeds it by more than 2^8 (always for the first finite maximum)
-        float m_prev = -CUDART_INF_F;
         if (wq == 0 && lane == 0) TSD_TR(11, Gj);
-        if (Gj > 0) {
-          // also for the first tile of an item, which takes nothing from the previous item: its
-          // write below must not overtake that item's last read of the same word
-          ok = ok && mbar_wait(bar(DEC + 4 * ((Gj - 1) & 3) + wq), ((Gj - 1) >> 2) & 1, abort_flag);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-          if (j > 0) m_prev = mref[r];
+        // (The first tile of an item waits too, although it takes nothing from the previous item: its decision must not be
+        // overtaken by that item's last one.)
+        for (uint32_t polls = 0; !__all_sync(0xffffffffu, decided == Gj); ++polls) {
+          if (polls == kSpinLimit) *abort_flag = 1u;
+          if ((polls & 255u) == 255u && *abort_flag) ok = false;
+          if (!__all_sync(0xffffffffu, ok)) break;
+          ld_decision(decision, m_prev, decided);
         }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (j == 0) m_prev = -CUDART_INF_F;
         const float m_new = fmaxf(m_prev, mx * c);
         const bool grow = m_new > m_prev + 8.f;
         const float m_use = grow ? m_new : m_prev;
-        mref[r] = m_use;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(DEC + 4 * (Gj & 3) + wq));
+        st_decision(decision, m_use, Gj + 1);
         if (wq == 0 && lane == 0) TSD_TR(12, Gj);
         const float alpha = grow ? ex2f(m_prev - m_new) : 1.f;  // what O has to be multiplied by
         if (m_mine != m_use) {
@@ -996,7 +1019,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
-          rescale_o_row<D>(t_lane + C::kO, alpha);
+          rescale_o_row<D>(t_lane + C::kO + (uint32_t)(D * (it % C::kNO)), alpha);
         }
         // P (bf16 pairs) into P buffer pb, free once the P V of tile t-2 has completed:
         // column i = keys 2i (low half), 2i+1
@@ -1130,7 +1153,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     for (int it = 0; it < (shared ? 0 : n_run) && ok; ++it) {
       int s, h, qt;
       item_coords(it, s, h, qt);
-      const int T = item_T[it], Gl = G + T - 1;
       if (tid == kFirstEpilogueWarp * 32) TSD_TR(5, 255 - it);
       ok = mbar_wait(bar(LPART + it % 3), (it / 3) & 1, abort_flag, 200);
       ok = __all_sync(0xffffffffu, ok);
@@ -1152,9 +1174,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         mbar_arrive(bar(OS_FREE));
       }
       ok = mbar_wait(bar(OS_FREE), it & 1, abort_flag);
-      // the softmax warps wrote the last P after the P V two tiles earlier had completed, so this
-      // barrier is at most one phase behind the one waited for
-      ok = ok && mbar_wait(bar(PV_DONE + (Gl & 3)), (Gl >> 2) & 1, abort_flag);
+      // The softmax warps wrote the last P after the P V two tiles earlier had completed, so with one O buffer the last tile's barrier
+      // is at most one phase behind the one waited for.  With two the P V of the next item may be further.
+      const int ob = it % C::kNO, last = G + item_T[it] - 1;
+      ok = ok && (C::kNO == 2 ? mbar_wait(bar(O_FULL + ob), (it / C::kNO) & 1, abort_flag)
+                              : mbar_wait(bar(PV_DONE + (last & 3)), (last >> 2) & 1, abort_flag));
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
@@ -1165,12 +1189,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 #pragma unroll
       for (int q4 = 0; q4 < D / 32; ++q4) {
         uint32_t ov[32];
-        TSD_TMEM_LD32(ov, 0, t_lane + C::kO + q4 * 32);
+        TSD_TMEM_LD32(ov, 0, t_lane + C::kO + (uint32_t)(D * ob) + q4 * 32);
         tmem_wait_ld();
         if (q4 == D / 32 - 1) {
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar(O_FREE));
+          if (lane == 0) mbar_arrive(bar(O_FREE + ob));
           if (tid == kFirstEpilogueWarp * 32) TSD_TR(2, 255 - it);
         }
         const uint32_t row_base = base + kOffO + (q4 >> 1) * kSub + (uint32_t)r * 128u;
@@ -1204,7 +1228,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         __syncwarp();
         if (!ok) break;
       }
-      G += T;
+      G += item_T[it];
     }
     // the staging buffer must outlive the last store's reads
     if (warp == kFirstEpilogueWarp && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -1401,7 +1425,7 @@ static int launch_tc(const AttnArgs& a) {
   }
   const MaskDims md = mask_dims(L);
   const int64_t n_items = (int64_t)L.batch * L.n_q_heads * md.n_qt;
-  if (!ok || n_items > 0x7fffffffLL / 4) return launch_attention_simt(a);  // strides the tensor maps cannot express
+  if (!ok || n_items > 0x7fffffffLL / 4 || md.bytes / 4 > 0xffffffffu) return launch_attention_simt(a);  // strides the tensor maps cannot express
   const int dev = current_device();
   if (dev < 0) return cuda_fail(cudaErrorInvalidDevice, "cudaGetDevice");
   const cudaError_t attr_err = allow_smem<D>(dev);
@@ -1411,7 +1435,7 @@ static int launch_tc(const AttnArgs& a) {
   p.lse = a.lse;
   p.status = a.status;
   p.S = L.batch; p.B = L.n_branches; p.R = L.rows_per_branch; p.Nc = L.n_cache; p.N = N;
-  p.Hq = L.n_q_heads; p.group = L.n_q_heads / L.n_kv_heads;
+  p.Hq = L.n_q_heads; p.Hkv = L.n_kv_heads; p.group = L.n_q_heads / L.n_kv_heads;
   p.recs_off = md.recs_off; p.n_qt = md.n_qt; p.rec_words = md.rec_words;
   p.n_items = (int)n_items;
   p.scale_log2e = D == 64 ? (float)(a.sm_scale * kLog2eExact * kSumsShrink) : a.sm_scale * kLog2e;

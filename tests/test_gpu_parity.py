@@ -333,7 +333,8 @@ def test_attention_head_dim_64_is_as_accurate_as_on_cuda_cores(S, Bn, R, Nc, sca
     assert tensor[0] <= 1.001 * cuda[0] and tensor[1] <= 1.1 * cuda[1], (tensor, cuda)
 
 
-@pytest.mark.parametrize("S,Bn,Nc,d", [(300, 2, 0, 128), (300, 2, 0, 64), (160, 2, 64, 128), (200, 4, 30, 64), (700, 2, 0, 128), (400, 1, 170, 128), (400, 1, 170, 64)])
+@pytest.mark.parametrize("S,Bn,Nc,d", [(300, 2, 0, 128), (300, 2, 0, 64), (160, 2, 64, 128), (200, 4, 30, 64), (700, 2, 0, 128), (400, 1, 170, 128), (400, 1, 170, 64),
+                                       (900, 2, 0, 64), (500, 4, 250, 64)])  # 64-wide heads: two O buffers in turn
 def test_attention_many_items_of_few_key_tiles(S, Bn, Nc, d):
     """Blocks that walk several work items of one or two key tiles: fewer than there are softmax warpgroups, so that
     some warpgroups pass an item without a tile of it while others are still at the one before."""
