@@ -31,6 +31,7 @@ namespace tsd {
 
 constexpr int kTopkUnroll = 4;            // chunks per thread per batch
 constexpr int kTopkSegChunks = 32768;     // chunks per segment at most (batch maxima: 32 KB of smem)
+constexpr int kTopkSmallChunks = 15360;   // chunks per row at most with 160 threads (15 KB of smem)
 constexpr int kMaxSegments = 32;
 constexpr int kMaxCluster = 8;            // blocks of a cluster at most (the portable size)
 constexpr int kPoolCap = 64;              // candidate pool of a block (entries)
@@ -258,7 +259,7 @@ struct Unpack<__nv_bfloat16> {
 };
 
 // grid.x = n_rows * n_seg; block = THREADS (256 when many blocks share an SM; 384 or 512 when there are so
-// few rows that two or three blocks have to keep the SM busy: more warps per row).
+// few rows that two or three blocks have to keep the SM busy: more warps per row; 160 where that lets all rows run at once).
 template <typename T, int K, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, int k, int n_seg,
@@ -268,7 +269,7 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   constexpr int E_ = Unpack<T>::kElems;
   constexpr int kTopkThreads = THREADS, kTopkWarps = THREADS / 32;
   constexpr int kTopkBatch = THREADS * kTopkUnroll;        // chunks per block per batch
-  constexpr int kTopkMaxIter = (kTopkSegChunks + kTopkBatch - 1) / kTopkBatch;  // batches per segment
+  constexpr int kTopkMaxIter = ((THREADS == 160 ? kTopkSmallChunks : kTopkSegChunks) + kTopkBatch - 1) / kTopkBatch;  // batches per segment
   __shared__ float s_bmax[kTopkMaxIter][kTopkThreads];  // per-thread batch maxima
   __shared__ __align__(16) float s_wmax[kTopkWarps];  // per-warp maxima
   __shared__ float s_wsum[kTopkWarps];                // per-warp sums on the block's exponent base
@@ -612,6 +613,12 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
   // 384 17.9, with 256 18.8; 444 x 126464 25.0 / 23.5 / 24.4; 960 x 126464 50.2 / 48.2 / 46.0.
   const int64_t units = n_rows * p.n_seg;
   p.threads = units <= 2 * kPlanSms ? 512 : (units <= 3 * kPlanSms ? 384 : 256);
+  // Long rows, a few more than 256 threads per row leave room for at one time, would be finished by a second wave of few blocks.
+  // fp32: 160 threads, of which 7 blocks run per SM, up to 1036 rows (of 50257, with 256 threads and with 160: 800 rows 37.0 and 30.7 us, 1024 rows
+  // 42.7 and 37.2, 1100 rows 43.8 and 47.2; of 32000: 800 rows 24.2 and 22.3).  bf16: 384, whose two waves are more even (of 126464, with
+  // 256 and 384: 640 rows 37.1 and 35.6, 740 rows 40.7 and 36.7, 800 rows 41.6 and 42.2; of 152064: 740 rows 45.8 and 41.4).
+  if (elems_per_chunk == 4 && units > 5 * kPlanSms && units <= 7 * kPlanSms && p.K <= 4 && chunks > 4096 && chunks <= kTopkSmallChunks) p.threads = 160;
+  if (elems_per_chunk == 8 && units > 4 * kPlanSms && units <= 5 * kPlanSms && chunks > 8192) p.threads = 384;
   // Rows that even 256 threads walk in one batch: with 512 threads 256 x 4096 fp32 takes 4.6 us and with 256 4.3, bf16 4.7 and 4.4,
   // 256 x 8192 bf16 4.8 and 4.6, 296 x 8000 bf16 5.2 and 4.9; 128 x 8000 and fewer rows the same (4.3).  128 x 16000: 5.0 and 5.8.
   if (chunks <= 1024) p.threads = 256;
@@ -634,6 +641,8 @@ static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   unsigned* tickets = reinterpret_cast<unsigned*>(static_cast<char*>(ws) + p.ticket_off);
   auto kernel = p.threads == 512 ? confidence_topk_kernel<T, K, 512>
               : p.threads == 384 ? confidence_topk_kernel<T, K, 384> : confidence_topk_kernel<T, K, 256>;
+  // (a block ranks its warps' maxima: it needs as many warps as candidates)
+  if constexpr (K <= 4 && sizeof(T) == 4) if (p.threads == 160) kernel = confidence_topk_kernel<T, K, 160>;
   return launch_clusters(p.n_seg <= kMaxCluster ? p.n_seg : 1, kernel, (unsigned)((a.n_rows + a.concurrent) * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
                 a.row_stride, a.k, p.n_seg, p.chunks_per_seg, a.conf, a.topk_idx, a.topk_prob, a.lse, partials, tickets,
                 p.prefetch, a.launch_next, a.concurrent ? (int)a.n_rows : 0);

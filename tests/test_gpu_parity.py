@@ -431,6 +431,16 @@ def test_topk_at_the_borders_of_its_plans(n, V):
     _check_topk(x, 3, rows=sorted({0, min(1, n - 1), n // 2, max(n - 2, 0), n - 1}))
 
 
+@pytest.mark.parametrize("dtype,n,V,k", [(torch.float32, 740, 17000, 3), (torch.float32, 741, 16388, 4), (torch.float32, 1036, 61441, 1),
+                                         (torch.float32, 1036, 61444, 2), (torch.float32, 1037, 17001, 3), (torch.float32, 900, 20000, 5),
+                                         (torch.bfloat16, 593, 65544, 3), (torch.bfloat16, 740, 65543, 8), (torch.bfloat16, 741, 65600, 2)])
+def test_topk_rows_of_two_uneven_waves(dtype, n, V, k):
+    # either side of the row counts, row lengths and candidates at which 160 (fp32) and 384 threads (bf16) are taken
+    g = torch.Generator(device=DEV).manual_seed(n)
+    x = (torch.randn((n, (V + 7) // 8 * 8), generator=g, device=DEV) * 3).to(dtype)[:, :V]
+    _check_topk(x, k, rows=sorted({0, n // 2, n - 2, n - 1}))
+
+
 @pytest.mark.parametrize("seed", range(10))
 def test_topk_random_rows_vocab_k_and_dtype(seed):
     # sizes drawn at random: one value per row up to a wide vocabulary, one row up to several waves of
