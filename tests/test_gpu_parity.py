@@ -441,6 +441,19 @@ def test_topk_rows_of_two_uneven_waves(dtype, n, V, k):
     _check_topk(x, k, rows=sorted({0, n // 2, n - 2, n - 1}))
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,V,pitch,shift", [(3, 40008, 40016, 0), (3, 40008, 40016, 16), (40, 70021, 70032, 0), (200, 50008, 50016, 0), (200, 50008, 50008, 0),
+                                             (300, 16389, 16400, 0), (300, 16389, 16400, 16), (2, 24, 32, 0), (500, 4104, 4112, 0)])
+def test_topk_loads_of_32_and_16_bytes(dtype, n, V, pitch, shift):
+    # rows that begin on 32 bytes and rows that do not, odd numbers of 16-byte chunks, segments, tails behind the last chunk
+    g = torch.Generator(device=DEV).manual_seed(V + shift)
+    buf = torch.full((n * pitch + 16,), float("inf"), dtype=dtype, device=DEV)      # what lies behind a row must not be read into it
+    first = shift // buf.element_size()                                            # `shift` in bytes
+    x = buf[first:first + n * pitch].view(n, pitch)[:, :V]
+    x.copy_(torch.randn((n, V), generator=g, device=DEV) * 3)
+    _check_topk(x, 4, rows=sorted({0, n // 2, n - 1}))
+
+
 @pytest.mark.parametrize("seed", range(10))
 def test_topk_random_rows_vocab_k_and_dtype(seed):
     # sizes drawn at random: one value per row up to a wide vocabulary, one row up to several waves of
