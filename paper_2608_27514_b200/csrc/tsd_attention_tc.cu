@@ -1153,6 +1153,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     for (int it = 0; it < (shared ? 0 : n_run) && ok; ++it) {
       int s, h, qt;
       item_coords(it, s, h, qt);
+      const int T = item_T[it], last = G + T - 1;
       if (tid == kFirstEpilogueWarp * 32) TSD_TR(5, 255 - it);
       ok = mbar_wait(bar(LPART + it % 3), (it / 3) & 1, abort_flag, 200);
       ok = __all_sync(0xffffffffu, ok);
@@ -1176,7 +1177,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       ok = mbar_wait(bar(OS_FREE), it & 1, abort_flag);
       // The softmax warps wrote the last P after the P V two tiles earlier had completed, so with one O buffer the last tile's barrier
       // is at most one phase behind the one waited for.  With two the P V of the next item may be further.
-      const int ob = it % C::kNO, last = G + item_T[it] - 1;
+      const int ob = it % C::kNO;
       ok = ok && (C::kNO == 2 ? mbar_wait(bar(O_FULL + ob), (it / C::kNO) & 1, abort_flag)
                               : mbar_wait(bar(PV_DONE + (last & 3)), (last >> 2) & 1, abort_flag));
       ok = __all_sync(0xffffffffu, ok);
@@ -1228,7 +1229,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         __syncwarp();
         if (!ok) break;
       }
-      G += item_T[it];
+      G += T;
     }
     // the staging buffer must outlive the last store's reads
     if (warp == kFirstEpilogueWarp && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
