@@ -671,11 +671,14 @@ static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   unsigned* tickets = reinterpret_cast<unsigned*>(static_cast<char*>(ws) + p.ticket_off);
   // bf16: 32-byte loads where every row (and, as segments are of whole pairs of chunks, every segment) begins on 32 bytes.  Decided for
   // all rows of a call alike: the order of a row's sum follows, and equal rows have to get equal results wherever they stand.
-  // Measured with 16- and 32-byte loads, 126464: 128 rows 12.2 and 11.6 us, 256 rows 17.3 and 16.7, 1024 rows 47.0 and 46.3, 16384 rows 648 and
-  // 626; 32 rows of 152064 6.2 and 5.9.  fp32 has half the arithmetic per byte and gains nothing (416 x 50257: 18.3 and 19.1).
+  // For rows in segments and for many rows: with 16- and 32-byte loads, 32 rows of 152064 6.25 and 5.93 us, 128 rows of 126464 12.2 and 11.6, 16384
+  // rows 648 and 626.  In between the pass alone gains too (320 rows 22.9 and 22.5, 1024 rows 47.0 and 46.3), but behind an attention
+  // kernel it loses (16 us of attention and 320 rows: 39.5 and 40.3; a joint pass of 1280 rows 110.4 and 111.2); the cause has not been found.
+  // fp32 has half the arithmetic per byte and gains nothing (416 x 50257: 18.3 and 19.1).
   auto kernel = pick_kernel<T, K, false>(p.threads);
   if constexpr (sizeof(T) == 2)
-    if (a.row_stride % 16 == 0 && reinterpret_cast<uintptr_t>(a.logits) % 32 == 0) kernel = pick_kernel<T, K, true>(p.threads);
+    if ((p.n_seg > 1 || a.n_rows >= 2048) && a.row_stride % 16 == 0 && reinterpret_cast<uintptr_t>(a.logits) % 32 == 0)
+      kernel = pick_kernel<T, K, true>(p.threads);
   return launch_clusters(p.n_seg <= kMaxCluster ? p.n_seg : 1, kernel, (unsigned)((a.n_rows + a.concurrent) * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
                 a.row_stride, a.k, p.n_seg, p.chunks_per_seg, a.conf, a.topk_idx, a.topk_prob, a.lse, partials, tickets,
                 p.prefetch, a.launch_next, a.concurrent ? (int)a.n_rows : 0);

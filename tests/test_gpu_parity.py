@@ -443,7 +443,7 @@ def test_topk_rows_of_two_uneven_waves(dtype, n, V, k):
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("n,V,pitch,shift", [(3, 40008, 40016, 0), (3, 40008, 40016, 16), (40, 70021, 70032, 0), (200, 50008, 50016, 0), (200, 50008, 50008, 0),
-                                             (300, 16389, 16400, 0), (300, 16389, 16400, 16), (2, 24, 32, 0), (500, 4104, 4112, 0)])
+                                             (300, 16389, 16400, 0), (300, 16389, 16400, 16), (2, 24, 32, 0), (2047, 4104, 4112, 0), (2048, 4104, 4112, 0), (2048, 4104, 4112, 16)])
 def test_topk_loads_of_32_and_16_bytes(dtype, n, V, pitch, shift):
     # rows that begin on 32 bytes and rows that do not, odd numbers of 16-byte chunks, segments, tails behind the last chunk
     g = torch.Generator(device=DEV).manual_seed(V + shift)
