@@ -22,7 +22,7 @@
 //               memory, fp32 accumulation in tensor memory.
 // All rows share one O accumulator, so the warpgroups agree on the exponent offset of a row
 // through a chain of decisions in tile order: the thread that owns row r in tile t waits for the
-// decision of tile t-1 (a word of shared memory per row that holds the offset and the tile), keeps that
+// decision of tile t-1 (a 64-bit word of shared memory per row that holds the offset and the tile), keeps that
 // offset unless the tile's maximum exceeds it by more than 2^8, publishes its decision and only
 // then starts on the exponentials.  The chain is short; the expensive part of the tiles overlaps.
 // A thread that moves the offset rescales the row of O before it publishes P (the P V of its tile
@@ -439,17 +439,20 @@ __device__ __forceinline__ float row_lse(const TcParams& p, float m, float l) {
   return (m + log2f(l)) * kLn2;
 }
 
-// A row's exponent offset and the count of tiles that have decided on it, in one word of shared memory: written by the thread that owns
-// the row in one tile, read by the one that owns it in the next.  (A barrier per warp with the offset beside it cost a test
-// of the barrier, a vote, the load and an arrival per tile, one behind the other: 512 items of 64-wide heads 65.3 us, with
-// the word 62.4, and with O in two buffers 59.5.)
+// A row's exponent offset and the count of tiles that have decided on it, in one 8-byte word of shared memory: written by the thread that
+// owns the row in one tile, read by the one that owns it in the next, which takes the offset as valid because the count beside it is.
+// One 64-bit access promises that; a vector of two 32-bit ones is two accesses in no stated order.
+// (A barrier per warp with the offset beside it cost a test of the barrier, a vote, the load and an arrival per tile, one behind
+// the other: 512 items of 64-wide heads 65.3 us, with the word 62.4, and with O in two buffers 59.5.)
 __device__ __forceinline__ void st_decision(uint32_t addr, float m, int count) {
-  asm volatile("st.volatile.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(__float_as_uint(m)), "r"(count) : "memory");
+  asm volatile("st.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(addr), "l"(pack2(__float_as_uint(m), (uint32_t)count)) : "memory");
 }
 __device__ __forceinline__ void ld_decision(uint32_t addr, float& m, int& count) {
-  uint32_t bits;
-  asm volatile("ld.volatile.shared.v2.b32 {%0, %1}, [%2];" : "=r"(bits), "=r"(count) : "r"(addr));
-  m = __uint_as_float(bits);
+  uint64_t word;
+  asm volatile("ld.relaxed.cta.shared::cta.b64 %0, [%1];" : "=l"(word) : "r"(addr) : "memory");
+  float count_bits;
+  unpack2(word, m, count_bits);
+  count = __float_as_int(count_bits);
 }
 
 // Rarely executed pieces of the softmax warps, kept out of line so that the loop over the key

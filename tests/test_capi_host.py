@@ -29,6 +29,16 @@ def test_exports_match_header(lib):
         assert hasattr(lib, name), name
 
 
+def test_a_decision_word_is_one_access():
+    # the attention kernel's softmax warps take a row's exponent offset as valid because the count beside it is, with no barrier in
+    # between: only a scalar 64-bit access hands both over together, a vector access is several in no stated order
+    src = open(os.path.join(ROOT, "paper_2608_27514_b200", "csrc", "tsd_attention_tc.cu")).read()
+    for name in ("st_decision", "ld_decision"):
+        body = re.search(r"void %s\(.*?\n}" % name, src, re.S).group(0)
+        ops = re.findall(r'"(?:st|ld)\.([a-z0-9_.:]*)', body)
+        assert len(ops) == 1 and re.fullmatch(r"(relaxed\.cta|volatile)\.shared(::cta)?\.b64", ops[0]), ops
+
+
 def test_strerror_and_status(lib):
     assert B.strerror(0) == "ok"
     assert "argument" in B.strerror(B.TSD_ERR_INVALID_ARG)
