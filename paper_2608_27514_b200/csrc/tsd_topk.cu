@@ -34,6 +34,8 @@ constexpr int kTopkSegChunks = 32768;     // chunks per segment at most (batch m
 constexpr int kTopkSmallChunks = 15360;   // chunks per row at most with 160 threads (15 KB of smem)
 constexpr int kMaxSegments = 32;
 constexpr int kMaxCluster = 8;            // blocks of a cluster at most (the portable size)
+// How a thread's chunks lie and are read: four single ones, or two pairs of neighbours in one load each or in two.
+enum { kSingle = 0, kPairs, kHalves };
 constexpr int kPoolCap = 64;              // candidate pool of a block (entries)
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -51,6 +53,15 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
   uint4 r;
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+  return r;
+}
+
+// One chunk of a pair that does not lie on 32 bytes.  Each of the pair's two loads takes half of every sector, so the second is to find
+// them in L1: past L1 they are fetched twice (4096 rows of 126464 that begin 16 bytes behind a multiple of 32: 194 us, so 167-177; 200 rows
+// 17.0 and 15.8).
+__device__ __forceinline__ uint4 ld_half(const uint4* p) {
+  uint4 r;
+  asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
   return r;
 }
 
@@ -266,7 +277,7 @@ struct Unpack<__nv_bfloat16> {
 
 // grid.x = n_rows * n_seg; block = THREADS (256 when many blocks share an SM; 384 or 512 when there are so
 // few rows that two or three blocks have to keep the SM busy: more warps per row; 160 where that lets all rows run at once).
-template <typename T, int K, int THREADS, bool WIDE>
+template <typename T, int K, int THREADS, int LOADS>
 __global__ void __launch_bounds__(THREADS)
 confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, int k, int n_seg,
                        int chunks_per_seg, float* __restrict__ conf, int32_t* __restrict__ topk_idx,
@@ -313,13 +324,14 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
   // ---- phase 1: stream.  Two register buffers: the loads of batch it+1 are in flight while
   // batch it is processed, so a block overlaps memory latency with its own arithmetic.
   float m = -CUDART_INF_F, e = 0.f, s = 0.f;
-  // chunk u of thread t in batch `it`
+  // Chunk u of thread t in batch `it`: single chunks, or pairs of them.  Which it is, and with it the order of the row's sum, follows from
+  // the plan alone, never from an address: the same values give the same bits wherever they lie.
   auto chunk = [&](int it, int t, int u) {
-    return c0 + it * kTopkBatch + (WIDE ? 2 * t + (u & 1) + (u >> 1) * 2 * kTopkThreads : t + u * kTopkThreads);
+    return c0 + it * kTopkBatch + (LOADS != kSingle ? 2 * t + (u & 1) + (u >> 1) * 2 * kTopkThreads : t + u * kTopkThreads);
   };
   const uint4 neg_inf = make_uint4(Unpack<T>::kNegInfWord, Unpack<T>::kNegInfWord, Unpack<T>::kNegInfWord, Unpack<T>::kNegInfWord);
   auto load_batch = [&](uint4 (&buf)[kTopkUnroll], int it) {  // past the segment: -inf adds nothing and is never a candidate
-    if constexpr (WIDE) {
+    if constexpr (LOADS == kPairs) {
 #pragma unroll
       for (int u = 0; u < kTopkUnroll; u += 2) {
         const int c = chunk(it, tid, u);
@@ -334,7 +346,7 @@ confidence_topk_kernel(const T* __restrict__ logits, int vocab, int64_t row_stri
 #pragma unroll
       for (int u = 0; u < kTopkUnroll; ++u) {
         const int c = chunk(it, tid, u);
-        buf[u] = c < c1 ? ld_stream(rowv + c) : neg_inf;
+        buf[u] = c < c1 ? (LOADS == kHalves ? ld_half(rowv + c) : ld_stream(rowv + c)) : neg_inf;
       }
     }
   };
@@ -655,13 +667,17 @@ static TopkPlan topk_plan(int64_t n_rows, int vocab, int k, int elems_per_chunk)
   return p;
 }
 
-template <typename T, int K, bool WIDE>
-static auto pick_kernel(int threads) {
-  auto kernel = threads == 512 ? confidence_topk_kernel<T, K, 512, WIDE>
-              : threads == 384 ? confidence_topk_kernel<T, K, 384, WIDE> : confidence_topk_kernel<T, K, 256, WIDE>;
+template <typename T, int K>
+static auto pick_kernel(int threads, int loads) {
+  auto kernel = threads == 512 ? confidence_topk_kernel<T, K, 512, kSingle>
+              : threads == 384 ? confidence_topk_kernel<T, K, 384, kSingle> : confidence_topk_kernel<T, K, 256, kSingle>;
   // (a block ranks its warps' maxima: it needs as many warps as candidates)
   if constexpr (K <= 4 && sizeof(T) == 4)
-    if (threads == 160) kernel = confidence_topk_kernel<T, K, 160, WIDE>;
+    if (threads == 160) kernel = confidence_topk_kernel<T, K, 160, kSingle>;
+  if constexpr (sizeof(T) == 2) {  // (rows in segments get 512 or 256 threads, 2048 rows and more 256)
+    if (loads == kPairs) kernel = threads == 512 ? confidence_topk_kernel<T, K, 512, kPairs> : confidence_topk_kernel<T, K, 256, kPairs>;
+    if (loads == kHalves) kernel = threads == 512 ? confidence_topk_kernel<T, K, 512, kHalves> : confidence_topk_kernel<T, K, 256, kHalves>;
+  }
   return kernel;
 }
 
@@ -669,16 +685,15 @@ template <typename T, int K>
 static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   Partial<K>* partials = reinterpret_cast<Partial<K>*>(ws);
   unsigned* tickets = reinterpret_cast<unsigned*>(static_cast<char*>(ws) + p.ticket_off);
-  // bf16: 32-byte loads where every row (and, as segments are of whole pairs of chunks, every segment) begins on 32 bytes.  Decided for
-  // all rows of a call alike: the order of a row's sum follows, and equal rows have to get equal results wherever they stand.
+  // bf16: chunks in pairs, read 32 bytes at a time where every row (and, as segments are of whole pairs, every segment) begins on 32 bytes.
   // For rows in segments and for many rows: with 16- and 32-byte loads, 32 rows of 152064 6.25 and 5.93 us, 128 rows of 126464 12.2 and 11.6, 16384
   // rows 648 and 626.  In between the pass alone gains too (320 rows 22.9 and 22.5, 1024 rows 47.0 and 46.3), but behind an attention
   // kernel it loses (16 us of attention and 320 rows: 39.5 and 40.3; a joint pass of 1280 rows 110.4 and 111.2); the cause has not been found.
   // fp32 has half the arithmetic per byte and gains nothing (416 x 50257: 18.3 and 19.1).
-  auto kernel = pick_kernel<T, K, false>(p.threads);
-  if constexpr (sizeof(T) == 2)
-    if ((p.n_seg > 1 || a.n_rows >= 2048) && a.row_stride % 16 == 0 && reinterpret_cast<uintptr_t>(a.logits) % 32 == 0)
-      kernel = pick_kernel<T, K, true>(p.threads);
+  int loads = kSingle;
+  if (sizeof(T) == 2 && (p.n_seg > 1 || a.n_rows >= 2048))
+    loads = a.row_stride % 16 == 0 && reinterpret_cast<uintptr_t>(a.logits) % 32 == 0 ? kPairs : kHalves;
+  auto kernel = pick_kernel<T, K>(p.threads, loads);
   return launch_clusters(p.n_seg <= kMaxCluster ? p.n_seg : 1, kernel, (unsigned)((a.n_rows + a.concurrent) * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,
                 a.row_stride, a.k, p.n_seg, p.chunks_per_seg, a.conf, a.topk_idx, a.topk_prob, a.lse, partials, tickets,
                 p.prefetch, a.launch_next, a.concurrent ? (int)a.n_rows : 0);

@@ -454,6 +454,30 @@ def test_topk_loads_of_32_and_16_bytes(dtype, n, V, pitch, shift):
     _check_topk(x, 4, rows=sorted({0, n // 2, n - 1}))
 
 
+@pytest.mark.parametrize("n,V,k", [(3, 40128, 3), (3, 40136, 1), (1, 2097288, 4), (40, 70021, 2), (200, 50008, 5), (300, 16389, 3), (2048, 4104, 8), (2050, 4099, 4)])
+def test_topk_bits_do_not_depend_on_where_the_rows_lie(n, V, k):
+    # the same values at addresses and pitches that are multiples of 32 bytes and of 16 only: rows in segments (an odd number of chunks
+    # for each, rounded to whole pairs: 40128 = 8 x 627 chunks, 2097288 = 9 x 29129), whole rows, many rows, ragged tails
+    g = torch.Generator(device=DEV).manual_seed(V + n)
+    x = (torch.randn((n, V), generator=g, device=DEV) * 3).bfloat16()
+    rows = sorted({0, n // 2, n - 1})
+    want = oracle.confidence_topk(_np(x[torch.as_tensor(rows, device=DEV)]), k)
+    ws = torch.empty(max(16, B.tsd_confidence_topk_workspace_bytes(n, V, k)), dtype=torch.uint8, device=DEV)
+    seen = []
+    for pitch, first in (((V + 15) // 16 * 16, 0), ((V + 15) // 16 * 16, 8), ((V + 15) // 16 * 16 + 8, 0), ((V + 15) // 16 * 16 + 8, 8)):
+        buf = torch.full((n * pitch + 16,), float("inf"), dtype=torch.bfloat16, device=DEV)  # what lies beside a row must not be read into it
+        y = buf[first:first + n * pitch].view(n, pitch)[:, :V]
+        y.copy_(x)
+        out = [torch.empty(shape, dtype=t, device=DEV) for shape, t in (((n,), torch.float32), ((n, k), torch.int32), ((n, k), torch.float32), ((n,), torch.float32))]
+        B.tsd_confidence_topk(y, k, *out, ws)
+        seen.append(out)
+    conf, idx, prob, lse = (_np(t)[rows] for t in seen[0])
+    assert np.array_equal(idx, want[1])
+    assert np.abs(conf - want[0]).max() <= 1e-5 and np.abs(prob - want[2]).max() <= 1e-5 and np.abs(lse - want[3]).max() <= 1e-4
+    for other in seen[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(seen[0], other))
+
+
 @pytest.mark.parametrize("seed", range(10))
 def test_topk_random_rows_vocab_k_and_dtype(seed):
     # sizes drawn at random: one value per row up to a wide vocabulary, one row up to several waves of
