@@ -690,8 +690,10 @@ static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   // rows 648 and 626.  In between the pass alone gains too (320 rows 22.9 and 22.5, 1024 rows 47.0 and 46.3), but behind an attention
   // kernel it loses (16 us of attention and 320 rows: 39.5 and 40.3; a joint pass of 1280 rows 110.4 and 111.2); the cause has not been found.
   // fp32 has half the arithmetic per byte and gains nothing (416 x 50257: 18.3 and 19.1).
+  // Segments too short to give most threads a pair keep single chunks (8 segments under 512 threads, single and in pairs: 8 rows of 32000, 500
+  // chunks per segment, 5.10 and 5.37 us; of 36000, 564 chunks, 5.19 and 5.33; of 40000, 626, 5.27 and 5.30; 18 rows of 48000, 750, 5.71 and 5.54).
   int loads = kSingle;
-  if (sizeof(T) == 2 && (p.n_seg > 1 || a.n_rows >= 2048))
+  if (sizeof(T) == 2 && (p.n_seg > 1 ? 4 * p.chunks_per_seg > 5 * p.threads : a.n_rows >= 2048))
     loads = a.row_stride % 16 == 0 && reinterpret_cast<uintptr_t>(a.logits) % 32 == 0 ? kPairs : kHalves;
   auto kernel = pick_kernel<T, K>(p.threads, loads);
   return launch_clusters(p.n_seg <= kMaxCluster ? p.n_seg : 1, kernel, (unsigned)((a.n_rows + a.concurrent) * p.n_seg), p.threads, 0, a.stream, static_cast<const T*>(a.logits), a.vocab,

@@ -454,10 +454,11 @@ def test_topk_loads_of_32_and_16_bytes(dtype, n, V, pitch, shift):
     _check_topk(x, 4, rows=sorted({0, n // 2, n - 1}))
 
 
-@pytest.mark.parametrize("n,V,k", [(3, 40128, 3), (3, 40136, 1), (1, 2097288, 4), (40, 70021, 2), (200, 50008, 5), (300, 16389, 3), (2048, 4104, 8), (2050, 4099, 4)])
+@pytest.mark.parametrize("n,V,k", [(3, 41664, 3), (3, 41672, 1), (1, 2097288, 4), (40, 70021, 2), (200, 50008, 5), (300, 16389, 3), (2048, 4104, 8), (2050, 4099, 4),
+                                   (8, 40960, 3), (8, 41088, 3)])  # segments just too short for pairs (640 chunks, 512 threads), and just long enough
 def test_topk_bits_do_not_depend_on_where_the_rows_lie(n, V, k):
     # the same values at addresses and pitches that are multiples of 32 bytes and of 16 only: rows in segments (an odd number of chunks
-    # for each, rounded to whole pairs: 40128 = 8 x 627 chunks, 2097288 = 9 x 29129), whole rows, many rows, ragged tails
+    # for each, rounded to whole pairs: 41664 = 8 x 651 chunks, 2097288 = 9 x 29129), whole rows, many rows, ragged tails
     g = torch.Generator(device=DEV).manual_seed(V + n)
     x = (torch.randn((n, V), generator=g, device=DEV) * 3).bfloat16()
     rows = sorted({0, n // 2, n - 1})
