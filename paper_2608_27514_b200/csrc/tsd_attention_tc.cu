@@ -1448,10 +1448,6 @@ static int launch_tc(const AttnArgs& a) {
   p.unscale_lo = (float)(unscale - (double)p.unscale_hi);
   p.concurrent = a.concurrent;
   p.next_at_once = a.next_at_once;
-  // one block per SM, each walking its share of the items; more blocks only when a block's share
-  // would not fit the per-block item table
-  const int sms = std::max(device_facts().sms, 1);
-  int64_t grid = std::min<int64_t>(n_items, sms);
   p.cut = blocks_per_item<D>(L);
   p.out = static_cast<__nv_bfloat16*>(a.out);
   p.os_b = a.os_b; p.os_r = a.os_r; p.os_h = a.os_h;
@@ -1460,7 +1456,10 @@ static int launch_tc(const AttnArgs& a) {
                                     mq, mkc, mvc, mkd, mvd, mo, p);
     return e != cudaSuccess ? cuda_fail(e, "attention_tc_kernel") : TSD_OK;
   }
-  grid = std::max<int64_t>(grid, (n_items + kMaxItems - 1) / kMaxItems);
+  // One block per SM, each walking its share of the items.  Where a share would not fit the block's item table, whole rounds of blocks: with
+  // only as many blocks as the table asks for, the last few of them would run by themselves, for as long as all the others.
+  const int64_t sms = std::max(device_facts().sms, 1);
+  const int64_t grid = std::min(n_items, sms * ((n_items + sms * kMaxItems - 1) / (sms * kMaxItems)));
   cudaError_t e = launch(attention_tc_kernel<D, false>, (unsigned)grid, kTcThreads, TcSmem<D>::kBytes, a.stream, mq, mkc, mvc, mkd,
                          mvd, mo, p);
   if (e != cudaSuccess) return cuda_fail(e, "attention_tc_kernel");

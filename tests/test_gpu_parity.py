@@ -343,6 +343,31 @@ def test_attention_many_items_of_few_key_tiles(S, Bn, Nc, d):
     _check_attention(cfg, W.attention_inputs(cfg, DEV), 0, cache_lens=lens, seqs=[0, 1, S // 2, S - 2, S - 1])
 
 
+@pytest.mark.parametrize("d", [128, 64])
+def test_attention_more_items_than_one_block_per_sm_has_room_for(d):
+    # a block's table holds 256 items: just above that the launch takes a second round of blocks, which has to be a whole one
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    full = sms * 256 // 4
+    ms = []
+    for S in (full, full + 1):
+        cfg = W.small(W.CONFIGS["cfg2"], S=S, B=1, R=32, Nc=70, Hq=4, Hkv=1, d=d)
+        attn = W.attention_inputs(cfg, DEV)
+        lens = torch.tensor([(7 * s) % 71 for s in range(S)], dtype=torch.int32, device=DEV)
+        if S > full:
+            _check_attention(cfg, attn, 0, cache_lens=lens, seqs=[0, 1, S // 2, S - 2, S - 1])
+        step, _ = _run_attention(cfg, attn, 0, cache_lens=lens)
+        start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        times = []
+        for _ in range(5):
+            start.record()
+            step.attention(attn["q"], attn["k_cache"], attn["v_cache"], attn["k_draft"], attn["v_draft"], attn["sm_scale"])
+            end.record()
+            torch.cuda.synchronize()
+            times.append(start.elapsed_time(end))
+        ms.append(min(times))
+    assert ms[1] < 1.5 * ms[0], ms              # with one block left over it would be twice as long
+
+
 @pytest.mark.parametrize("S,Bn,R,Nc,Hq,Hkv,d,lens", [
     (1, 3, 32, 1500, 8, 4, 128, None),                  # 8 items in 8 parts, rows past the last branch
     (1, 6, 64, 1500, 4, 2, 128, [1499]),                # 12 items in 8 parts of 3 or 4 tiles
