@@ -1457,7 +1457,8 @@ static int launch_tc(const AttnArgs& a) {
     return e != cudaSuccess ? cuda_fail(e, "attention_tc_kernel") : TSD_OK;
   }
   // One block per SM, each walking its share of the items.  Where a share would not fit the block's item table, whole rounds of blocks: with
-  // only as many blocks as the table asks for, the last few of them would run by themselves, for as long as all the others.
+  // only as many blocks as the table asks for, the last few of them would run by themselves, for as long as all the others (37888 and 38144
+  // items of 8 tiles on 148 SMs: 1.56 and 2.71-2.83 ms; in whole rounds 1.56 and 1.59).
   const int64_t sms = std::max(device_facts().sms, 1);
   const int64_t grid = std::min(n_items, sms * ((n_items + sms * kMaxItems - 1) / (sms * kMaxItems)));
   cudaError_t e = launch(attention_tc_kernel<D, false>, (unsigned)grid, kTcThreads, TcSmem<D>::kBytes, a.stream, mq, mkc, mvc, mkd,

@@ -365,7 +365,7 @@ def test_attention_more_items_than_one_block_per_sm_has_room_for(d):
             torch.cuda.synchronize()
             times.append(start.elapsed_time(end))
         ms.append(min(times))
-    assert ms[1] < 1.5 * ms[0], ms              # with one block left over it would be twice as long
+    assert ms[1] < 1.25 * ms[0], ms             # with one block left over: 1.5 to 1.8
 
 
 @pytest.mark.parametrize("S,Bn,R,Nc,Hq,Hkv,d,lens", [
