@@ -172,11 +172,12 @@ int tsd_verify_attention(const tsd_layout* layout, const void* mask,
  * Every wait inside the attention kernel is bounded: a block whose wait runs out
  * ORs TSD_STATUS_TIMEOUT into the status word, stops issuing work and returns,
  * so the context stays usable and tsd_check_status() gives TSD_ERR_TIMEOUT.
- * This call launches one warp that runs that same bounded wait on a barrier
- * nothing will ever complete, with a limit of `poll_limit` polls (1..65536; a
- * few dozen microseconds at most), so that a caller, or a test, can see the
- * whole path work (kernel returns by itself, status word, decoding) without
- * making anything hang or fault.
+ * This call launches two warps that run those same bounded waits (on a barrier
+ * nothing will ever complete, and for a word another warp never writes; before
+ * that they hand such words to each other, which has to succeed), with a limit
+ * of `poll_limit` polls (1..65536; some milliseconds at most), so that a caller,
+ * or a test, can see the whole path work (kernel returns by itself, status
+ * word, decoding) without making anything hang or fault.
  *   status   device uint32, required: receives TSD_STATUS_TIMEOUT.
  * ------------------------------------------------------------------------- */
 int tsd_selftest_bounded_wait(uint32_t* status, uint32_t poll_limit, tsd_stream_t stream);

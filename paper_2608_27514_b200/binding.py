@@ -281,7 +281,7 @@ def tsd_gather_accepted_kv(accepted_node, rows_per_branch, k_draft, v_draft, k_o
 
 
 def tsd_selftest_bounded_wait(status, poll_limit=64, stream=None):
-    """Runs the library's bounded barrier wait on a barrier nothing completes; sets TSD_STATUS_TIMEOUT."""
+    """Runs the library's bounded device waits on what never comes; sets TSD_STATUS_TIMEOUT if each gives up as it should."""
     _check(lib().tsd_selftest_bounded_wait(_ptr(status), int(poll_limit), _stream(stream)),
            "tsd_selftest_bounded_wait")
 

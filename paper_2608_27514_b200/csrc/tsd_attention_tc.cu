@@ -42,7 +42,7 @@
 // its own.  Bound by the serial chain of one item otherwise: 28 items of 81 key tiles took 40.6 us on 28 SMs and take 18.7 on 112,
 // 56 items 41.6 -> 27.6, 16 items of 81 tiles 40.8 -> 18.2 (64-wide heads: 4 items of 34 tiles 24.3 -> 11.7).  A
 // kernel of its own, so that the loops of whole items keep their registers (in one kernel: 256 items 31.7 -> 36.4 us).
-// Every mbarrier wait is bounded: on expiry the block raises TSD_STATUS_TIMEOUT, stops issuing
+// Every wait, on an mbarrier or for a decision, is bounded: on expiry the block raises TSD_STATUS_TIMEOUT, stops issuing
 // work, waits (bounded) for its copies in flight, frees its tensor memory and returns.
 #include <cuda.h>
 #include <math_constants.h>
@@ -453,6 +453,20 @@ __device__ __forceinline__ void ld_decision(uint32_t addr, float& m, int& count)
   float count_bits;
   unpack2(word, m, count_bits);
   count = __float_as_int(count_bits);
+}
+// Waits, warp by warp, until `count` tiles have decided on every lane's row.  The caller has read the word once (m, decided).  Bounded as
+// mbar_wait is (it leaves within 256 polls behind the limit): false for the whole warp when the block is aborting.  (In this form the kernel
+// is what it was with the loop in place; leaving at the limit itself cost 128-wide heads 0.5-1 %.)
+__device__ __forceinline__ bool decision_wait(uint32_t addr, int count, float& m, int& decided, volatile uint32_t* abort_flag,
+                                              uint32_t limit = kSpinLimit) {
+  bool ok = true;
+  for (uint32_t polls = 0; !__all_sync(0xffffffffu, decided == count); ++polls) {
+    if (polls == limit) *abort_flag = 1u;
+    if ((polls & 255u) == 255u && *abort_flag) ok = false;
+    if (!__all_sync(0xffffffffu, ok)) break;
+    ld_decision(addr, m, decided);
+  }
+  return __all_sync(0xffffffffu, ok);
 }
 
 // Rarely executed pieces of the softmax warps, kept out of line so that the loop over the key
@@ -973,13 +987,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         if (wq == 0 && lane == 0) TSD_TR(11, Gj);
         // (The first tile of an item waits too, although it takes nothing from the previous item: its decision must not be
         // overtaken by that item's last one.)
-        for (uint32_t polls = 0; !__all_sync(0xffffffffu, decided == Gj); ++polls) {
-          if (polls == kSpinLimit) *abort_flag = 1u;
-          if ((polls & 255u) == 255u && *abort_flag) ok = false;
-          if (!__all_sync(0xffffffffu, ok)) break;
-          ld_decision(decision, m_prev, decided);
-        }
-        ok = __all_sync(0xffffffffu, ok);
+        ok = decision_wait(decision, Gj, m_prev, decided, abort_flag);
         if (!ok) break;
         if (j == 0) m_prev = -CUDART_INF_F;
         const float m_new = fmaxf(m_prev, mx * c);
@@ -1256,22 +1264,41 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   if (p.concurrent) grid_wait();
 }
 
-// The bounded wait of this file on a barrier that nothing ever completes: it gives up after
-// `poll_limit` polls, the block notes it and returns by itself, as a block of the attention kernel
-// does when one of its waits runs out.
+// The bounded waits of this file, for a decision that never comes and on a barrier that nothing ever completes: each gives up at
+// its limit, the block notes it and returns by itself, as a block of the attention kernel does when one of its waits
+// runs out.  Before that two warps hand decisions to each other in turn, and none of those waits may run out.  The time-out is
+// reported only if all of this went as it should.
 __global__ void bounded_wait_selftest_kernel(uint32_t* status, uint32_t poll_limit) {
-  __shared__ uint64_t bar_mem;
-  __shared__ uint32_t abort_word;
-  const uint32_t b = smem_u32(&bar_mem);
+  __shared__ uint64_t bar_mem, words[32];
+  __shared__ volatile uint32_t abort_word[2];
+  const uint32_t b = smem_u32(&bar_mem), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, word = smem_u32(&words[lane]);
   if (threadIdx.x == 0) {
-    abort_word = 0;
+    abort_word[0] = abort_word[1] = 0;
     mbar_init(b, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 0) st_decision(word, 0.f, 0);
   __syncthreads();
-  const bool ok = mbar_wait(b, 0, &abort_word, 0, poll_limit);
+  auto offset = [&](int count) { return (float)(count * 33 + (int)lane); };
+  constexpr int kTurns = 1000;
+  float m;
+  int decided;
+  bool handed = true;
+  for (int t = (int)warp; t < kTurns && handed; t += 2) {
+    ld_decision(word, m, decided);
+    handed = decision_wait(word, t, m, decided, &abort_word[1]) && (t == 0 || m == offset(t));
+    handed = __all_sync(0xffffffffu, handed);
+    st_decision(word, offset(t + 1), t + 1);
+  }
+  handed = __syncthreads_and(handed);
+  ld_decision(word, m, decided);
+  const bool came = decision_wait(word, kTurns + 1, m, decided, abort_word, poll_limit);
+  const bool noted = __syncthreads_and(abort_word[0] != 0);
+  if (threadIdx.x == 0) abort_word[0] = 0;
   __syncthreads();
-  if (threadIdx.x == 0 && (!ok || abort_word) && status) atomicOr(status, TSD_STATUS_TIMEOUT);
+  const bool done = mbar_wait(b, 0, abort_word, 0, poll_limit);
+  const bool all = __syncthreads_and(handed && !came && noted && !done && abort_word[0]);
+  if (threadIdx.x == 0 && all) atomicOr(status, TSD_STATUS_TIMEOUT);
 }
 
 // ------------------------------------------------------------------------------ host side
@@ -1479,7 +1506,7 @@ extern "C" int tsd_attention_trace_read(long long* dst) {
 
 extern "C" int tsd_selftest_bounded_wait(uint32_t* status, uint32_t poll_limit, tsd_stream_t stream) {
   if (!status || poll_limit < 1 || poll_limit > (1u << 16)) return TSD_ERR_INVALID_ARG;
-  tsd::bounded_wait_selftest_kernel<<<1, 32, 0, stream>>>(status, poll_limit);
+  tsd::bounded_wait_selftest_kernel<<<1, 64, 0, stream>>>(status, poll_limit);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return tsd::cuda_fail(e, "bounded_wait_selftest_kernel");
   return TSD_OK;

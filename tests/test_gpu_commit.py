@@ -256,6 +256,14 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable()
     assert B.tsd_check_status(step.status) == B.TSD_OK
 
 
+@pytest.mark.parametrize("poll_limit", [1, 255, 256, 257, 4096])
+def test_every_bounded_wait_gives_up_at_its_limit(poll_limit):
+    # the limit either side of the polls at which a wait also looks for another one's time-out
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    B.tsd_selftest_bounded_wait(status, poll_limit)
+    assert B.tsd_check_status(status) == B.TSD_ERR_TIMEOUT
+
+
 @pytest.mark.parametrize("S,Bn,R,k,width,depth,rule", [(1, 1, 32, 1, 1, 1, B.TSD_ACCEPT_EXACT), (3, 10, 32, 4, 3, 3, B.TSD_ACCEPT_TOP1),
                                                        (2, 7, 64, 3, 2, 3, B.TSD_ACCEPT_TOPK), (2, 9, 32, 5, 3, 2, B.TSD_ACCEPT_PROB),
                                                        (5, 4, 128, 8, 32, 4, B.TSD_ACCEPT_EXACT), (2, 256, 32, 3, 8, 40, B.TSD_ACCEPT_PROB)])
