@@ -7,8 +7,9 @@
 // draft tile only the (query branch, key branch) pairs whose bit is set are visible, everything
 // else gets weight 0.  Tiles of branches a query tile cannot see are never loaded.
 //
-// Tensor memory (all 512 columns): O (128 columns, fp32), Q of the current and of the next item
-// (2 x 64 columns, bf16 pairs), three S buffers (3 x 64) and two P buffers (2 x 32).
+// Tensor memory (all 512 columns at head_dim 128): O (128 columns, fp32), Q of the current and of the next item
+// (2 x 64 columns, bf16 pairs), three S buffers (3 x 64) and two P buffers (2 x 32).  At head_dim 64: two O (2 x 64),
+// Q in 2 x 32 columns, P in 2 x 64 (two parts).
 //   S = Q K^T : tcgen05.mma with A = Q from TENSOR MEMORY, B = K (K-major) from 128B-swizzled
 //               shared memory.  An MMA whose A operand comes from shared memory is limited by
 //               shared-memory bandwidth (4 KB of A + 2 KB of B per 128x64x16 step: 48 clocks
@@ -20,7 +21,7 @@
 //               block keeps the tensor pipe fed by itself.
 //   O += P V  : tcgen05.mma, A = P from tensor memory, B = V (head_dim contiguous) from shared
 //               memory, fp32 accumulation in tensor memory.
-// All rows share one O accumulator, so the warpgroups agree on the exponent offset of a row
+// The rows of an item share one O accumulator, so the warpgroups agree on the exponent offset of a row
 // through a chain of decisions in tile order: the thread that owns row r in tile t waits for the
 // decision of tile t-1 (a 64-bit word of shared memory per row that holds the offset and the tile), keeps that
 // offset unless the tile's maximum exceeds it by more than 2^8, publishes its decision and only
@@ -93,7 +94,7 @@ static_assert(kKeys == kKeyTile, "the mask blob lists tiles of this many keys");
 // of O and Q is free, so P is kept as the sum of two bf16 (high part, residual: 2^-17 relative) and P V issues
 // one MMA more per 16 keys: the outputs' error against fp64 is then that of fp32 weights up to bf16 roundings that fall the other
 // way (relative, 2-norm: 1.6594e-3 for either; over drawn sizes the two are apart by 2e-5 of the error at most).
-// (4 sequences x 16 branches x 32 rows, 32/8 heads, 1472 cached keys: 65.6 us; on CUDA cores, where this head
+// (4 sequences x 16 branches x 32 rows, 32/8 heads, 1472 cached keys: 60.2 us; on CUDA cores, where this head
 // size ran before: 5.96 ms.)
 template <int D>
 struct TcCols {

@@ -689,6 +689,9 @@ static cudaError_t run_plan(const TopkArgs& a, const TopkPlan& p, void* ws) {
   // For rows in segments and for many rows: with 16- and 32-byte loads, 32 rows of 152064 6.25 and 5.93 us, 128 rows of 126464 12.2 and 11.6, 16384
   // rows 648 and 626.  In between the pass alone gains too (320 rows 22.9 and 22.5, 1024 rows 47.0 and 46.3), but behind an attention
   // kernel it loses (16 us of attention and 320 rows: 39.5 and 40.3; a joint pass of 1280 rows 110.4 and 111.2); the cause has not been found.
+  // Rows in segments gain there (steps of 152064, single chunks and pairs: 96 rows and 96 items 26.1 and 25.6 us, 160 and 160 40.4 and 39.3, 192 and
+  // 192 41.6 and 40.5), except where a few run beside a short attention (32 items of 12 tiles: 32 rows 16.0 and 16.5, 64 rows 17.4 and 17.55).
+  // The rule does not look at the position, because a step has to give the bits of its single calls.
   // fp32 has half the arithmetic per byte and gains nothing (416 x 50257: 18.3 and 19.1).
   // Segments too short to give most threads a pair keep single chunks (8 segments under 512 threads, single and in pairs: 8 rows of 32000, 500
   // chunks per segment, 5.10 and 5.37 us; of 36000, 564 chunks, 5.19 and 5.33; of 40000, 626, 5.27 and 5.30; 18 rows of 48000, 750, 5.71 and 5.54).
