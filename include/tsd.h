@@ -175,9 +175,9 @@ int tsd_verify_attention(const tsd_layout* layout, const void* mask,
  * This call launches two warps that run those same bounded waits (on a barrier
  * nothing will ever complete, and for a word another warp never writes; before
  * that they hand such words to each other, which has to succeed), with a limit
- * of `poll_limit` polls (1..65536; some milliseconds at most), so that a caller,
- * or a test, can see the whole path work (kernel returns by itself, status
- * word, decoding) without making anything hang or fault.
+ * of `poll_limit` polls (1..65536, some 10 us each), so that a caller, or a
+ * test, can see the whole path work (kernel returns by itself, status word,
+ * decoding) without making anything hang or fault.
  *   status   device uint32, required: receives TSD_STATUS_TIMEOUT.
  * ------------------------------------------------------------------------- */
 int tsd_selftest_bounded_wait(uint32_t* status, uint32_t poll_limit, tsd_stream_t stream);

@@ -110,7 +110,10 @@ struct TcCols {
 // tiles in halves: 27.6 us, 40 tiles less than 41.6; 28 in quarters: 18.7, 60 tiles less than 40.6.  Two thirds of it is the way of the
 // columns between the SMs, ~20 bytes per clock and SM.  64 items of 14 tiles would gain nothing: 12.7 whole, 13.0 in halves.)
 constexpr int kMeetTiles = 7;
-constexpr uint32_t kSpinLimit = 1u << 21;
+constexpr uint32_t kSpinLimit = 1u << 21;      // polls of a barrier; each may suspend the warp for 4 us
+// Polls of a decision (0.09 us each) for one of a barrier: the warp that owes the decision may itself be in a barrier wait for its keys, and
+// whoever waits for it must not give up first.
+constexpr uint32_t kDecisionPolls = 64;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr double kLog2eExact = 1.4426950408889634;
@@ -459,7 +462,7 @@ __device__ __forceinline__ void ld_decision(uint32_t addr, float& m, int& count)
 // mbar_wait is (it leaves within 256 polls behind the limit): false for the whole warp when the block is aborting.  (In this form the kernel
 // is what it was with the loop in place; leaving at the limit itself cost 128-wide heads 0.5-1 %.)
 __device__ __forceinline__ bool decision_wait(uint32_t addr, int count, float& m, int& decided, volatile uint32_t* abort_flag,
-                                              uint32_t limit = kSpinLimit) {
+                                              uint32_t limit = kSpinLimit * kDecisionPolls) {
   bool ok = true;
   for (uint32_t polls = 0; !__all_sync(0xffffffffu, decided == count); ++polls) {
     if (polls == limit) *abort_flag = 1u;
@@ -1267,8 +1270,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
 // The bounded waits of this file, for a decision that never comes and on a barrier that nothing ever completes: each gives up at
 // its limit, the block notes it and returns by itself, as a block of the attention kernel does when one of its waits
-// runs out.  Before that two warps hand decisions to each other in turn, and none of those waits may run out.  The time-out is
-// reported only if all of this went as it should.
+// runs out.  Before that two warps hand decisions to each other in turn, and none of those waits may run out; and the wait for a decision has to
+// be the longer one.  The time-out is reported only if all of this went as it should.
 __global__ void bounded_wait_selftest_kernel(uint32_t* status, uint32_t poll_limit) {
   __shared__ uint64_t bar_mem, words[32];
   __shared__ volatile uint32_t abort_word[2];
@@ -1293,12 +1296,16 @@ __global__ void bounded_wait_selftest_kernel(uint32_t* status, uint32_t poll_lim
   }
   handed = __syncthreads_and(handed);
   ld_decision(word, m, decided);
-  const bool came = decision_wait(word, kTurns + 1, m, decided, abort_word, poll_limit);
+  const long long begin = clock64();
+  const bool came = decision_wait(word, kTurns + 1, m, decided, abort_word, poll_limit * kDecisionPolls);
+  const long long decision_clocks = clock64() - begin;
   const bool noted = __syncthreads_and(abort_word[0] != 0);
   if (threadIdx.x == 0) abort_word[0] = 0;
   __syncthreads();
+  const long long again = clock64();
   const bool done = mbar_wait(b, 0, abort_word, 0, poll_limit);
-  const bool all = __syncthreads_and(handed && !came && noted && !done && abort_word[0]);
+  const bool outlasted = decision_clocks >= clock64() - again;
+  const bool all = __syncthreads_and(handed && !came && noted && !done && abort_word[0] && outlasted);
   if (threadIdx.x == 0 && all) atomicOr(status, TSD_STATUS_TIMEOUT);
 }
 

@@ -258,7 +258,8 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable()
 
 @pytest.mark.parametrize("poll_limit", [1, 255, 256, 257, 4096])
 def test_every_bounded_wait_gives_up_at_its_limit(poll_limit):
-    # the limit either side of the polls at which a wait also looks for another one's time-out
+    # the limit either side of the polls at which a wait also looks for another one's time-out; the self-test reports nothing if the wait
+    # for a decision gave up before one on a barrier would have, or if two warps could not hand decisions to each other
     status = torch.zeros(1, dtype=torch.int32, device=DEV)
     B.tsd_selftest_bounded_wait(status, poll_limit)
     assert B.tsd_check_status(status) == B.TSD_ERR_TIMEOUT
